@@ -151,12 +151,22 @@ def _ptr(t: Optional[torch.Tensor]):
         raise ValueError("the SPA library takes device tensors only")
     if not t.is_contiguous():
         raise ValueError("tensors must be contiguous")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# handle of the current stream as an integer: torch.cuda.current_stream() builds a Stream object first (3 us a call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def current_stream_handle() -> int:
+    if _raw_stream is None or _device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    return stream.cuda_stream if stream is not None else current_stream_handle()
 
 
 def _check(rc: int, where: str):
@@ -351,10 +361,7 @@ def block_buffers(**fields) -> SpaBlockBuffers:
     """A spa_block_buffers filled from tensors (device pointers), scalars and None (NULL)."""
     b = SpaBlockBuffers()
     for name, v in fields.items():
-        if isinstance(v, torch.Tensor):
-            p = _ptr(v)
-            v = p.value if p is not None else None
-        setattr(b, name, v)
+        setattr(b, name, _ptr(v) if isinstance(v, torch.Tensor) else v)
     return b
 
 

@@ -7,6 +7,7 @@ computes or sequences.  Nothing synchronises; N_p stays on the device.
 """
 from __future__ import annotations
 
+import ctypes
 from typing import Optional
 
 import torch
@@ -23,7 +24,7 @@ class SpaBlock:
                  fused: Optional[bool] = None, one_pass: bool = False):
         if not torch.cuda.is_available():
             raise RuntimeError("SpaBlock needs a CUDA device; there is no CPU path")
-        L.lib()
+        self._lib = L.lib()
         self.B, self.N, self.C, self.H = B, N, C, H
         self.tdtype = torch.float32 if dtype == "f32" else torch.bfloat16
         cap = capacity if capacity is not None else max(B * N, 1)
@@ -37,6 +38,7 @@ class SpaBlock:
             flags |= L.SPA_FLAG_UNFUSED
         self.p = L.make_params(B, N, C, H, dtype, cap, flags, tau)
         self.cap = cap
+        self._inplace = bool(flags & L.SPA_FLAG_INPLACE)
         dev = torch.device(device)
         T = self.tdtype
         e = lambda *s, dt=T: torch.empty(*s, dtype=dt, device=dev)
@@ -73,10 +75,11 @@ class SpaBlock:
             self.dW_o = e(C, C, dt=torch.float32)
             self.db_o = e(C, dt=torch.float32)
         self._saved = None            # (W_qkv, W_o) of the last forward()
-        self._seg = (self.cu, B)      # attention segments: the images, unless forward() is given others
         self._keep = None             # tensors of the last call that the enqueued work still reads
-        self._container_len = 0       # > 0: the library builds the container cuts itself (forward(container_len=L))
+        self._n_max = {}              # container length -> upper bound of the number of containers
         self.container_seg = None
+        self._bufs = self._fixed_buffers(backward)  # segments: the images, unless forward() is given others
+        self._args = (ctypes.byref(self.p), ctypes.byref(self._bufs))
 
     def __del__(self):
         try:
@@ -87,13 +90,15 @@ class SpaBlock:
         except Exception:
             pass
 
-    def _buffers(self, **extra):
-        seg, n_seg = self._seg
+    def _fixed_buffers(self, backward):
+        """The block's own buffers as the library's struct, filled once: a call sets only the tensors it is given.
+        (Filling all of it anew cost 10 us of the 38 us a forward call of one image spent on the host.)"""
         f = dict(scores=self.scores, mask=self.mask, cu_seqlens=self.cu, idx=self.idx, inv=self.inv, x_packed=self.xp,
                  qkv=self.qkv, attn_out=self.ao, lse=self.lse, z=self.z, workspace=self.workspace, d_status=self.status,
-                 pack_state=self.pack_state, container_len=self._container_len,
-                 seg_offsets=None if seg is self.cu else seg, n_seg=n_seg)
-        f.update(extra)
+                 pack_state=self.pack_state)
+        if backward:
+            f.update(dz=self.dz, d_attn_out=self.dao, dqkv=self.dqkv, dx_packed=self.dxp, dW_qkv=self.dW_qkv,
+                     db_qkv=self.db_qkv, dW_o=self.dW_o, db_o=self.db_o, workspace_side=self.workspace_side)
         return L.block_buffers(**f)
 
     # ------------------------------------------------------------------ forward
@@ -103,36 +108,41 @@ class SpaBlock:
         feature map); `seg_offsets` (int32, ascending, ending at N_p): attention segments other than the images;
         `container_len` = L > 0: the paper's containers, their cuts built on the device by the library (the segment
         array is owned here).  The backward pass uses the same segments."""
-        inplace = bool(self.p.flags & L.SPA_FLAG_INPLACE)
-        y = x if inplace else (self.y if y is None else y)
-        self._container_len = int(container_len)
+        ptr, b = L._ptr, self._bufs
+        y = x if self._inplace else (self.y if y is None else y)
         if container_len > 0:
-            n_max = L.spa_container_max_segments(self.p, container_len)
+            n_max = self._n_max.get(container_len)
+            if n_max is None:
+                n_max = self._n_max[container_len] = L.spa_container_max_segments(self.p, container_len)
             if self.container_seg is None or self.container_seg.numel() != n_max + 1:
                 self.container_seg = torch.zeros(n_max + 1, dtype=torch.int32, device=self.cu.device)
             seg_offsets = self.container_seg
-        self._seg = (self.cu, self.B) if seg_offsets is None else (seg_offsets, int(seg_offsets.numel()) - 1)
+        b.container_len = int(container_len)
+        if seg_offsets is None:
+            b.seg_offsets, b.n_seg = None, self.B
+        else:
+            b.seg_offsets, b.n_seg = ptr(seg_offsets), int(seg_offsets.numel()) - 1
         self._saved = (W_qkv, W_o)
         self._keep = (x, w_g, W_qkv, b_qkv, W_o, b_o, s_up, order, seg_offsets, y)
-        L.spa_block_fwd(self.p, self._buffers(x=x, w_g=w_g, b_g=float(b_g), s_up=s_up, W_qkv=W_qkv, b_qkv=b_qkv, W_o=W_o,
-                                              b_o=b_o, order=order, y=y))
+        b.x, b.w_g, b.b_g, b.s_up, b.order, b.y = ptr(x), ptr(w_g), float(b_g), ptr(s_up), ptr(order), ptr(y)
+        b.W_qkv, b.b_qkv, b.W_o, b.b_o = ptr(W_qkv), ptr(b_qkv), ptr(W_o), ptr(b_o)
+        L._check(self._lib.spa_block_fwd(*self._args, L.current_stream_handle()), "spa_block_fwd")
         return y
 
     # ------------------------------------------------------------------ backward
-    def _backward_fields(self, dY, dX):
+    def _backward(self, dY, dX, overlap, trainable):
+        b = self._bufs
         W_qkv, W_o = self._saved
-        return dict(W_qkv=W_qkv, W_o=W_o, dY=dY, dz=self.dz, d_attn_out=self.dao, dqkv=self.dqkv, dx_packed=self.dxp,
-                    dX=dX, dW_qkv=self.dW_qkv, db_qkv=self.db_qkv, dW_o=self.dW_o, db_o=self.db_o,
-                    workspace_side=self.workspace_side)
+        b.W_qkv, b.W_o, b.dY, b.dX = L._ptr(W_qkv), L._ptr(W_o), L._ptr(dY), L._ptr(dX)
+        b.overlap, b.trainable = overlap, trainable
+        L._check(self._lib.spa_block_bwd(*self._args, L.current_stream_handle()), "spa_block_bwd")
+        return dX
 
     def backward(self, dY, dX=None, overlap=True):
         """Gradients for the last forward(): returns dX; parameter gradients land in dW_qkv, db_qkv,
         dW_o, db_o (fp32).  No gradient reaches the gate (hard threshold).  With overlap=True the two
         weight-gradient products run on the library's second stream and are joined before the call returns."""
-        dX = self.dX if dX is None else dX
-        L.spa_block_bwd(self.p, self._buffers(overlap=self._overlap if overlap else None,
-                                              **self._backward_fields(dY, dX)))
-        return dX
+        return self._backward(dY, self.dX if dX is None else dX, self._overlap if overlap else None, 0)
 
     def backward_trainable(self, dY, x, w_g, labels=None, alpha: float = 1.0, s_up=None, dX=None):
         """backward() extended by the gradient that reaches the gate (Sec. 3.2 Eq. 4-5, Sec. 3.3 Eq. 10): the
@@ -149,11 +159,12 @@ class SpaBlock:
             self.db_g = torch.empty(1, dtype=torch.float32, device=dev)
             self.loss = torch.zeros(1, dtype=torch.float32, device=dev)
             self.train_ws = torch.empty(max(L.spa_train_workspace_bytes(self.p), 256), dtype=torch.uint8, device=dev)
-        L.spa_block_bwd(self.p, self._buffers(x=x, w_g=w_g, s_up=s_up, trainable=1, labels=labels, alpha=float(alpha),
-                                              ds=self.ds, ds_up=self.ds_up, dw_g=self.dw_g, db_g=self.db_g,
-                                              loss=self.loss, train_workspace=self.train_ws,
-                                              **self._backward_fields(dY, dX)))
-        return dX
+            b = self._bufs
+            b.ds, b.ds_up, b.dw_g, b.db_g = L._ptr(self.ds), L._ptr(self.ds_up), L._ptr(self.dw_g), L._ptr(self.db_g)
+            b.loss, b.train_workspace = L._ptr(self.loss), L._ptr(self.train_ws)
+        b = self._bufs
+        b.x, b.w_g, b.s_up, b.labels, b.alpha = L._ptr(x), L._ptr(w_g), L._ptr(s_up), L._ptr(labels), float(alpha)
+        return self._backward(dY, dX, None, 1)
 
     def read_status(self) -> int:
         """Blocking: the device status word (0 = ok)."""
