@@ -2,305 +2,336 @@
 // tokens attend only to tokens of the same image; the 2L^2C term of Eq. 9).  The path of the fp32
 // workload and the bring-up reference of the tensor-core kernels.
 //
-// Work split: a CTA owns 64 consecutive packed rows and one head, wherever segment boundaries fall;
-// it walks the key range spanned by the segments of its rows in tiles of 64 staged in shared memory
-// as fp32, and each thread masks the keys outside its own row's segment.  A row is owned by
-// kSplit = d/32 adjacent lanes, each holding 32 of the d head dimensions in registers; dot products
-// are completed with one shuffle.  No padding token is ever computed, nothing is atomically
-// accumulated, and every sum runs in a fixed order.
+// Work split: a CTA owns 32 consecutive packed rows and one head, wherever segment boundaries fall, and walks the
+// rows of the other side that the segments of its rows span, in tiles of 64 staged in shared memory as fp32, two
+// tiles in flight.  128 threads form a grid of 8 x 16: a product tile of 32 x 64 is 4 x 4 values per thread (8
+// vector reads of shared memory per 64 multiply-adds), its softmax statistics are shuffles among 16 lanes, and the
+// second product gives a thread 4 rows x D / 16 head dimensions.  Small problems are bound by the length of one CTA's
+// chain: 32-row tiles halve it and double the CTAs.  (235 rows of 3 heads: 7 us forward, 15 us backward,
+// where one thread per row, one key after the other, took 32 and 90; 1 568 rows of 6 heads: 22 us forward, before 75.)  No padding token is ever
+// computed, nothing is atomically accumulated, and every sum runs in a fixed order.
 #include <math_constants.h>
 
+#include "simt_stage.cuh"
 #include "spa_common.cuh"
 
 namespace spa {
 namespace {
 
-constexpr int kRows = 64;   // packed rows per CTA and rows per staged tile
-constexpr int kPart = 32;   // head dimensions held by one thread
+constexpr int kR = 32;          // packed rows per CTA
+constexpr int kT = 64;          // rows of a streamed tile
+constexpr int kThreads = 128;
+constexpr int kTX = 16, kTY = 8;  // thread (ty, tx): rows ty + 8 i (i < 4), streamed rows tx + 16 j (j < 4)
+constexpr int kLdP = kT + 4;    // leading dimension of the probability tiles
+template <int D> constexpr int kLd = D + 4;  // rows 4 banks apart
 
-// Stage rows [row0, row0 + kRows) of one head's slice (column offset col0 of a [*, ld] matrix) as fp32.
-template <typename T, int D>
-__device__ __forceinline__ void stage_rows(float (*dst)[D], const T* __restrict__ src, long long ld, int col0, int row0,
-                                           int row_end, int tid, int nthreads) {
-  constexpr int E = Vec16<T>::kElems;
-  constexpr int CPR = D / E;
-  for (int c = tid; c < kRows * CPR; c += nthreads) {
-    const int r = c / CPR, cc = c % CPR;
-    float f[E];
-    if (row0 + r < row_end) {
-      const uint4 v = *reinterpret_cast<const uint4*>(src + (long long)(row0 + r) * ld + col0 + cc * E);
-      Vec16<T>::to_float(v, f);
-    } else {
+// Rows [row0, row0 + kRows) of one head's slice (column col0 of a [*, ld] matrix); rows from row_end on become zero.
+template <typename T, int D, int kRows>
+__device__ __forceinline__ void stage_rows(float* dst, const T* __restrict__ src, long long ld, int col0, int row0, int row_end,
+                                           int tid) {
+  constexpr int E = Vec16<T>::kElems, kPer = D / E;
 #pragma unroll
-      for (int e = 0; e < E; ++e) f[e] = 0.f;
-    }
-#pragma unroll
-    for (int e = 0; e < E; ++e) dst[r][cc * E + e] = f[e];
+  for (int c = tid; c < kRows * kPer; c += kThreads) {
+    const int r = c / kPer, cc = (c % kPer) * E;
+    stage16<T>(dst + r * kLd<D> + cc, src + (long long)(row0 + r) * ld + col0 + cc, row0 + r < row_end, src);
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void load_part(float* dst, const T* __restrict__ src) {  // kPart contiguous elements
-  constexpr int E = Vec16<T>::kElems;
+// s[i][j] += a_row(ty + 8 i) . b_row(tx + 16 j) over D
+template <int D>
+__device__ __forceinline__ void dots(float (*s)[4], const float* a, const float* b, int ty, int tx) {
 #pragma unroll
-  for (int c = 0; c < kPart / E; ++c) Vec16<T>::to_float(*reinterpret_cast<const uint4*>(src + c * E), dst + c * E);
+  for (int e = 0; e < D; e += 4) {
+    float4 av[4], bv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const float4*>(a + (ty + kTY * i) * kLd<D> + e);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(b + (tx + kTX * j) * kLd<D> + e);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        s[i][j] = fmaf(av[i].x, bv[j].x, s[i][j]);
+        s[i][j] = fmaf(av[i].y, bv[j].y, s[i][j]);
+        s[i][j] = fmaf(av[i].z, bv[j].z, s[i][j]);
+        s[i][j] = fmaf(av[i].w, bv[j].w, s[i][j]);
+      }
+  }
 }
 
-template <typename T>
-__device__ __forceinline__ void store_part(T* dst, const float* src) {
-  constexpr int E = Vec16<T>::kElems;
+// o[i][d] += sum over the tile's rows k < n of p[ty + 8 i][k] * v[k][tx * (D / 16) + d]
+template <int D>
+__device__ __forceinline__ void weighted(float (*o)[D / kTX], const float* p, const float* v, int n, int ty, int tx) {
+  constexpr int W = D / kTX;  // 2 or 4
+  for (int k = 0; k < n; k += 4) {  // p is zero from row n on
+    float4 pv[4];
 #pragma unroll
-  for (int c = 0; c < kPart / E; ++c) *reinterpret_cast<uint4*>(dst + c * E) = Vec16<T>::from_float(src + c * E);
+    for (int i = 0; i < 4; ++i) pv[i] = *reinterpret_cast<const float4*>(p + (ty + kTY * i) * kLdP + k);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      float w[W];
+      const float* src = v + (k + u) * kLd<D> + tx * W;
+      if (W == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(src);
+        w[0] = t.x; w[1] = t.y; w[W - 2] = t.z; w[W - 1] = t.w;
+      } else {
+        const float2 t = *reinterpret_cast<const float2*>(src);
+        w[0] = t.x; w[1] = t.y;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float pi = u == 0 ? pv[i].x : u == 1 ? pv[i].y : u == 2 ? pv[i].z : pv[i].w;
+#pragma unroll
+        for (int d = 0; d < W; ++d) o[i][d] = fmaf(pi, w[d], o[i][d]);
+      }
+    }
+  }
 }
 
-template <int kSplit>
-__device__ __forceinline__ float split_sum(float v) {
-  if (kSplit >= 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
-  if (kSplit >= 4) v += __shfl_xor_sync(0xffffffffu, v, 2);
+// W consecutive values of one row
+template <typename T, int W> __device__ __forceinline__ void store_row(T* dst, const float* v) {
+#pragma unroll
+  for (int d = 0; d < W; ++d) dst[d] = from_f32<T>(v[d]);
+}
+template <> __device__ __forceinline__ void store_row<float, 4>(float* dst, const float* v) {
+  *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <> __device__ __forceinline__ void store_row<float, 2>(float* dst, const float* v) {
+  *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
+}
+
+__device__ __forceinline__ float max16(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float sum16(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-__device__ __forceinline__ float dot_part(const float* a, const float* __restrict__ b_smem) {
-  float s = 0.f;
-#pragma unroll
-  for (int e = 0; e < kPart; e += 4) {
-    const float4 b = *reinterpret_cast<const float4*>(b_smem + e);
-    s = fmaf(a[e], b.x, s); s = fmaf(a[e + 1], b.y, s); s = fmaf(a[e + 2], b.z, s); s = fmaf(a[e + 3], b.w, s);
-  }
-  return s;
-}
-
-__device__ __forceinline__ void axpy_part(float* acc, float w, const float* __restrict__ b_smem) {
-#pragma unroll
-  for (int e = 0; e < kPart; e += 4) {
-    const float4 b = *reinterpret_cast<const float4*>(b_smem + e);
-    acc[e] = fmaf(w, b.x, acc[e]); acc[e + 1] = fmaf(w, b.y, acc[e + 1]);
-    acc[e + 2] = fmaf(w, b.z, acc[e + 2]); acc[e + 3] = fmaf(w, b.w, acc[e + 3]);
-  }
-}
-
-// CTA-wide range of "other side" rows: from the segment start of the first row to the segment end
-// of the last valid row of this CTA.
-__device__ __forceinline__ void cta_range(const RowSeg& mine, int i, int i0, int Np, bool leader, int* range_smem) {
-  const int last = (i0 + kRows - 1 < Np - 1) ? i0 + kRows - 1 : Np - 1;
-  if (leader && i == i0) range_smem[0] = mine.lo;
-  if (leader && i == last) range_smem[1] = mine.hi;
+// Segments of the CTA's 32 rows in seg_s[32] (threads 0-31 search one each); returns the range they span together.
+__device__ __forceinline__ RowSeg tile_segments(RowSeg* seg_s, const int32_t* __restrict__ seg, int n_seg, int Np, int i0,
+                                                int tid) {
+  if (tid < kR) seg_s[tid] = row_segment(seg, n_seg, Np, i0 + tid);
   __syncthreads();
+  const int last = i0 + kR - 1 < Np - 1 ? kR - 1 : Np - 1 - i0;
+  return RowSeg{seg_s[0].lo, seg_s[last].hi};
 }
 
 // ------------------------------------------------------------------------------------ forward
+template <int D> constexpr int kFwdFloats = (kR + 4 * kT) * kLd<D> + kR * kLdP;  // Q, two stages of K and V, P
+
 template <typename T, int D>
-__global__ void __launch_bounds__(kRows * (D / kPart))
+__global__ void __launch_bounds__(kThreads)
 attn_fwd_simt_kernel(const T* __restrict__ qkv, const int32_t* __restrict__ seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ ao, float* __restrict__ lse) {
   pdl_entry();
-  constexpr int kSplit = D / kPart;
-  constexpr int kThreads = kRows * kSplit;
-  __shared__ __align__(16) float Ks[kRows][D];
-  __shared__ __align__(16) float Vs[kRows][D];
-  __shared__ int range[2];
+  constexpr int W = D / kTX;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ RowSeg seg_s[kR];
+  float* Qs = sm;
+  float* KV = sm + kR * kLd<D>;              // stage s: K at s * 2 tiles, V behind it
+  float* Ps = KV + 4 * kT * kLd<D>;
+  constexpr int kTile = kT * kLd<D>;
   const int Np = packed_rows(seg, n_seg, capacity);
-  const int i0 = blockIdx.x * kRows;
+  const int i0 = blockIdx.x * kR;
   if (i0 >= Np) return;
-  const int tid = threadIdx.x, r = tid / kSplit, part = tid % kSplit, h = blockIdx.y;
-  const int i = i0 + r;
+  const int tid = threadIdx.x, tx = tid % kTX, ty = tid / kTX, h = blockIdx.y;
   const long long ld = 3LL * C;
-  const RowSeg mine = row_segment(seg, n_seg, Np, i);
-  cta_range(mine, i, i0, Np, part == 0, range);
-  const int kv_lo = range[0], kv_hi = range[1];
+  stage_rows<T, D, kR>(Qs, qkv, ld, h * D, i0, Np, tid);
+  const RowSeg all = tile_segments(seg_s, seg, n_seg, Np, i0, tid);
+  auto stage = [&](int t) {
+    const int kv0 = all.lo + t * kT;
+    float* dst = KV + (t & 1) * 2 * kTile;
+    stage_rows<T, D, kT>(dst, qkv, ld, C + h * D, kv0, all.hi, tid);
+    stage_rows<T, D, kT>(dst + kTile, qkv, ld, 2 * C + h * D, kv0, all.hi, tid);
+    cp_async_commit();
+  };
+  const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
+  stage(0);
 
-  float q[kPart], o[kPart];
+  float o[4][W] = {}, m[4], l[4] = {};
+  RowSeg mine[4];
 #pragma unroll
-  for (int e = 0; e < kPart; ++e) { q[e] = 0.f; o[e] = 0.f; }
-  if (i < Np) {
-    load_part<T>(q, qkv + (long long)i * ld + h * D + part * kPart);
+  for (int i = 0; i < 4; ++i) { m[i] = -CUDART_INF_F; mine[i] = seg_s[ty + kTY * i]; }
+  for (int t = 0; t < n_tiles; ++t) {
+    if (t + 1 < n_tiles) { stage(t + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+    __syncthreads();
+    const int kv0 = all.lo + t * kT;
+    const float* Ks = KV + (t & 1) * 2 * kTile;
+    float s[4][4] = {};
+    dots<D>(s, Qs, Ks, ty, tx);
 #pragma unroll
-    for (int e = 0; e < kPart; ++e) q[e] *= scale;
-  }
-  float m = -CUDART_INF_F, l = 0.f;
-
-  for (int kv0 = kv_lo; kv0 < kv_hi; kv0 += kRows) {
-    __syncthreads();
-    stage_rows<T, D>(Ks, qkv, ld, C + h * D, kv0, kv_hi, tid, kThreads);
-    stage_rows<T, D>(Vs, qkv, ld, 2 * C + h * D, kv0, kv_hi, tid, kThreads);
-    __syncthreads();
-    const int jmax = kv_hi - kv0 < kRows ? kv_hi - kv0 : kRows;
-    for (int j0 = 0; j0 < jmax; j0 += 8) {
-      float s[8];
+    for (int i = 0; i < 4; ++i) {
       float cm = -CUDART_INF_F;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = j0 + u;  // rows >= jmax are zero-filled and masked below
-        float v = split_sum<kSplit>(dot_part(q, &Ks[j][part * kPart]));
-        const int ja = kv0 + j;
-        s[u] = (j < jmax && ja >= mine.lo && ja < mine.hi) ? v : -CUDART_INF_F;
-        cm = fmaxf(cm, s[u]);
+      for (int j = 0; j < 4; ++j) {
+        const int ja = kv0 + tx + kTX * j;
+        s[i][j] = (ja >= mine[i].lo && ja < mine[i].hi) ? s[i][j] * scale : -CUDART_INF_F;
+        cm = fmaxf(cm, s[i][j]);
       }
-      if (cm > -CUDART_INF_F) {
-        const float m_new = fmaxf(m, cm);
-        const float alpha = expf(m - m_new);
-        l *= alpha;
+      const float m_new = fmaxf(m[i], max16(cm));
+      const float m_use = m_new == -CUDART_INF_F ? 0.f : m_new;  // no key of this row so far
+      const float alpha = expf(m[i] - m_use);
+      float rs = 0.f;
 #pragma unroll
-        for (int e = 0; e < kPart; ++e) o[e] *= alpha;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const float pj = expf(s[u] - m_new);
-          l += pj;
-          axpy_part(o, pj, &Vs[j0 + u][part * kPart]);
-        }
-        m = m_new;
+      for (int j = 0; j < 4; ++j) {
+        const float p = expf(s[i][j] - m_use);
+        rs += p;
+        Ps[(ty + kTY * i) * kLdP + tx + kTX * j] = p;
       }
+      l[i] = l[i] * alpha + sum16(rs);
+#pragma unroll
+      for (int d = 0; d < W; ++d) o[i][d] *= alpha;
+      m[i] = m_new;
     }
+    __syncwarp();  // the rows of P that this warp reads are the ones its own lanes wrote
+    const int n = all.hi - kv0 < kT ? all.hi - kv0 : kT;
+    weighted<D>(o, Ps, Ks + kTile, n, ty, tx);
+    __syncthreads();  // the stage is free for the tile after next
   }
-  if (i < Np) {
-    const float inv_l = 1.f / l;
 #pragma unroll
-    for (int e = 0; e < kPart; ++e) o[e] *= inv_l;
-    store_part<T>(ao + (long long)i * C + h * D + part * kPart, o);
-    if (part == 0) lse[(long long)h * capacity + i] = m + logf(l);
+  for (int i = 0; i < 4; ++i) {
+    const int row = i0 + ty + kTY * i;
+    if (row >= Np) continue;
+    const float inv_l = 1.f / l[i];
+#pragma unroll
+    for (int d = 0; d < W; ++d) o[i][d] *= inv_l;
+    store_row<T, W>(ao + (long long)row * C + h * D + tx * W, o[i]);
+    if (tx == 0) lse[(long long)h * capacity + row] = m[i] + logf(l[i]);
   }
 }
 
-// ------------------------------------------------------------------------------------ backward, dQ
+// ------------------------------------------------------------------------------------ backward
+// One launch for both passes, which need nothing of each other (D_i = dO_i . O_i is taken by either from the rows it
+// holds), so that they share the GPU: blockIdx.z = 0: own rows are queries, streamed rows keys,
+//   S = Q K^T, dP = dO V^T, dS = P (dP - D), dQ += dS K;
+// blockIdx.z = 1: own rows are keys, streamed rows queries, everything transposed: dV += P^T dO, dK += dS^T Q.
+template <int D> constexpr int kBwdFloats = (2 * kR + 4 * kT) * kLd<D> + 2 * kR * kLdP + 4 * kT;
+
 template <typename T, int D>
-__global__ void __launch_bounds__(kRows * (D / kPart))
-attn_bwd_dq_simt_kernel(const T* __restrict__ qkv, const T* __restrict__ ao, const float* __restrict__ lse,
-                        const T* __restrict__ dao, const int32_t* __restrict__ seg, int n_seg, int capacity, int C,
-                        float scale, T* __restrict__ dqkv) {
+__global__ void __launch_bounds__(kThreads)
+attn_bwd_simt_kernel(const T* __restrict__ qkv, const T* __restrict__ ao, const float* __restrict__ lse,
+                     const T* __restrict__ dao, const int32_t* __restrict__ seg, int n_seg, int capacity, int C,
+                     float scale, T* __restrict__ dqkv) {
   pdl_entry();
-  constexpr int kSplit = D / kPart;
-  constexpr int kThreads = kRows * kSplit;
-  __shared__ __align__(16) float Ks[kRows][D];
-  __shared__ __align__(16) float Vs[kRows][D];
-  __shared__ int range[2];
+  constexpr int W = D / kTX, E = Vec16<T>::kElems;
+  constexpr int kTile = kT * kLd<D>;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ RowSeg seg_s[kR];
+  float* A1 = sm;                       // Q | K of the own rows
+  float* A2 = A1 + kR * kLd<D>;         // dO | V
+  float* Y = A2 + kR * kLd<D>;          // stage s: K | Q at s * 2 tiles, V | dO behind it
+  float* Ps = Y + 4 * kTile;            // P^T (second pass)
+  float* Ds = Ps + kR * kLdP;           // dS | dS^T
+  float* st = Ds + kR * kLdP;           // second pass, stage s: lse_i at s * 2 * kT, D_i behind it
+  const bool dq = blockIdx.z == 0;
   const int Np = packed_rows(seg, n_seg, capacity);
-  const int i0 = blockIdx.x * kRows;
+  const int i0 = blockIdx.x * kR;
   if (i0 >= Np) return;
-  const int tid = threadIdx.x, r = tid / kSplit, part = tid % kSplit, h = blockIdx.y;
-  const int i = i0 + r;
+  const int tid = threadIdx.x, tx = tid % kTX, ty = tid / kTX, h = blockIdx.y;
   const long long ld = 3LL * C;
-  const RowSeg mine = row_segment(seg, n_seg, Np, i);
-  cta_range(mine, i, i0, Np, part == 0, range);
-  const int kv_lo = range[0], kv_hi = range[1];
-
-  float q[kPart], dO[kPart], dq[kPart];
-  float Di = 0.f, lse_i = 0.f;
+  // D of packed row i: eight or sixteen 16-byte loads, all in flight together
+  auto row_D = [&](int i) {
+    float s = 0.f;
+    const T* po = ao + (long long)i * C + h * D;
+    const T* pg = dao + (long long)i * C + h * D;
 #pragma unroll
-  for (int e = 0; e < kPart; ++e) { q[e] = 0.f; dO[e] = 0.f; dq[e] = 0.f; }
-  if (i < Np) {
-    load_part<T>(q, qkv + (long long)i * ld + h * D + part * kPart);
-    load_part<T>(dO, dao + (long long)i * C + h * D + part * kPart);
-    float ov[kPart];
-    load_part<T>(ov, ao + (long long)i * C + h * D + part * kPart);
+    for (int c = 0; c < D / E; ++c) {
+      float a[E], b[E];
+      Vec16<T>::to_float(*reinterpret_cast<const uint4*>(po + c * E), a);
+      Vec16<T>::to_float(*reinterpret_cast<const uint4*>(pg + c * E), b);
 #pragma unroll
-    for (int e = 0; e < kPart; ++e) Di = fmaf(dO[e], ov[e], Di);
-    lse_i = lse[(long long)h * capacity + i];
-  }
-  Di = split_sum<kSplit>(Di);
+      for (int e = 0; e < E; ++e) s = fmaf(a[e], b[e], s);
+    }
+    return s;
+  };
+  stage_rows<T, D, kR>(A1, qkv, ld, (dq ? 0 : C) + h * D, i0, Np, tid);
+  if (dq) stage_rows<T, D, kR>(A2, dao, (long long)C, h * D, i0, Np, tid);
+  else stage_rows<T, D, kR>(A2, qkv, ld, 2 * C + h * D, i0, Np, tid);
+  const RowSeg all = tile_segments(seg_s, seg, n_seg, Np, i0, tid);
+  auto stage = [&](int t) {
+    const int y0 = all.lo + t * kT;
+    float* dst = Y + (t & 1) * 2 * kTile;
+    stage_rows<T, D, kT>(dst, qkv, ld, (dq ? C : 0) + h * D, y0, all.hi, tid);
+    if (dq) stage_rows<T, D, kT>(dst + kTile, qkv, ld, 2 * C + h * D, y0, all.hi, tid);
+    else stage_rows<T, D, kT>(dst + kTile, dao, (long long)C, h * D, y0, all.hi, tid);
+    cp_async_commit();
+    if (!dq && tid < kT) {
+      float* s2 = st + (t & 1) * 2 * kT;
+      const bool in = y0 + tid < all.hi;
+      s2[tid] = in ? lse[(long long)h * capacity + y0 + tid] : 0.f;
+      s2[kT + tid] = in ? row_D(y0 + tid) : 0.f;
+    }
+  };
+  const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
+  stage(0);
 
-  for (int kv0 = kv_lo; kv0 < kv_hi; kv0 += kRows) {
-    __syncthreads();
-    stage_rows<T, D>(Ks, qkv, ld, C + h * D, kv0, kv_hi, tid, kThreads);
-    stage_rows<T, D>(Vs, qkv, ld, 2 * C + h * D, kv0, kv_hi, tid, kThreads);
-    __syncthreads();
-    const int jmax = kv_hi - kv0 < kRows ? kv_hi - kv0 : kRows;
-    for (int j = 0; j < jmax; ++j) {
-      const float s = scale * split_sum<kSplit>(dot_part(q, &Ks[j][part * kPart]));
-      const float dp = split_sum<kSplit>(dot_part(dO, &Vs[j][part * kPart]));
-      const int ja = kv0 + j;
-      const bool ok = ja >= mine.lo && ja < mine.hi;
-      const float pj = ok ? expf(s - lse_i) : 0.f;
-      axpy_part(dq, pj * (dp - Di), &Ks[j][part * kPart]);
+  RowSeg mine[4];
+  float my_lse[4] = {}, my_D[4] = {};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) mine[i] = seg_s[ty + kTY * i];
+  if (dq) {
+    // lane tx < 4 fetches row ty + 8 tx, the others take it from there
+    const int r = i0 + ty + kTY * (tx & 3);
+    const float dv = r < Np ? row_D(r) : 0.f, lv = r < Np ? lse[(long long)h * capacity + r] : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      my_D[i] = __shfl_sync(0xffffffffu, dv, i, kTX);
+      my_lse[i] = __shfl_sync(0xffffffffu, lv, i, kTX);
     }
   }
-  if (i < Np) {
-#pragma unroll
-    for (int e = 0; e < kPart; ++e) dq[e] *= scale;
-    store_part<T>(dqkv + (long long)i * ld + h * D + part * kPart, dq);
-  }
-}
-
-// ------------------------------------------------------------------------------------ backward, dK and dV
-template <typename T, int D>
-__global__ void __launch_bounds__(kRows * (D / kPart))
-attn_bwd_dkv_simt_kernel(const T* __restrict__ qkv, const T* __restrict__ ao, const float* __restrict__ lse,
-                         const T* __restrict__ dao, const int32_t* __restrict__ seg, int n_seg, int capacity, int C,
-                         float scale, T* __restrict__ dqkv) {
-  pdl_entry();
-  constexpr int kSplit = D / kPart;
-  constexpr int kThreads = kRows * kSplit;
-  constexpr int E = Vec16<T>::kElems;
-  __shared__ __align__(16) float Qs[kRows][D];
-  __shared__ __align__(16) float dOs[kRows][D];
-  __shared__ float lse_s[kRows], D_s[kRows];
-  __shared__ int range[2];
-  const int Np = packed_rows(seg, n_seg, capacity);
-  const int j0 = blockIdx.x * kRows;
-  if (j0 >= Np) return;
-  const int tid = threadIdx.x, r = tid / kSplit, part = tid % kSplit, h = blockIdx.y;
-  const int j = j0 + r;
-  const long long ld = 3LL * C;
-  const RowSeg mine = row_segment(seg, n_seg, Np, j);
-  cta_range(mine, j, j0, Np, part == 0, range);
-  const int q_lo = range[0], q_hi = range[1];
-
-  float k[kPart], v[kPart], dk[kPart], dv[kPart];
-#pragma unroll
-  for (int e = 0; e < kPart; ++e) { k[e] = 0.f; v[e] = 0.f; dk[e] = 0.f; dv[e] = 0.f; }
-  if (j < Np) {
-    load_part<T>(k, qkv + (long long)j * ld + C + h * D + part * kPart);
-    load_part<T>(v, qkv + (long long)j * ld + 2 * C + h * D + part * kPart);
-  }
-
-  for (int q0 = q_lo; q0 < q_hi; q0 += kRows) {
+  float acc1[4][W] = {}, acc2[4][W] = {};  // dQ | dK and dV
+  for (int t = 0; t < n_tiles; ++t) {
+    if (t + 1 < n_tiles) { stage(t + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
     __syncthreads();
-    stage_rows<T, D>(Qs, qkv, ld, h * D, q0, q_hi, tid, kThreads);
-    stage_rows<T, D>(dOs, dao, (long long)C, h * D, q0, q_hi, tid, kThreads);
-    if (tid < kRows) {  // D_i = dO_i . O_i and lse_i of the staged query rows
-      const int i = q0 + tid;
-      float Di = 0.f, li = 0.f;
-      if (i < q_hi) {
-        const T* orow = ao + (long long)i * C + h * D;
-        const T* grow = dao + (long long)i * C + h * D;
+    const int y0 = all.lo + t * kT;
+    const float* Y1 = Y + (t & 1) * 2 * kTile;
+    const float* Y2 = Y1 + kTile;
+    const float* s2 = st + (t & 1) * 2 * kT;
+    float s[4][4] = {}, dp[4][4] = {};
+    dots<D>(s, A1, Y1, ty, tx);
+    dots<D>(dp, A2, Y2, ty, tx);
 #pragma unroll
-        for (int c = 0; c < D / E; ++c) {
-          float a[E], b[E];
-          Vec16<T>::to_float(*reinterpret_cast<const uint4*>(orow + c * E), a);
-          Vec16<T>::to_float(*reinterpret_cast<const uint4*>(grow + c * E), b);
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int e = 0; e < E; ++e) Di = fmaf(a[e], b[e], Di);
-        }
-        li = lse[(long long)h * capacity + i];
+      for (int j = 0; j < 4; ++j) {
+        const int c = tx + kTX * j, ya = y0 + c;
+        const float l = dq ? my_lse[i] : s2[c], Dv = dq ? my_D[i] : s2[kT + c];
+        const float p = (ya >= mine[i].lo && ya < mine[i].hi) ? expf(s[i][j] * scale - l) : 0.f;
+        if (!dq) Ps[(ty + kTY * i) * kLdP + c] = p;
+        Ds[(ty + kTY * i) * kLdP + c] = p * (dp[i][j] - Dv);
       }
-      D_s[tid] = Di;
-      lse_s[tid] = li;
-    }
-    __syncthreads();
-    const int imax = q_hi - q0 < kRows ? q_hi - q0 : kRows;
-    for (int ii = 0; ii < imax; ++ii) {
-      const float s = scale * split_sum<kSplit>(dot_part(k, &Qs[ii][part * kPart]));
-      const float dp = split_sum<kSplit>(dot_part(v, &dOs[ii][part * kPart]));
-      const int ia = q0 + ii;
-      const bool ok = ia >= mine.lo && ia < mine.hi;
-      const float pij = ok ? expf(s - lse_s[ii]) : 0.f;
-      axpy_part(dv, pij, &dOs[ii][part * kPart]);
-      axpy_part(dk, pij * (dp - D_s[ii]), &Qs[ii][part * kPart]);
-    }
+    __syncwarp();  // the rows of P and dS that this warp reads are the ones its own lanes wrote
+    const int n = all.hi - y0 < kT ? all.hi - y0 : kT;
+    weighted<D>(acc1, Ds, Y1, n, ty, tx);
+    if (!dq) weighted<D>(acc2, Ps, Y2, n, ty, tx);
+    __syncthreads();  // the stage is free for the tile after next
   }
-  if (j < Np) {
 #pragma unroll
-    for (int e = 0; e < kPart; ++e) dk[e] *= scale;
-    store_part<T>(dqkv + (long long)j * ld + C + h * D + part * kPart, dk);
-    store_part<T>(dqkv + (long long)j * ld + 2 * C + h * D + part * kPart, dv);
+  for (int i = 0; i < 4; ++i) {
+    const int row = i0 + ty + kTY * i;
+    if (row >= Np) continue;
+    T* dst = dqkv + (long long)row * ld + h * D + tx * W;
+#pragma unroll
+    for (int d = 0; d < W; ++d) acc1[i][d] *= scale;
+    store_row<T, W>(dst + (dq ? 0 : C), acc1[i]);
+    if (!dq) store_row<T, W>(dst + 2 * C, acc2[i]);
   }
 }
 
 template <typename T, int D>
 int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao, float* lse,
                cudaStream_t st) {
-  dim3 grid((p.capacity + kRows - 1) / kRows, p.H);
-  launch_pdl(attn_fwd_simt_kernel<T, D>, grid, kRows * (D / kPart), 0, st, (const T*)qkv, seg, n_seg, p.capacity, p.C,
-                                                                  softmax_scale_of(p), (T*)ao, lse);
+  auto kern = attn_fwd_simt_kernel<T, D>;
+  constexpr int kSmem = kFwdFloats<D> * (int)sizeof(float);
+  static DeviceOnce attr;
+  cudaError_t e = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem); });
+  if (e != cudaSuccess) { set_cuda_error(e, "attn_fwd_simt_kernel"); return SPA_ERR_CUDA; }
+  launch_pdl(kern, dim3((p.capacity + kR - 1) / kR, p.H), kThreads, kSmem, st, (const T*)qkv, seg, n_seg, p.capacity, p.C,
+             softmax_scale_of(p), (T*)ao, lse);
   SPA_CUDA_CHECK_LAUNCH("attn_fwd_simt_kernel");
   return SPA_OK;
 }
@@ -308,15 +339,14 @@ int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_s
 template <typename T, int D>
 int bwd_launch(const spa_params& p, const void* qkv, const void* ao, const float* lse, const void* dao,
                const int32_t* seg, int n_seg, void* dqkv, cudaStream_t st) {
-  dim3 grid((p.capacity + kRows - 1) / kRows, p.H);
-  const float scale = softmax_scale_of(p);
-  launch_pdl(attn_bwd_dq_simt_kernel<T, D>, grid, kRows * (D / kPart), 0, st, (const T*)qkv, (const T*)ao, lse, (const T*)dao,
-                                                                     seg, n_seg, p.capacity, p.C, scale, (T*)dqkv);
-  SPA_CUDA_CHECK_LAUNCH("attn_bwd_dq_simt_kernel");
-  launch_pdl(attn_bwd_dkv_simt_kernel<T, D>, grid, kRows * (D / kPart), 0, st, (const T*)qkv, (const T*)ao, lse,
-                                                                      (const T*)dao, seg, n_seg, p.capacity, p.C,
-                                                                      scale, (T*)dqkv);
-  SPA_CUDA_CHECK_LAUNCH("attn_bwd_dkv_simt_kernel");
+  auto kern = attn_bwd_simt_kernel<T, D>;
+  constexpr int kSmem = kBwdFloats<D> * (int)sizeof(float);
+  static DeviceOnce attr;
+  cudaError_t e = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem); });
+  if (e != cudaSuccess) { set_cuda_error(e, "attn_bwd_simt_kernel"); return SPA_ERR_CUDA; }
+  launch_pdl(kern, dim3((p.capacity + kR - 1) / kR, p.H, 2), kThreads, kSmem, st, (const T*)qkv, (const T*)ao, lse,
+             (const T*)dao, seg, n_seg, p.capacity, p.C, softmax_scale_of(p), (T*)dqkv);
+  SPA_CUDA_CHECK_LAUNCH("attn_bwd_simt_kernel");
   return SPA_OK;
 }
 
