@@ -321,14 +321,14 @@ int spa_gelu_bwd(const spa_params* p, const void* dh, const void* u, int32_t n_c
 
 /* ---- The block as one unit (Sec. 3.2: gate -> select and pack -> attention on the packed tokens -> unpack; Eq. 9
  * counts it as one).  spa_block_fwd and spa_block_bwd issue the calls above in order on `stream`; they choose the
- * fused calls where spa_fused_scatter_supported() allows (unless SPA_FLAG_UNFUSED), and spa_block_bwd runs the two
+ * products that scatter their rows to the tokens themselves (unless SPA_FLAG_UNFUSED), and spa_block_bwd runs the two
  * weight-gradient products on a second stream beside the attention backward when `overlap` is given.  Nothing
  * synchronises with the host, so both can be recorded into one CUDA graph.
  *
  * All pointers are device memory owned by the caller and sized as in the single calls (packed buffers: `capacity`
  * rows).  Which fields may be NULL:
  *   s_up, order, seg_offsets (NULL: the images are the attention segments), b_qkv, b_o, pack_state;
- *   z, dx_packed            when the fused calls apply (the products write y and dX rows themselves);
+ *   z, dx_packed            unless SPA_FLAG_UNFUSED (or, dx_packed, `trainable`) asks for the separate kernels;
  *   every backward field    for spa_block_fwd;
  *   labels .. train_workspace unless `trainable` is non-zero.
  * The forward pass leaves scores, mask, cu_seqlens, idx, inv, x_packed, qkv, attn_out, lse for the backward pass. */

@@ -28,13 +28,13 @@ class SpaBlock:
         self.B, self.N, self.C, self.H = B, N, C, H
         self.tdtype = torch.float32 if dtype == "f32" else torch.bfloat16
         cap = capacity if capacity is not None else max(B * N, 1)
-        # fused unpack: the projection and the QKV input gradient scatter their rows to the tokens themselves
-        # (tensor-core problems only); None = use it where the library offers it
+        # fused unpack: the projection and the QKV input gradient scatter their rows to the tokens themselves; False =
+        # separate kernels.  `self.fused`: the single calls that do so apply too (tensor-core problems)
         can_fuse = L.spa_fused_scatter_supported(L.make_params(B, N, C, H, dtype, cap, flags, tau))
         if fused and not can_fuse:
             raise ValueError("the fused scatter calls do not apply to this problem (needs bf16 tensor-core sizes)")
         self.fused = can_fuse if fused is None else bool(fused)
-        if not self.fused:
+        if fused is False:
             flags |= L.SPA_FLAG_UNFUSED
         self.p = L.make_params(B, N, C, H, dtype, cap, flags, tau)
         self.cap = cap

@@ -51,6 +51,21 @@ int check_heads(const spa_params* p) {
 // bf16 problems run on the tensor-core kernels unless the caller asks for the fp32-FMA ones
 inline bool use_tc(const spa_params* p) { return p->dtype == SPA_BF16 && !(p->flags & SPA_FLAG_SIMT_ONLY); }
 
+// linear layers that the bf16 tensor-core kernels do not take: fp32 data, or bf16 on the fp32-FMA kernels
+int linear_fwd_other(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out, const int32_t* cu,
+                     void* out, int32_t* d_status, void* stream, const int32_t* row_map = nullptr, bool accumulate = false) {
+  cudaStream_t st = (cudaStream_t)stream;
+  return p.dtype == SPA_F32 ? launch_linear_fwd_f32(p, a, W, bias, n_in, n_out, cu, out, d_status, st, row_map, accumulate)
+                            : launch_linear_fwd_simt(p, a, W, bias, n_in, n_out, cu, out, st, row_map, accumulate);
+}
+int linear_bwd_other(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out, const int32_t* cu,
+                     void* da, float* dW, float* db, int32_t* d_status, void* stream, const int32_t* row_map = nullptr,
+                     bool accumulate = false) {
+  cudaStream_t st = (cudaStream_t)stream;
+  return p.dtype == SPA_F32 ? launch_linear_bwd_f32(p, a, W, dout, n_in, n_out, cu, da, dW, db, d_status, st, row_map, accumulate)
+                            : launch_linear_bwd_simt(p, a, W, dout, n_in, n_out, cu, da, dW, db, st, row_map, accumulate);
+}
+
 #define SPA_REQUIRE(cond, code) do { if (!(cond)) return (code); } while (0)
 #define SPA_PTR(ptr) SPA_REQUIRE((ptr) != nullptr && aligned16(ptr), SPA_ERR_INVALID_ARG)
 #define SPA_OPT_PTR(ptr) SPA_REQUIRE((ptr) == nullptr || aligned16(ptr), SPA_ERR_INVALID_ARG)
@@ -163,7 +178,7 @@ int spa_packed_qkv(const spa_params* p, const void* x_packed, const void* W_qkv,
                               (cudaStream_t)stream);
     if (rc != SPA_ERR_UNSUPPORTED) return rc;  // geometry the TMA path cannot describe: fp32-FMA kernels
   }
-  return launch_linear_fwd_simt(*p, x_packed, W_qkv, b_qkv, p->C, 3 * p->C, cu_seqlens, qkv, (cudaStream_t)stream);
+  return linear_fwd_other(*p, x_packed, W_qkv, b_qkv, p->C, 3 * p->C, cu_seqlens, qkv, d_status, stream);
 }
 
 int spa_packed_proj(const spa_params* p, const void* a, const void* W_o, const void* b_o, const int32_t* cu_seqlens,
@@ -175,7 +190,7 @@ int spa_packed_proj(const spa_params* p, const void* a, const void* W_o, const v
     rc = launch_linear_fwd_tc(*p, a, W_o, b_o, p->C, p->C, cu_seqlens, z, d_status, (cudaStream_t)stream);
     if (rc != SPA_ERR_UNSUPPORTED) return rc;
   }
-  return launch_linear_fwd_simt(*p, a, W_o, b_o, p->C, p->C, cu_seqlens, z, (cudaStream_t)stream);
+  return linear_fwd_other(*p, a, W_o, b_o, p->C, p->C, cu_seqlens, z, d_status, stream);
 }
 
 int spa_packed_attention_fwd(const spa_params* p, const void* qkv, const int32_t* seg_offsets, int32_t n_seg,
@@ -285,7 +300,7 @@ int spa_packed_linear_bwd(const spa_params* p, const void* a, const void* W, con
                               (cudaStream_t)stream);
     if (rc != SPA_ERR_UNSUPPORTED) return rc;
   }
-  return launch_linear_bwd_simt(*p, a, W, dout, n_in, n_out, cu_seqlens, da, dW, db, (cudaStream_t)stream);
+  return linear_bwd_other(*p, a, W, dout, n_in, n_out, cu_seqlens, da, dW, db, d_status, stream);
 }
 
 int spa_fused_scatter_supported(const spa_params* p) {
@@ -380,7 +395,7 @@ int spa_packed_linear(const spa_params* p, const void* a, const void* W, const v
                               accumulate != 0);
     if (rc != SPA_ERR_UNSUPPORTED) return rc;
   }
-  return launch_linear_fwd_simt(*p, a, W, b, n_in, n_out, cu_seqlens, out, (cudaStream_t)stream, accumulate != 0);
+  return linear_fwd_other(*p, a, W, b, n_in, n_out, cu_seqlens, out, d_status, stream, nullptr, accumulate != 0);
 }
 
 int spa_layer_norm(const spa_params* p, const void* x, const void* gamma, const void* beta, float eps, void* y,
@@ -451,8 +466,23 @@ int spa_overlap_destroy(spa_overlap* ov) {
 }
 
 namespace {
-inline bool block_fused(const spa_params* p) {
-  return !(p->flags & SPA_FLAG_UNFUSED) && spa_fused_scatter_supported(p) != 0;
+inline bool block_fused(const spa_params* p) { return !(p->flags & SPA_FLAG_UNFUSED); }
+// The two products that scatter their rows to the tokens: tensor-core problems, else the fp32-FMA kernels.
+int proj_scatter(const spa_params* p, const spa_block_buffers* b, void* y, void* stream) {
+  if (spa_fused_scatter_supported(p))
+    return spa_packed_proj_scatter(p, b->attn_out, b->W_o, b->b_o, b->idx, b->cu_seqlens, y, b->d_status, stream);
+  SPA_PTR(b->attn_out); SPA_PTR(b->W_o); SPA_PTR(b->idx); SPA_PTR(b->cu_seqlens); SPA_PTR(y); SPA_OPT_PTR(b->b_o);
+  return linear_fwd_other(*p, b->attn_out, b->W_o, b->b_o, p->C, p->C, b->cu_seqlens, y, b->d_status, stream, b->idx,
+                          (p->flags & SPA_FLAG_RESIDUAL) != 0);
+}
+int qkv_bwd_scatter(const spa_params* p, const spa_block_buffers* b, float* dW, float* db, void* ws, void* stream) {
+  if (spa_fused_scatter_supported(p))
+    return spa_packed_linear_bwd_scatter(p, b->x_packed, b->W_qkv, b->dqkv, p->C, 3 * p->C, b->idx, b->cu_seqlens, b->dX, dW, db,
+                                         ws, b->d_status, stream);
+  SPA_PTR(b->dqkv); SPA_PTR(b->W_qkv); SPA_PTR(b->x_packed); SPA_PTR(b->idx); SPA_PTR(b->cu_seqlens); SPA_PTR(b->dX);
+  SPA_OPT_PTR(dW); SPA_OPT_PTR(db);
+  return linear_bwd_other(*p, b->x_packed, b->W_qkv, b->dqkv, p->C, 3 * p->C, b->cu_seqlens, b->dX, dW, db, b->d_status, stream,
+                          b->idx, (p->flags & SPA_FLAG_RESIDUAL) != 0);
 }
 // the second stream starts after everything enqueued on the main stream so far
 inline int fork_side(const spa_overlap* ov, cudaStream_t main) {
@@ -501,7 +531,7 @@ int spa_block_fwd(const spa_params* p, const spa_block_buffers* b, void* stream)
   const int32_t n_seg = b->container_len > 0 ? spa_container_max_segments(p, b->container_len)
                                              : (b->seg_offsets != nullptr ? b->n_seg : p->B);
   SPA_STEP(spa_packed_attention_fwd(p, b->qkv, seg, n_seg, b->attn_out, b->lse, b->d_status, stream));
-  if (fused) return spa_packed_proj_scatter(p, b->attn_out, b->W_o, b->b_o, b->idx, b->cu_seqlens, y, b->d_status, stream);
+  if (fused) return proj_scatter(p, b, y, stream);
   SPA_STEP(spa_packed_proj(p, b->attn_out, b->W_o, b->b_o, b->cu_seqlens, b->z, b->d_status, stream));
   return spa_unpack_scatter(p, b->z, inplace ? nullptr : b->x, b->idx, b->inv, b->cu_seqlens, y, b->d_status, stream);
 }
@@ -556,8 +586,7 @@ int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream)
     void* ws = ov != nullptr ? nullptr : b->workspace;
     if (fused) {
       // the input gradient scatters its rows to the selected tokens itself: no packed dx, no scatter kernel
-      rc = spa_packed_linear_bwd_scatter(p, b->x_packed, b->W_qkv, b->dqkv, C, 3 * C, b->idx, b->cu_seqlens, b->dX, dW,
-                                         db, ws, b->d_status, stream);
+      rc = qkv_bwd_scatter(p, b, dW, db, ws, stream);
     } else {
       rc = spa_packed_linear_bwd(p, b->x_packed, b->W_qkv, b->dqkv, C, 3 * C, b->cu_seqlens, b->dx_packed, dW, db,
                                  ov != nullptr ? b->workspace : ws, b->d_status, stream);

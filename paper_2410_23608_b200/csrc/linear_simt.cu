@@ -1,8 +1,7 @@
 // fp32-FMA linear layers on the packed tokens (QKV / output projection and their gradients; the
-// 3LC^2 and NC^2 terms of Eq. 9).  This is the path of the fp32 workload, whose 1e-4 tolerance a
-// single-pass reduced-precision tensor-core product cannot meet, and the reference path the
-// tensor-core kernels are brought up against.  One generic tiled kernel covers all three products
-// by taking element strides:  out[m][n] = sum_k A(m,k) * B(n,k).
+// 3LC^2 and NC^2 terms of Eq. 9) for bf16 data: the path that SPA_FLAG_SIMT_ONLY selects to cross-check the
+// tensor-core kernels, and that serves layers narrower than they cover.  (fp32 data: linear_f32.cu.)  One generic
+// tiled kernel covers all three products by taking element strides:  out[m][n] = sum_k A(m,k) * B(n,k).
 #include "spa_common.cuh"
 
 namespace spa {
@@ -17,7 +16,8 @@ template <typename T, typename TO>
 __global__ void __launch_bounds__(kThreads)
 gemm_simt_kernel(const T* __restrict__ A, long long sAm, long long sAk, const T* __restrict__ Bm, long long sBn,
                  long long sBk, const T* __restrict__ bias, TO* __restrict__ out, long long ldo, int M, int N, int K,
-                 const int32_t* __restrict__ cu, int n_seg, int capacity, int dyn_which, int accumulate) {
+                 const int32_t* __restrict__ cu, int n_seg, int capacity, int dyn_which, int accumulate,
+                 const int32_t* __restrict__ row_map) {
   pdl_entry();
   if (dyn_which != 0) {
     const int rows = packed_rows(cu, n_seg, capacity);
@@ -65,14 +65,15 @@ gemm_simt_kernel(const T* __restrict__ A, long long sAm, long long sAk, const T*
   for (int i = 0; i < 4; ++i) {
     const int m = m0 + ty * 4 + i;
     if (m >= M) continue;
+    const long long mo = row_map != nullptr ? __ldg(row_map + m) : m;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int n = n0 + tx * 4 + j;
       if (n >= N) continue;
       float v = acc[i][j];
       if (bias != nullptr) v += to_f32<T>(bias[n]);
-      if (accumulate) v += to_f32<TO>(out[(long long)m * ldo + n]);  // residual: the product joins what the row holds
-      out[(long long)m * ldo + n] = from_f32<TO>(v);
+      if (accumulate) v += to_f32<TO>(out[mo * ldo + n]);  // residual: the product joins what the row holds
+      out[mo * ldo + n] = from_f32<TO>(v);
     }
   }
 }
@@ -98,53 +99,48 @@ colsum_kernel(const T* __restrict__ dout, int n_out, const int32_t* __restrict__
 template <typename T, typename TO>
 void launch_gemm(const T* A, long long sAm, long long sAk, const T* Bm, long long sBn, long long sBk, const T* bias,
                  TO* out, long long ldo, int M, int N, int K, const int32_t* cu, int n_seg, int capacity,
-                 int dyn_which, cudaStream_t st, int accumulate = 0) {
+                 int dyn_which, cudaStream_t st, int accumulate = 0, const int32_t* row_map = nullptr) {
   dim3 grid((N + kTile - 1) / kTile, (M + kTile - 1) / kTile);
   launch_pdl(gemm_simt_kernel<T, TO>, grid, kThreads, 0, st, A, sAm, sAk, Bm, sBn, sBk, bias, out, ldo, M, N, K, cu, n_seg,
-                                                    capacity, dyn_which, accumulate);
+                                                    capacity, dyn_which, accumulate, row_map);
 }
 
-template <typename T>
-int linear_fwd(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
-               const int32_t* cu, void* out, cudaStream_t st, bool accumulate) {
-  launch_gemm<T, T>((const T*)a, n_in, 1, (const T*)W, n_in, 1, (const T*)bias, (T*)out, n_out, p.capacity, n_out,
-                    n_in, cu, p.B, p.capacity, 1, st, accumulate ? 1 : 0);
-  SPA_CUDA_CHECK_LAUNCH("gemm_simt_kernel(fwd)");
-  return SPA_OK;
-}
-
-template <typename T>
-int linear_bwd(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out,
-               const int32_t* cu, void* da, float* dW, float* db, cudaStream_t st) {
-  if (da != nullptr) {  // da[m][j] = sum_o dout[m][o] W[o][j]
-    launch_gemm<T, T>((const T*)dout, n_out, 1, (const T*)W, 1, n_in, nullptr, (T*)da, n_in, p.capacity, n_in, n_out,
-                      cu, p.B, p.capacity, 1, st);
-    SPA_CUDA_CHECK_LAUNCH("gemm_simt_kernel(dgrad)");
-  }
-  if (dW != nullptr) {  // dW[o][j] = sum_i dout[i][o] a[i][j]
-    launch_gemm<T, float>((const T*)dout, 1, n_out, (const T*)a, 1, n_in, nullptr, dW, n_in, n_out, n_in, p.capacity,
-                          cu, p.B, p.capacity, 2, st);
-    SPA_CUDA_CHECK_LAUNCH("gemm_simt_kernel(wgrad)");
-  }
-  if (db != nullptr) {
-    launch_pdl(colsum_kernel<T>, (n_out + 63) / 64, kThreads, 0, st, (const T*)dout, n_out, cu, p.B, p.capacity, db);
-    SPA_CUDA_CHECK_LAUNCH("colsum_kernel");
-  }
-  return SPA_OK;
-}
+using bf16 = __nv_bfloat16;
 
 }  // namespace
 
 int launch_linear_fwd_simt(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
-                           const int32_t* cu, void* out, cudaStream_t st, bool accumulate) {
-  return p.dtype == SPA_F32 ? linear_fwd<float>(p, a, W, bias, n_in, n_out, cu, out, st, accumulate)
-                            : linear_fwd<__nv_bfloat16>(p, a, W, bias, n_in, n_out, cu, out, st, accumulate);
+                           const int32_t* cu, void* out, cudaStream_t st, const int32_t* row_map, bool accumulate) {
+  launch_gemm<bf16, bf16>((const bf16*)a, n_in, 1, (const bf16*)W, n_in, 1, (const bf16*)bias, (bf16*)out, n_out, p.capacity, n_out,
+                          n_in, cu, p.B, p.capacity, 1, st, accumulate ? 1 : 0, row_map);
+  SPA_CUDA_CHECK_LAUNCH("gemm_simt_kernel(fwd)");
+  return SPA_OK;
 }
 
 int launch_linear_bwd_simt(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out,
-                           const int32_t* cu, void* da, float* dW, float* db, cudaStream_t st) {
-  return p.dtype == SPA_F32 ? linear_bwd<float>(p, a, W, dout, n_in, n_out, cu, da, dW, db, st)
-                            : linear_bwd<__nv_bfloat16>(p, a, W, dout, n_in, n_out, cu, da, dW, db, st);
+                           const int32_t* cu, void* da, float* dW, float* db, cudaStream_t st, const int32_t* row_map,
+                           bool accumulate) {
+  if (da != nullptr) {  // da[m][j] = sum_o dout[m][o] W[o][j]
+    launch_gemm<bf16, bf16>((const bf16*)dout, n_out, 1, (const bf16*)W, 1, n_in, nullptr, (bf16*)da, n_in, p.capacity, n_in, n_out,
+                            cu, p.B, p.capacity, 1, st, accumulate ? 1 : 0, row_map);
+    SPA_CUDA_CHECK_LAUNCH("gemm_simt_kernel(dgrad)");
+  }
+  if (dW != nullptr) {  // dW[o][j] = sum_i dout[i][o] a[i][j]
+    launch_gemm<bf16, float>((const bf16*)dout, 1, n_out, (const bf16*)a, 1, n_in, nullptr, dW, n_in, n_out, n_in, p.capacity,
+                             cu, p.B, p.capacity, 2, st);
+    SPA_CUDA_CHECK_LAUNCH("gemm_simt_kernel(wgrad)");
+  }
+  return db != nullptr ? launch_colsum_simt(p, dout, n_out, cu, db, st) : SPA_OK;
+}
+
+int launch_colsum_simt(const spa_params& p, const void* dout, int n_out, const int32_t* cu, float* db, cudaStream_t st) {
+  const int grid = (n_out + 63) / 64;
+  if (p.dtype == SPA_F32)
+    launch_pdl(colsum_kernel<float>, grid, kThreads, 0, st, (const float*)dout, n_out, cu, p.B, p.capacity, db);
+  else
+    launch_pdl(colsum_kernel<bf16>, grid, kThreads, 0, st, (const bf16*)dout, n_out, cu, p.B, p.capacity, db);
+  SPA_CUDA_CHECK_LAUNCH("colsum_kernel");
+  return SPA_OK;
 }
 
 }  // namespace spa

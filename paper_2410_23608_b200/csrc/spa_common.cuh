@@ -198,11 +198,21 @@ int launch_layer_norm_bwd(const spa_params& p, const void* dy, const void* x, co
 int launch_gelu(const spa_params& p, const void* u, const void* dh, int n_cols, void* out, cudaStream_t st);
 int launch_copy_tokens(const spa_params& p, const void* src, void* dst, cudaStream_t st);  // dst[B*N][C] = src
 
-// out[M][n_out] = a[M][n_in] W[n_out][n_in]^T + bias, M = packed rows (device)
+// out[M][n_out] = a[M][n_in] W[n_out][n_in]^T + bias, M = packed rows (device); row_map: output row i is written to row
+// row_map[i] of `out`, added to its contents if `accumulate`.  _simt: bf16 data on fp32 FMAs; _f32: fp32 data.
 int launch_linear_fwd_simt(const spa_params& p, const void* a, const void* W, const void* bias, int n_in,
-                           int n_out, const int32_t* cu, void* out, cudaStream_t st, bool accumulate = false);
+                           int n_out, const int32_t* cu, void* out, cudaStream_t st, const int32_t* row_map = nullptr,
+                           bool accumulate = false);
 int launch_linear_bwd_simt(const spa_params& p, const void* a, const void* W, const void* dout, int n_in,
-                           int n_out, const int32_t* cu, void* da, float* dW, float* db, cudaStream_t st);
+                           int n_out, const int32_t* cu, void* da, float* dW, float* db, cudaStream_t st,
+                           const int32_t* row_map = nullptr, bool accumulate = false);
+int launch_colsum_simt(const spa_params& p, const void* dout, int n_out, const int32_t* cu, float* db, cudaStream_t st);
+int launch_linear_fwd_f32(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
+                          const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st,
+                          const int32_t* row_map = nullptr, bool accumulate = false);
+int launch_linear_bwd_f32(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out,
+                          const int32_t* cu, void* da, float* dW, float* db, int32_t* d_status, cudaStream_t st,
+                          const int32_t* row_map = nullptr, bool accumulate = false);
 int launch_attention_fwd_simt(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao,
                               float* lse, cudaStream_t st);
 int launch_attention_bwd_simt(const spa_params& p, const void* qkv, const void* ao, const float* lse,
