@@ -166,6 +166,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   };
 
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -176,11 +178,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         k_range(c.z, k_begin, k_end, k_step);
         for (int k0 = k_begin; k0 < k_end; k0 += k_step, ++it) {
           const int s = it % kStages;
-          if (it >= kStages && !ptx::mbar_wait(empty_bar(s), ((it / kStages) - 1) & 1)) {
-            record_status(d_status, SPA_ERR_TIMEOUT);
-            *abort_flag = 1;
-          }
-          if (*abort_flag) break;
+          if (it >= kStages) wait(empty_bar(s), ((it / kStages) - 1) & 1);
           const uint32_t a_dst = smem_base + s * kStage, b_dst = a_dst + kABytes;
           ptx::mbar_expect_tx(full_bar(s), kStage);
           if (!kAMn) {
@@ -207,28 +205,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     int it = 0, tl = 0;  // k-block counter, tile counter of this CTA
-    bool dead = false;   // warp-uniform: a wait of this warp ran out, or another role gave up
-    for (int tile = blockIdx.x; tile < total && !dead; tile += gridDim.x, ++tl) {
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+    for (int tile = blockIdx.x; tile < total && !__any_sync(0xffffffffu, *abort_flag != 0); tile += gridDim.x, ++tl) {
       const TileCoord c = coord(tile);
       int k_begin, k_end, k_step;
       k_range(c.z, k_begin, k_end, k_step);
       const int acc = tl & 1;
-      if (tl >= 2 && !__all_sync(0xffffffffu, ptx::mbar_wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1))) {
-        if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
-        break;
-      }
+      if (tl >= 2) wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1);
       ptx::tc_fence_after_sync();
       const uint32_t tmem_d = tmem_base + acc * BN;
       bool first = true;
       for (int k0 = k_begin; k0 < k_end; k0 += k_step, ++it) {
         const int s = it % kStages;
-        if (__any_sync(0xffffffffu, *abort_flag != 0)) { dead = true; break; }
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(full_bar(s), (it / kStages) & 1))) {
-          if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
-          dead = true;
-          break;
-        }
+        wait(full_bar(s), (it / kStages) & 1);
         const uint32_t a_src = smem_base + s * kStage, b_src = a_src + kABytes;
         const int k_valid = k_end - k0;
         if ((kAMn || kBMn) && k_valid < BK) {
@@ -270,15 +258,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint8_t* stage = smem_al + kStages * kStage + 128 + (warp - 2) * 2048;  // this warp's transposition buffer
     int tl = 0;
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++tl) {
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
       const TileCoord c = coord(tile);
       const int acc = tl & 1;
-      const bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(tmem_full_bar(acc), (tl >> 1) & 1) && !*abort_flag);
-      if (!ok) {
-        if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
-        break;
-      }
-      ptx::tc_fence_after_sync();
       // Thread `lane` receives row (q*32 + lane) of the accumulator.  Written straight from there, every
       // store instruction would touch 32 rows with 16 bytes each; instead the warp turns 64-byte row
       // segments around in its private 2 KB of shared memory, so that a store instruction covers 8 rows
@@ -293,8 +274,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int grow = c.m0 + q * 32 + my_row + 8 * j;
         orow[j] = (row_map != nullptr && grow < M) ? (long long)__ldg(row_map + grow) : (long long)grow;
       }
+      // the bias of the tile comes to L1 under the main loop: fetched where it is added, each 32 columns waited for L2
+      if (bias != nullptr && lane < BN / 64 && c.n0 + lane * 64 < N) prefetch_l1(bias + c.n0 + lane * 64);
+      wait(tmem_full_bar(acc), (tl >> 1) & 1);
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      ptx::tc_fence_after_sync();
 #pragma unroll 1
       for (int cc = 0; cc < BN / 32; ++cc) {
+        uint4 old[4];  // what the rows hold, under the read of the accumulator
+        if (sizeof(OutT) == 2 && accumulate) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (c.m0 + q * 32 + my_row + 8 * j < M && c.n0 + cc * 32 + my_chunk * 8 < N)
+              old[j] = *reinterpret_cast<const uint4*>(obase + orow[j] * ldo + c.n0 + cc * 32 + my_chunk * 8);
+        }
         uint32_t r[32];
         ptx::tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + cc * 32, r);
         ptx::tmem_ld_wait();
@@ -331,7 +324,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               uint4* dst = reinterpret_cast<uint4*>(obase + orow[j] * ldo + gcol);
               if (sizeof(OutT) == 2 && accumulate) {
                 float fa[8], fb[8];
-                Vec16<__nv_bfloat16>::to_float(*dst, fa);
+                Vec16<__nv_bfloat16>::to_float(old[j], fa);
                 Vec16<__nv_bfloat16>::to_float(v4, fb);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) fa[e] += fb[e];

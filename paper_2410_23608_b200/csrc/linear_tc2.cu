@@ -86,7 +86,7 @@ constexpr int kPairStages = 5;
 constexpr int kPairEpiWarps = 8;   // two per TMEM lane quarter: they split the 32-column groups of a tile
 constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;  // warp 0: TMA, warp 1: MMA (leader) + TMEM owner, then the epilogue warps
 constexpr int kPairStage = PM * PK * 2 + (PN / 2) * PK * 2;  // 32 KB
-constexpr int kPairSmem = kPairStages * kPairStage + 1024 + 256 + kPairEpiWarps * 2048;  // ring, alignment slack, barriers, transposition
+constexpr int kPairSmem = kPairStages * kPairStage + 1024 + 256 + kPairEpiWarps * 4096;  // ring, alignment slack, barriers, transposition
 
 // kBMn: B = W is MN-major (input gradient: K = n_out rows of W, N = n_in contiguous); otherwise K-major
 // (forward: N = n_out rows of W, K = n_in contiguous).  A is always K-major, the output bf16.
@@ -138,6 +138,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int tiles_m = (M + 2 * PM - 1) / (2 * PM);
   const int total = tiles_m * tiles_n;
   const int k_blocks = (K + PK - 1) / PK;
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one per CTA)
@@ -148,11 +149,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int n0 = (tile % tiles_n) * PN + (int)rank * (PN / 2);
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kPairStages;
-          if (it >= kPairStages && !ptx::mbar_wait(empty_bar(s), ((it / kPairStages) - 1) & 1)) {
-            record_status(d_status, SPA_ERR_TIMEOUT);
-            *abort_flag = 1;
-          }
-          if (*abort_flag) break;
+          if (it >= kPairStages) wait(empty_bar(s), ((it / kPairStages) - 1) & 1);
           const uint32_t a_dst = smem_base + s * kPairStage, b_dst = a_dst + PM * PK * 2;
           const uint32_t lead_full = ptx2::map_to_cta(full_bar(s), 0);
           ptx2::mbar_expect_tx_cluster(lead_full, kPairStage);
@@ -172,27 +169,17 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // ------------------------------------------------------------------ MMA issuer: the leader's, for the pair
     if (rank == 0) {
       int it = 0, tl = 0;
-      bool dead = false;
-      for (int tile = pair; tile < total && !dead; tile += n_pairs, ++tl) {
-        if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      for (int tile = pair; tile < total && !__any_sync(0xffffffffu, *abort_flag != 0); tile += n_pairs, ++tl) {
         const int acc = tl & 1;
-        if (tl >= 2 && !__all_sync(0xffffffffu, ptx::mbar_wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1))) {
-          if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
-          break;
-        }
+        if (tl >= 2) wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1);
         ptx::tc_fence_after_sync();
         const uint32_t tmem_d = tmem_base + acc * PN;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kPairStages;
-          if (__any_sync(0xffffffffu, *abort_flag != 0)) { dead = true; break; }
-          if (!__all_sync(0xffffffffu, ptx::mbar_wait(full_bar(s), (it / kPairStages) & 1))) {
-            if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
-            dead = true;
-            break;
-          }
+          wait(full_bar(s), (it / kPairStages) & 1);
           ptx::tc_fence_after_sync();
           const uint32_t a_src = smem_base + s * kPairStage, b_src = a_src + PM * PK * 2;
-          if (lane == 0) {
+          if (ptx::elect_one()) {
 #pragma unroll
             for (int k = 0; k < PK / 16; ++k) {
               const uint64_t adesc = ptx::smem_desc_sw128(a_src + k * 32, 16, 1024);
@@ -201,69 +188,76 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               ptx2::mma_bf16_pair(tmem_d, adesc, bdesc, kIdesc, (kb == 0 && k == 0) ? 0u : 1u);
             }
             ptx2::mma_commit_pair(empty_bar(s));
+            if (kb == k_blocks - 1) ptx2::mma_commit_pair(tmem_full_bar(acc));
           }
           __syncwarp();
         }
-        if (lane == 0 && !dead && k_blocks > 0) ptx2::mma_commit_pair(tmem_full_bar(acc));
       }
     }
   } else {
     // ------------------------------------------------------------------ epilogue warps (both CTAs)
     const int q = warp & 3;  // TMEM lane quarter this warp may read
     const int half = (warp - 2) >> 2;  // which of the two warps of that quarter: even or odd 32-column groups
-    uint8_t* stage = smem_al + kPairStages * kPairStage + 256 + (warp - 2) * 2048;  // this warp's transposition buffer
+    uint8_t* stage = smem_al + kPairStages * kPairStage + 256 + (warp - 2) * 4096;  // this warp's transposition buffer
     const uint32_t lead_empty[2] = {ptx2::map_to_cta(tmem_empty_bar(0), 0), ptx2::map_to_cta(tmem_empty_bar(1), 0)};
-    const int my_chunk = lane & 3, my_row = lane >> 2;
+    const int my_chunk = lane & 7, my_row = lane >> 3;
     int tl = 0;
     for (int tile = pair; tile < total; tile += n_pairs, ++tl) {
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
       const int m0 = (tile / tiles_n) * 2 * PM + (int)rank * PM;
       const int n0 = (tile % tiles_n) * PN;
       const int acc = tl & 1;
-      const bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(tmem_full_bar(acc), (tl >> 1) & 1) && !*abort_flag);
-      if (!ok) {
-        if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
-        break;
-      }
-      ptx::tc_fence_after_sync();
-      long long orow[4];  // destination rows of the four rows this lane stores
+      long long orow[8];  // destination rows of the eight rows this lane stores
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int grow = m0 + q * 32 + my_row + 8 * j;
+      for (int j = 0; j < 8; ++j) {
+        const int grow = m0 + q * 32 + my_row + 4 * j;
         orow[j] = (row_map != nullptr && grow < M) ? (long long)__ldg(row_map + grow) : (long long)grow;
       }
+      // the bias of the tile comes to L1 under the main loop: fetched where it is added, each 64 columns waited for L2
+      if (bias != nullptr && lane < PN / 64 && n0 + lane * 64 < N) prefetch_l1(bias + n0 + lane * 64);
+      wait(tmem_full_bar(acc), (tl >> 1) & 1);
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      ptx::tc_fence_after_sync();
+      // Thread `lane` receives one accumulator row; 64 columns (128 bytes of the output) at a time are turned around in
+      // the warp's 4 KB, so that a store instruction covers four whole 128-byte lines.
 #pragma unroll 1
-      for (int cc = half; cc < PN / 32; cc += 2) {
-        if (n0 + cc * 32 >= N) break;  // warp-uniform: columns past the layer's width
-        uint32_t r[32];
-        ptx::tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * PN + cc * 32, r);
+      for (int cc = half; cc < PN / 64; cc += 2) {
+        if (n0 + cc * 64 >= N) break;  // warp-uniform: columns past the layer's width
+        const int gcol = n0 + cc * 64 + my_chunk * 8;
+        uint4 old[8];  // what the rows hold, under the reads of the accumulator
+        if (accumulate) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (m0 + q * 32 + my_row + 4 * j < M && gcol < N) old[j] = *reinterpret_cast<const uint4*>(out + orow[j] * ldo + gcol);
+        }
+        uint32_t r[64];
+        const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + acc * PN + cc * 64;
+        ptx::tmem_ld_32x32(at, r);
+        ptx::tmem_ld_32x32(at + 32, r + 32);
         ptx::tmem_ld_wait();
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {  // 16-byte chunk i of this row's 64-byte segment
+        for (int i = 0; i < 8; ++i) {  // 16-byte chunk i of this row's 128-byte segment
           float v[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[i * 8 + e]);
-          const int col = n0 + cc * 32 + i * 8;
+          const int col = n0 + cc * 64 + i * 8;
           if (bias != nullptr && col < N) {
             float b[8];
             Vec16<__nv_bfloat16>::to_float(__ldg(reinterpret_cast<const uint4*>(bias + col)), b);
 #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] += b[e];
           }
-          *reinterpret_cast<uint4*>(stage + lane * 64 + ((i ^ ((lane >> 1) & 3)) << 4)) = Vec16<__nv_bfloat16>::from_float(v);
+          *reinterpret_cast<uint4*>(stage + lane * 128 + ((i ^ (lane & 7)) << 4)) = Vec16<__nv_bfloat16>::from_float(v);
         }
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int rr = my_row + 8 * j;
-          const uint4 v4 = *reinterpret_cast<const uint4*>(stage + rr * 64 + ((my_chunk ^ ((rr >> 1) & 3)) << 4));
-          const int grow = m0 + q * 32 + rr;
-          const int gcol = n0 + cc * 32 + my_chunk * 8;
-          if (grow < M && gcol < N) {
+        for (int j = 0; j < 8; ++j) {
+          const int rr = my_row + 4 * j;
+          const uint4 v4 = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((my_chunk ^ (rr & 7)) << 4));
+          if (m0 + q * 32 + rr < M && gcol < N) {
             uint4* dst = reinterpret_cast<uint4*>(out + orow[j] * ldo + gcol);
             if (accumulate) {
               float fa[8], fb[8];
-              Vec16<__nv_bfloat16>::to_float(*dst, fa);
+              Vec16<__nv_bfloat16>::to_float(old[j], fa);
               Vec16<__nv_bfloat16>::to_float(v4, fb);
 #pragma unroll
               for (int e = 0; e < 8; ++e) fa[e] += fb[e];
