@@ -161,7 +161,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
   pdl_entry();
   const bool staged = n_seg < kSegStage;
   if (staged)
-    for (int i = tid; i <= n_seg; i += kFwdThreads) seg_s[i] = __ldg(seg + i);
+    for (int i = tid; i <= n_seg; i += kFwdThreads) seg_s[i] = ld_dep(seg + i);
   const int Np = packed_rows(seg, n_seg, capacity);
   const int n_items = ((Np + kQ - 1) / kQ) * H;
   if ((int)blockIdx.x >= n_items) return;
@@ -563,7 +563,7 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   pdl_entry();
   const bool staged = n_seg < kSegStage;
   if (staged)
-    for (int i = tid; i <= n_seg; i += kBwdThreads) seg_s[i] = __ldg(seg + i);
+    for (int i = tid; i <= n_seg; i += kBwdThreads) seg_s[i] = ld_dep(seg + i);
   const int Np = packed_rows(seg, n_seg, capacity);
   const int n_items = ((Np + 127) / 128) * H;
   if ((int)blockIdx.x >= n_items) return;
@@ -1027,7 +1027,7 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
   pdl_entry();
   const bool staged = n_seg < kSegStage;
   if (staged)
-    for (int i = tid; i <= n_seg; i += kBwdThreads) seg_s[i] = __ldg(seg + i);
+    for (int i = tid; i <= n_seg; i += kBwdThreads) seg_s[i] = ld_dep(seg + i);
   const int Np = packed_rows(seg, n_seg, capacity);
   const int n_items = ((Np + 127) / 128) * H;
   if ((int)blockIdx.x >= n_items) return;
@@ -1430,8 +1430,8 @@ attn_bwd_short_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_c
   }
   pdl_entry();
   const int Np = packed_rows(seg, n_seg, capacity);
-  const int lo = __ldg(seg + s_idx);
-  int hi = __ldg(seg + s_idx + 1);
+  const int lo = ld_dep(seg + s_idx);
+  int hi = ld_dep(seg + s_idx + 1);
   hi = hi < Np ? hi : Np;
   const int n = hi - lo;  // rows of this segment
   if (n <= 0 || n > kShortMax) return;  // empty, or one for the two-pass kernels

@@ -34,6 +34,11 @@ template <int BN> constexpr int kStageBytes = 3 * (kAPlane + kBPlane<BN>);
 template <int BN> constexpr int kLdT = BN + 4;  // finished tile in shared memory, fp32
 template <int BN> constexpr int kSmem = kStages * kStageBytes<BN> + 1024 + 64;
 
+__device__ __forceinline__ float4 ld_values(const float* p) {
+  const uint4 v = ld_dep16(p);
+  return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+
 struct Tile8 { float4 a, b; };  // eight consecutive values of a line
 
 // Two values into their three bf16 parts, packed pairwise.  A value beyond bf16's range keeps its infinite first part.
@@ -68,8 +73,8 @@ template <int R, bool kMn> struct Operand {
       row += r0; k += k0;
       const float* p = src + (kMn ? (long long)k * ld + row : (long long)row * ld + k);
       const bool in0 = row < rows && k < k_end, in1 = kMn ? (row + 4 < rows && k < k_end) : (row < rows && k + 4 < k_end);
-      t[i].a = in0 ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      t[i].b = in1 ? __ldg(reinterpret_cast<const float4*>(p + 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      t[i].a = in0 ? ld_values(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+      t[i].b = in1 ? ld_values(p + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
   __device__ static __forceinline__ void store(const Tile8* t, uint8_t* plane0, int tid) {
@@ -277,7 +282,7 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
       }
       const int m = m0 + r;
-      float4* dst = reinterpret_cast<float4*>(out + (row_map != nullptr ? (long long)__ldg(row_map + m) : (long long)m) * ldo + n0 + c);
+      float4* dst = reinterpret_cast<float4*>(out + (row_map != nullptr ? (long long)ld_dep(row_map + m) : (long long)m) * ldo + n0 + c);
       if (accumulate) {
         const float4 w = *dst;
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;

@@ -65,7 +65,7 @@ gemm_simt_kernel(const T* __restrict__ A, long long sAm, long long sAk, const T*
   for (int i = 0; i < 4; ++i) {
     const int m = m0 + ty * 4 + i;
     if (m >= M) continue;
-    const long long mo = row_map != nullptr ? __ldg(row_map + m) : m;
+    const long long mo = row_map != nullptr ? ld_dep(row_map + m) : m;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int n = n0 + tx * 4 + j;

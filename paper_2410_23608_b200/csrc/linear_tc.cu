@@ -166,7 +166,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   };
 
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -178,7 +179,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         k_range(c.z, k_begin, k_end, k_step);
         for (int k0 = k_begin; k0 < k_end; k0 += k_step, ++it) {
           const int s = it % kStages;
-          if (it >= kStages) wait(empty_bar(s), ((it / kStages) - 1) & 1);
+          if (it >= kStages) wait_lane(empty_bar(s), ((it / kStages) - 1) & 1);
           const uint32_t a_dst = smem_base + s * kStage, b_dst = a_dst + kABytes;
           ptx::mbar_expect_tx(full_bar(s), kStage);
           if (!kAMn) {
@@ -272,7 +273,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int grow = c.m0 + q * 32 + my_row + 8 * j;
-        orow[j] = (row_map != nullptr && grow < M) ? (long long)__ldg(row_map + grow) : (long long)grow;
+        orow[j] = (row_map != nullptr && grow < M) ? (long long)ld_dep(row_map + grow) : (long long)grow;
       }
       // the bias of the tile comes to L1 under the main loop: fetched where it is added, each 32 columns waited for L2
       if (bias != nullptr && lane < BN / 64 && c.n0 + lane * 64 < N) prefetch_l1(bias + c.n0 + lane * 64);

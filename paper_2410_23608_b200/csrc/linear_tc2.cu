@@ -138,7 +138,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int tiles_m = (M + 2 * PM - 1) / (2 * PM);
   const int total = tiles_m * tiles_n;
   const int k_blocks = (K + PK - 1) / PK;
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one per CTA)
@@ -149,7 +150,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int n0 = (tile % tiles_n) * PN + (int)rank * (PN / 2);
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kPairStages;
-          if (it >= kPairStages) wait(empty_bar(s), ((it / kPairStages) - 1) & 1);
+          if (it >= kPairStages) wait_lane(empty_bar(s), ((it / kPairStages) - 1) & 1);
           const uint32_t a_dst = smem_base + s * kPairStage, b_dst = a_dst + PM * PK * 2;
           const uint32_t lead_full = ptx2::map_to_cta(full_bar(s), 0);
           ptx2::mbar_expect_tx_cluster(lead_full, kPairStage);
@@ -210,7 +211,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int grow = m0 + q * 32 + my_row + 4 * j;
-        orow[j] = (row_map != nullptr && grow < M) ? (long long)__ldg(row_map + grow) : (long long)grow;
+        orow[j] = (row_map != nullptr && grow < M) ? (long long)ld_dep(row_map + grow) : (long long)grow;
       }
       // the bias of the tile comes to L1 under the main loop: fetched where it is added, each 64 columns waited for L2
       if (bias != nullptr && lane < PN / 64 && n0 + lane * 64 < N) prefetch_l1(bias + n0 + lane * 64);

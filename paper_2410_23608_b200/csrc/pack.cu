@@ -62,14 +62,14 @@ select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ ma
   int cnt = 0;
   const uint4* mask16 = reinterpret_cast<const uint4*>(mask);
   if (!kOrdered) {
-    for (int k = tid; k < (tile_start >> 4); k += kPackThreads) cnt += count_nonzero_bytes(__ldg(mask16 + k));
+    for (int k = tid; k < (tile_start >> 4); k += kPackThreads) cnt += count_nonzero_bytes(ld_dep16(mask16 + k));
   } else {
     // whole images before the tile's first image: any order visits the same bytes; then the positions of
     // that image which the given order visits before the tile
     const int img0 = (tile_start / N) * N;
-    for (int k = tid; k < (img0 >> 4); k += kPackThreads) cnt += count_nonzero_bytes(__ldg(mask16 + k));
-    for (int k = (img0 & ~15) + tid; k < img0; k += kPackThreads) cnt += mask[k] != 0;
-    for (int j = tid; j < tile_start - img0; j += kPackThreads) cnt += mask[img0 + __ldg(order + j)] != 0;
+    for (int k = tid; k < (img0 >> 4); k += kPackThreads) cnt += count_nonzero_bytes(ld_dep16(mask16 + k));
+    for (int k = (img0 & ~15) + tid; k < img0; k += kPackThreads) cnt += ld_dep(mask + k) != 0;
+    for (int j = tid; j < tile_start - img0; j += kPackThreads) cnt += ld_dep(mask + img0 + __ldg(order + j)) != 0;
   }
   cnt = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
   if (lane == 0) warp_cnt[wid] = cnt;
@@ -79,7 +79,7 @@ select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ ma
   const bool in_tile = tid < tile && t < rows;
   int tok = t;  // the token that position t of the visiting order stands for
   if (kOrdered && in_tile) tok = (t / N) * N + __ldg(order + t % N);
-  const bool sel = in_tile && mask[tok] != 0;
+  const bool sel = in_tile && ld_dep(mask + tok) != 0;
   const unsigned ballot = __ballot_sync(0xffffffffu, sel);
   if (lane == 0) warp_sel[wid] = __popc(ballot);
   __syncthreads();
@@ -153,7 +153,7 @@ unpack_scatter_kernel(const uint4* __restrict__ z16, const uint4* __restrict__ x
       if (k < total) {
         const long long t = k / Q;
         const int q = (int)(k - t * Q);
-        const int i = __ldg(inv + t);
+        const int i = ld_dep(inv + t);
         if (i >= 0 && i < Np) {
           v[u] = ld_nc16(z16 + (size_t)i * Q + q);
           if (kResidual) v[u] = add16<T>(v[u], ld_nc16(x16 + k));
@@ -189,7 +189,7 @@ row_scatter_kernel(const uint4* __restrict__ src16, const uint4* addp, const int
       if (k < total) {
         const long long i = k / Q;
         const int q = (int)(k - i * Q);
-        o[u] = (size_t)__ldg(idx + i) * Q + q;
+        o[u] = (size_t)ld_dep(idx + i) * Q + q;
         v[u] = ld_nc16(src16 + k);
         if (kAdd) v[u] = add16<T>(v[u], addp[o[u]]);
       }
@@ -220,7 +220,7 @@ unpack_scatter_bwd_kernel(const uint4* __restrict__ dY16, const int32_t* __restr
       if (k < total) {
         const long long t = k / Q;
         const int q = (int)(k - t * Q);
-        const int i = __ldg(inv + t);
+        const int i = ld_dep(inv + t);
         if (i >= 0 && i < Np) o[u] = (long long)i * Q + q;
         else if (copy_pass_through) o[u] = -1;
         if (o[u] != -2) v[u] = ld_nc16(dY16 + k);
@@ -286,7 +286,7 @@ container_offsets_kernel(const int32_t* __restrict__ cu, int B, int L, int n_max
   __shared__ int carry_s;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int n = B + 1;
-  for (int i = tid; i < n; i += kCutThreads) cu_s[i] = __ldg(cu + i);
+  for (int i = tid; i < n; i += kCutThreads) cu_s[i] = ld_dep(cu + i);
   if (tid == 0) carry_s = 0;
   __syncthreads();
   for (int base = 0; base < n; base += kCutThreads) {

@@ -89,7 +89,7 @@ pack_bwd_gated_kernel(const uint4* __restrict__ dxp16, const uint4* __restrict__
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (kTrainThreads / 32);
   for (int i = blockIdx.x * (kTrainThreads / 32) + (threadIdx.x >> 5); i < Np; i += warps) {
-    const long long t = __ldg(idx + i);
+    const long long t = ld_dep(idx + i);
     const float p = sigmoid_f(scores[t]);
     float dot = 0.f;
     for (int q = lane; q < Q; q += 32) {

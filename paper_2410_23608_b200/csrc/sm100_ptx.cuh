@@ -65,6 +65,13 @@ __device__ __forceinline__ void mbar_wait_or_abort(uint32_t bar, uint32_t parity
   if (d_status != nullptr) atomicCAS(d_status, 0, timeout_code);
   *abort_flag = 1;
 }
+// The same by all lanes of a warp, which are converged again when it returns: lanes may have polled a different number of
+// times, and elect_one() in a diverged warp would elect a lane of each part.
+__device__ __forceinline__ void mbar_wait_or_abort_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* d_status,
+                                                        int timeout_code) {
+  mbar_wait_or_abort(bar, parity, abort_flag, d_status, timeout_code);
+  __syncwarp();
+}
 
 // True in exactly one lane of a converged warp (all 32 lanes must execute it together).  Work that one thread has to
 // issue (tensor-core products, bulk copies) is written as `if (elect_one()) ...` inside code that the whole warp

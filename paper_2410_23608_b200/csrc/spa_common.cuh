@@ -13,9 +13,27 @@ namespace spa {
 
 constexpr int kNumSMs = 148;  // B200: two dies of 74 SMs
 
+// Loads of what an earlier kernel of the stream wrote.  Not the read-only path (__ldg): under programmatic dependent
+// launch the writer may still run when this kernel starts, and a read-only load is free to move above the wait.
+__device__ __forceinline__ int32_t ld_dep(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_dep(const uint8_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_dep16(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 // Number of valid packed rows: the device-resident total, clamped to the allocated rows.
 __device__ __forceinline__ int packed_rows(const int32_t* __restrict__ offsets, int n_seg, int capacity) {
-  int n = __ldg(offsets + n_seg);
+  int n = ld_dep(offsets + n_seg);
   return n < capacity ? n : capacity;
 }
 
@@ -91,7 +109,7 @@ __device__ __forceinline__ int find_segment(const int32_t* __restrict__ offsets,
   int lo = 0, hi = n_seg;  // invariant: offsets[lo] <= i < offsets[hi]
   while (hi - lo > 1) {
     int mid = (lo + hi) >> 1;
-    if (__ldg(offsets + mid) <= i) lo = mid; else hi = mid;
+    if (ld_dep(offsets + mid) <= i) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -103,8 +121,8 @@ __device__ __forceinline__ RowSeg row_segment(const int32_t* __restrict__ seg, i
   RowSeg r{0, 0};
   if (i < Np) {
     const int s = find_segment(seg, n_seg, i);
-    r.lo = __ldg(seg + s);
-    const int hi = __ldg(seg + s + 1);
+    r.lo = ld_dep(seg + s);
+    const int hi = ld_dep(seg + s + 1);
     r.hi = hi < Np ? hi : Np;
   }
   return r;
