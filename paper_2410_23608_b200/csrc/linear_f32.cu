@@ -269,14 +269,7 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
       const int r = z + (e / (BN / 4)) * split, c = (e % (BN / 4)) * 4;
       if (n0 + c >= N) continue;
       const float* src = tile + r * kLd + c;
-      float4 v = *reinterpret_cast<const float4*>(src);
-      if (split > 1) {
-        v = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int s = 0; s < split; ++s) {
-          const float4 w = ld_dsmem4(src, s);
-          v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-        }
-      }
+      float4 v = split > 1 ? sum_dsmem4(src, split) : *reinterpret_cast<const float4*>(src);
       if (bias != nullptr) {
         const float4 w = __ldg(reinterpret_cast<const float4*>(bias + n0 + c));
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
@@ -292,9 +285,7 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
     if (kAMn && sums)
       for (int e = tid; e < my_rows; e += kThreads) {
         const int r = z + e * split;
-        float v = 0.f;
-        for (int s = 0; s < split; ++s) v += split > 1 ? ld_dsmem(tile_sum + r, s) : tile_sum[r];
-        colsum[m0 + r] = v;
+        colsum[m0 + r] = split > 1 ? sum_dsmem(tile_sum + r, split) : tile_sum[r];
       }
   }
   if (split > 1) cluster_sync_all(); else __syncthreads();  // nobody leaves while a partial tile is still being read

@@ -404,12 +404,12 @@ colsum_partial_kernel(const __nv_bfloat16* __restrict__ dout, int n_out, const i
 
 // out[e] = sum over the splits that hold rows (in split order) of part[s][e]; zero if there are none.
 // Two arrays in one launch: the weight-gradient partials (a few splits: a thread adds them in split order) and,
-// optionally, the bias-gradient partials, which have row chunks of their own - up to hundreds of them for a few
-// thousand outputs, so there a warp owns four outputs: lane l adds chunks l, l + 32, ... in order and a fixed shuffle
+// optionally, the bias-gradient partials, one per row chunk or (rows_per_chunk2 = 0) tiles_n2 per split - up to hundreds
+// of them for a few thousand outputs, so there a warp owns four outputs: lane l adds chunks l, l + 32, ... in order and a fixed shuffle
 // tree adds the lanes.  The first ceil(n2 / 32) blocks take the second array.
 __global__ void __launch_bounds__(256)
 split_reduce_kernel(const float* __restrict__ part, long long n, const float* __restrict__ part2, long long n2,
-                    int splits, int rows_per_chunk2, const int32_t* __restrict__ cu, int n_seg, int capacity,
+                    int splits, int rows_per_chunk2, int tiles_n2, const int32_t* __restrict__ cu, int n_seg, int capacity,
                     float* __restrict__ out, float* __restrict__ out2) {
   pdl_entry();
   const int rows = packed_rows(cu, n_seg, capacity);
@@ -418,7 +418,7 @@ split_reduce_kernel(const float* __restrict__ part, long long n, const float* __
   const long long n4 = n >> 2, m4 = n2 >> 2;
   const int nb2 = (int)((m4 + 7) / 8);
   if ((int)blockIdx.x < nb2) {
-    const int valid2 = (rows + rows_per_chunk2 - 1) / rows_per_chunk2;
+    const int valid2 = rows_per_chunk2 > 0 ? (rows + rows_per_chunk2 - 1) / rows_per_chunk2 : valid1 * tiles_n2;
     const long long j = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (j >= m4) return;
     const int lane = threadIdx.x & 31;
@@ -463,7 +463,7 @@ SplitPlan plan_splits(int capacity, int n_in, int n_out) {
   int splits = (2 * kNumSMs) / tiles;
   const int max_by_rows = (capacity + BK - 1) / BK;
   if (splits > max_by_rows) splits = max_by_rows;
-  if (splits > 32) splits = 32;
+  if (splits > 31) splits = 31;  // the bias partials fit beside them in a workspace of 32
   if (splits < 1) splits = 1;
   int kps = (capacity + splits - 1) / splits;
   kps = ((kps + BK - 1) / BK) * BK;
@@ -473,10 +473,15 @@ SplitPlan plan_splits(int capacity, int n_in, int n_out) {
 
 size_t wgrad_workspace_bytes(int capacity, int n_in, int n_out) {
   const SplitPlan sp = plan_splits(capacity, n_in, n_out);
-  size_t w = (size_t)sp.splits * n_out * n_in * sizeof(float);
-  w = (w + 255) & ~(size_t)255;
-  return w + (size_t)kColsumChunks * n_out * sizeof(float) + 256;
+  const PairWgradPlan pl = pair_wgrad_plan(capacity, n_in, n_out);
+  auto bytes = [&](int splits, int sums) {
+    return (((size_t)splits * n_out * n_in * sizeof(float) + 255) & ~(size_t)255) + (size_t)sums * n_out * sizeof(float) + 256;
+  };
+  const size_t one = bytes(sp.splits, kColsumChunks), two = bytes(pl.splits, pl.splits * pl.tiles_n);
+  return one > two ? one : two;
 }
+
+inline bool wgrad_on_pairs(const spa_params& p) { return !(p.flags & SPA_FLAG_NO_CTA_PAIRS); }
 
 template <int BN, bool kAMn, bool kBMn, typename OutT>
 int launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, OutT* out, long long ldo,
@@ -551,19 +556,27 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
     if (rc != SPA_OK) return rc;
   }
   if (dW == nullptr && db == nullptr) return SPA_OK;
+  const PairWgradPlan pl = pair_wgrad_plan(p.capacity, n_in, n_out);
+  // CTA pairs where there are enough of their 256 x 256 tiles and enough rows to split between them (768 x 768 over 9 216
+  // rows: 18 us on pairs, 30 on clusters; 1 536 x 512 over 3 402: 17 either way; 1 536 x 384 over 1 568: 14 and 12)
+  if (dW != nullptr && wgrad_on_pairs(p) && (pl.tiles < 9 || p.capacity < 128 * BK))
+    return launch_wgrad_cluster(p, a, dout, n_in, n_out, cu, dW, db, d_status, st);
   const SplitPlan sp = plan_splits(p.capacity, n_in, n_out);
+  const bool pair = dW != nullptr && wgrad_on_pairs(p);
+  const int splits = pair ? pl.splits : sp.splits;
   float* part_w = reinterpret_cast<float*>(workspace);
-  size_t off = ((size_t)sp.splits * n_out * n_in * sizeof(float) + 255) & ~(size_t)255;
+  size_t off = ((size_t)splits * n_out * n_in * sizeof(float) + 255) & ~(size_t)255;
   float* part_b = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) + off);
   const long long n_w = (long long)n_out * n_in;
   const int rpc = colsum_rows_per_chunk(p.capacity);
-  if (db != nullptr) {  // db[j] = sum_i dout[i][j]: partial sums per row chunk, added up by the reduction below
+  if (db != nullptr && !pair) {  // db[j] = sum_i dout[i][j]: partial sums per row chunk, added up by the reduction below
     dim3 grid((n_out + 63) / 64, (p.capacity + rpc - 1) / rpc);
     launch_pdl(colsum_partial_kernel, grid, 256, 0, st, (const __nv_bfloat16*)dout, n_out, cu, p.B, p.capacity, rpc, part_b);
     SPA_CUDA_CHECK_LAUNCH("colsum_partial_kernel");
   }
   if (dW != nullptr) {  // dW[n_out][n_in] = sum_i dout[i][:]^T a[i][:]
-    int rc = launch_gemm<128, true, true, float>(tmA2, tmB2, nullptr, part_w, n_in, n_w, n_out, n_in, p.capacity,
+    int rc = pair ? launch_wgrad_pair(p, a, dout, n_in, n_out, cu, part_w, db != nullptr ? part_b : nullptr, pl, d_status, st)
+                  : launch_gemm<128, true, true, float>(tmA2, tmB2, nullptr, part_w, n_in, n_w, n_out, n_in, p.capacity,
                                                         cu, p.B, p.capacity, 2, sp.k_per_split, sp.splits, sp.splits,
                                                         nullptr, 0, d_status, st, "gemm_tc_kernel(wgrad)");
     if (rc != SPA_OK) return rc;
@@ -571,12 +584,12 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
     int grid = (int)((n_w / 4 + 255) / 256);
     if (grid > kNumSMs * 8) grid = kNumSMs * 8;
     grid += (int)((n_b / 4 + 7) / 8);  // the blocks of the bias gradient come first
-    launch_pdl(split_reduce_kernel, grid, 256, 0, st, part_w, n_w, part_b, n_b, sp.splits, rpc, cu, p.B, p.capacity, dW,
-               db);
+    launch_pdl(split_reduce_kernel, grid, 256, 0, st, part_w, n_w, part_b, n_b, splits, pair ? 0 : rpc, pl.tiles_n, cu, p.B, p.capacity,
+               dW, db);
     SPA_CUDA_CHECK_LAUNCH("split_reduce_kernel");
   } else {  // db alone
     launch_pdl(split_reduce_kernel, (n_out / 4 + 7) / 8, 256, 0, st, (const float*)nullptr, 0LL, (const float*)part_b,
-               (long long)n_out, 0, rpc, cu, p.B, p.capacity, (float*)nullptr, db);
+               (long long)n_out, 0, rpc, 0, cu, p.B, p.capacity, (float*)nullptr, db);
     SPA_CUDA_CHECK_LAUNCH("split_reduce_kernel(db)");
   }
   return SPA_OK;

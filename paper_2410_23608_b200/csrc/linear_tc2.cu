@@ -48,6 +48,9 @@ __device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t cluster_bar, uin
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_bar) {  // publishes this CTA's writes to the pair
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
 // tiled load into this CTA's shared memory, completion counted on a barrier of the pair (leader's)
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, uint32_t cluster_bar, int x, int y) {
   asm volatile(
@@ -285,7 +288,248 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   }
 }
 
+// ------------------------------------------------------------------------------------------------ weight gradient
+// dW[n_out][n_in] = dout^T a on CTA pairs: both operands MN-major, K = the device-side packed row count, split over the
+// pairs that are resident at once.  The splits are dealt the 64-row blocks of K in turn (split z takes blocks z, z + S,
+// ...) and each leaves its fp32 tile in the workspace for the fixed-order reduction.  A pair reads 32 KB per CTA and
+// k-block for 256 x 256 x 64 products, half of what two 128 x 128 tiles on an SM need, which were bound by it.
+//   Rows past the last packed one: the last k-block of K is loaded on a barrier of each CTA's own, its producer warp
+//   zeroes the lines, and only then reports the stage to the leader.
+//   Bias gradient: db[m] = sum_k dout[k][m] is the product with a matrix of ones, 16 columns wide, into TMEM columns
+//   behind the tile's; the tiles of a row of tiles take the k-blocks of it in turn (every sum of bf16 values is exact
+//   up to the fp32 additions, as before).  A column-sum kernel over dout cost 9-11 us where this adds under 1.
+// One accumulator: all tiles x splits are resident at once (up to layers of 4.8 M weights), so there is no next tile
+// whose main loop an epilogue could run under.
+constexpr int kWgSmem = kPairSmem + 1024;  // and the 8 x 64 block of ones
+
+__global__ void __launch_bounds__(kPairThreads)
+wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ part,
+                  float* __restrict__ part_b, int M, int N, int splits, const int32_t* __restrict__ cu, int n_seg,
+                  int capacity, int32_t* d_status) {
+  constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(2 * PM, PN, true, true);
+  constexpr uint32_t kIdescOnes = ptx::idesc_bf16_f32(2 * PM, 16, true, false);
+  constexpr int kBars = kPairStages * kPairStage;
+  pdl_launch_dependents();
+
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* smem_al = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
+  const uint32_t ones_s = smem_base + kBars, bar_base = ones_s + 1024;
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (kPairStages + s); };
+  const uint32_t tmem_full_bar = bar_base + 8u * (2 * kPairStages), tmem_empty_bar = tmem_full_bar + 8, tail_bar = tmem_full_bar + 16;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kBars + 1024 + 192);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kBars + 1024 + 196);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = ptx2::cluster_ctarank();  // 0 = leader
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  if (threadIdx.x == 0) {
+    ptx::prefetch_tensormap(&tmA);
+    ptx::prefetch_tensormap(&tmB);
+    for (int s = 0; s < kPairStages; ++s) {
+      ptx::mbar_init(full_bar(s), 2);
+      ptx::mbar_init(empty_bar(s), 1);
+    }
+    ptx::mbar_init(tmem_full_bar, 1);
+    ptx::mbar_init(tmem_empty_bar, 2 * kPairEpiWarps);
+    ptx::mbar_init(tail_bar, 1);
+    *abort_flag = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 2) {  // 8 rows of 64 ones: the same under any swizzle
+    for (int i = lane; i < 64; i += 32)
+      *reinterpret_cast<uint4*>(smem_al + kBars + i * 16) = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
+    ptx::fence_proxy_async_smem();
+  }
+  if (warp == 1) ptx2::tmem_alloc_pair(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), 2 * PN);
+  ptx::tc_fence_before_sync();
+  __syncthreads();
+  ptx2::cluster_sync();  // both CTAs' barriers exist before either signals the other
+  ptx::tc_fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+
+  pdl_wait();  // everything above touched no global memory
+  const int K = packed_rows(cu, n_seg, capacity);
+  const int tiles_n = (N + PN - 1) / PN, tiles_m = (M + 2 * PM - 1) / (2 * PM);
+  const int k_blocks = (K + PK - 1) / PK;
+  const int n_splits = k_blocks < splits ? k_blocks : splits;
+  const int total = tiles_m * tiles_n * n_splits;
+  struct Item { int m0, n0, n_t, z; };  // first row and column of the pair's tile, its column of tiles, its split
+  auto item_of = [&](int i) {
+    Item c;
+    c.n_t = i % tiles_n;
+    const int rest = i / tiles_n;
+    c.m0 = (rest % tiles_m) * 2 * PM;
+    c.z = rest / tiles_m;
+    c.n0 = c.n_t * PN;
+    return c;
+  };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ TMA producer (one per CTA)
+    int it = 0, tails = 0;
+    for (int i = pair; i < total && !__any_sync(0xffffffffu, *abort_flag != 0); i += n_pairs) {
+      const Item c = item_of(i);
+      const int m0 = c.m0 + (int)rank * PM, n0 = c.n0 + (int)rank * (PN / 2);
+      for (int kb = c.z; kb < k_blocks; kb += n_splits, ++it) {
+        const int s = it % kPairStages, k0 = kb * PK;
+        const uint32_t a_dst = smem_base + s * kPairStage, b_dst = a_dst + PM * PK * 2;
+        const uint32_t lead_full = ptx2::map_to_cta(full_bar(s), 0);
+        const bool tail = k0 + PK > K;
+        if (lane == 0) {
+          if (it >= kPairStages) wait_lane(empty_bar(s), ((it / kPairStages) - 1) & 1);
+          if (!tail) {
+            ptx2::mbar_expect_tx_cluster(lead_full, kPairStage);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ptx2::tma_load_2d_pair(a_dst + j * (PK * 128), &tmA, lead_full, m0 + 64 * j, k0);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ptx2::tma_load_2d_pair(b_dst + j * (PK * 128), &tmB, lead_full, n0 + 64 * j, k0);
+          } else {
+            ptx::mbar_expect_tx(tail_bar, kPairStage);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ptx::tma_load_2d(a_dst + j * (PK * 128), &tmA, tail_bar, m0 + 64 * j, k0);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ptx::tma_load_2d(b_dst + j * (PK * 128), &tmB, tail_bar, n0 + 64 * j, k0);
+          }
+        }
+        __syncwarp();
+        if (tail) {
+          wait(tail_bar, tails & 1);
+          ++tails;
+          const int first = K - k0;  // lines of the four boxes from here on hold no packed row
+          for (int q = lane; q < 4 * (PK - first) * 8; q += 32) {
+            const int box = q / ((PK - first) * 8), r = q % ((PK - first) * 8);
+            *reinterpret_cast<uint4*>(smem_al + s * kPairStage + box * (PK * 128) + (first + r / 8) * 128 + (r % 8) * 16) = make_uint4(0, 0, 0, 0);
+          }
+          ptx::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) ptx2::mbar_arrive_release_cluster(lead_full);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer: the leader's, for the pair
+    if (rank == 0) {
+      const uint64_t ones_desc = ptx::smem_desc_sw128(ones_s, 16, 1024);
+      int it = 0, tl = 0;
+      for (int i = pair; i < total && !__any_sync(0xffffffffu, *abort_flag != 0); i += n_pairs, ++tl) {
+        const Item c = item_of(i);
+        if (tl > 0) wait(tmem_empty_bar, (tl - 1) & 1);
+        ptx::tc_fence_after_sync();
+        bool first = true, first_sum = true;
+        for (int kb = c.z; kb < k_blocks; kb += n_splits, ++it) {
+          const int s = it % kPairStages;
+          wait(full_bar(s), (it / kPairStages) & 1);
+          ptx::tc_fence_after_sync();
+          const uint32_t a_src = smem_base + s * kPairStage, b_src = a_src + PM * PK * 2;
+          const bool sum = part_b != nullptr && (kb / n_splits) % tiles_n == c.n_t;
+          if (ptx::elect_one()) {
+#pragma unroll
+            for (int k = 0; k < PK / 16; ++k)
+              ptx2::mma_bf16_pair(tmem, ptx::smem_desc_sw128(a_src + k * 2048, PK * 128, 1024),
+                                  ptx::smem_desc_sw128(b_src + k * 2048, PK * 128, 1024), kIdesc, (first && k == 0) ? 0u : 1u);
+            if (sum) {
+#pragma unroll
+              for (int k = 0; k < PK / 16; ++k)
+                ptx2::mma_bf16_pair(tmem + PN, ptx::smem_desc_sw128(a_src + k * 2048, PK * 128, 1024), ones_desc, kIdescOnes,
+                                    (first_sum && k == 0) ? 0u : 1u);
+            }
+            ptx2::mma_commit_pair(empty_bar(s));
+            if (kb + n_splits >= k_blocks) ptx2::mma_commit_pair(tmem_full_bar);
+          }
+          first = false;
+          first_sum = first_sum && !sum;
+          __syncwarp();
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue warps (both CTAs)
+    const int q = warp & 3;            // TMEM lane quarter this warp may read
+    const int half = (warp - 2) >> 2;  // which of the two warps of that quarter: even or odd 32-column groups
+    uint8_t* stage = smem_al + kBars + 1024 + 256 + (warp - 2) * 4096;  // this warp's transposition buffer
+    const uint32_t lead_empty = ptx2::map_to_cta(tmem_empty_bar, 0);
+    const int my_chunk = lane & 7, my_row = lane >> 3;
+    int tl = 0;
+    for (int i = pair; i < total; i += n_pairs, ++tl) {
+      const Item c = item_of(i);
+      const int m0 = c.m0 + (int)rank * PM + q * 32;
+      float* obase = part + (long long)c.z * M * N;
+      wait(tmem_full_bar, tl & 1);
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      ptx::tc_fence_after_sync();
+      const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
+      // Thread `lane` receives one accumulator row; 32 columns (128 bytes) at a time are turned around in the warp's
+      // 4 KB, so that a store instruction covers four whole 128-byte lines.
+#pragma unroll 1
+      for (int cc = half; cc < PN / 32; cc += 2) {
+        if (c.n0 + cc * 32 >= N) break;  // warp-uniform: columns past the layer's width
+        uint32_t r[32];
+        ptx::tmem_ld_32x32(lanes + cc * 32, r);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          *reinterpret_cast<uint4*>(stage + lane * 128 + ((e ^ (lane & 7)) << 4)) = make_uint4(r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]);
+        __syncwarp();
+        const int gcol = c.n0 + cc * 32 + my_chunk * 4;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int rr = my_row + 4 * j;
+          const uint4 v = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((my_chunk ^ (rr & 7)) << 4));
+          if (m0 + rr < M && gcol < N) *reinterpret_cast<uint4*>(obase + (long long)(m0 + rr) * N + gcol) = v;
+        }
+        __syncwarp();
+      }
+      if (part_b != nullptr && half == 0) {
+        uint32_t r[16];
+        ptx::tmem_ld_32x16(lanes + PN, r);
+        ptx::tmem_ld_wait();
+        // k-blocks of this split: z, z + S, ...; the tile has taken those whose turn falls on its column of tiles
+        const int mine = (k_blocks - c.z + n_splits - 1) / n_splits;
+        if (m0 + lane < M) part_b[((long long)c.z * tiles_n + c.n_t) * M + m0 + lane] = mine > c.n_t ? __uint_as_float(r[0]) : 0.f;
+      }
+      ptx::tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) ptx2::mbar_arrive_cluster(lead_empty);  // this warp has drained its quarter of the accumulator
+    }
+  }
+  // nobody leaves while the peer may still read this CTA's operands or signal its barriers
+  ptx::tc_fence_before_sync();
+  __syncthreads();
+  ptx2::cluster_sync();
+  if (warp == 1) {
+    ptx::tc_fence_after_sync();
+    ptx2::tmem_dealloc_pair(tmem, 2 * PN);
+  }
+}
+
 constexpr int kMaxPairs = kNumSMs / 2;
+
+// `pairs` clusters of two CTAs
+template <typename... KArgs, typename... Args>
+int launch_clusters(void (*kern)(KArgs...), int pairs, int smem, cudaStream_t st, const char* what, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * pairs);
+  cfg.blockDim = dim3(kPairThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  if (e != cudaSuccess) { set_cuda_error(e, what); return SPA_ERR_CUDA; }
+  SPA_CUDA_CHECK_LAUNCH(what);
+  return SPA_OK;
+}
 
 template <bool kBMn>
 int launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, __nv_bfloat16* out, long long ldo,
@@ -297,28 +541,40 @@ int launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloa
   if (ea != cudaSuccess) { set_cuda_error(ea, what); return SPA_ERR_CUDA; }
   const long long tiles = (long long)((N + PN - 1) / PN) * ((capacity + 2 * PM - 1) / (2 * PM));
   const int pairs = (int)(tiles < kMaxPairs ? (tiles < 1 ? 1 : tiles) : kMaxPairs);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(kPairThreads);
-  cfg.dynamicSmemBytes = kPairSmem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl_enabled() ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, bias, out, ldo, N, K, cu, n_seg, capacity, row_map, accumulate,
-                                     d_status);
-  if (e != cudaSuccess) { set_cuda_error(e, what); return SPA_ERR_CUDA; }
-  SPA_CUDA_CHECK_LAUNCH(what);
-  return SPA_OK;
+  return launch_clusters(kern, pairs, kPairSmem, st, what, tmA, tmB, bias, out, ldo, N, K, cu, n_seg, capacity, row_map, accumulate,
+                         d_status);
 }
 
 }  // namespace
+
+PairWgradPlan pair_wgrad_plan(int capacity, int n_in, int n_out) {
+  PairWgradPlan pl;
+  pl.tiles_n = (n_in + PN - 1) / PN;
+  pl.tiles = pl.tiles_n * ((n_out + 2 * PM - 1) / (2 * PM));
+  // as many splits as keep all tiles x splits resident; at least four k-blocks each when half of the capacity is in
+  // use (a split costs a tile of partial sums written and read); 31 leave room for the bias partials in a workspace of
+  // 32 splits
+  int s = kMaxPairs / pl.tiles;
+  const int by_rows = (capacity / 2 + 4 * PK - 1) / (4 * PK);
+  if (s > by_rows) s = by_rows;
+  if (s > 31) s = 31;
+  pl.splits = s < 1 ? 1 : s;
+  return pl;
+}
+
+int launch_wgrad_pair(const spa_params& p, const void* a, const void* dout, int n_in, int n_out, const int32_t* cu, float* part,
+                      float* part_b, const PairWgradPlan& pl, int32_t* d_status, cudaStream_t st) {
+  CUtensorMap tmA, tmB;
+  if (!make_tmap_bf16_2d(&tmA, dout, n_out, p.capacity, (uint64_t)n_out * 2, 64, PK) ||
+      !make_tmap_bf16_2d(&tmB, a, n_in, p.capacity, (uint64_t)n_in * 2, 64, PK))
+    return SPA_ERR_UNSUPPORTED;
+  static DeviceOnce smem_attr;
+  cudaError_t ea = smem_attr.run([&] { return cudaFuncSetAttribute(wgrad_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem); });
+  if (ea != cudaSuccess) { set_cuda_error(ea, "wgrad_pair_kernel"); return SPA_ERR_CUDA; }
+  const int tiles = pl.tiles * pl.splits;
+  return launch_clusters(wgrad_pair_kernel, tiles < kMaxPairs ? tiles : kMaxPairs, kWgSmem, st, "wgrad_pair_kernel", tmA, tmB, part,
+                         part_b, n_out, n_in, pl.splits, cu, p.B, p.capacity, d_status);
+}
 
 // The pair kernels pay off where the 128 x 128 tiles are operand-feed bound: wide layers with enough
 // rows for several 256 x 256 tiles per pair.

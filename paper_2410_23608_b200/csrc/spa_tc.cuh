@@ -25,6 +25,17 @@ int launch_linear_fwd_pair(const spa_params& p, const void* a, const void* W, co
 int launch_linear_dgrad_pair(const spa_params& p, const void* W, const void* dout, int n_in, int n_out, const int32_t* cu,
                              void* da, int32_t* d_status, cudaStream_t st, const int32_t* row_map, bool accumulate);
 
+// weight gradient on CTA pairs: `splits` partial tiles [splits][n_out][n_in] and, with part_b, splits * tiles_n partial bias
+// gradients [.][n_out]; the splits that have rows (at most the number of 64-row blocks) are written
+struct PairWgradPlan { int splits, tiles_n, tiles; };
+PairWgradPlan pair_wgrad_plan(int capacity, int n_in, int n_out);
+int launch_wgrad_pair(const spa_params& p, const void* a, const void* dout, int n_in, int n_out, const int32_t* cu, float* part,
+                      float* part_b, const PairWgradPlan& pl, int32_t* d_status, cudaStream_t st);
+
+// weight gradient (and db unless NULL) of the narrower layers, K split over clusters, no scratch
+int launch_wgrad_cluster(const spa_params& p, const void* a, const void* dout, int n_in, int n_out, const int32_t* cu, float* dW,
+                         float* db, int32_t* d_status, cudaStream_t st);
+
 bool tc_attention_fwd_supported(const spa_params& p);
 int launch_attention_fwd_tc(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao, float* lse,
                             int32_t* d_status, cudaStream_t st);
