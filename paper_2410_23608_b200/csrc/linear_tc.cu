@@ -518,7 +518,7 @@ size_t tc_linear_workspace_bytes(const spa_params& p) {
 int launch_linear_fwd_tc(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
                          const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st, const int32_t* row_map,
                          bool accumulate) {
-  if (tc_pair_linear_supported(p, n_in, n_out))
+  if (tc_pair_linear_supported(p, n_in, n_out, n_out))
     return launch_linear_fwd_pair(p, a, W, bias, n_in, n_out, cu, out, d_status, st, row_map, accumulate);
   CUtensorMap tmA, tmB;
   if (!make_tmap_bf16_2d(&tmA, a, n_in, p.capacity, (uint64_t)n_in * 2, BK, BM) ||
@@ -540,11 +540,7 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
   if (dW != nullptr && (!make_tmap_bf16_2d(&tmA2, dout, n_out, p.capacity, (uint64_t)n_out * 2, 64, BK) ||
                         !make_tmap_bf16_2d(&tmB2, a, n_in, p.capacity, (uint64_t)n_in * 2, 64, BK)))
     return SPA_ERR_UNSUPPORTED;
-  // A pair CTA owns its SM (all 512 TMEM columns, 175 KB of shared memory).  A call that asks for da alone is
-  // the pattern of a caller that runs the weight gradients beside it on another stream: there the one-CTA
-  // kernel, which shares an SM with them, gives the shorter step; a call that computes everything in
-  // sequence takes the pair kernel for da.
-  const bool pair_dgrad = da != nullptr && (dW != nullptr || db != nullptr) && tc_pair_linear_supported(p, n_in, n_out);
+  const bool pair_dgrad = da != nullptr && tc_pair_linear_supported(p, n_in, n_out, n_in);
   if (pair_dgrad) {
     int rc = launch_linear_dgrad_pair(p, W, dout, n_in, n_out, cu, da, d_status, st, row_map, accumulate);
     if (rc != SPA_OK) return rc;

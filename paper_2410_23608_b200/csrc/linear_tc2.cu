@@ -576,11 +576,13 @@ int launch_wgrad_pair(const spa_params& p, const void* a, const void* dout, int 
                          part_b, n_out, n_in, pl.splits, cu, p.B, p.capacity, d_status);
 }
 
-// The pair kernels pay off where the 128 x 128 tiles are operand-feed bound: wide layers with enough
-// rows for several 256 x 256 tiles per pair.
-bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out) {
+// The pair kernels pay off where every pair gets a 256 x 256 tile (half of the allocated rows stands for the packed
+// ones): 15 120 rows 256 -> 768 13.7 us against 15.0 on single CTAs, 6 272 rows 384 -> 1 152 11.2 against 12.2; with
+// fewer tiles the smaller ones spread better (6 272 rows 384 -> 384: 7.9 against 6.5).
+bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out, int n_cols) {
   if (p.flags & SPA_FLAG_NO_CTA_PAIRS) return false;
-  return n_in % 8 == 0 && n_out % 8 == 0 && n_in >= 512 && n_out >= 512 && p.capacity >= 4096 && tensor_maps_available();
+  const long long tiles = (long long)((p.capacity / 2 + 2 * PM - 1) / (2 * PM)) * ((n_cols + PN - 1) / PN);
+  return n_in % 8 == 0 && n_out % 8 == 0 && tiles >= kMaxPairs && tensor_maps_available();
 }
 
 int launch_linear_fwd_pair(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,

@@ -18,7 +18,7 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
                          cudaStream_t st, const int32_t* row_map = nullptr, bool accumulate = false);
 
 // CTA-pair variants (cta_group::2, 256 x 256 tiles) of the forward product and the input gradient
-bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out);
+bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out, int n_cols);  // n_cols: width of the result
 int launch_linear_fwd_pair(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
                            const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st, const int32_t* row_map,
                            bool accumulate);
