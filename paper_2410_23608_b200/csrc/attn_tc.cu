@@ -17,6 +17,8 @@
 #include <math_constants.h>
 
 #include <mutex>
+#include <unordered_map>
+#include <vector>
 
 #include "sm100_ptx.cuh"
 #include "spa_tc.cuh"
@@ -99,21 +101,136 @@ __device__ __forceinline__ void copy_tile_out(const uint8_t* tile, __nv_bfloat16
   }
 }
 
-template <int D> __host__ __device__ constexpr int fwd_smem_bytes() {
-  // Q + 2 x (K, V), alignment slack, barriers, row-max exchange, segment offsets
-  return 5 * 128 * D * 2 + 1024 + 128 + 2048 + kSegStage * 4 + 64;
+// ---- work items -------------------------------------------------------------------------------------------------
+// The persistent kernels draw their (row tile, head) items from a counter in global memory, longest rows of key tiles
+// first: static strides left the last CTA busy for 1.36 times the mean (detection, 210 to 1 680 rows per segment).
+constexpr int kMaxOrder = 512;  // row tiles that are put in order of length; beyond, there are items enough to even out
+
+// Position of the row tiles [first, n_tiles) in that order (ties in ascending order, so that all CTAs agree):
+// tile[rank], less first.  By kThreads threads behind named barrier `id`, offsets staged; about 1 000 clocks, which fit under the loads of a CTA's first item.
+struct __align__(16) ItemOrder { uint4 cost16[kMaxOrder / 16]; uint16_t tile[kMaxOrder]; };
+template <int kThreads>
+__device__ __forceinline__ void order_items(ItemOrder* o, const int32_t* s_off, int n_seg, int Np, int first, int n_tiles, int id) {
+  uint8_t* cost = reinterpret_cast<uint8_t*>(o->cost16);
+  const int n = n_tiles - first;
+  for (int i = threadIdx.x; i < ((n + 15) & ~15); i += kThreads) {
+    int c = 0;
+    if (i < n) {
+      const int r0 = (first + i) * 128, last = r0 + 127 < Np - 1 ? r0 + 127 : Np - 1;
+      c = (row_segment_staged(s_off, n_seg, Np, last).hi - row_segment_staged(s_off, n_seg, Np, r0).lo + 127) >> 7;
+    }
+    cost[i] = (uint8_t)(c < 255 ? c : 255);
+  }
+  ptx::named_barrier(id, kThreads);
+  for (int i = threadIdx.x; i < n; i += kThreads) {
+    const uint32_t mine = cost[i] * 0x01010101u;
+    int rank = 0;
+    for (int w = 0; w < (n + 15) / 16; ++w) {
+      const uint4 v = o->cost16[w];
+      const uint32_t c[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int below = i - 16 * w - 4 * u;  // tiles of this word in front of tile i
+        const uint32_t front = below >= 4 ? 0x01010101u : (below > 0 ? 0x01010101u & ((1u << (8 * below)) - 1u) : 0u);
+        rank += __popc((__vcmpgtu4(c[u], mine) & 0x01010101u) | (__vcmpeq4(c[u], mine) & front));
+      }
+    }
+    o->tile[rank] = (uint16_t)i;
+  }
 }
 
+// The next item for this CTA, after its first.  The first `given` items (whole row tiles) go to the CTAs of their number,
+// the others are drawn: every CTA draws until it gets a number past the last item, so that a launch takes n_items - given
+// + gridDim.x numbers and the counter wraps to zero with the last of them, for the next launch of the stream.  Without a
+// counter: a static stride.
+__device__ __forceinline__ int draw_item(unsigned* counter, int given, int n_items, int& own) {
+  own += gridDim.x;
+  if (counter == nullptr || n_items <= given) return own;
+  return (int)atomicInc(counter, (unsigned)(n_items - given) + gridDim.x - 1u) + given;
+}
+
+// Segment of packed row `row` (lane l of a converged warp asks for row0 + l); rows from Np on get an empty range.  A
+// 32-way search for the warp's first row, then the offsets behind it, 32 at a time, looked up with shuffles.
+template <typename Load>
+__device__ __forceinline__ RowSeg warp_row_segment(Load off, int n_seg, int Np, int row0) {
+  const int lane = threadIdx.x & 31, row = row0 + lane;
+  RowSeg r{0, 0};
+  if (row0 >= Np) return r;  // the same for the whole warp
+  int lo = 0, n = n_seg;     // off(lo) <= row0, and the segment sought is one of the n from lo on
+  while (n > 1) {
+    const int step = (n + 31) >> 5, at = lo + lane * step;
+    const unsigned le = __ballot_sync(0xffffffffu, lane * step < n && off(at) <= row0);
+    const int k = 31 - __clz(le);  // lane 0 always counts
+    n = n - k * step < step ? n - k * step : step;
+    lo += k * step;
+  }
+  int seg = -1;
+  for (int base = lo;; base += 32) {
+    const int at = base + 1 + lane;
+    const int end = at <= n_seg ? off(at) : 0x7fffffff;  // end of segment base + lane
+    int c = 0;                                           // segments of this group that end at or before the row
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1)
+      if (__shfl_sync(0xffffffffu, end, c + s - 1) <= row) c += s;
+    const int last_end = __shfl_sync(0xffffffffu, end, 31);
+    if (c == 31 && last_end <= row) c = 32;
+    const int hi = __shfl_sync(0xffffffffu, end, c & 31);
+    int start = __shfl_sync(0xffffffffu, end, (c + 31) & 31);
+    if (c == 0) start = off(base);
+    if (seg < 0 && c < 32) { seg = base + c; r.lo = start; r.hi = hi; }
+    if (__all_sync(0xffffffffu, seg >= 0 || row >= Np)) break;
+  }
+  if (row >= Np) return RowSeg{0, 0};
+  if (r.hi > Np) r.hi = Np;
+  return r;
+}
+
+constexpr int kFwdSegStage = 2048;
+constexpr int kEarlySegments = 256;  // eight offsets a lane: their loads are in flight together
+
+// c[j] of lane 4 i + k becomes c[k] of lane 4 i + j
+__device__ __forceinline__ void transpose_quads(uint4 (&c)[4], int lane) {
+  auto swap = [&](uint4& a, uint4& b, int bit) {  // lanes without the bit give b for the other's a
+    const bool up = (lane & bit) != 0;
+    const uint4 give = up ? a : b;
+    uint4 got;
+    got.x = __shfl_xor_sync(0xffffffffu, give.x, bit);
+    got.y = __shfl_xor_sync(0xffffffffu, give.y, bit);
+    got.z = __shfl_xor_sync(0xffffffffu, give.z, bit);
+    got.w = __shfl_xor_sync(0xffffffffu, give.w, bit);
+    (up ? a : b) = got;
+  };
+  swap(c[0], c[1], 1);
+  swap(c[2], c[3], 1);
+  swap(c[0], c[2], 2);
+  swap(c[1], c[3], 2);
+}
+template <int D> struct FwdSmem {
+  // 2 x Q, 2 x K, 2 x V
+  static constexpr int kTile = HeadTile<D>::kTileBytes;
+  static constexpr int kBar = 6 * kTile;                   // 13 barriers, TMEM slot, abort flag, four item slots
+  static constexpr int kXch = kBar + 256;                  // row maxima: [2 tile parities][2 halves][128 rows]
+  static constexpr int kXl = kXch + 2048;                  // row sums: [2 halves][128 rows]
+  static constexpr int kSeg = kXl + 1024;                  // staged segment offsets
+  static constexpr int kOrder = kSeg + (kFwdSegStage + 4) * 4;
+  static constexpr int kBytes = kOrder + (int)sizeof(ItemOrder) + 1024;  // and the alignment of the base
+};
+
+// One persistent pipeline per CTA over all tiles of all its items.  Phases are counted over the whole run, nothing is set
+// up per item and no barrier joins the CTA: while the softmax warps finish an item (normalise, store), the next item's Q,
+// K and V are on their way and its first S product is computed.  What bounds it is the exponentials of the key loop
+// (2 900 clocks per tile with two CTAs on an SM, 71 % of the rate of the unit that computes them); with a prologue per
+// item and static strides an item cost 4 700 to 7 100 clocks outside its loop.  Before and after: 16 segments of 210 to
+// 1 680 rows, 8 heads of 32: 84 -> 67 us; of 64: 74 -> 55; 32 segments of 58 to 518 rows, 12 heads of 64: 40 -> 34;
+// 128 segments of 98 to 196 rows, 12 heads of 64: 54 -> 51; one segment of 98 rows: 6.0 us, as before.
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 2)
 attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __restrict__ seg, int n_seg, int capacity,
                    int C, int H, float scale_log2e, __nv_bfloat16* __restrict__ ao, float* __restrict__ lse,
-                   int32_t* d_status) {
+                   unsigned* counter, bool even_items, int32_t* d_status) {
   using HT = HeadTile<D>;
+  using SM = FwdSmem<D>;
   constexpr int kTile = HT::kTileBytes;
-  // A CTA takes the work items blockIdx.x, blockIdx.x + gridDim.x, ... of the (tile, head) pairs that the device-side
-  // row count leaves (heads fastest, so that CTAs running side by side share their K / V tiles in L2): no CTA is
-  // launched for rows that do not exist, and TMEM and the staged segment offsets are set up once per CTA.
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool is_softmax = warp < kSoftmaxThreads / 32;  // warps 0-7; warp 8 issues the copies and the products
   // warps w and w + 4 may touch the same quarter of the TMEM lanes: they share 32 query rows and split
@@ -123,331 +240,425 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_al = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-  const uint32_t q_s = smem_base;
-  auto k_s = [&](int st) { return smem_base + kTile * (1 + 2 * st); };
-  auto v_s = [&](int st) { return smem_base + kTile * (2 + 2 * st); };
-  const uint32_t bar_base = smem_base + 5 * kTile;
-  const uint32_t bar_q = bar_base, bar_s = bar_base + 40, bar_o = bar_base + 48;
-  const uint32_t bar_sfree = bar_base + 56;   // 8 arrivals: every softmax warp holds its part of S_t in registers
-  const uint32_t bar_pready = bar_base + 64;  // 8 arrivals: every softmax warp has written its part of P_t
-  auto bar_k = [&](int st) { return bar_base + 8 + 8 * st; };
-  auto bar_v = [&](int st) { return bar_base + 24 + 8 * st; };
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + 5 * kTile + 72);
-  volatile int* abort_any = reinterpret_cast<volatile int*>(smem_al + 5 * kTile + 76);
-  volatile int* range = reinterpret_cast<volatile int*>(smem_al + 5 * kTile + 80);
-  // [2 tile parities][4 quarters]: written by the two warps of a quarter before their barrier, read after it
-  volatile int* abort_pair = reinterpret_cast<volatile int*>(smem_al + 5 * kTile + 88);
-  float* xch = reinterpret_cast<float*>(smem_al + 5 * kTile + 128);  // [2 tile parities][2 halves][128 rows]
-  int32_t* seg_s = reinterpret_cast<int32_t*>(smem_al + 5 * kTile + 128 + 2048);  // [kSegStage + 1]
+  auto q_s = [&](int b) { return smem_base + kTile * b; };
+  auto k_s = [&](int st) { return smem_base + kTile * (2 + st); };
+  auto v_s = [&](int st) { return smem_base + kTile * (4 + st); };
+  const uint32_t bar = smem_base + SM::kBar;
+  auto bar_q = [&](int b) { return bar + 8 * b; };            // Q of an item has landed
+  auto bar_item = [&](int b) { return bar + 32 + 8 * b; };    // the item slot is filled
+  auto bar_k = [&](int st) { return bar + 48 + 8 * st; };
+  auto bar_v = [&](int st) { return bar + 64 + 8 * st; };
+  const uint32_t bar_s = bar + 80, bar_o = bar + 88;
+  const uint32_t bar_sfree = bar + 96;    // 8 arrivals: every softmax warp holds its part of S_t in registers
+  const uint32_t bar_pready = bar + 104;  // 8 arrivals: every softmax warp has written its part of P_t
+  const uint32_t bar_order = bar + 16;    // 8 arrivals: the order of the items is there
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + SM::kBar + 112);
+  const uint32_t abort_any = bar + 116;
+  auto item_slot = [&](int item) { return bar + 128 + 16 * (item & 3); };  // {q0, h, kv_lo, n_tiles}; 64 bytes on: {valid lines of the last tile, valid rows}
+  float* xch = reinterpret_cast<float*>(smem_al + SM::kXch);
+  float* xl = reinterpret_cast<float*>(smem_al + SM::kXl);
+  int32_t* seg_s = reinterpret_cast<int32_t*>(smem_al + SM::kSeg);
+  ItemOrder* order = reinterpret_cast<ItemOrder*>(smem_al + SM::kOrder);
 
-  // The thread that sets the barriers up is the one that later issues the copies counted on them (program order: no
-  // copy can meet a barrier that is not initialised yet).
-  auto init_barriers = [&]() {
-    ptx::mbar_init(bar_q, 1);
-    for (int s = 0; s < 2; ++s) { ptx::mbar_init(bar_k(s), 1); ptx::mbar_init(bar_v(s), 1); }
+  // The thread that sets the barriers up belongs to the warp that later issues the copies counted on them.
+  if (tid == kSoftmaxThreads) {
+    ptx::prefetch_tensormap(&tm);
+    for (int b = 0; b < 2; ++b) {
+      ptx::mbar_init(bar_q(b), 1);
+      ptx::mbar_init(bar_item(b), 1);
+      ptx::mbar_init(bar_k(b), 1);
+      ptx::mbar_init(bar_v(b), 1);
+    }
     ptx::mbar_init(bar_s, 1);
     ptx::mbar_init(bar_o, 1);
     ptx::mbar_init(bar_sfree, kSoftmaxThreads / 32);
     ptx::mbar_init(bar_pready, kSoftmaxThreads / 32);
-    *abort_any = 0;
-    for (int i = 0; i < 8; ++i) abort_pair[i] = 0;
+    ptx::mbar_init(bar_order, kSoftmaxThreads / 32);
+    ptx::sts_s32(abort_any, 0);
     ptx::fence_mbar_init();
-  };
-  // everything up to the wait touches no global memory, so it runs under the previous kernel's tail
-  if (tid == kSoftmaxThreads) {
-    ptx::prefetch_tensormap(&tm);
-    init_barriers();
   }
-  pdl_entry();
-  const bool staged = n_seg < kSegStage;
+  pdl_entry();  // everything up to the wait touches no global memory
+  const bool staged = n_seg < kFwdSegStage;
   if (staged)
     for (int i = tid; i <= n_seg; i += kFwdThreads) seg_s[i] = ld_dep(seg + i);
   const int Np = packed_rows(seg, n_seg, capacity);
-  const int n_items = ((Np + kQ - 1) / kQ) * H;
+  const int row_tiles = (Np + kQ - 1) / kQ, n_items = row_tiles * H;
   if ((int)blockIdx.x >= n_items) return;
   if (warp == 0) ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
-  bool cta_failed = false;
-  for (int item = blockIdx.x; item < n_items && !cta_failed; item += gridDim.x) {
-  const int h = item % H, q0 = (item / H) * kQ;
-  if (tid == kSoftmaxThreads) {
-    if (item != (int)blockIdx.x) {  // every phase of the previous item has completed: the barriers start over
-      ptx::mbar_inval(bar_q);
-      for (int s = 0; s < 2; ++s) { ptx::mbar_inval(bar_k(s)); ptx::mbar_inval(bar_v(s)); }
-      ptx::mbar_inval(bar_s);
-      ptx::mbar_inval(bar_o);
-      ptx::mbar_inval(bar_sfree);
-      ptx::mbar_inval(bar_pready);
-      init_barriers();
+  // Items are drawn behind the whole row tiles that the CTAs start with; longest first where their lengths differ, where
+  // they are few enough to be put in order, and where CTAs take 1.5 of them or more (below that, who ends first takes
+  // the rest: with 300 to 320 items for 296 CTAs the order cost 3 %, with 432 it was even, with 576 it gained 6 %).
+  const bool draws = counter != nullptr && n_items > (int)gridDim.x;
+  const int given = draws ? (int)gridDim.x / H * H : n_items;
+  const bool ordered = !even_items && draws && staged && 2 * n_items >= 3 * (int)gridDim.x && row_tiles - given / H <= kMaxOrder;
+  // The issuing warp gets the key rows of the CTA's first item straight from the offsets, of which a lane takes a few,
+  // and starts its copies before the CTA comes together.
+  const bool early = !is_softmax && n_seg < kEarlySegments && !(draws && (int)blockIdx.x >= given);
+  int early_lo = 0, early_hi = Np;
+  if (early) {
+    const int q0 = (int)blockIdx.x / H * kQ, h = (int)blockIdx.x % H;
+#pragma unroll 4
+    for (int i = lane; i <= n_seg; i += 32) {
+      const int o = ld_dep(seg + i);
+      if (o <= q0 && o > early_lo) early_lo = o;
+      if (o > q0 + kQ - 1 && o < early_hi) early_hi = o;
     }
-    // the Q tile depends only on q0: fetch it under the segment search
-    ptx::mbar_expect_tx(bar_q, kTile);
-    ptx::tma_load_2d(q_s, &tm, bar_q, h * D, q0);
+    early_lo = __reduce_max_sync(0xffffffffu, early_lo);
+    early_hi = __reduce_min_sync(0xffffffffu, early_hi);
+    if (ptx::elect_one()) {
+      ptx::mbar_expect_tx(bar_q(0), kTile);
+      ptx::tma_load_2d(q_s(0), &tm, bar_q(0), h * D, q0);
+      ptx::mbar_expect_tx(bar_k(0), kTile);
+      ptx::tma_load_2d(k_s(0), &tm, bar_k(0), C + h * D, early_lo);
+      ptx::mbar_expect_tx(bar_v(0), kTile);
+      ptx::tma_load_2d(v_s(0), &tm, bar_v(0), 2 * C + h * D, early_lo);
+    }
+    __syncwarp();
   }
   ptx::tc_fence_before_sync();
   __syncthreads();  // barriers, TMEM address and staged offsets are visible
   ptx::tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-
-  const int row = q0 + rl;
-  RowSeg mine{0, 0};
-  if (is_softmax) {
-    mine = staged ? row_segment_staged(seg_s, n_seg, Np, row) : row_segment(seg, n_seg, Np, row);
-    if (half == 0) {
-      const int last = (q0 + kQ - 1 < Np - 1) ? q0 + kQ - 1 : Np - 1;
-      if (row == q0) range[0] = mine.lo;
-      if (row == last) range[1] = mine.hi;
-    }
-  }
-  __syncthreads();
   const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;  // TMEM lanes this warp may touch
-  float lse_m = 0.f;
-  constexpr int kCols = kKV / 2;  // key columns of each tile owned by this thread
-  constexpr int kDh = D / 2;      // head dimensions of O owned by this thread
-  const int col0 = half * kCols;
-  const int kv_lo = range[0], kv_hi = range[1];
-  const int n_tiles = (kv_hi - kv_lo + kKV - 1) / kKV;
+  auto off = [&](int i) { return staged ? seg_s[i] : ld_dep(seg + i); };
 
   constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(kQ, kKV, false, false);
   constexpr uint32_t kIdescO = ptx::idesc_bf16_f32(kQ, D, false, true);
+  // Bounded; nobody branches on a wait that gave up inside an item (see mbar_wait_or_abort)
+  auto wait = [&](uint32_t b, uint32_t parity) { ptx::mbar_wait_or_abort_warp(b, parity, abort_any, d_status, SPA_ERR_TIMEOUT); };
 
-  // Bounded wait that also gives up as soon as any thread of the CTA has reported a failure.
-  auto wait = [&](uint32_t bar, uint32_t parity) {
-    for (uint32_t i = 0; i < ptx::kWaitLimit; ++i) {
-      if (ptx::mbar_try_wait(bar, parity)) return true;
-      if ((i & 255u) == 255u && *abort_any) return false;
-    }
-    return false;
-  };
-
-  // every lane polls (measured faster than one lane polling for the warp); the warp takes one answer
-  auto wait_w = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, wait(bar, parity)) != 0; };
   if (!is_softmax) {
     // ---------------------------------------------------------------- copies and products: one warp, whose lanes
-    // all follow the tiles and take every wait together; one elected lane issues (see ptx::elect_one)
-    auto load_k = [&](int t) {
-      if (ptx::elect_one()) {
-        ptx::mbar_expect_tx(bar_k(t & 1), kTile);
-        ptx::tma_load_2d(k_s(t & 1), &tm, bar_k(t & 1), C + h * D, kv_lo + t * kKV);
+    // all follow the tiles and take every wait together; one elected lane issues (see ptx::elect_one).  Three cursors
+    // run over the same sequence of tiles: the one whose P V product is next, the one whose S product is next, and the
+    // one whose K tile is loaded next, which draws the items.
+    struct Cursor { int item, t, n_tiles, h, kv0, q0; };  // item number of this CTA, tile of it; n_tiles 0: past the end
+    int own = blockIdx.x, drawn = blockIdx.x;             // static stride without a counter; a number drawn a tile ahead
+    if (draws && (int)blockIdx.x >= given) {
+      if (lane == 0) drawn = draw_item(counter, given, n_items, own);
+    }
+    bool order_ready = false;
+    bool more = true;                                     // numbers are drawn until one lies past the last item
+    auto announce = [&](const Cursor& c) {
+      if (lane == 0) {
+        const uint32_t slot = item_slot(c.item);
+        ptx::sts_s32(slot, c.q0);
+        ptx::sts_s32(slot + 4, c.h);
+        ptx::sts_s32(slot + 8, c.kv0);
+        ptx::sts_s32(slot + 12, c.n_tiles);
+        ptx::sts_s32(slot + 64, Np - (c.kv0 + (c.n_tiles - 1) * kKV));
+        ptx::sts_s32(slot + 68, Np - c.q0);
+        ptx::mbar_arrive(bar_item(c.item & 1));
+        // the next number, a tile before it is needed
+        if (c.n_tiles == 1) drawn = draw_item(counter, given, n_items, own);
+      }
+    };
+    auto next_item = [&](Cursor& c) {
+      const int v = __shfl_sync(0xffffffffu, drawn, 0);
+      ++c.item;
+      c.t = 0;
+      c.n_tiles = 0;
+      if (v < n_items) {
+        const int rank = v / H;
+        c.h = v - rank * H;
+        const bool by_order = ordered && v >= given;
+        if (by_order && !order_ready) {
+          wait(bar_order, 0);
+          order_ready = true;
+        }
+        const int at = by_order ? order->tile[rank - given / H] : 0;  // tile number, less the given ones
+        c.q0 = (by_order ? given / H + at : rank) * kQ;
+        int lo, hi;
+        const int last = c.q0 + kQ - 1 < Np - 1 ? c.q0 + kQ - 1 : Np - 1;
+        if (staged) {  // both ends at once
+          const RowSeg s = row_segment_staged(seg_s, n_seg, Np, lane < 16 ? c.q0 : last);
+          lo = __shfl_sync(0xffffffffu, s.lo, 0);
+          hi = __shfl_sync(0xffffffffu, s.hi, 16);
+        } else {
+          const int r1 = last >= 31 ? last - 31 : 0;
+          lo = __shfl_sync(0xffffffffu, warp_row_segment(off, n_seg, Np, c.q0).lo, 0);
+          hi = __shfl_sync(0xffffffffu, warp_row_segment(off, n_seg, Np, r1).hi, last - r1);
+        }
+        c.kv0 = lo;
+        c.n_tiles = (hi - lo + kKV - 1) / kKV;
+      } else {
+        more = false;
+      }
+      announce(c);
+      // Q of the item two before is no longer needed: this cursor is at most two tiles ahead of the last S columns that
+      // the softmax warps have taken
+      if (c.n_tiles > 0 && ptx::elect_one()) {
+        ptx::mbar_expect_tx(bar_q(c.item & 1), kTile);
+        ptx::tma_load_2d(q_s(c.item & 1), &tm, bar_q(c.item & 1), c.h * D, c.q0);
       }
       __syncwarp();
     };
-    auto load_v = [&](int t) {
+    auto advance = [&](Cursor& c) {
+      if (++c.t < c.n_tiles) {
+        c.kv0 += kKV;
+        if (c.t == c.n_tiles - 1 && lane == 0) drawn = draw_item(counter, given, n_items, own);
+      } else {
+        next_item(c);
+      }
+    };
+    auto load = [&](const Cursor& c, int g, bool v) {  // K or V of tile g
+      const int st = g & 1;
+      const uint32_t b = v ? bar_v(st) : bar_k(st);
       if (ptx::elect_one()) {
-        ptx::mbar_expect_tx(bar_v(t & 1), kTile);
-        ptx::tma_load_2d(v_s(t & 1), &tm, bar_v(t & 1), 2 * C + h * D, kv_lo + t * kKV);
+        ptx::mbar_expect_tx(b, kTile);
+        ptx::tma_load_2d(v ? v_s(st) : k_s(st), &tm, b, (v ? 2 : 1) * C + c.h * D, c.kv0);
       }
       __syncwarp();
     };
-    auto issue_qk = [&](int t) {  // S = Q K_t^T into TMEM; bar_s completes when it is done
-      if (!wait_w(bar_k(t & 1), (t >> 1) & 1)) return false;
+    auto issue_qk = [&](const Cursor& c, int g) {  // S = Q K^T of tile g into TMEM; bar_s completes when it is done
+      if (c.t == 0) wait(bar_q(c.item & 1), (c.item >> 1) & 1);
+      wait(bar_k(g & 1), (g >> 1) & 1);
       ptx::tc_fence_after_sync();
-      const uint32_t ka = k_s(t & 1);
+      const uint32_t qa = q_s(c.item & 1), ka = k_s(g & 1);
       if (ptx::elect_one()) {
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
-          ptx::mma_bf16(tmem + kColS, HT::kmajor(q_s, k), HT::kmajor(ka, k), kIdescS, k != 0 ? 1u : 0u);
+          ptx::mma_bf16(tmem + kColS, HT::kmajor(qa, k), HT::kmajor(ka, k), kIdescS, k != 0 ? 1u : 0u);
         ptx::mma_commit(bar_s);
       }
       __syncwarp();
-      return true;
     };
-    int loads_k = 0, loads_v = 0;  // tiles whose loads have been issued
-    bool ok = true;
-    if (n_tiles > 0) {
-      load_k(0);
-      load_v(0);
-      loads_k = loads_v = 1;
-      if (n_tiles > 1) { load_k(1); loads_k = 2; }
-      ok = wait_w(bar_q, 0) && issue_qk(0);
+    Cursor ck{-1, 0, 0, 0, 0, 0};
+    if (early) {
+      ck = Cursor{0, 0, (early_hi - early_lo + kKV - 1) / kKV, (int)blockIdx.x % H, early_lo, (int)blockIdx.x / H * kQ};
+      announce(ck);
+    } else {
+      next_item(ck);
     }
-    for (int t = 0; ok && t < n_tiles; ++t) {
-      // every softmax thread holds its S_t columns: the S columns and K stage t & 1 are free
-      if (!(ok = wait_w(bar_sfree, t & 1))) break;
-      if (t + 1 < n_tiles) {
-        if (!(ok = issue_qk(t + 1))) break;  // runs on the tensor core under the softmax of tile t
-        if (t + 2 < n_tiles) { load_k(t + 2); loads_k = t + 3; }
+    Cursor cp = ck, cs = ck;  // tiles of the next P V product, the next S product; ck: of the next K load
+    int g = 0, gk = 0, gv = 0;  // number of the tile of cp; tiles whose K and V loads have been issued
+    if (cp.n_tiles > 0) {
+      if (!early) {
+        load(cp, 0, false);
+        load(cp, 0, true);
       }
-      // P_t is in TMEM, O has been rescaled where needed, and the previous P V product has completed
-      if (!(ok = wait_w(bar_pready, t & 1))) break;
-      if (!(ok = wait_w(bar_v(t & 1), (t >> 1) & 1))) break;
+      gk = gv = 1;
+      const bool same = cp.n_tiles > 1;  // a second item's number may still be on its way: after the first product
+      if (!same) issue_qk(cs, 0);
+      advance(ck);
+      if (ck.n_tiles > 0) {
+        load(ck, 1, false);
+        gk = 2;
+      }
+      if (same) issue_qk(cs, 0);
+      cs = ck;
+    }
+    while (cp.n_tiles > 0 && !__any_sync(0xffffffffu, ptx::lds_s32(abort_any) != 0)) {
+      // every softmax thread holds its columns of S of tile g: the S columns and K stage g & 1 are free
+      wait(bar_sfree, g & 1);
+      const Cursor cn = cs;  // tile g + 1
+      if (cs.n_tiles > 0) {
+        issue_qk(cs, g + 1);  // runs on the tensor core under the softmax of tile g
+        advance(ck);
+        if (ck.n_tiles > 0) {
+          load(ck, g + 2, false);
+          gk = g + 3;
+        }
+        cs = ck;
+      }
+      // P of tile g is in TMEM, O has been rescaled where needed, and the P V product before has completed
+      wait(bar_pready, g & 1);
+      wait(bar_v(g & 1), (g >> 1) & 1);
       ptx::tc_fence_after_sync();
-      const uint32_t va = v_s(t & 1);
+      const uint32_t va = v_s(g & 1);
       if (ptx::elect_one()) {
 #pragma unroll
         for (int k = 0; k < kKV / 16; ++k)
-          ptx::mma_bf16_ts(tmem + kColO, tmem + kColP + k * 8, HT::mnmajor(va, k), kIdescO, (k != 0 || t > 0) ? 1u : 0u);
+          ptx::mma_bf16_ts(tmem + kColO, tmem + kColP + k * 8, HT::mnmajor(va, k), kIdescO, (k != 0 || cp.t > 0) ? 1u : 0u);
         ptx::mma_commit(bar_o);
       }
       __syncwarp();
-      if (t + 1 < n_tiles) { load_v(t + 1); loads_v = t + 2; }  // its stage held V of tile t - 1
+      if (cn.n_tiles > 0) {  // its V stage held V of tile g - 1
+        load(cn, g + 1, true);
+        gv = g + 2;
+      }
+      cp = cn;
+      ++g;
     }
-    if (!ok && lane == 0) {
-      record_status(d_status, SPA_ERR_TIMEOUT);
-      *abort_any = 1;
-      // let outstanding loads land before shared memory is released
-      for (int t = loads_k > 2 ? loads_k - 2 : 0; t < loads_k; ++t) ptx::mbar_wait(bar_k(t & 1), (t >> 1) & 1);
-      for (int t = loads_v > 2 ? loads_v - 2 : 0; t < loads_v; ++t) ptx::mbar_wait(bar_v(t & 1), (t >> 1) & 1);
-      ptx::mbar_wait(bar_q, 0);
+    if (__any_sync(0xffffffffu, ptx::lds_s32(abort_any) != 0) && lane == 0) {
+      // let outstanding loads land before shared memory is released; the numbers drawn have to add up all the same
+      for (int i = gv > 2 ? gv - 2 : 0; i < gv; ++i) ptx::mbar_wait(bar_v(i & 1), (i >> 1) & 1);
+      for (int i = gk > 2 ? gk - 2 : 0; i < gk; ++i) ptx::mbar_wait(bar_k(i & 1), (i >> 1) & 1);
+      const int q_last = ck.n_tiles > 0 ? ck.item : ck.item - 1;  // last item whose Q tile has been asked for
+      for (int i = q_last > 1 ? q_last - 1 : 0; i <= q_last; ++i) ptx::mbar_wait(bar_q(i & 1), (i >> 1) & 1);
+      while (more && draws && drawn < n_items) drawn = draw_item(counter, given, n_items, own);
     }
+    __syncwarp();
   } else {
     // ---------------------------------------------------------------- online softmax: two threads per query row
-    float m = -CUDART_INF_F, l = 0.f;  // m: the maximum the stored P and O refer to (may lag the true one by kRescaleGap)
-    const unsigned span = (unsigned)(mine.hi - mine.lo);
-    auto fail = [&](int slot) {
-      record_status(d_status, SPA_ERR_TIMEOUT);
-      abort_pair[slot * 4 + quarter] = 1;
-      *abort_any = 1;
-    };
-    for (int t = 0; t < n_tiles; ++t) {
-      const int st = t & 1;
-      const int kv0 = kv_lo + t * kKV;
-      // ---- S_t into registers: TMEM loads in flight together, one wait
-      if (!wait_w(bar_s, t & 1)) fail(t & 1);
-      ptx::tc_fence_after_sync();
-      uint32_t s[kCols];
-#pragma unroll
-      for (int c = 0; c < kCols / 32; ++c) ptx::tmem_ld_32x32(tmem + lane_base + kColS + col0 + c * 32, s + c * 32);
-      ptx::tmem_ld_wait();
-      // Which of this thread's groups of 32 key columns meet its row's segment at all (the others take no
-      // arithmetic: their P is zero); the mask is applied only where a boundary of the segment crosses a group.
-      // This half's row maximum is handed to the partner thread through shared memory.
-      const int kc0 = kv0 + col0;
-      bool need[kCols / 32];
-#pragma unroll
-      for (int c = 0; c < kCols / 32; ++c) {
-        const int g0 = kc0 + c * 32;
-        need[c] = g0 < mine.hi && g0 + 32 > mine.lo;
-        if (need[c] && !(g0 >= mine.lo && g0 + 32 <= mine.hi)) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if ((unsigned)(g0 + j - mine.lo) >= span) s[c * 32 + j] = 0xff800000u;  // -inf
-        }
-      }
-      float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-#pragma unroll
-      for (int c = 0; c < kCols / 32; ++c) {
-        if (need[c]) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) mx[u] = fmaxf(mx[u], __uint_as_float(s[c * 32 + j + u]));
-          }
-        }
-      }
-      float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-      xch[((t & 1) * 2 + half) * 128 + rl] = mt;
-      ptx::tc_fence_before_sync();
-      ptx::named_barrier(1 + quarter, 64);  // the two warps that share these 32 rows
-      if (abort_pair[(t & 1) * 4 + quarter]) break;
-      if (lane == 0) ptx::mbar_arrive(bar_sfree);
-
-      // ---- this half row's P (exp2 domain): one fma, one ex2 and one add per key.  The maximum that P and O
-      // refer to is raised only when the true one has grown by more than kRescaleGap, so O (accumulated in
-      // TMEM over all tiles) is rescaled rarely; sums and outputs are exact for any such reference value.
-      mt = fmaxf(mt, xch[((t & 1) * 2 + (half ^ 1)) * 128 + rl]);
-      const float m_cand = fmaxf(m, mt * scale_log2e);  // the scale is positive: max commutes with it
-      const bool raise = m_cand > m + kRescaleGap;      // also the first tile that has a key of this row
-      const float m_new = raise ? m_cand : m;
-      const float m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
-      const float alpha = raise ? ptx::ex2_approx(m - m_use) : 1.f;
-      float rs0 = 0.f, rs1 = 0.f;
-      uint32_t pk[kCols / 2];
-#pragma unroll
-      for (int c = 0; c < kCols / 32; ++c) {
-        if (need[c]) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const float p0 = ptx::ex2_approx(fmaf(__uint_as_float(s[c * 32 + j]), scale_log2e, -m_use));  // -inf -> 0
-            const float p1 = ptx::ex2_approx(fmaf(__uint_as_float(s[c * 32 + j + 1]), scale_log2e, -m_use));
-            rs0 += p0;
-            rs1 += p1;
-            __nv_bfloat162 b = __floats2bfloat162_rn(p0, p1);  // low half = even key
-            pk[c * 16 + (j >> 1)] = *reinterpret_cast<uint32_t*>(&b);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) pk[c * 16 + j] = 0u;
-        }
-      }
-      // ---- the previous P V product must have completed before P is overwritten or O rescaled
-      if (t > 0) {
-        if (!wait_w(bar_o, (t - 1) & 1)) fail((t + 1) & 1);
-        ptx::tc_fence_after_sync();
-        if (__any_sync(0xffffffffu, raise)) {
-          uint32_t r[kDh];
-          if (kDh == 32) ptx::tmem_ld_32x32(tmem + lane_base + kColO + half * kDh, r);
-          else ptx::tmem_ld_32x16(tmem + lane_base + kColO + half * kDh, r);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < kDh; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-          if (kDh == 32) ptx::tmem_st_32x32(tmem + lane_base + kColO + half * kDh, r);
-          else ptx::tmem_st_32x16(tmem + lane_base + kColO + half * kDh, r);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kCols / 32; ++c)
-        ptx::tmem_st_32x16(tmem + lane_base + kColP + (col0 >> 1) + c * 16, pk + c * 16);
-      ptx::tmem_st_wait();
-      l = l * alpha + (rs0 + rs1);
-      m = m_new;
-      // ---- V lines past the last valid packed row must not reach the product
-      if (kv0 + kKV > Np) {
-        if (!wait(bar_v(st), (t >> 1) & 1)) fail((t + 1) & 1);
-        const int first = Np - kv0;  // >= 1
-        constexpr int kChunks = HT::kRowBytes / 16;
-        for (int c = tid; c < (kKV - first) * kChunks; c += kSoftmaxThreads)
-          *reinterpret_cast<uint4*>(smem_al + kTile * (2 + 2 * st) + (first + c / kChunks) * HT::kRowBytes +
-                                    (c % kChunks) * 16) = make_uint4(0, 0, 0, 0);
-        ptx::fence_proxy_async_smem();
-      }
-      ptx::tc_fence_before_sync();
+    constexpr int kCols = kKV / 2;  // key columns of each tile owned by this thread
+    constexpr int kDh = D / 2;      // head dimensions of O owned by this thread
+    const int col0 = half * kCols;
+    int g = 0;                      // tiles so far
+    if (ordered) {
+      order_items<kSoftmaxThreads>(order, seg_s, n_seg, Np, given / H, row_tiles, 5);
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(bar_pready);
+      if (lane == 0) ptx::mbar_arrive(bar_order);
     }
-    // the last product completes O
-    const bool gave_up = __shfl_sync(0xffffffffu, *abort_any, 0) != 0;  // one answer per warp
-    if (n_tiles > 0 && !gave_up && !wait_w(bar_o, (n_tiles - 1) & 1)) fail(0);
-    xch[half * 128 + rl] = l;  // the two halves of a row share the reference maximum but kept separate sums
-    lse_m = m;
-  }
-  ptx::tc_fence_before_sync();
-  __syncthreads();  // nobody reports a failure from here on: the branches below are taken by all threads or by none
-  ptx::tc_fence_after_sync();
-  const bool failed = *abort_any != 0;
-  if (!failed && is_softmax) {
-    // normalised rows go to the Q tile's shared memory (idle now: every product has completed) as bf16 and
-    // leave from there as whole lines
-    uint32_t r[kDh];
-    if (n_tiles > 0) {
+    for (int it = 0;; ++it) {
+      wait(bar_item(it & 1), (it >> 1) & 1);
+      // four slots: this one is read again behind the loop, when the item two further on may have been announced
+      int left = ptx::lds_s32(item_slot(it) + 12);  // tiles still to come
+      // the two warps of a quarter leave together, at the end or after a failure
+      if (ptx::named_barrier_or(1 + quarter, 64, left == 0 || ptx::lds_s32(abort_any) != 0)) break;
+      RowSeg mine;
+      if (staged) mine = row_segment_staged(seg_s, n_seg, Np, ptx::lds_s32(item_slot(it)) + rl);
+      else mine = warp_row_segment(off, n_seg, Np, ptx::lds_s32(item_slot(it)) + quarter * 32);
+      // the row's segment relative to this thread's first key column of the tile; it moves down tile by tile
+      int lo = mine.lo - ptx::lds_s32(item_slot(it) + 8) - col0, hi = mine.hi - mine.lo + lo;
+      bool first = true;
+      float m = -CUDART_INF_F, l = 0.f;  // m: the maximum the stored P and O refer to (may lag the true one by kRescaleGap)
+      for (; left > 0; --left, ++g, lo -= kKV, hi -= kKV) {
+        // ---- S_t into registers: TMEM loads in flight together, one wait
+        wait(bar_s, g & 1);
+        ptx::tc_fence_after_sync();
+        uint32_t s[kCols];
+#pragma unroll
+        for (int c = 0; c < kCols / 32; ++c) ptx::tmem_ld_32x32(tmem + lane_base + kColS + col0 + c * 32, s + c * 32);
+        ptx::tmem_ld_wait();
+        // Which of this thread's groups of 32 key columns meet its row's segment at all (the others take no
+        // arithmetic: their P is zero); the mask is applied only where a boundary of the segment crosses a group.
+        // This half's row maximum is handed to the partner thread through shared memory.
+        bool need[kCols / 32];
+#pragma unroll
+        for (int c = 0; c < kCols / 32; ++c) {
+          need[c] = c * 32 < hi && c * 32 + 32 > lo;
+          if (need[c] && !(c * 32 >= lo && c * 32 + 32 <= hi)) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if ((unsigned)(c * 32 + j - lo) >= (unsigned)(hi - lo)) s[c * 32 + j] = 0xff800000u;  // -inf
+          }
+        }
+        float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+        for (int c = 0; c < kCols / 32; ++c) {
+          if (need[c]) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u) mx[u] = fmaxf(mx[u], __uint_as_float(s[c * 32 + j + u]));
+            }
+          }
+        }
+        float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        xch[((g & 1) * 2 + half) * 128 + rl] = mt;
+        ptx::tc_fence_before_sync();
+        ptx::named_barrier(1 + quarter, 64);  // the two warps that share these 32 rows
+        if (lane == 0) ptx::mbar_arrive(bar_sfree);
+
+        // ---- this half row's P (exp2 domain): one fma, one ex2 and one add per key.  The maximum that P and O
+        // refer to is raised only when the true one has grown by more than kRescaleGap, so O (accumulated in
+        // TMEM over all tiles) is rescaled rarely; sums and outputs are exact for any such reference value.
+        mt = fmaxf(mt, xch[((g & 1) * 2 + (half ^ 1)) * 128 + rl]);
+        const float m_cand = fmaxf(m, mt * scale_log2e);  // the scale is positive: max commutes with it
+        const bool raise = m_cand > m + kRescaleGap;      // also the first tile that has a key of this row
+        const float m_new = raise ? m_cand : m;
+        const float m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
+        const float alpha = raise ? ptx::ex2_approx(m - m_use) : 1.f;
+        float rs0 = 0.f, rs1 = 0.f;
+        uint32_t pk[kCols / 2];
+#pragma unroll
+        for (int c = 0; c < kCols / 32; ++c) {
+          if (need[c]) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+              const float p0 = ptx::ex2_approx(fmaf(__uint_as_float(s[c * 32 + j]), scale_log2e, -m_use));  // -inf -> 0
+              const float p1 = ptx::ex2_approx(fmaf(__uint_as_float(s[c * 32 + j + 1]), scale_log2e, -m_use));
+              rs0 += p0;
+              rs1 += p1;
+              __nv_bfloat162 b = __floats2bfloat162_rn(p0, p1);  // low half = even key
+              pk[c * 16 + (j >> 1)] = *reinterpret_cast<uint32_t*>(&b);
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) pk[c * 16 + j] = 0u;
+          }
+        }
+        // ---- the previous P V product must have completed before P is overwritten or O rescaled (before the first
+        // tile of an item it has: the item before waited for it)
+        __syncwarp();
+        if (!first) {
+          wait(bar_o, (g - 1) & 1);
+          ptx::tc_fence_after_sync();
+          if (__any_sync(0xffffffffu, raise)) {
+            uint32_t r[kDh];
+            if (kDh == 32) ptx::tmem_ld_32x32(tmem + lane_base + kColO + half * kDh, r);
+            else ptx::tmem_ld_32x16(tmem + lane_base + kColO + half * kDh, r);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < kDh; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
+            if (kDh == 32) ptx::tmem_st_32x32(tmem + lane_base + kColO + half * kDh, r);
+            else ptx::tmem_st_32x16(tmem + lane_base + kColO + half * kDh, r);
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < kCols / 32; ++c)
+          ptx::tmem_st_32x16(tmem + lane_base + kColP + (col0 >> 1) + c * 16, pk + c * 16);
+        ptx::tmem_st_wait();
+        l = l * alpha + (rs0 + rs1);
+        m = m_new;
+        first = false;
+        // ---- V lines past the last valid packed row must not reach the product (an item's last tile may have some)
+        const int line0 = left == 1 ? ptx::lds_s32(item_slot(it) + 16 * 4) : kKV;
+        if (line0 < kKV) {
+          const int st = g & 1;
+          wait(bar_v(st), (g >> 1) & 1);
+          constexpr int kChunks = HT::kRowBytes / 16;
+          for (int c = tid; c < (kKV - line0) * kChunks; c += kSoftmaxThreads)
+            *reinterpret_cast<uint4*>(smem_al + kTile * (4 + st) + (line0 + c / kChunks) * HT::kRowBytes +
+                                      (c % kChunks) * 16) = make_uint4(0, 0, 0, 0);
+          ptx::fence_proxy_async_smem();
+        }
+        ptx::tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar_pready);
+      }
+      // ---- the last product completes O: normalised, and stored as bf16 from the registers, a 32-byte sector per
+      // thread and instruction
+      const int q0 = ptx::lds_s32(item_slot(it)), h = ptx::lds_s32(item_slot(it) + 4), row = q0 + rl;
+      xl[half * 128 + rl] = l;  // the two halves of a row share the reference maximum but kept separate sums
+      wait(bar_o, (g - 1) & 1);
+      ptx::tc_fence_after_sync();
+      uint32_t r[kDh];
       if (kDh == 32) ptx::tmem_ld_32x32(tmem + lane_base + kColO + half * kDh, r);
       else ptx::tmem_ld_32x16(tmem + lane_base + kColO + half * kDh, r);
       ptx::tmem_ld_wait();
-    } else {
+      ptx::tc_fence_before_sync();
+      ptx::named_barrier(1 + quarter, 64);
+      const int rows = ptx::lds_s32(item_slot(it) + 68);
+      const float l_row = xl[half * 128 + rl] + xl[(half ^ 1) * 128 + rl], inv_l = 1.f / l_row;
+      uint4 o16[kDh / 8];
 #pragma unroll
-      for (int e = 0; e < kDh; ++e) r[e] = 0u;
+      for (int c = 0; c < kDh / 8; ++c) {
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[c * 8 + e]) * inv_l;
+        o16[c] = Vec16<__nv_bfloat16>::from_float(v);
+      }
+      if constexpr (kDh == 32) {  // four lanes take a row's 64 bytes: 8 rows per store instead of 32
+        transpose_quads(o16, lane);
+        __nv_bfloat16* dst = ao + (long long)(q0 + quarter * 32 + (lane & ~3)) * C + h * D + half * kDh + (lane & 3) * 8;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (quarter * 32 + (lane & ~3) + j < rows) *reinterpret_cast<uint4*>(dst + (long long)j * C) = o16[j];
+      } else if (rl < rows) {
+        st_global32(ao + (long long)row * C + h * D + half * kDh, o16[0], o16[1],
+                    (reinterpret_cast<uintptr_t>(ao) & 31u) == 0);  // rows and heads are whole sectors then
+      }
+      if (half == 0 && rl < rows) lse[(long long)h * capacity + row] = (m + log2f(l_row)) * 0.6931471805599453f;
+      __syncwarp();
     }
-    const float l_row = xch[half * 128 + rl] + xch[(half ^ 1) * 128 + rl];
-    const float inv_l = row < Np ? 1.f / l_row : 0.f;
-    const int rot = chunk_rot<D>(rl);
-#pragma unroll
-    for (int c = 0; c < kDh / 8; ++c) {
-      float v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = row < Np ? __uint_as_float(r[c * 8 + e]) * inv_l : 0.f;
-      *reinterpret_cast<uint4*>(smem_al + rl * HT::kRowBytes + (((half * (kDh / 8) + c) ^ rot) << 4)) =
-          Vec16<__nv_bfloat16>::from_float(v);
-    }
-    if (half == 0 && row < Np) lse[(long long)h * capacity + row] = (lse_m + log2f(l_row)) * 0.6931471805599453f;
   }
-  __syncthreads();
-  if (!failed) copy_tile_out<D, kFwdThreads>(smem_al, ao + h * D, C, q0, Np, tid);
-  cta_failed = failed;
   ptx::tc_fence_before_sync();
-  __syncthreads();  // the tile's memory and the barriers are free for the next item
-  }
+  __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after_sync();
-    ptx::tmem_dealloc(*tmem_slot, kTmemCols);
+    ptx::tmem_dealloc(tmem, kTmemCols);
   }
 }
 
@@ -1665,6 +1876,12 @@ int bwd_launch(const spa_params& p, const void* qkv, const void* ao, const float
   return SPA_OK;
 }
 
+// The counter that a launch on stream `st` draws its items from, or nullptr (then items are assigned by a static stride).
+// Launches of a stream run one after the other and each leaves its counter at zero, so a stream needs one counter: it is
+// found by the stream's id, which is never reused.  A launch that is being recorded gets one for itself, since its graph
+// may be replayed beside anything: 12 288 of them, then nullptr.
+unsigned* item_counter(cudaStream_t st);
+
 template <int D>
 int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao, float* lse,
                int32_t* d_status, cudaStream_t st) {
@@ -1672,14 +1889,16 @@ int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_s
   if (!make_tmap_bf16_2d(&tm, qkv, 3ull * p.C, p.capacity, 6ull * p.C, D, 128, D * 2)) return SPA_ERR_UNSUPPORTED;
   auto kern = attn_fwd_tc_kernel<D>;
   static DeviceOnce attr;
-  cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem_bytes<D>()); });
+  cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::kBytes); });
   if (ea != cudaSuccess) { set_cuda_error(ea, "attn_fwd_tc_kernel"); return SPA_ERR_CUDA; }
-  // a persistent grid: two CTAs per SM (87 KB of shared memory, 256 TMEM columns each), never more than work items
+  // a persistent grid: two CTAs per SM (at most 112 KB of shared memory, 256 TMEM columns each), never more than work items
   const long long items = (long long)p.H * ((p.capacity + kQ - 1) / kQ);
   const int grid = (int)(items < 2 * kNumSMs ? items : 2 * kNumSMs);
-  launch_pdl(kern, grid, kFwdThreads, fwd_smem_bytes<D>(), st, tm, seg, n_seg, p.capacity, p.C, p.H,
-                                                      softmax_scale_of(p) * 1.4426950408889634f,
-                                                      (__nv_bfloat16*)ao, lse, d_status);
+  // Short segments make items of nearly the same length: putting them in order gained nothing up to segment slots of
+  // 400 rows (and cost 1 us in front of short items), and 8 to 12 % from 576 rows on.
+  const bool even_items = (long long)p.capacity <= 512ll * (n_seg > 0 ? n_seg : 1);
+  launch_pdl(kern, grid, kFwdThreads, FwdSmem<D>::kBytes, st, tm, seg, n_seg, p.capacity, p.C, p.H,
+             softmax_scale_of(p) * 1.4426950408889634f, (__nv_bfloat16*)ao, lse, items > grid ? item_counter(st) : nullptr, even_items, d_status);
   SPA_CUDA_CHECK_LAUNCH("attn_fwd_tc_kernel");
   return SPA_OK;
 }
@@ -1721,11 +1940,98 @@ int launch_attention_fwd_tc(const spa_params& p, const void* qkv, const int32_t*
 // device, with that device current, and cached.
 static __device__ __align__(256) unsigned char g_static_scratch[SPA_STATIC_SCRATCH_BYTES];
 
+// Item counters of the persistent attention kernels: zero when the library is loaded and after every launch.  A stream
+// has one, since its launches follow one another; a recorded launch has one of its own, since graphs may run side by side,
+// and gives it back with its graph.  A launch that finds none left strides over its items.
+static constexpr int kStreamCounters = 4096, kRecordedCounters = 12288;
+static __device__ unsigned g_item_counters[kStreamCounters + kRecordedCounters];
+
 namespace spa {
 namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mutex;
 void* g_scratch_ptr[kMaxDevices] = {};
+}  // namespace
+
+namespace {
+struct RecordedCounters {  // of one device; never destroyed: graphs may outlive every static object
+  std::vector<int> free_list;
+  int used = 0;
+};
+struct RecordedCounter { int dev, index; };
+
+std::mutex g_counter_mutex;
+unsigned* g_counter_ptr[kMaxDevices] = {};
+std::unordered_map<unsigned long long, int>& g_stream_counter = *new std::unordered_map<unsigned long long, int>;  // by stream id
+RecordedCounters* const g_recorded = new RecordedCounters[kMaxDevices];
+
+void give_back_counter(void* p) {  // by the driver, when nothing that holds the recorded launch is left
+  RecordedCounter* r = static_cast<RecordedCounter*>(p);
+  {
+    std::lock_guard<std::mutex> lock(g_counter_mutex);
+    g_recorded[r->dev].free_list.push_back(r->index);
+  }
+  delete r;
+}
+
+unsigned* item_counter(cudaStream_t st) {
+  int dev = -1;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaGraph_t graph = nullptr;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices ||
+      cudaStreamGetCaptureInfo(st, &capture, &id, &graph) != cudaSuccess ||
+      (capture == cudaStreamCaptureStatusNone && cudaStreamGetId(st, &id) != cudaSuccess)) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  RecordedCounter* recorded = nullptr;
+  unsigned* counter = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_counter_mutex);
+    if (g_counter_ptr[dev] == nullptr) {
+      void* p = nullptr;
+      if (capture != cudaStreamCaptureStatusNone || cudaGetSymbolAddress(&p, g_item_counters) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      g_counter_ptr[dev] = static_cast<unsigned*>(p);
+    }
+    if (capture == cudaStreamCaptureStatusNone) {
+      auto it = g_stream_counter.find(id);
+      if (it != g_stream_counter.end()) return g_counter_ptr[dev] + it->second;
+      const int n = (int)g_stream_counter.size();
+      if (n >= kStreamCounters) return nullptr;
+      g_stream_counter.emplace(id, n);
+      return g_counter_ptr[dev] + n;
+    }
+    RecordedCounters& pool = g_recorded[dev];
+    int index = -1;
+    if (!pool.free_list.empty()) {
+      index = pool.free_list.back();
+      pool.free_list.pop_back();
+    } else if (pool.used < kRecordedCounters) {
+      index = pool.used++;
+    } else {
+      return nullptr;
+    }
+    recorded = new RecordedCounter{dev, index};
+    counter = g_counter_ptr[dev] + kStreamCounters + index;
+  }
+  // outside the lock: dropping the object calls give_back_counter
+  cudaUserObject_t obj = nullptr;
+  if (cudaUserObjectCreate(&obj, recorded, give_back_counter, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+    cudaGetLastError();
+    give_back_counter(recorded);
+    return nullptr;
+  }
+  if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+    cudaGetLastError();
+    cudaUserObjectRelease(obj, 1);
+    return nullptr;
+  }
+  return counter;
+}
 }  // namespace
 
 // Device address of g_static_scratch on the current device (looked up on first use).

@@ -166,8 +166,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   };
 
-  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer

@@ -141,8 +141,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int tiles_m = (M + 2 * PM - 1) / (2 * PM);
   const int total = tiles_m * tiles_n;
   const int k_blocks = (K + PK - 1) / PK;
-  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one per CTA)
@@ -365,8 +365,8 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     c.n0 = c.n_t * PN;
     return c;
   };
-  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one per CTA)

@@ -70,7 +70,7 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const int k_blocks = (K + BK - 1) / BK;
   const int mine = z < k_blocks ? (k_blocks - z + split - 1) / split : 0;  // k-blocks z, z + split, ...
   const bool with_sums = db != nullptr && blockIdx.x == 0;
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, abort_flag, d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
 
   if (warp == 0) {
     if (lane == 0) {

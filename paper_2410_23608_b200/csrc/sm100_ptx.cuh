@@ -49,25 +49,35 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
   return false;
 }
 
+// A word of shared memory that other threads write, by its 32-bit address (no generic pointer to keep in registers)
+__device__ __forceinline__ int lds_s32(uint32_t addr) {
+  int v;
+  asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts_s32(uint32_t addr, int v) {
+  asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
 // Wait inside a pipeline loop: returns once the phase has completed.  After kWaitLimit polls, or when another thread of
-// the CTA has given up, it returns all the same with *abort_flag set; the caller goes on without looking (every later
+// the CTA has given up, it returns all the same with the abort flag (an address in shared memory) set; the caller goes on without looking (every later
 // wait then returns at once, the loops end, and results are dropped after the CTA's next barrier), so a warp never
 // diverges here and the ready case is one instruction and a branch: with a poll of the flag and two votes around it a
 // satisfied wait took 160 clocks of a GEMM's 668 per k-block.
-__device__ __forceinline__ void mbar_wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* d_status,
+__device__ __forceinline__ void mbar_wait_or_abort(uint32_t bar, uint32_t parity, uint32_t abort_flag, int32_t* d_status,
                                                    int timeout_code) {
   if (mbar_try_wait(bar, parity)) return;
 #pragma unroll 1
   for (uint32_t i = 0; i < kWaitLimit; ++i) {
     if (mbar_try_wait(bar, parity)) return;
-    if ((i & 63u) == 0u && *abort_flag) return;
+    if ((i & 63u) == 0u && lds_s32(abort_flag)) return;
   }
   if (d_status != nullptr) atomicCAS(d_status, 0, timeout_code);
-  *abort_flag = 1;
+  sts_s32(abort_flag, 1);
 }
 // The same by all lanes of a warp, which are converged again when it returns: lanes may have polled a different number of
 // times, and elect_one() in a diverged warp would elect a lane of each part.
-__device__ __forceinline__ void mbar_wait_or_abort_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* d_status,
+__device__ __forceinline__ void mbar_wait_or_abort_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag, int32_t* d_status,
                                                         int timeout_code) {
   mbar_wait_or_abort(bar, parity, abort_flag, d_status, timeout_code);
   __syncwarp();
@@ -90,6 +100,18 @@ __device__ __forceinline__ bool elect_one() {
 // Barrier `id` (1-15; 0 is __syncthreads) among `threads` threads (a multiple of 32) of the CTA.
 __device__ __forceinline__ void named_barrier(uint32_t id, uint32_t threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// The same, returning whether any of the threads passed true (all of them get the same answer).
+__device__ __forceinline__ bool named_barrier_or(uint32_t id, uint32_t threads, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "barrier.cta.red.or.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r) : "r"(id), "r"(threads), "r"(v ? 1u : 0u) : "memory");
+  return r != 0;
 }
 
 // ---- fences -------------------------------------------------------------------------------------

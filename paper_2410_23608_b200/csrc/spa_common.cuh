@@ -96,6 +96,16 @@ __device__ __forceinline__ uint4 ld_nc16(const void* p) {  // streaming 16-byte 
   return v;
 }
 
+// 32 bytes in one store where they are a whole sector, else two of 16
+__device__ __forceinline__ void st_global32(void* p, const uint4& a, const uint4& b, bool sector) {
+  if (!sector) {
+    static_cast<uint4*>(p)[0] = a;
+    static_cast<uint4*>(p)[1] = b;
+    return;
+  }
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+}
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ float warp_sum(float v) {
