@@ -206,9 +206,10 @@ __device__ __forceinline__ void transpose_quads(uint4 (&c)[4], int lane) {
   swap(c[1], c[3], 2);
 }
 template <int D> struct FwdSmem {
-  // 2 x Q, 2 x K, 2 x V
+  // Q, 2 x K, 2 x V.  Two CTAs stay below 196 KB of an SM: with 228 (a second Q tile) the kernels that run before and after
+  // on the same SMs lost 3 to 5 us, the gate and the packing most (128 images of 196 tokens, forward: 88 -> 92 us).
   static constexpr int kTile = HeadTile<D>::kTileBytes;
-  static constexpr int kBar = 6 * kTile;                   // 13 barriers, TMEM slot, abort flag, four item slots
+  static constexpr int kBar = 5 * kTile;                   // 12 barriers, TMEM slot, abort flag, four item slots
   static constexpr int kXch = kBar + 256;                  // row maxima: [2 tile parities][2 halves][128 rows]
   static constexpr int kXl = kXch + 2048;                  // row sums: [2 halves][128 rows]
   static constexpr int kSeg = kXl + 1024;                  // staged segment offsets
@@ -240,11 +241,11 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_al = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-  auto q_s = [&](int b) { return smem_base + kTile * b; };
-  auto k_s = [&](int st) { return smem_base + kTile * (2 + st); };
-  auto v_s = [&](int st) { return smem_base + kTile * (4 + st); };
+  const uint32_t q_s = smem_base;
+  auto k_s = [&](int st) { return smem_base + kTile * (1 + st); };
+  auto v_s = [&](int st) { return smem_base + kTile * (3 + st); };
   const uint32_t bar = smem_base + SM::kBar;
-  auto bar_q = [&](int b) { return bar + 8 * b; };            // Q of an item has landed
+  const uint32_t bar_q = bar;                                 // Q of an item has landed
   auto bar_item = [&](int b) { return bar + 32 + 8 * b; };    // the item slot is filled
   auto bar_k = [&](int st) { return bar + 48 + 8 * st; };
   auto bar_v = [&](int st) { return bar + 64 + 8 * st; };
@@ -264,11 +265,11 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
   if (tid == kSoftmaxThreads) {
     ptx::prefetch_tensormap(&tm);
     for (int b = 0; b < 2; ++b) {
-      ptx::mbar_init(bar_q(b), 1);
       ptx::mbar_init(bar_item(b), 1);
       ptx::mbar_init(bar_k(b), 1);
       ptx::mbar_init(bar_v(b), 1);
     }
+    ptx::mbar_init(bar_q, 1);
     ptx::mbar_init(bar_s, 1);
     ptx::mbar_init(bar_o, 1);
     ptx::mbar_init(bar_sfree, kSoftmaxThreads / 32);
@@ -306,8 +307,8 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
     early_lo = __reduce_max_sync(0xffffffffu, early_lo);
     early_hi = __reduce_min_sync(0xffffffffu, early_hi);
     if (ptx::elect_one()) {
-      ptx::mbar_expect_tx(bar_q(0), kTile);
-      ptx::tma_load_2d(q_s(0), &tm, bar_q(0), h * D, q0);
+      ptx::mbar_expect_tx(bar_q, kTile);
+      ptx::tma_load_2d(q_s, &tm, bar_q, h * D, q0);
       ptx::mbar_expect_tx(bar_k(0), kTile);
       ptx::tma_load_2d(k_s(0), &tm, bar_k(0), C + h * D, early_lo);
       ptx::mbar_expect_tx(bar_v(0), kTile);
@@ -385,12 +386,15 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
         more = false;
       }
       announce(c);
-      // Q of the item two before is no longer needed: this cursor is at most two tiles ahead of the last S columns that
-      // the softmax warps have taken
-      if (c.n_tiles > 0 && ptx::elect_one()) {
-        ptx::mbar_expect_tx(bar_q(c.item & 1), kTile);
-        ptx::tma_load_2d(q_s(c.item & 1), &tm, bar_q(c.item & 1), c.h * D, c.q0);
+      __syncwarp();
+    };
+    int q_item = early ? 0 : -1;  // last item whose Q tile has been asked for
+    auto load_q = [&](const Cursor& c) {  // the S products of the item before have completed
+      if (ptx::elect_one()) {
+        ptx::mbar_expect_tx(bar_q, kTile);
+        ptx::tma_load_2d(q_s, &tm, bar_q, c.h * D, c.q0);
       }
+      q_item = c.item;
       __syncwarp();
     };
     auto advance = [&](Cursor& c) {
@@ -411,14 +415,14 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
       __syncwarp();
     };
     auto issue_qk = [&](const Cursor& c, int g) {  // S = Q K^T of tile g into TMEM; bar_s completes when it is done
-      if (c.t == 0) wait(bar_q(c.item & 1), (c.item >> 1) & 1);
+      if (c.t == 0) wait(bar_q, c.item & 1);
       wait(bar_k(g & 1), (g >> 1) & 1);
       ptx::tc_fence_after_sync();
-      const uint32_t qa = q_s(c.item & 1), ka = k_s(g & 1);
+      const uint32_t ka = k_s(g & 1);
       if (ptx::elect_one()) {
 #pragma unroll
         for (int k = 0; k < D / 16; ++k)
-          ptx::mma_bf16(tmem + kColS, HT::kmajor(qa, k), HT::kmajor(ka, k), kIdescS, k != 0 ? 1u : 0u);
+          ptx::mma_bf16(tmem + kColS, HT::kmajor(q_s, k), HT::kmajor(ka, k), kIdescS, k != 0 ? 1u : 0u);
         ptx::mma_commit(bar_s);
       }
       __syncwarp();
@@ -432,8 +436,18 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
     }
     Cursor cp = ck, cs = ck;  // tiles of the next P V product, the next S product; ck: of the next K load
     int g = 0, gk = 0, gv = 0;  // number of the tile of cp; tiles whose K and V loads have been issued
+    // Tile `last` is the last whose S product has been issued.  If the next one opens an item, its Q tile takes the memory
+    // of the one before as soon as that product is done, which is before the softmax warps have read its columns; it lands
+    // under their exponentials.
+    auto next_q = [&](int last) {
+      if (cs.n_tiles > 0 && cs.t == 0) {
+        wait(bar_s, last & 1);
+        load_q(cs);
+      }
+    };
     if (cp.n_tiles > 0) {
       if (!early) {
+        load_q(cp);
         load(cp, 0, false);
         load(cp, 0, true);
       }
@@ -447,6 +461,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
       }
       if (same) issue_qk(cs, 0);
       cs = ck;
+      next_q(0);
     }
     while (cp.n_tiles > 0 && !__any_sync(0xffffffffu, ptx::lds_s32(abort_any) != 0)) {
       // every softmax thread holds its columns of S of tile g: the S columns and K stage g & 1 are free
@@ -479,13 +494,13 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
       }
       cp = cn;
       ++g;
+      next_q(g);
     }
     if (__any_sync(0xffffffffu, ptx::lds_s32(abort_any) != 0) && lane == 0) {
       // let outstanding loads land before shared memory is released; the numbers drawn have to add up all the same
       for (int i = gv > 2 ? gv - 2 : 0; i < gv; ++i) ptx::mbar_wait(bar_v(i & 1), (i >> 1) & 1);
       for (int i = gk > 2 ? gk - 2 : 0; i < gk; ++i) ptx::mbar_wait(bar_k(i & 1), (i >> 1) & 1);
-      const int q_last = ck.n_tiles > 0 ? ck.item : ck.item - 1;  // last item whose Q tile has been asked for
-      for (int i = q_last > 1 ? q_last - 1 : 0; i <= q_last; ++i) ptx::mbar_wait(bar_q(i & 1), (i >> 1) & 1);
+      if (q_item >= 0) ptx::mbar_wait(bar_q, q_item & 1);
       while (more && draws && drawn < n_items) drawn = draw_item(counter, given, n_items, own);
     }
     __syncwarp();
@@ -610,7 +625,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
           wait(bar_v(st), (g >> 1) & 1);
           constexpr int kChunks = HT::kRowBytes / 16;
           for (int c = tid; c < (kKV - line0) * kChunks; c += kSoftmaxThreads)
-            *reinterpret_cast<uint4*>(smem_al + kTile * (4 + st) + (line0 + c / kChunks) * HT::kRowBytes +
+            *reinterpret_cast<uint4*>(smem_al + kTile * (3 + st) + (line0 + c / kChunks) * HT::kRowBytes +
                                       (c % kChunks) * 16) = make_uint4(0, 0, 0, 0);
           ptx::fence_proxy_async_smem();
         }
@@ -1891,7 +1906,7 @@ int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_s
   static DeviceOnce attr;
   cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::kBytes); });
   if (ea != cudaSuccess) { set_cuda_error(ea, "attn_fwd_tc_kernel"); return SPA_ERR_CUDA; }
-  // a persistent grid: two CTAs per SM (at most 112 KB of shared memory, 256 TMEM columns each), never more than work items
+  // a persistent grid: two CTAs per SM (at most 94 KB of shared memory, 256 TMEM columns each), never more than work items
   const long long items = (long long)p.H * ((p.capacity + kQ - 1) / kQ);
   const int grid = (int)(items < 2 * kNumSMs ? items : 2 * kNumSMs);
   // Short segments make items of nearly the same length: putting them in order gained nothing up to segment slots of
