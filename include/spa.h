@@ -406,6 +406,40 @@ int spa_block_fwd(const spa_params* p, const spa_block_buffers* b, void* stream)
  * is ordered before whatever is enqueued on `stream` next. */
 int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream);
 
+/* ---- The pre-norm transformer block around SPA as one unit -----------------------------------------------------
+ * out = y1 + W2 gelu(W1 LN2(y1)), y1 = x + scatter(SPA(LN1(x))).  `blk` holds the buffers and weights of the attention part
+ * (its x, y, dY and dX are not used: z, y1, dy1 and dX below stand in their place). */
+typedef struct spa_layer_buffers {
+  const spa_block_buffers* blk;
+  int32_t hidden;             /* width of the feed-forward network                                   */
+  float eps;
+  /* inputs of the forward pass */
+  const void* x;              /* T[B][N][C]                                                          */
+  const void *g1, *be1;       /* T[C] LayerNorm before the attention                                 */
+  const void *g2, *be2;       /* T[C] LayerNorm before the feed-forward network                      */
+  const void *W1, *b1;        /* T[hidden][C], T[hidden]                                             */
+  const void *W2, *b2;        /* T[C][hidden], T[C]                                                  */
+  const int32_t* cu_all;      /* int32[B+1] = 0, N, 2N, ...: every token is a row                    */
+  /* results and intermediates of the forward pass */
+  void *z, *y1, *t, *out;     /* T[B][N][C]                                                          */
+  void *u, *h;                /* T[B*N][hidden]: W1 t + b1, gelu(u)                                  */
+  float *m1, *r1, *m2, *r2;   /* float[B*N] mean and 1/std of the rows of x and y1                   */
+  /* backward pass */
+  const void* d_out;          /* T[B][N][C]                                                          */
+  void* dh;                   /* T[B*N][hidden]: gradient to u                                       */
+  void *dt, *dy1, *dX;        /* T[B][N][C]                                                          */
+  float *dW1, *db1, *dW2, *db2, *dg1, *dbe1, *dg2, *dbe2;
+  void* workspace;            /* at least spa_workspace_bytes(), spa_train_workspace_bytes() and
+                                 32 (hidden C + max(hidden, C)) floats + 1 KB                        */
+} spa_layer_buffers;
+
+/* Forward pass of the block.  blk->pack_state, order, s_up, seg_offsets and container_len are not looked at. */
+int spa_layer_fwd(const spa_params* p, const spa_layer_buffers* l, void* stream);
+
+/* Backward pass for the last spa_layer_fwd on the same buffers: dX, dW1, db1, dW2, db2, the LayerNorms' dg and dbe, and
+ * blk's dW_qkv, db_qkv, dW_o, db_o.  No gradient reaches the gate. */
+int spa_layer_bwd(const spa_params* p, const spa_layer_buffers* l, void* stream);
+
 /* ---- Diagnostics (the paper has no counterpart) ----------------------------------------------------------------
  * spa_probe_exp2: n_ctas CTAs of 512 threads evaluate base-2 exponentials with the instruction the softmax kernels
  * use, 8 * iters per thread; *n_exp (host, may be NULL) receives the total count.  Timed by the caller, it gives the

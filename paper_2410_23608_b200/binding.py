@@ -32,7 +32,7 @@ EXPORTS = (
     "spa_fused_scatter_supported", "spa_gate_prefill", "spa_unpack_prefill", "spa_packed_proj_scatter", "spa_packed_linear_bwd_scatter",
     "spa_select_pack_ordered", "spa_train_workspace_bytes", "spa_score_pool", "spa_select_loss", "spa_select_pack_bwd_gated", "spa_gate_bwd",
     "spa_packed_linear", "spa_layer_norm", "spa_layer_norm_bwd", "spa_gelu", "spa_gelu_bwd",
-    "spa_overlap_create", "spa_overlap_destroy", "spa_block_fwd", "spa_block_bwd",
+    "spa_overlap_create", "spa_overlap_destroy", "spa_block_fwd", "spa_block_bwd", "spa_layer_fwd", "spa_layer_bwd",
     "spa_probe_exp2", "spa_probe_wait_expiry", "spa_probe_mma_issue", "spa_pack_state_bytes", "spa_gate_select_pack_supported",
     "spa_gate_select_pack", "spa_container_max_segments", "spa_container_offsets",
 )
@@ -67,6 +67,15 @@ class SpaBlockBuffers(C.Structure):
                 ("trainable", C.c_int32), ("labels", C.c_void_p), ("alpha", C.c_float), ("ds", C.c_void_p),
                 ("ds_up", C.c_void_p), ("dw_g", C.c_void_p), ("db_g", C.c_void_p), ("loss", C.c_void_p),
                 ("train_workspace", C.c_void_p), ("container_len", C.c_int32)]
+
+
+class SpaLayerBuffers(C.Structure):
+    """spa_layer_buffers of include/spa.h, field for field."""
+    _fields_ = ([("blk", C.POINTER(SpaBlockBuffers)), ("hidden", C.c_int32), ("eps", C.c_float)] +
+                [(n, C.c_void_p) for n in (
+                    "x", "g1", "be1", "g2", "be2", "W1", "b1", "W2", "b2", "cu_all", "z", "y1", "t", "out", "u", "h", "m1", "r1",
+                    "m2", "r2", "d_out", "dh", "dt", "dy1", "dX", "dW1", "db1", "dW2", "db2", "dg1", "dbe1", "dg2", "dbe2",
+                    "workspace")])
 
 
 def make_params(B, N, Cc, H, dtype, capacity=None, flags=0, tau=0.0, softmax_scale=0.0) -> SpaParams:
@@ -120,6 +129,8 @@ def lib() -> C.CDLL:
         L.spa_overlap_destroy.argtypes = [vp]
         L.spa_block_fwd.argtypes = [pp, C.POINTER(SpaBlockBuffers), vp]
         L.spa_block_bwd.argtypes = [pp, C.POINTER(SpaBlockBuffers), vp]
+        L.spa_layer_fwd.argtypes = [pp, C.POINTER(SpaLayerBuffers), vp]
+        L.spa_layer_bwd.argtypes = [pp, C.POINTER(SpaLayerBuffers), vp]
         L.spa_pack_state_bytes.restype = C.c_size_t
         L.spa_pack_state_bytes.argtypes = [pp]
         L.spa_gate_select_pack_supported.argtypes = [pp]

@@ -11,14 +11,22 @@ namespace {
 constexpr int kRestThreads = 256;
 constexpr int kLnChunks = 4;  // 16-byte chunks of a row per lane: C <= 128 chunks (1024 bf16 / 512 fp32 channels)
 
-template <typename T>
+// LayerNorm of every token row.  kGate: the SPA gate reads the normalised (rounded) row from the same registers - scores
+// and mask as spa_gate writes them - and the row itself is passed on to `copy` (the residual stream that the attention
+// adds to): one pass over x instead of three kernels that read x or its normalisation again.
+template <typename T, bool kGate>
 __global__ void __launch_bounds__(kRestThreads)
 layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, const T* __restrict__ beta, float eps,
-                  int rows, int C, uint4* __restrict__ y16, float* __restrict__ mean, float* __restrict__ rstd) {
+                  int rows, int C, uint4* __restrict__ y16, float* __restrict__ mean, float* __restrict__ rstd,
+                  const T* __restrict__ w_g, float b_g, float tau, float* __restrict__ scores, uint8_t* __restrict__ mask,
+                  uint4* __restrict__ copy16) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
   const int lane = threadIdx.x & 31, Q = C / E;
   const int warps = gridDim.x * (kRestThreads / 32);
+  const uint4* g16 = reinterpret_cast<const uint4*>(gamma);
+  const uint4* b16 = reinterpret_cast<const uint4*>(beta);
+  const uint4* w16 = reinterpret_cast<const uint4*>(w_g);
   for (int t = blockIdx.x * (kRestThreads / 32) + (threadIdx.x >> 5); t < rows; t += warps) {
     float v[kLnChunks][E];
     float s = 0.f;
@@ -26,7 +34,9 @@ layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, co
     for (int k = 0; k < kLnChunks; ++k) {
       const int q = lane + 32 * k;
       if (q < Q) {
-        Vec16<T>::to_float(ld_nc16(x16 + (long long)t * Q + q), v[k]);
+        const uint4 raw = ld_nc16(x16 + (long long)t * Q + q);
+        if (kGate) copy16[(long long)t * Q + q] = raw;
+        Vec16<T>::to_float(raw, v[k]);
 #pragma unroll
         for (int e = 0; e < E; ++e) s += v[k][e];
       }
@@ -41,16 +51,29 @@ layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, co
       }
     const float rs = rsqrtf(warp_sum(ss) / C + eps);
     if (lane == 0) { mean[t] = mu; rstd[t] = rs; }
+    float dot = 0.f;
 #pragma unroll
     for (int k = 0; k < kLnChunks; ++k) {
       const int q = lane + 32 * k;
       if (q < Q) {
-        float o[E];
+        float o[E], g[E], b[E];
+        Vec16<T>::to_float(__ldg(g16 + q), g);
+        Vec16<T>::to_float(__ldg(b16 + q), b);
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-          o[e] = (v[k][e] - mu) * rs * to_f32<T>(gamma[q * E + e]) + to_f32<T>(beta[q * E + e]);
-        y16[(long long)t * Q + q] = Vec16<T>::from_float(o);
+        for (int e = 0; e < E; ++e) o[e] = (v[k][e] - mu) * rs * g[e] + b[e];
+        const uint4 out = Vec16<T>::from_float(o);
+        y16[(long long)t * Q + q] = out;
+        if (kGate) {
+          Vec16<T>::to_float(out, o);
+          Vec16<T>::to_float(__ldg(w16 + q), g);
+#pragma unroll
+          for (int e = 0; e < E; ++e) dot = fmaf(o[e], g[e], dot);
+        }
       }
+    }
+    if (kGate) {
+      const float sc = warp_sum(dot) + b_g;
+      if (lane == 0) { scores[t] = sc; mask[t] = sc > tau ? 1 : 0; }
     }
   }
 }
@@ -59,11 +82,14 @@ layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, co
 // branch's gradient).  Per-CTA sums of dy xh (dgamma) and dy (dbeta) go to part[blockIdx][2C].
 // kCh = 16-byte chunks of a row per lane (ceil(C / (32 chunks))): sized exactly, so that narrow rows do not
 // carry the registers of wide ones and several CTAs share an SM.
+// dy_row (optional): row t of dy is packed row dy_row[t], or zero where that is negative (the gradient reaches selected
+// tokens only).  dz_row / dz16 (optional): dx row t goes to packed row dz_row[t] as well, where that is not negative.
 template <typename T, int kCh>
 __global__ void __launch_bounds__(kRestThreads)
 layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ x16, const T* __restrict__ gamma,
                       const float* __restrict__ mean, const float* __restrict__ rstd, const uint4* add16, int rows,
-                      int C, uint4* dx16, float* __restrict__ part) {
+                      int C, uint4* dx16, float* __restrict__ part, const int32_t* __restrict__ dy_row,
+                      const int32_t* __restrict__ dz_row, uint4* __restrict__ dz16) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
   extern __shared__ float acc_s[];  // [8 warps][2C]
@@ -75,6 +101,20 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
     for (int e = 0; e < E; ++e) { ag[k][e] = 0.f; ab[k][e] = 0.f; }
   const int warps = gridDim.x * (kRestThreads / 32);
   for (int t = blockIdx.x * (kRestThreads / 32) + warp; t < rows; t += warps) {
+    const int src = dy_row != nullptr ? ld_dep(dy_row + t) : t;
+    const int dz = dz_row != nullptr ? ld_dep(dz_row + t) : -1;
+    if (src < 0) {  // no gradient into this row: what the residual branch brings, or nothing
+#pragma unroll
+      for (int k = 0; k < kCh; ++k) {
+        const int q = lane + 32 * k;
+        if (q < Q) {
+          const uint4 v = add16 != nullptr ? add16[(long long)t * Q + q] : make_uint4(0u, 0u, 0u, 0u);
+          dx16[(long long)t * Q + q] = v;
+          if (dz >= 0) dz16[(long long)dz * Q + q] = v;
+        }
+      }
+      continue;
+    }
     const float mu = mean[t], rs = rstd[t];
     float g[kCh][E], xh[kCh][E];
     float s1 = 0.f, s2 = 0.f;
@@ -82,13 +122,14 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
     for (int k = 0; k < kCh; ++k) {
       const int q = lane + 32 * k;
       if (q < Q) {
-        float dy[E], xv[E];
-        Vec16<T>::to_float(ld_nc16(dy16 + (long long)t * Q + q), dy);
+        float dy[E], xv[E], gm[E];
+        Vec16<T>::to_float(ld_nc16(dy16 + (long long)src * Q + q), dy);
         Vec16<T>::to_float(ld_nc16(x16 + (long long)t * Q + q), xv);
+        Vec16<T>::to_float(__ldg(reinterpret_cast<const uint4*>(gamma) + q), gm);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           xh[k][e] = (xv[e] - mu) * rs;
-          g[k][e] = dy[e] * to_f32<T>(gamma[q * E + e]);
+          g[k][e] = dy[e] * gm[e];
           s1 += g[k][e];
           s2 = fmaf(g[k][e], xh[k][e], s2);
           ag[k][e] = fmaf(dy[e], xh[k][e], ag[k][e]);
@@ -110,7 +151,9 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
 #pragma unroll
           for (int e = 0; e < E; ++e) o[e] += a[e];
         }
-        dx16[(long long)t * Q + q] = Vec16<T>::from_float(o);
+        const uint4 v = Vec16<T>::from_float(o);
+        dx16[(long long)t * Q + q] = v;
+        if (dz >= 0) dz16[(long long)dz * Q + q] = v;
       }
     }
   }
@@ -130,11 +173,6 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
     for (int w = 0; w < kRestThreads / 32; ++w) s += acc_s[w * 2 * C + c];
     part[(long long)blockIdx.x * 2 * C + c] = s;
   }
-}
-
-__device__ __forceinline__ float gelu_f(float u) { return 0.5f * u * (1.f + erff(u * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad_f(float u) {
-  return 0.5f * (1.f + erff(u * 0.70710678118654752f)) + u * 0.3989422804014327f * __expf(-0.5f * u * u);
 }
 
 // out = gelu(u) (kBwd = false) or out = dh * gelu'(u) (kBwd = true), over `total` 16-byte chunks
@@ -180,22 +218,28 @@ bool layer_norm_supported(const spa_params& p) { return p.C / (p.dtype == SPA_F3
 
 int launch_layer_norm(const spa_params& p, const void* x, const void* gamma, const void* beta, float eps, void* y,
                       float* mean, float* rstd, cudaStream_t st) {
+  return launch_layer_norm_gate(p, x, gamma, beta, eps, y, mean, rstd, nullptr, 0.f, nullptr, nullptr, nullptr, st);
+}
+
+int launch_layer_norm_gate(const spa_params& p, const void* x, const void* gamma, const void* beta, float eps, void* y,
+                           float* mean, float* rstd, const void* w_g, float b_g, float* scores, uint8_t* mask, void* copy,
+                           cudaStream_t st) {
   const int rows = p.B * p.N;
   if (rows == 0) return SPA_OK;
   if (!layer_norm_supported(p)) return SPA_ERR_UNSUPPORTED;
-  if (p.dtype == SPA_F32)
-    launch_pdl(layer_norm_kernel<float>, ln_grid(rows), kRestThreads, 0, st, (const uint4*)x, (const float*)gamma,
-               (const float*)beta, eps, rows, p.C, (uint4*)y, mean, rstd);
-  else
-    launch_pdl(layer_norm_kernel<__nv_bfloat16>, ln_grid(rows), kRestThreads, 0, st, (const uint4*)x,
-               (const __nv_bfloat16*)gamma, (const __nv_bfloat16*)beta, eps, rows, p.C, (uint4*)y, mean, rstd);
+#define SPA_LN(T, G)                                                                                                  \
+  launch_pdl(layer_norm_kernel<T, G>, ln_grid(rows), kRestThreads, 0, st, (const uint4*)x, (const T*)gamma,           \
+             (const T*)beta, eps, rows, p.C, (uint4*)y, mean, rstd, (const T*)w_g, b_g, p.tau, scores, mask, (uint4*)copy)
+  if (p.dtype == SPA_F32) { if (w_g != nullptr) SPA_LN(float, true); else SPA_LN(float, false); }
+  else { if (w_g != nullptr) SPA_LN(__nv_bfloat16, true); else SPA_LN(__nv_bfloat16, false); }
+#undef SPA_LN
   SPA_CUDA_CHECK_LAUNCH("layer_norm_kernel");
   return SPA_OK;
 }
 
 int launch_layer_norm_bwd(const spa_params& p, const void* dy, const void* x, const void* gamma, const float* mean,
                           const float* rstd, const void* add, void* dx, float* dgamma, float* dbeta, void* workspace,
-                          cudaStream_t st) {
+                          cudaStream_t st, const int32_t* dy_row, const int32_t* dz_row, void* dz) {
   const int rows = p.B * p.N;
   if (rows == 0) return SPA_OK;
   if (!layer_norm_supported(p)) return SPA_ERR_UNSUPPORTED;
@@ -211,7 +255,7 @@ int launch_layer_norm_bwd(const spa_params& p, const void* dy, const void* x, co
     e = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024); }); \
     if (e == cudaSuccess)                                                                                             \
       launch_pdl(kern, grid, kRestThreads, smem, st, (const uint4*)dy, (const uint4*)x, (const T*)gamma, mean, rstd, \
-                 (const uint4*)add, rows, p.C, (uint4*)dx, part);                                                     \
+                 (const uint4*)add, rows, p.C, (uint4*)dx, part, dy_row, dz_row, (uint4*)dz);                          \
   } while (0)
 #define SPA_LN_BWD_T(T)                                                                                               \
   do {                                                                                                                \

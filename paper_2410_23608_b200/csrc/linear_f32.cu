@@ -101,13 +101,13 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t addr, int k, bool mn) 
 }
 
 // dyn_which: 1 = M is the device-side packed row count, 2 = K is.
-// row_map (optional): output row i goes to row row_map[i] of `out`; accumulate: the result joins what that row holds.
+// row_map (optional): output row i goes to row row_map[i] of `out`; add, u, h: LinearEpilogue.
 // colsum (optional, wgrad): colsum[m] = sum_k A(m,k), by the CTAs of the first column of tiles from the lines they load.
 template <int BN, bool kAMn, bool kBMn>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restrict__ Bm, long long ldb,
-                const float* __restrict__ bias, float* __restrict__ out, long long ldo, int M, int N, int K,
-                const int32_t* __restrict__ cu, int n_seg, int capacity, int dyn_which, int accumulate,
+                const float* __restrict__ bias, float* out, long long ldo, int M, int N, int K,
+                const int32_t* __restrict__ cu, int n_seg, int capacity, int dyn_which, const float* add, const float* u, float* h,
                 const int32_t* __restrict__ row_map, float* __restrict__ colsum, int32_t* d_status) {
   using OpA = Operand<BM, kAMn>;
   using OpB = Operand<BN, kBMn>;
@@ -275,12 +275,18 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
       }
       const int m = m0 + r;
-      float4* dst = reinterpret_cast<float4*>(out + (row_map != nullptr ? (long long)ld_dep(row_map + m) : (long long)m) * ldo + n0 + c);
-      if (accumulate) {
-        const float4 w = *dst;
+      const long long at = (row_map != nullptr ? (long long)ld_dep(row_map + m) : (long long)m) * ldo + n0 + c;
+      if (add != nullptr) {
+        const float4 w = *reinterpret_cast<const float4*>(add + at);
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
       }
-      *dst = v;
+      if (u != nullptr) {
+        const float4 w = *reinterpret_cast<const float4*>(u + at);
+        v.x *= gelu_grad_f(w.x); v.y *= gelu_grad_f(w.y); v.z *= gelu_grad_f(w.z); v.w *= gelu_grad_f(w.w);
+      }
+      *reinterpret_cast<float4*>(out + at) = v;
+      if (h != nullptr)
+        *reinterpret_cast<float4*>(h + at) = make_float4(gelu_f(v.x), gelu_f(v.y), gelu_f(v.z), gelu_f(v.w));
     }
     if (kAMn && sums)
       for (int e = tid; e < my_rows; e += kThreads) {
@@ -299,7 +305,8 @@ struct Gemm {
   const void *A, *B, *bias;
   void* out;
   long long lda, ldb, ldo;
-  int M, N, K, dyn_which, accumulate;
+  int M, N, K, dyn_which;
+  LinearEpilogue epi;
   const int32_t *cu, *row_map;
   int n_seg, capacity;
   float* colsum;
@@ -331,7 +338,7 @@ template <int BN, bool kAMn, bool kBMn> int launch_tile(const Gemm& g, int split
   cfg.attrs = attr;
   cfg.numAttrs = n;
   e = cudaLaunchKernelEx(&cfg, kern, (const float*)g.A, g.lda, (const float*)g.B, g.ldb, (const float*)g.bias, (float*)g.out, g.ldo,
-                         g.M, g.N, g.K, g.cu, g.n_seg, g.capacity, g.dyn_which, g.accumulate, g.row_map, g.colsum, g.d_status);
+                         g.M, g.N, g.K, g.cu, g.n_seg, g.capacity, g.dyn_which, (const float*)g.epi.add, (const float*)g.epi.u, (float*)g.epi.h, g.row_map, g.colsum, g.d_status);
   if (e != cudaSuccess) { set_cuda_error(e, what); return SPA_ERR_CUDA; }
   SPA_CUDA_CHECK_LAUNCH(what);
   return SPA_OK;
@@ -358,21 +365,21 @@ template <bool kAMn, bool kBMn> int launch_gemm(const Gemm& g, cudaStream_t st, 
 
 int launch_linear_fwd_f32(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
                           const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st, const int32_t* row_map,
-                          bool accumulate) {
-  const Gemm g{a, W, bias, out, n_in, n_in, n_out, p.capacity, n_out, n_in, 1, accumulate ? 1 : 0, cu, row_map, p.B, p.capacity, nullptr, d_status};
+                          const LinearEpilogue& epi) {
+  const Gemm g{a, W, bias, out, n_in, n_in, n_out, p.capacity, n_out, n_in, 1, epi, cu, row_map, p.B, p.capacity, nullptr, d_status};
   return launch_gemm<false, false>(g, st, "gemm_f32_kernel(fwd)");
 }
 
 int launch_linear_bwd_f32(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out,
                           const int32_t* cu, void* da, float* dW, float* db, int32_t* d_status, cudaStream_t st,
-                          const int32_t* row_map, bool accumulate) {
+                          const int32_t* row_map, const LinearEpilogue& epi) {
   if (da != nullptr) {  // da[m][j] = sum_o dout[m][o] W[o][j]
-    const Gemm g{dout, W, nullptr, da, n_out, n_in, n_in, p.capacity, n_in, n_out, 1, accumulate ? 1 : 0, cu, row_map, p.B, p.capacity, nullptr, d_status};
+    const Gemm g{dout, W, nullptr, da, n_out, n_in, n_in, p.capacity, n_in, n_out, 1, epi, cu, row_map, p.B, p.capacity, nullptr, d_status};
     const int rc = launch_gemm<false, true>(g, st, "gemm_f32_kernel(dgrad)");
     if (rc != SPA_OK) return rc;
   }
   if (dW != nullptr) {  // dW[o][j] = sum_i dout[i][o] a[i][j]; db beside it
-    const Gemm g{dout, a, nullptr, dW, n_out, n_in, n_in, n_out, n_in, p.capacity, 2, 0, cu, nullptr, p.B, p.capacity, db, d_status};
+    const Gemm g{dout, a, nullptr, dW, n_out, n_in, n_in, n_out, n_in, p.capacity, 2, {}, cu, nullptr, p.B, p.capacity, db, d_status};
     return launch_gemm<true, true>(g, st, "gemm_f32_kernel(wgrad)");
   }
   return db != nullptr ? launch_colsum_simt(p, dout, n_out, cu, db, st) : SPA_OK;

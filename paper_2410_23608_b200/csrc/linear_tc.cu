@@ -90,14 +90,14 @@ struct TileCoord { int m0, n0, z, n_t; };
 // that the device-side row count leaves; two accumulator stages in TMEM let the epilogue of one tile
 // overlap the main loop of the next, and the TMA ring runs ahead across tile boundaries.
 // row_map (optional): output row i goes to row row_map[i] of `out` (the unpack scatter fused into the
-// epilogue); with `accumulate` the bf16 result is added to what that row holds.
-template <int BN, bool kAMn, bool kBMn, typename OutT>
+// epilogue).  epi: what a bf16 result goes through on its way out (RowEpilogue; split-K partials go as they are).
+template <int BN, bool kAMn, bool kBMn, typename OutT, int kKind>
 __global__ void __launch_bounds__(kGemmThreads)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __nv_bfloat16* __restrict__ bias, OutT* __restrict__ out, long long ldo,
                long long split_stride, int M, int N, int K, const int32_t* __restrict__ cu, int n_seg, int capacity,
                int dyn_which, int k_per_split, int k_interleave, const int32_t* __restrict__ row_map,
-               int accumulate, int32_t* d_status) {
+               RowEpilogue<kKind> epi, int32_t* d_status) {
   constexpr int kStage = stage_bytes<BN>();
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(BM, BN, kAMn, kBMn);
   pdl_launch_dependents();
@@ -282,12 +282,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       ptx::tc_fence_after_sync();
 #pragma unroll 1
       for (int cc = 0; cc < BN / 32; ++cc) {
-        uint4 old[4];  // what the rows hold, under the read of the accumulator
-        if (sizeof(OutT) == 2 && accumulate) {
+        uint4 old[4];  // what the results are combined with, under the read of the accumulator
+        if constexpr (sizeof(OutT) == 2) {
 #pragma unroll
           for (int j = 0; j < 4; ++j)
             if (c.m0 + q * 32 + my_row + 8 * j < M && c.n0 + cc * 32 + my_chunk * 8 < N)
-              old[j] = *reinterpret_cast<const uint4*>(obase + orow[j] * ldo + c.n0 + cc * 32 + my_chunk * 8);
+              epi.fetch(obase, old[j], orow[j] * ldo + c.n0 + cc * 32 + my_chunk * 8);
         }
         uint32_t r[32];
         ptx::tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + cc * 32, r);
@@ -322,17 +322,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int grow = c.m0 + q * 32 + rr;
             const int gcol = c.n0 + cc * 32 + ps * kSegCols + my_chunk * (16 / (int)sizeof(OutT));
             if (grow < M && gcol < N) {
-              uint4* dst = reinterpret_cast<uint4*>(obase + orow[j] * ldo + gcol);
-              if (sizeof(OutT) == 2 && accumulate) {
-                float fa[8], fb[8];
-                Vec16<__nv_bfloat16>::to_float(old[j], fa);
-                Vec16<__nv_bfloat16>::to_float(v4, fb);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) fa[e] += fb[e];
-                *dst = Vec16<__nv_bfloat16>::from_float(fa);
-              } else {
-                *dst = v4;
-              }
+              if constexpr (sizeof(OutT) == 2) epi.finish(obase, orow[j] * ldo + gcol, v4, old[j]);
+              else *reinterpret_cast<uint4*>(obase + orow[j] * ldo + gcol) = v4;
             }
           }
           __syncwarp();
@@ -483,12 +474,12 @@ size_t wgrad_workspace_bytes(int capacity, int n_in, int n_out) {
 
 inline bool wgrad_on_pairs(const spa_params& p) { return !(p.flags & SPA_FLAG_NO_CTA_PAIRS); }
 
-template <int BN, bool kAMn, bool kBMn, typename OutT>
+template <int BN, bool kAMn, bool kBMn, typename OutT, int kKind>
 int launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, OutT* out, long long ldo,
                 long long split_stride, int M, int N, int K, const int32_t* cu, int n_seg, int capacity, int dyn_which,
-                int k_per_split, int splits, int k_interleave, const int32_t* row_map, int accumulate,
+                int k_per_split, int splits, int k_interleave, const int32_t* row_map, RowEpilogue<kKind> epi,
                 int32_t* d_status, cudaStream_t st, const char* what) {
-  auto kern = gemm_tc_kernel<BN, kAMn, kBMn, OutT>;
+  auto kern = gemm_tc_kernel<BN, kAMn, kBMn, OutT, kKind>;
   static DeviceOnce attr;  // per instantiation and device
   cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes<BN>()); });
   if (ea != cudaSuccess) { set_cuda_error(ea, what); return SPA_ERR_CUDA; }
@@ -497,7 +488,7 @@ int launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloa
   long long tiles = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM) * splits;
   const int grid = (int)(tiles < 2 * kNumSMs ? (tiles < 1 ? 1 : tiles) : 2 * kNumSMs);
   launch_pdl(kern, grid, kGemmThreads, gemm_smem_bytes<BN>(), st, tmA, tmB, bias, out, ldo, split_stride, M, N, K, cu,
-             n_seg, capacity, dyn_which, k_per_split, k_interleave, row_map, accumulate, d_status);
+             n_seg, capacity, dyn_which, k_per_split, k_interleave, row_map, epi, d_status);
   SPA_CUDA_CHECK_LAUNCH(what);
   return SPA_OK;
 }
@@ -517,22 +508,26 @@ size_t tc_linear_workspace_bytes(const spa_params& p) {
 
 int launch_linear_fwd_tc(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
                          const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st, const int32_t* row_map,
-                         bool accumulate) {
+                         const LinearEpilogue& epi) {
   if (tc_pair_linear_supported(p, n_in, n_out, n_out))
-    return launch_linear_fwd_pair(p, a, W, bias, n_in, n_out, cu, out, d_status, st, row_map, accumulate);
+    return launch_linear_fwd_pair(p, a, W, bias, n_in, n_out, cu, out, d_status, st, row_map, epi);
   CUtensorMap tmA, tmB;
   if (!make_tmap_bf16_2d(&tmA, a, n_in, p.capacity, (uint64_t)n_in * 2, BK, BM) ||
       !make_tmap_bf16_2d(&tmB, W, n_in, n_out, (uint64_t)n_in * 2, BK, 128))
     return SPA_ERR_UNSUPPORTED;
-  return launch_gemm<128, false, false, __nv_bfloat16>(tmA, tmB, (const __nv_bfloat16*)bias,
-                                                              (__nv_bfloat16*)out, n_out, 0, p.capacity, n_out, n_in,
-                                                              cu, p.B, p.capacity, 1, n_in, 1, 0, row_map,
-                                                              accumulate ? 1 : 0, d_status, st, "gemm_tc_kernel(fwd)");
+  auto go = [&](auto row_epi) {
+    return launch_gemm<128, false, false, __nv_bfloat16>(tmA, tmB, (const __nv_bfloat16*)bias, (__nv_bfloat16*)out, n_out, 0,
+                                                         p.capacity, n_out, n_in, cu, p.B, p.capacity, 1, n_in, 1, 0, row_map,
+                                                         row_epi, d_status, st, "gemm_tc_kernel(fwd)");
+  };
+  if (epi.h != nullptr) return go(RowEpilogue<kEpiGelu>{(__nv_bfloat16*)epi.h});
+  if (epi.add != nullptr && epi.add != out) return go(RowEpilogue<kEpiAdd>{(__nv_bfloat16*)const_cast<void*>(epi.add)});
+  return go(RowEpilogue<kEpiOwn>{epi.add != nullptr ? (__nv_bfloat16*)out : nullptr});
 }
 
 int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out,
                          const int32_t* cu, void* da, float* dW, float* db, void* workspace, int32_t* d_status,
-                         cudaStream_t st, const int32_t* row_map, bool accumulate) {
+                         cudaStream_t st, const int32_t* row_map, const LinearEpilogue& epi) {
   CUtensorMap tmA, tmB, tmA2, tmB2;
   if (da != nullptr && (!make_tmap_bf16_2d(&tmA, dout, n_out, p.capacity, (uint64_t)n_out * 2, BK, BM) ||
                         !make_tmap_bf16_2d(&tmB, W, n_in, n_out, (uint64_t)n_in * 2, 64, BK)))
@@ -542,13 +537,16 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
     return SPA_ERR_UNSUPPORTED;
   const bool pair_dgrad = da != nullptr && tc_pair_linear_supported(p, n_in, n_out, n_in);
   if (pair_dgrad) {
-    int rc = launch_linear_dgrad_pair(p, W, dout, n_in, n_out, cu, da, d_status, st, row_map, accumulate);
+    int rc = launch_linear_dgrad_pair(p, W, dout, n_in, n_out, cu, da, d_status, st, row_map, epi);
     if (rc != SPA_OK) return rc;
   } else if (da != nullptr) {  // da[M][n_in] = dout[M][n_out] W[n_out][n_in]
-    int rc = launch_gemm<128, false, true, __nv_bfloat16>(tmA, tmB, nullptr, (__nv_bfloat16*)da, n_in, 0,
-                                                                 p.capacity, n_in, n_out, cu, p.B, p.capacity, 1, n_out,
-                                                                 1, 0, row_map, accumulate ? 1 : 0, d_status, st,
-                                                                 "gemm_tc_kernel(dgrad)");
+    auto go = [&](auto row_epi) {
+      return launch_gemm<128, false, true, __nv_bfloat16>(tmA, tmB, nullptr, (__nv_bfloat16*)da, n_in, 0, p.capacity, n_in, n_out, cu,
+                                                          p.B, p.capacity, 1, n_out, 1, 0, row_map, row_epi, d_status, st,
+                                                          "gemm_tc_kernel(dgrad)");
+    };
+    int rc = epi.u != nullptr ? go(RowEpilogue<kEpiGeluGrad>{(__nv_bfloat16*)const_cast<void*>(epi.u)})
+                              : go(RowEpilogue<kEpiOwn>{epi.add != nullptr ? (__nv_bfloat16*)da : nullptr});
     if (rc != SPA_OK) return rc;
   }
   if (dW == nullptr && db == nullptr) return SPA_OK;
@@ -574,7 +572,7 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
     int rc = pair ? launch_wgrad_pair(p, a, dout, n_in, n_out, cu, part_w, db != nullptr ? part_b : nullptr, pl, d_status, st)
                   : launch_gemm<128, true, true, float>(tmA2, tmB2, nullptr, part_w, n_in, n_w, n_out, n_in, p.capacity,
                                                         cu, p.B, p.capacity, 2, sp.k_per_split, sp.splits, sp.splits,
-                                                        nullptr, 0, d_status, st, "gemm_tc_kernel(wgrad)");
+                                                        nullptr, RowEpilogue<kEpiOwn>{nullptr}, d_status, st, "gemm_tc_kernel(wgrad)");
     if (rc != SPA_OK) return rc;
     const long long n_b = db != nullptr ? n_out : 0;
     int grid = (int)((n_w / 4 + 255) / 256);

@@ -93,13 +93,13 @@ constexpr int kPairSmem = kPairStages * kPairStage + 1024 + 256 + kPairEpiWarps 
 
 // kBMn: B = W is MN-major (input gradient: K = n_out rows of W, N = n_in contiguous); otherwise K-major
 // (forward: N = n_out rows of W, K = n_in contiguous).  A is always K-major, the output bf16.
-// M is the device-side packed row count.  row_map / accumulate as in the single-CTA kernel.
-template <bool kBMn>
+// M is the device-side packed row count.  row_map and epi as in the single-CTA kernel.
+template <bool kBMn, int kKind>
 __global__ void __launch_bounds__(kPairThreads)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __nv_bfloat16* __restrict__ bias, __nv_bfloat16* __restrict__ out, long long ldo, int N, int K,
                  const int32_t* __restrict__ cu, int n_seg, int capacity, const int32_t* __restrict__ row_map,
-                 int accumulate, int32_t* d_status) {
+                 RowEpilogue<kKind> epi, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(2 * PM, PN, false, kBMn);
   pdl_launch_dependents();
 
@@ -227,12 +227,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       for (int cc = half; cc < PN / 64; cc += 2) {
         if (n0 + cc * 64 >= N) break;  // warp-uniform: columns past the layer's width
         const int gcol = n0 + cc * 64 + my_chunk * 8;
-        uint4 old[8];  // what the rows hold, under the reads of the accumulator
-        if (accumulate) {
+        uint4 old[8];  // what the results are combined with, under the reads of the accumulator
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (m0 + q * 32 + my_row + 4 * j < M && gcol < N) old[j] = *reinterpret_cast<const uint4*>(out + orow[j] * ldo + gcol);
-        }
+        for (int j = 0; j < 8; ++j)
+          if (m0 + q * 32 + my_row + 4 * j < M && gcol < N) epi.fetch(out, old[j], orow[j] * ldo + gcol);
         uint32_t r[64];
         const uint32_t at = tmem_base + ((uint32_t)(q * 32) << 16) + acc * PN + cc * 64;
         ptx::tmem_ld_32x32(at, r);
@@ -257,19 +255,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int j = 0; j < 8; ++j) {
           const int rr = my_row + 4 * j;
           const uint4 v4 = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((my_chunk ^ (rr & 7)) << 4));
-          if (m0 + q * 32 + rr < M && gcol < N) {
-            uint4* dst = reinterpret_cast<uint4*>(out + orow[j] * ldo + gcol);
-            if (accumulate) {
-              float fa[8], fb[8];
-              Vec16<__nv_bfloat16>::to_float(old[j], fa);
-              Vec16<__nv_bfloat16>::to_float(v4, fb);
-#pragma unroll
-              for (int e = 0; e < 8; ++e) fa[e] += fb[e];
-              *dst = Vec16<__nv_bfloat16>::from_float(fa);
-            } else {
-              *dst = v4;
-            }
-          }
+          if (m0 + q * 32 + rr < M && gcol < N) epi.finish(out, orow[j] * ldo + gcol, v4, old[j]);
         }
         __syncwarp();
       }
@@ -531,18 +517,17 @@ int launch_clusters(void (*kern)(KArgs...), int pairs, int smem, cudaStream_t st
   return SPA_OK;
 }
 
-template <bool kBMn>
+template <bool kBMn, int kKind>
 int launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, __nv_bfloat16* out, long long ldo,
-                int N, int K, const int32_t* cu, int n_seg, int capacity, const int32_t* row_map, int accumulate,
+                int N, int K, const int32_t* cu, int n_seg, int capacity, const int32_t* row_map, RowEpilogue<kKind> epi,
                 int32_t* d_status, cudaStream_t st, const char* what) {
-  auto kern = gemm_pair_kernel<kBMn>;
+  auto kern = gemm_pair_kernel<kBMn, kKind>;
   static DeviceOnce smem_attr;  // per instantiation and device
   cudaError_t ea = smem_attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem); });
   if (ea != cudaSuccess) { set_cuda_error(ea, what); return SPA_ERR_CUDA; }
   const long long tiles = (long long)((N + PN - 1) / PN) * ((capacity + 2 * PM - 1) / (2 * PM));
   const int pairs = (int)(tiles < kMaxPairs ? (tiles < 1 ? 1 : tiles) : kMaxPairs);
-  return launch_clusters(kern, pairs, kPairSmem, st, what, tmA, tmB, bias, out, ldo, N, K, cu, n_seg, capacity, row_map, accumulate,
-                         d_status);
+  return launch_clusters(kern, pairs, kPairSmem, st, what, tmA, tmB, bias, out, ldo, N, K, cu, n_seg, capacity, row_map, epi, d_status);
 }
 
 }  // namespace
@@ -587,24 +572,34 @@ bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out, int n_co
 
 int launch_linear_fwd_pair(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
                            const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st, const int32_t* row_map,
-                           bool accumulate) {
+                           const LinearEpilogue& epi) {
   CUtensorMap tmA, tmB;
   if (!make_tmap_bf16_2d(&tmA, a, n_in, p.capacity, (uint64_t)n_in * 2, PK, PM) ||
       !make_tmap_bf16_2d(&tmB, W, n_in, n_out, (uint64_t)n_in * 2, PK, PN / 2))
     return SPA_ERR_UNSUPPORTED;
-  return launch_pair<false>(tmA, tmB, (const __nv_bfloat16*)bias, (__nv_bfloat16*)out, n_out, n_out, n_in, cu, p.B, p.capacity,
-                            row_map, accumulate ? 1 : 0, d_status, st, "gemm_pair_kernel(fwd)");
+  auto go = [&](auto row_epi) {
+    return launch_pair<false>(tmA, tmB, (const __nv_bfloat16*)bias, (__nv_bfloat16*)out, n_out, n_out, n_in, cu, p.B, p.capacity,
+                              row_map, row_epi, d_status, st, "gemm_pair_kernel(fwd)");
+  };
+  if (epi.h != nullptr) return go(RowEpilogue<kEpiGelu>{(__nv_bfloat16*)epi.h});
+  if (epi.add != nullptr && epi.add != out) return go(RowEpilogue<kEpiAdd>{(__nv_bfloat16*)const_cast<void*>(epi.add)});
+  return go(RowEpilogue<kEpiOwn>{epi.add != nullptr ? (__nv_bfloat16*)out : nullptr});
 }
 
 // da[M][n_in] = dout[M][n_out] W[n_out][n_in]
 int launch_linear_dgrad_pair(const spa_params& p, const void* W, const void* dout, int n_in, int n_out, const int32_t* cu,
-                             void* da, int32_t* d_status, cudaStream_t st, const int32_t* row_map, bool accumulate) {
+                             void* da, int32_t* d_status, cudaStream_t st, const int32_t* row_map,
+                             const LinearEpilogue& epi) {
   CUtensorMap tmA, tmB;
   if (!make_tmap_bf16_2d(&tmA, dout, n_out, p.capacity, (uint64_t)n_out * 2, PK, PM) ||
       !make_tmap_bf16_2d(&tmB, W, n_in, n_out, (uint64_t)n_in * 2, 64, PK))
     return SPA_ERR_UNSUPPORTED;
-  return launch_pair<true>(tmA, tmB, nullptr, (__nv_bfloat16*)da, n_in, n_in, n_out, cu, p.B, p.capacity, row_map,
-                           accumulate ? 1 : 0, d_status, st, "gemm_pair_kernel(dgrad)");
+  auto go = [&](auto row_epi) {
+    return launch_pair<true>(tmA, tmB, nullptr, (__nv_bfloat16*)da, n_in, n_in, n_out, cu, p.B, p.capacity, row_map, row_epi,
+                             d_status, st, "gemm_pair_kernel(dgrad)");
+  };
+  return epi.u != nullptr ? go(RowEpilogue<kEpiGeluGrad>{(__nv_bfloat16*)const_cast<void*>(epi.u)})
+                          : go(RowEpilogue<kEpiOwn>{epi.add != nullptr ? (__nv_bfloat16*)da : nullptr});
 }
 
 }  // namespace spa

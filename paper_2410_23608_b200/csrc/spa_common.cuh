@@ -108,6 +108,24 @@ __device__ __forceinline__ void st_global32(void* p, const uint4& a, const uint4
 }
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
+// The exact (erf) GELU and its derivative
+__device__ __forceinline__ float gelu_f(float u) { return 0.5f * u * (1.f + erff(u * 0.70710678118654752f)); }
+__device__ __forceinline__ float gelu_grad_f(float u) {
+  return 0.5f * (1.f + erff(u * 0.70710678118654752f)) + u * 0.3989422804014327f * __expf(-0.5f * u * u);
+}
+
+// Standard normal distribution function and density, Phi(u) and phi(u), from Abramowitz and Stegun 7.1.26: erfc(x) =
+// t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) e^(-x^2), t = 1 / (1 + 0.3275911 x), |error| <= 1.5e-7, x >= 0 (the tail is
+// the product itself, so it keeps its relative accuracy).  About half of erff's instructions.
+__device__ __forceinline__ void normal_cdf_pdf(float u, float& cdf, float& pdf) {
+  const float x = fabsf(u) * 0.70710678118654752f;
+  const float e = __expf(-x * x);
+  const float t = __fdividef(1.f, fmaf(0.3275911f, x, 1.f));
+  const float tail = 0.5f * t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f) * e;
+  cdf = u < 0.f ? tail : 1.f - tail;
+  pdf = 0.3989422804014327f * e;
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -222,14 +240,26 @@ size_t layer_norm_workspace_bytes(const spa_params& p);
 bool layer_norm_supported(const spa_params& p);
 int launch_layer_norm(const spa_params& p, const void* x, const void* gamma, const void* beta, float eps, void* y,
                       float* mean, float* rstd, cudaStream_t st);
+// with the gate on the normalised rows (scores, mask) and a copy of x
+int launch_layer_norm_gate(const spa_params& p, const void* x, const void* gamma, const void* beta, float eps, void* y,
+                           float* mean, float* rstd, const void* w_g, float b_g, float* scores, uint8_t* mask, void* copy,
+                           cudaStream_t st);
+// dy_row (optional): row t of dy is dy[dy_row[t]], zero where negative; dz_row, dz (optional): dz[dz_row[t]] = dx[t] too
 int launch_layer_norm_bwd(const spa_params& p, const void* dy, const void* x, const void* gamma, const float* mean,
                           const float* rstd, const void* add, void* dx, float* dgamma, float* dbeta, void* workspace,
-                          cudaStream_t st);
+                          cudaStream_t st, const int32_t* dy_row = nullptr, const int32_t* dz_row = nullptr,
+                          void* dz = nullptr);
 int launch_gelu(const spa_params& p, const void* u, const void* dh, int n_cols, void* out, cudaStream_t st);
 int launch_copy_tokens(const spa_params& p, const void* src, void* dst, cudaStream_t st);  // dst[B*N][C] = src
 
+// What a linear layer's result goes through on its way out, row by row (rows as they are written, after row_map):
+//   add   result += add                 (a residual branch; may be `out` itself)
+//   u     result *= gelu'(u)            (the input gradient through the activation; u has the result's shape)
+//   h     h = gelu(result) beside it    (h has the result's shape)
+struct LinearEpilogue { const void* add = nullptr; const void* u = nullptr; void* h = nullptr; };
+
 // out[M][n_out] = a[M][n_in] W[n_out][n_in]^T + bias, M = packed rows (device); row_map: output row i is written to row
-// row_map[i] of `out`, added to its contents if `accumulate`.  _simt: bf16 data on fp32 FMAs; _f32: fp32 data.
+// row_map[i] of `out`.  _simt: bf16 data on fp32 FMAs; _f32: fp32 data.
 int launch_linear_fwd_simt(const spa_params& p, const void* a, const void* W, const void* bias, int n_in,
                            int n_out, const int32_t* cu, void* out, cudaStream_t st, const int32_t* row_map = nullptr,
                            bool accumulate = false);
@@ -239,10 +269,10 @@ int launch_linear_bwd_simt(const spa_params& p, const void* a, const void* W, co
 int launch_colsum_simt(const spa_params& p, const void* dout, int n_out, const int32_t* cu, float* db, cudaStream_t st);
 int launch_linear_fwd_f32(const spa_params& p, const void* a, const void* W, const void* bias, int n_in, int n_out,
                           const int32_t* cu, void* out, int32_t* d_status, cudaStream_t st,
-                          const int32_t* row_map = nullptr, bool accumulate = false);
+                          const int32_t* row_map = nullptr, const LinearEpilogue& epi = {});
 int launch_linear_bwd_f32(const spa_params& p, const void* a, const void* W, const void* dout, int n_in, int n_out,
                           const int32_t* cu, void* da, float* dW, float* db, int32_t* d_status, cudaStream_t st,
-                          const int32_t* row_map = nullptr, bool accumulate = false);
+                          const int32_t* row_map = nullptr, const LinearEpilogue& epi = {});
 int launch_attention_fwd_simt(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao,
                               float* lse, cudaStream_t st);
 int launch_attention_bwd_simt(const spa_params& p, const void* qkv, const void* ao, const float* lse,
