@@ -431,6 +431,8 @@ typedef struct spa_layer_buffers {
   float *dW1, *db1, *dW2, *db2, *dg1, *dbe1, *dg2, *dbe2;
   void* workspace;            /* at least spa_workspace_bytes(), spa_train_workspace_bytes() and
                                  32 (hidden C + max(hidden, C)) floats + 1 KB                        */
+  void* workspace_side;       /* a second area of that size: the weight gradients then run on the second
+                                 stream of blk->overlap; or NULL                                     */
 } spa_layer_buffers;
 
 /* Forward pass of the block.  blk->pack_state, order, s_up, seg_offsets and container_len are not looked at. */

@@ -75,7 +75,7 @@ class SpaLayerBuffers(C.Structure):
                 [(n, C.c_void_p) for n in (
                     "x", "g1", "be1", "g2", "be2", "W1", "b1", "W2", "b2", "cu_all", "z", "y1", "t", "out", "u", "h", "m1", "r1",
                     "m2", "r2", "d_out", "dh", "dt", "dy1", "dX", "dW1", "db1", "dW2", "db2", "dg1", "dbe1", "dg2", "dbe2",
-                    "workspace")])
+                    "workspace", "workspace_side")])
 
 
 def make_params(B, N, Cc, H, dtype, capacity=None, flags=0, tau=0.0, softmax_scale=0.0) -> SpaParams:

@@ -634,7 +634,7 @@ int linear_fwd_epi(const spa_params* p, const void* a, const void* W, const void
 // ... and the gradients of one; da *= gelu'(u)
 int linear_bwd_gelu(const spa_params* p, const void* a, const void* W, const void* dout, int n_in, int n_out, const int32_t* cu,
                     void* da, const void* u, float* dW, float* db, void* workspace, int32_t* d_status, void* stream) {
-  SPA_PTR(a); SPA_PTR(W); SPA_PTR(dout); SPA_PTR(cu); SPA_PTR(da); SPA_PTR(u); SPA_PTR(dW); SPA_PTR(db); SPA_OPT_PTR(workspace);
+  SPA_PTR(a); SPA_PTR(W); SPA_PTR(dout); SPA_PTR(cu); SPA_PTR(da); SPA_PTR(u); SPA_OPT_PTR(dW); SPA_OPT_PTR(db); SPA_OPT_PTR(workspace);
   const int es = p->dtype == SPA_F32 ? 4 : 2;
   SPA_REQUIRE(n_in > 0 && n_out > 0, SPA_ERR_INVALID_ARG);
   SPA_REQUIRE((n_in * es) % 16 == 0 && (n_out * es) % 16 == 0, SPA_ERR_UNSUPPORTED);
@@ -703,17 +703,46 @@ int spa_layer_bwd(const spa_params* p, const spa_layer_buffers* l, void* stream)
   SPA_REQUIRE(l->dg1 != nullptr && l->dbe1 != nullptr && l->dg2 != nullptr && l->dbe2 != nullptr && l->workspace != nullptr,
               SPA_ERR_INVALID_ARG);
   if (p->B == 0) return SPA_OK;
-  SPA_STEP(linear_bwd_gelu(p, l->h, l->W2, l->d_out, Hd, C, l->cu_all, l->dh, l->u, l->dW2, l->db2, l->workspace, b->d_status, stream));
-  SPA_STEP(spa_packed_linear_bwd(p, l->t, l->W1, l->dh, C, Hd, l->cu_all, l->dt, l->dW1, l->db1, l->workspace, b->d_status, stream));
-  SPA_STEP(launch_layer_norm_bwd(*p, l->dt, l->y1, l->g2, l->m2, l->r2, l->d_out, l->dy1, l->dg2, l->dbe2, l->workspace, st, nullptr,
-                                 b->inv, b->dz));
-  SPA_STEP(spa_packed_linear_bwd(p, b->attn_out, b->W_o, b->dz, C, C, b->cu_seqlens, b->d_attn_out, b->dW_o, b->db_o, l->workspace,
-                                 b->d_status, stream));
-  SPA_STEP(spa_packed_attention_bwd(p, b->qkv, b->attn_out, b->lse, b->d_attn_out, b->cu_seqlens, p->B, b->dqkv, l->workspace,
-                                    b->d_status, stream));
-  SPA_STEP(spa_packed_linear_bwd(p, b->x_packed, b->W_qkv, b->dqkv, C, 3 * C, b->cu_seqlens, b->dx_packed, b->dW_qkv, b->db_qkv,
-                                 l->workspace, b->d_status, stream));
-  return launch_layer_norm_bwd(*p, b->dx_packed, l->x, l->g1, l->m1, l->r1, l->dy1, l->dX, l->dg1, l->dbe1, l->workspace, st, b->inv);
+  // the weight gradients on the second stream where there is one, each beside the input gradient of its layer and what
+  // follows (as in spa_block_bwd)
+  const spa_overlap* ov = l->workspace_side != nullptr ? b->overlap : nullptr;
+  void* side = ov != nullptr ? (void*)ov->side : stream;
+  void* ws_side = ov != nullptr ? l->workspace_side : l->workspace;
+  bool forked = false;
+  auto fork = [&]() -> int {
+    if (ov == nullptr) return SPA_OK;
+    forked = true;
+    return fork_side(ov, st);
+  };
+  auto run = [&]() -> int {
+    SPA_STEP(fork());
+    SPA_STEP(spa_packed_linear_bwd(p, l->h, l->W2, l->d_out, Hd, C, l->cu_all, nullptr, l->dW2, l->db2, ws_side, b->d_status, side));
+    SPA_STEP(linear_bwd_gelu(p, l->h, l->W2, l->d_out, Hd, C, l->cu_all, l->dh, l->u, nullptr, nullptr, l->workspace, b->d_status, stream));
+    SPA_STEP(fork());
+    SPA_STEP(spa_packed_linear_bwd(p, l->t, l->W1, l->dh, C, Hd, l->cu_all, nullptr, l->dW1, l->db1, ws_side, b->d_status, side));
+    SPA_STEP(spa_packed_linear_bwd(p, l->t, l->W1, l->dh, C, Hd, l->cu_all, l->dt, nullptr, nullptr, l->workspace, b->d_status, stream));
+    SPA_STEP(launch_layer_norm_bwd(*p, l->dt, l->y1, l->g2, l->m2, l->r2, l->d_out, l->dy1, l->dg2, l->dbe2, l->workspace, st, nullptr,
+                                   b->inv, b->dz));
+    SPA_STEP(fork());
+    SPA_STEP(spa_packed_linear_bwd(p, b->attn_out, b->W_o, b->dz, C, C, b->cu_seqlens, nullptr, b->dW_o, b->db_o, ws_side, b->d_status,
+                                   side));
+    SPA_STEP(spa_packed_linear_bwd(p, b->attn_out, b->W_o, b->dz, C, C, b->cu_seqlens, b->d_attn_out, nullptr, nullptr, l->workspace,
+                                   b->d_status, stream));
+    SPA_STEP(spa_packed_attention_bwd(p, b->qkv, b->attn_out, b->lse, b->d_attn_out, b->cu_seqlens, p->B, b->dqkv, l->workspace,
+                                      b->d_status, stream));
+    SPA_STEP(fork());
+    SPA_STEP(spa_packed_linear_bwd(p, b->x_packed, b->W_qkv, b->dqkv, C, 3 * C, b->cu_seqlens, nullptr, b->dW_qkv, b->db_qkv, ws_side,
+                                   b->d_status, side));
+    SPA_STEP(spa_packed_linear_bwd(p, b->x_packed, b->W_qkv, b->dqkv, C, 3 * C, b->cu_seqlens, b->dx_packed, nullptr, nullptr,
+                                   l->workspace, b->d_status, stream));
+    return launch_layer_norm_bwd(*p, b->dx_packed, l->x, l->g1, l->m1, l->r1, l->dy1, l->dX, l->dg1, l->dbe1, l->workspace, st, b->inv);
+  };
+  rc = run();
+  if (forked) {  // joined on every path, so that a recording stream is never left forked
+    const int rj = join_side(ov, st);
+    if (rc == SPA_OK) rc = rj;
+  }
+  return rc;
 }
 #undef SPA_STEP
 

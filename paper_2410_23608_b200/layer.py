@@ -38,10 +38,11 @@ class SpaLayer:
         # split-K partials of the widest weight gradient (at most 32 splits) and the per-CTA sums of the LayerNorm backward
         ws = max(L.spa_workspace_bytes(self.p), 32 * self.hidden * C * 4 + 32 * max(self.hidden, C) * 4 + 1024,
                  L.spa_train_workspace_bytes(self.p))
-        self.workspace = torch.empty(ws, dtype=torch.uint8, device=dev)
+        self.workspace, self.workspace_side = (torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(2))
+        self.blk._bufs.overlap = self.blk._overlap  # the weight gradients on the library's second stream
         self._lib = L.lib()
         own = ("cu_all", "z", "y1", "t", "out", "u", "h", "m1", "r1", "m2", "r2", "dh", "dt", "dy1", "dX", "dW1", "db1", "dW2", "db2",
-               "dg1", "dbe1", "dg2", "dbe2", "workspace")
+               "dg1", "dbe1", "dg2", "dbe2", "workspace", "workspace_side")
         self._bufs = L.SpaLayerBuffers(blk=ctypes.pointer(self.blk._bufs), hidden=self.hidden, eps=eps,
                                        **{k: L._ptr(getattr(self, k)) for k in own})
         self._args = (ctypes.byref(self.p), ctypes.byref(self._bufs))
