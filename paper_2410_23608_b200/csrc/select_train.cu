@@ -61,17 +61,36 @@ select_loss_kernel(const float* __restrict__ scores, const uint8_t* __restrict__
 }
 
 // out[j] = sum over blocks of part[block * stride + j] for j < n_out; columns n_out .. n_out + n_out2 - 1 go to out2.
-// One warp per column: lane l adds blocks l, l + 32, ... in order, then the lanes combine in a fixed tree.
-__global__ void __launch_bounds__(kTrainThreads)
+// kWide: 32 columns per CTA, a lane each, so that every load is a whole line; warp w adds blocks w, w + 32, ... in order, then
+// the warps' sums in a fixed tree.  Otherwise one warp per column: lane l adds blocks l, l + 32, ..., then a fixed tree.  (A warp
+// per column read a 32-byte sector for 4 bytes: 296 blocks of 1 536 columns.)
+constexpr int kSumThreads = 1024;
+template <bool kWide>
+__global__ void __launch_bounds__(kWide ? kSumThreads : kTrainThreads)
 partial_sum_kernel(const float* __restrict__ part, int n_blocks, int stride, int n_out, float* __restrict__ out, int n_out2,
                    float* __restrict__ out2) {
   pdl_entry();
-  const int j = blockIdx.x * (kTrainThreads / 32) + (threadIdx.x >> 5);
-  if (j >= n_out + n_out2) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float s = 0.f;
-  for (int b = threadIdx.x & 31; b < n_blocks; b += 32) s += part[(long long)b * stride + j];
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) {
+  int j;
+  if (kWide) {
+    __shared__ float sums[kSumThreads / 32][33];
+    j = blockIdx.x * 32 + lane;
+    if (j < n_out + n_out2) {
+#pragma unroll 8
+      for (int b = warp; b < n_blocks; b += kSumThreads / 32) s += part[(long long)b * stride + j];
+    }
+    sums[warp][lane] = s;
+    __syncthreads();
+    j = blockIdx.x * 32 + warp;
+    s = warp_sum(sums[lane][warp]);  // a warp takes a column
+  } else {
+    j = blockIdx.x * (kTrainThreads / 32) + warp;
+    if (j >= n_out + n_out2) return;
+    for (int b = lane; b < n_blocks; b += 32) s += part[(long long)b * stride + j];
+    s = warp_sum(s);
+  }
+  if (lane == 0 && j < n_out + n_out2) {
     if (j < n_out) out[j] = s; else out2[j - n_out] = s;
   }
 }
@@ -220,8 +239,11 @@ int launch_partial_sum(const float* part, int n_blocks, int stride, int n_out, f
                        cudaStream_t st) {
   if (out2 == nullptr) n_out2 = 0;
   const int cols = n_out + n_out2;
-  launch_pdl(partial_sum_kernel, (cols + kTrainThreads / 32 - 1) / (kTrainThreads / 32), kTrainThreads, 0, st, part, n_blocks,
-             stride, n_out, out, n_out2, out2);
+  if (cols >= 32)
+    launch_pdl(partial_sum_kernel<true>, (cols + 31) / 32, kSumThreads, 0, st, part, n_blocks, stride, n_out, out, n_out2, out2);
+  else
+    launch_pdl(partial_sum_kernel<false>, (cols + kTrainThreads / 32 - 1) / (kTrainThreads / 32), kTrainThreads, 0, st, part, n_blocks,
+               stride, n_out, out, n_out2, out2);
   SPA_CUDA_CHECK_LAUNCH("partial_sum_kernel");
   return SPA_OK;
 }
