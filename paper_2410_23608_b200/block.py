@@ -164,7 +164,7 @@ class SpaBlock:
             b.loss, b.train_workspace = L._ptr(self.loss), L._ptr(self.train_ws)
         b = self._bufs
         b.x, b.w_g, b.s_up, b.labels, b.alpha = L._ptr(x), L._ptr(w_g), L._ptr(s_up), L._ptr(labels), float(alpha)
-        return self._backward(dY, dX, None, 1)
+        return self._backward(dY, dX, self._overlap, 1)
 
     def read_status(self) -> int:
         """Blocking: the device status word (0 = ok)."""

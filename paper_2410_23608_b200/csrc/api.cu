@@ -543,8 +543,8 @@ int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream)
   const int C = p->C;
   cudaStream_t main = (cudaStream_t)stream;
   // the weight gradients feed nothing downstream: with `overlap` they run on the second stream, with a scratch
-  // area of their own, beside the attention backward and the input gradients.  The trainable path keeps one stream.
-  const spa_overlap* ov = b->trainable ? nullptr : b->overlap;
+  // area of their own, beside the attention backward and the input gradients.
+  const spa_overlap* ov = b->overlap;
   SPA_REQUIRE(ov == nullptr || b->workspace_side != nullptr || spa_workspace_bytes(p) == 0, SPA_ERR_INVALID_ARG);
   const bool fused = block_fused(p) && !b->trainable;
   const int32_t* seg = b->seg_offsets != nullptr ? b->seg_offsets : b->cu_seqlens;
@@ -599,15 +599,13 @@ int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream)
       }
     }
   }
+  if (rc == SPA_OK && rc_side == SPA_OK && b->trainable)
+    rc = spa_gate_bwd(p, b->x, b->w_g, b->scores, b->s_up, b->ds, b->dX, b->dw_g, b->db_g, b->ds_up, b->train_workspace, stream);
   if (forked) {  // joined on every path, so that a recording stream is never left forked
     const int rj = join_side(ov, main);
     if (rc == SPA_OK) rc = rc_side != SPA_OK ? rc_side : rj;
   }
-  if (rc != SPA_OK) return rc;
-  if (b->trainable)
-    SPA_STEP(spa_gate_bwd(p, b->x, b->w_g, b->scores, b->s_up, b->ds, b->dX, b->dw_g, b->db_g, b->ds_up,
-                          b->train_workspace, stream));
-  return SPA_OK;
+  return rc;
 }
 namespace {
 // A linear layer whose result goes through `epi` on its way out, whichever kernels the problem takes: where they cannot
