@@ -91,7 +91,7 @@ struct TileCoord { int m0, n0, z, n_t; };
 // overlap the main loop of the next, and the TMA ring runs ahead across tile boundaries.
 // row_map (optional): output row i goes to row row_map[i] of `out` (the unpack scatter fused into the
 // epilogue).  epi: what a bf16 result goes through on its way out (RowEpilogue; split-K partials go as they are).
-template <int BN, bool kAMn, bool kBMn, typename OutT, int kKind>
+template <int BN, bool kDyn, bool kAMn, bool kBMn, typename OutT, int kKind>
 __global__ void __launch_bounds__(kGemmThreads)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __nv_bfloat16* __restrict__ bias, OutT* __restrict__ out, long long ldo,
@@ -99,7 +99,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                int dyn_which, int k_per_split, int k_interleave, const int32_t* __restrict__ row_map,
                RowEpilogue<kKind> epi, int32_t* d_status) {
   constexpr int kStage = stage_bytes<BN>();
-  constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(BM, BN, kAMn, kBMn);
   pdl_launch_dependents();
 
   extern __shared__ uint8_t smem_raw[];
@@ -136,8 +135,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int rows = packed_rows(cu, n_seg, capacity);
     if (dyn_which == 1) M = rows; else if (dyn_which == 2) K = rows;
   }
-  const int tiles_n = (N + BN - 1) / BN;
   const int tiles_m = (M + BM - 1) / BM;
+  const int bn = kDyn && (long long)tiles_m * ((N + BN - 1) / BN) <= kNumSMs ? BN / 2 : BN;  // see tile_width
+  const int tiles_n = (N + bn - 1) / bn;
+  const uint32_t idesc = bn == BN ? ptx::idesc_bf16_f32(BM, BN, kAMn, kBMn) : ptx::idesc_bf16_f32(BM, 64, kAMn, kBMn);
   // Split-K: contiguous spans of k_per_split, or (k_interleave > 0) that many splits dealt the BK-blocks of K in
   // turn - split z takes blocks z, z + splits, ... - so that the splits get equal work whatever K turns out to be.
   const int k_blocks = (K + BK - 1) / BK;
@@ -150,7 +151,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int rest = tile / tiles_n;
     c.m0 = (rest % tiles_m) * BM;
     c.z = rest / tiles_m;
-    c.n0 = c.n_t * BN;
+    c.n0 = c.n_t * bn;
     return c;
   };
   auto k_range = [&](int z, int& k_begin, int& k_end, int& k_step) {
@@ -181,7 +182,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const int s = it % kStages;
           if (it >= kStages) wait_lane(empty_bar(s), ((it / kStages) - 1) & 1);
           const uint32_t a_dst = smem_base + s * kStage, b_dst = a_dst + kABytes;
-          ptx::mbar_expect_tx(full_bar(s), kStage);
+          ptx::mbar_expect_tx(full_bar(s), kABytes + bn * BK * 2);
           if (!kAMn) {
             ptx::tma_load_2d(a_dst, &tmA, full_bar(s), k0, c.m0);
           } else {
@@ -190,11 +191,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               ptx::tma_load_2d(a_dst + j * (BK * 128), &tmA, full_bar(s), c.m0 + 64 * j, k0);
           }
           if (!kBMn) {
-            ptx::tma_load_2d(b_dst, &tmB, full_bar(s), k0, c.n0);
+            constexpr int kBox = kDyn ? 64 : BN;  // rows of W per copy
+#pragma unroll
+            for (int j = 0; j < BN / kBox; ++j)
+              if (j * kBox < bn) ptx::tma_load_2d(b_dst + j * (kBox * 128), &tmB, full_bar(s), k0, c.n0 + kBox * j);
           } else {
 #pragma unroll
             for (int j = 0; j < BN / 64; ++j)
-              ptx::tma_load_2d(b_dst + j * (BK * 128), &tmB, full_bar(s), c.n0 + 64 * j, k0);
+              if (j * 64 < bn) ptx::tma_load_2d(b_dst + j * (BK * 128), &tmB, full_bar(s), c.n0 + 64 * j, k0);
           }
         }
       }
@@ -229,7 +233,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 *reinterpret_cast<uint4*>(smem_al + s * kStage + j * (BK * 128) + (k_valid + q / 8) * 128 + (q % 8) * 16) =
                     make_uint4(0, 0, 0, 0);
           if (kBMn)
-            for (int j = 0; j < BN / 64; ++j)
+            for (int j = 0; j < bn / 64; ++j)
               for (int q = lane; q < n_lines * 8; q += 32)
                 *reinterpret_cast<uint4*>(smem_al + s * kStage + kABytes + j * (BK * 128) + (k_valid + q / 8) * 128 +
                                           (q % 8) * 16) = make_uint4(0, 0, 0, 0);
@@ -244,7 +248,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                         : ptx::smem_desc_sw128(a_src + k * 32, 16, 1024);
             const uint64_t bdesc = kBMn ? ptx::smem_desc_sw128(b_src + k * 2048, BK * 128, 1024)
                                         : ptx::smem_desc_sw128(b_src + k * 32, 16, 1024);
-            ptx::mma_bf16(tmem_d, adesc, bdesc, kIdesc, (first && k == 0) ? 0u : 1u);
+            ptx::mma_bf16(tmem_d, adesc, bdesc, idesc, (first && k == 0) ? 0u : 1u);
           }
           ptx::mma_commit(empty_bar(s));
         }
@@ -276,12 +280,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         orow[j] = (row_map != nullptr && grow < M) ? (long long)ld_dep(row_map + grow) : (long long)grow;
       }
       // the bias of the tile comes to L1 under the main loop: fetched where it is added, each 32 columns waited for L2
-      if (bias != nullptr && lane < BN / 64 && c.n0 + lane * 64 < N) prefetch_l1(bias + c.n0 + lane * 64);
+      if (bias != nullptr && lane < bn / 64 && c.n0 + lane * 64 < N) prefetch_l1(bias + c.n0 + lane * 64);
       wait(tmem_full_bar(acc), (tl >> 1) & 1);
       if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
       ptx::tc_fence_after_sync();
 #pragma unroll 1
-      for (int cc = 0; cc < BN / 32; ++cc) {
+      for (int cc = 0; cc < bn / 32; ++cc) {
         uint4 old[4];  // what the results are combined with, under the read of the accumulator
         if constexpr (sizeof(OutT) == 2) {
 #pragma unroll
@@ -474,23 +478,43 @@ size_t wgrad_workspace_bytes(int capacity, int n_in, int n_out) {
 
 inline bool wgrad_on_pairs(const spa_params& p) { return !(p.flags & SPA_FLAG_NO_CTA_PAIRS); }
 
-template <int BN, bool kAMn, bool kBMn, typename OutT, int kKind>
+template <int BN, bool kDyn, bool kAMn, bool kBMn, typename OutT, int kKind>
 int launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, OutT* out, long long ldo,
                 long long split_stride, int M, int N, int K, const int32_t* cu, int n_seg, int capacity, int dyn_which,
                 int k_per_split, int splits, int k_interleave, const int32_t* row_map, RowEpilogue<kKind> epi,
                 int32_t* d_status, cudaStream_t st, const char* what) {
-  auto kern = gemm_tc_kernel<BN, kAMn, kBMn, OutT, kKind>;
+  auto kern = gemm_tc_kernel<BN, kDyn, kAMn, kBMn, OutT, kKind>;
   static DeviceOnce attr;  // per instantiation and device
   cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes<BN>()); });
   if (ea != cudaSuccess) { set_cuda_error(ea, what); return SPA_ERR_CUDA; }
   // persistent grid: two CTAs per SM (99 KB of shared memory and 256 TMEM columns each), never more
   // CTAs than there are tiles when every allocated row is in use
-  long long tiles = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM) * splits;
+  long long tiles = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM) * splits * (kDyn ? 2 : 1);
   const int grid = (int)(tiles < 2 * kNumSMs ? (tiles < 1 ? 1 : tiles) : 2 * kNumSMs);
   launch_pdl(kern, grid, kGemmThreads, gemm_smem_bytes<BN>(), st, tmA, tmB, bias, out, ldo, split_stride, M, N, K, cu,
              n_seg, capacity, dyn_which, k_per_split, k_interleave, row_map, epi, d_status);
   SPA_CUDA_CHECK_LAUNCH(what);
   return SPA_OK;
+}
+
+// Tiles of 64 columns where that leaves every tile a CTA of its own from the start (two per SM): twice the SMs share the
+// operands' way into shared memory, which bounds the main loop, and the epilogue.  98 rows 384 -> 1 152: 5.9 -> 4.8 us; 1 568
+// rows 1 536 -> 384: 10.6 -> 9.4; past that line they lose up to 40 % (3 120 rows 2 304 -> 768: 16.3 -> 23.2).  The rows that
+// there are decide, the host knows the capacity, of which about half is filled: up to 148 wide tiles for all of it narrow ones,
+// up to twice as many the kernel chooses (0.3 us slower with wide tiles than the kernel that has no choice), above wide ones.
+enum TileWidth { kNarrow, kByRows, kWide };
+inline TileWidth tile_width(int capacity, int n_cols) {
+  const long long wide = (long long)((capacity + BM - 1) / BM) * ((n_cols + 127) / 128);
+  return wide <= kNumSMs ? kNarrow : (wide <= 2 * kNumSMs ? kByRows : kWide);
+}
+template <bool kBMn, int kKind>
+int launch_width(TileWidth width, const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, __nv_bfloat16* out,
+                 const spa_params& p, int n_cols, int k, const int32_t* cu, const int32_t* row_map, RowEpilogue<kKind> epi,
+                 int32_t* d_status, cudaStream_t st, const char* what) {
+  auto run = width == kNarrow   ? launch_gemm<64, false, false, kBMn, __nv_bfloat16, kKind>
+             : width == kByRows ? launch_gemm<128, true, false, kBMn, __nv_bfloat16, kKind>
+                                : launch_gemm<128, false, false, kBMn, __nv_bfloat16, kKind>;
+  return run(tmA, tmB, bias, out, n_cols, 0, p.capacity, n_cols, k, cu, p.B, p.capacity, 1, k, 1, 0, row_map, epi, d_status, st, what);
 }
 
 }  // namespace
@@ -511,14 +535,14 @@ int launch_linear_fwd_tc(const spa_params& p, const void* a, const void* W, cons
                          const LinearEpilogue& epi) {
   if (tc_pair_linear_supported(p, n_in, n_out, n_out))
     return launch_linear_fwd_pair(p, a, W, bias, n_in, n_out, cu, out, d_status, st, row_map, epi);
+  const TileWidth width = tile_width(p.capacity, n_out);
   CUtensorMap tmA, tmB;
   if (!make_tmap_bf16_2d(&tmA, a, n_in, p.capacity, (uint64_t)n_in * 2, BK, BM) ||
-      !make_tmap_bf16_2d(&tmB, W, n_in, n_out, (uint64_t)n_in * 2, BK, 128))
+      !make_tmap_bf16_2d(&tmB, W, n_in, n_out, (uint64_t)n_in * 2, BK, width == kWide ? 128 : 64))
     return SPA_ERR_UNSUPPORTED;
   auto go = [&](auto row_epi) {
-    return launch_gemm<128, false, false, __nv_bfloat16>(tmA, tmB, (const __nv_bfloat16*)bias, (__nv_bfloat16*)out, n_out, 0,
-                                                         p.capacity, n_out, n_in, cu, p.B, p.capacity, 1, n_in, 1, 0, row_map,
-                                                         row_epi, d_status, st, "gemm_tc_kernel(fwd)");
+    return launch_width<false>(width, tmA, tmB, (const __nv_bfloat16*)bias, (__nv_bfloat16*)out, p, n_out, n_in, cu, row_map, row_epi,
+                               d_status, st, "gemm_tc_kernel(fwd)");
   };
   if (epi.h != nullptr) return go(RowEpilogue<kEpiGelu>{(__nv_bfloat16*)epi.h});
   if (epi.add != nullptr && epi.add != out) return go(RowEpilogue<kEpiAdd>{(__nv_bfloat16*)const_cast<void*>(epi.add)});
@@ -541,9 +565,8 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
     if (rc != SPA_OK) return rc;
   } else if (da != nullptr) {  // da[M][n_in] = dout[M][n_out] W[n_out][n_in]
     auto go = [&](auto row_epi) {
-      return launch_gemm<128, false, true, __nv_bfloat16>(tmA, tmB, nullptr, (__nv_bfloat16*)da, n_in, 0, p.capacity, n_in, n_out, cu,
-                                                          p.B, p.capacity, 1, n_out, 1, 0, row_map, row_epi, d_status, st,
-                                                          "gemm_tc_kernel(dgrad)");
+      return launch_width<true>(tile_width(p.capacity, n_in), tmA, tmB, nullptr, (__nv_bfloat16*)da, p, n_in, n_out, cu, row_map, row_epi,
+                                d_status, st, "gemm_tc_kernel(dgrad)");
     };
     int rc = epi.u != nullptr ? go(RowEpilogue<kEpiGeluGrad>{(__nv_bfloat16*)const_cast<void*>(epi.u)})
                               : go(RowEpilogue<kEpiOwn>{epi.add != nullptr ? (__nv_bfloat16*)da : nullptr});
@@ -570,7 +593,7 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
   }
   if (dW != nullptr) {  // dW[n_out][n_in] = sum_i dout[i][:]^T a[i][:]
     int rc = pair ? launch_wgrad_pair(p, a, dout, n_in, n_out, cu, part_w, db != nullptr ? part_b : nullptr, pl, d_status, st)
-                  : launch_gemm<128, true, true, float>(tmA2, tmB2, nullptr, part_w, n_in, n_w, n_out, n_in, p.capacity,
+                  : launch_gemm<128, false, true, true, float>(tmA2, tmB2, nullptr, part_w, n_in, n_w, n_out, n_in, p.capacity,
                                                         cu, p.B, p.capacity, 2, sp.k_per_split, sp.splits, sp.splits,
                                                         nullptr, RowEpilogue<kEpiOwn>{nullptr}, d_status, st, "gemm_tc_kernel(wgrad)");
     if (rc != SPA_OK) return rc;

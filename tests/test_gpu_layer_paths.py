@@ -31,3 +31,26 @@ def test_layer_paths(ci, B, flag):
                            ("db1", lay.db1, bwd["db1"]), ("dg1", lay.dg1, bwd["dg1"]), ("dbe2", lay.dbe2, bwd["dbe2"]),
                            ("dW_qkv", lay.blk.dW_qkv, bwd["dW_qkv"])):
         assert_close(host(got), ref, dt, name, scale_max_abs=True)
+
+
+# rows around the line between narrow and wide tiles of the single-CTA products (148 wide tiles), remainders of both
+@pytest.mark.parametrize("rows,n_in,n_out", [(1, 64, 72), (129, 136, 64), (2368, 72, 1024), (2369, 64, 1024), (2432, 64, 1032),
+                                             (6272, 384, 384), (18944, 64, 128), (18945, 64, 120)])
+@pytest.mark.parametrize("slack", [0, 300, 20000])   # capacity past the rows: narrow tiles, chosen by the rows, wide
+def test_linear_tile_widths(rows, n_in, n_out, slack):
+    from paper_2410_23608_b200 import binding as L
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    cap = rows + slack
+    p = L.make_params(1, cap, 64, 2, "bf16", cap, flags=L.SPA_FLAG_NO_CTA_PAIRS)
+    cu = torch.tensor([0, rows], dtype=torch.int32, device="cuda")
+    a, W, b, dout = rnd(cap, n_in), rnd(n_out, n_in), rnd(n_out), rnd(cap, n_out)
+    a[rows:], dout[rows:] = float("nan"), float("nan")
+    out, da = torch.full((cap, n_out), 7.0, device="cuda").bfloat16(), torch.full((cap, n_in), 7.0, device="cuda").bfloat16()
+    ws, status = torch.empty(64 << 20, dtype=torch.uint8, device="cuda"), torch.zeros(4, dtype=torch.int32, device="cuda")
+    L.spa_packed_linear(p, a, W, b, n_in, n_out, cu, out, d_status=status)
+    L.spa_packed_linear_bwd(p, a, W, dout, n_in, n_out, cu, da, None, None, ws, d_status=status)
+    assert L.spa_read_status(status) == 0
+    for got, ref in ((out[:rows], a[:rows].double() @ W.double().T + b.double()), (da[:rows], dout[:rows].double() @ W.double())):
+        assert float(((got.double() - ref).abs() / (1e-2 * ref.abs() + 1e-2 * ref.abs().mean())).max()) < 1
+    assert bool((out[rows:] == 7).all()) and bool((da[rows:] == 7).all())
