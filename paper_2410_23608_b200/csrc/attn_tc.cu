@@ -18,7 +18,6 @@
 
 #include <mutex>
 #include <unordered_map>
-#include <vector>
 
 #include "sm100_ptx.cuh"
 #include "spa_tc.cuh"
@@ -141,7 +140,7 @@ __device__ __forceinline__ void order_items(ItemOrder* o, const int32_t* s_off, 
 
 // The next item for this CTA, after its first.  The first `given` items (whole row tiles) go to the CTAs of their number,
 // the others are drawn: every CTA draws until it gets a number past the last item, so that a launch takes n_items - given
-// + gridDim.x numbers and the counter wraps to zero with the last of them, for the next launch of the stream.  Without a
+// + gridDim.x numbers and the counter wraps to zero with the last of them, for the next launch.  Without a
 // counter: a static stride.
 __device__ __forceinline__ int draw_item(unsigned* counter, int given, int n_items, int& own) {
   own += gridDim.x;
@@ -1891,11 +1890,8 @@ int bwd_launch(const spa_params& p, const void* qkv, const void* ao, const float
   return SPA_OK;
 }
 
-// The counter that a launch on stream `st` draws its items from, or nullptr (then items are assigned by a static stride).
-// Launches of a stream run one after the other and each leaves its counter at zero, so a stream needs one counter: it is
-// found by the stream's id, which is never reused.  A launch that is being recorded gets one for itself, since its graph
-// may be replayed beside anything: 12 288 of them, then nullptr.
-unsigned* item_counter(cudaStream_t st);
+// The counter that a launch which writes `out` draws its items from, or nullptr (then a static stride assigns them).
+unsigned* item_counter(const void* out, cudaStream_t st);
 
 template <int D>
 int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao, float* lse,
@@ -1913,7 +1909,7 @@ int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_s
   // 400 rows (and cost 1 us in front of short items), and 8 to 12 % from 576 rows on.
   const bool even_items = (long long)p.capacity <= 512ll * (n_seg > 0 ? n_seg : 1);
   launch_pdl(kern, grid, kFwdThreads, FwdSmem<D>::kBytes, st, tm, seg, n_seg, p.capacity, p.C, p.H,
-             softmax_scale_of(p) * 1.4426950408889634f, (__nv_bfloat16*)ao, lse, items > grid ? item_counter(st) : nullptr, even_items, d_status);
+             softmax_scale_of(p) * 1.4426950408889634f, (__nv_bfloat16*)ao, lse, items > grid ? item_counter(ao, st) : nullptr, even_items, d_status);
   SPA_CUDA_CHECK_LAUNCH("attn_fwd_tc_kernel");
   return SPA_OK;
 }
@@ -1955,11 +1951,13 @@ int launch_attention_fwd_tc(const spa_params& p, const void* qkv, const int32_t*
 // device, with that device current, and cached.
 static __device__ __align__(256) unsigned char g_static_scratch[SPA_STATIC_SCRATCH_BYTES];
 
-// Item counters of the persistent attention kernels: zero when the library is loaded and after every launch.  A stream
-// has one, since its launches follow one another; a recorded launch has one of its own, since graphs may run side by side,
-// and gives it back with its graph.  A launch that finds none left strides over its items.
-static constexpr int kStreamCounters = 4096, kRecordedCounters = 12288;
-static __device__ unsigned g_item_counters[kStreamCounters + kRecordedCounters];
+// Item counters of the attention forward kernel: zero when the library is loaded and after every launch.  A launch uses the
+// one that belongs to its output array: two launches that write the same array cannot run side by side, on whatever
+// streams or in whatever graphs they are.  (One per recorded launch, given back by a user object of its graph, made every
+// replay of the graph 40 to 100 us slower.)  An array keeps its counter while the library is loaded; the arrays past the
+// first 16 384 get none, and their launches stride over the items.
+static constexpr int kCounters = 16384;
+static __device__ unsigned g_item_counters[kCounters];
 
 namespace spa {
 namespace {
@@ -1969,83 +1967,37 @@ void* g_scratch_ptr[kMaxDevices] = {};
 }  // namespace
 
 namespace {
-struct RecordedCounters {  // of one device; never destroyed: graphs may outlive every static object
-  std::vector<int> free_list;
-  int used = 0;
-};
-struct RecordedCounter { int dev, index; };
-
 std::mutex g_counter_mutex;
-unsigned* g_counter_ptr[kMaxDevices] = {};
-std::unordered_map<unsigned long long, int>& g_stream_counter = *new std::unordered_map<unsigned long long, int>;  // by stream id
-RecordedCounters* const g_recorded = new RecordedCounters[kMaxDevices];
+struct DeviceCounters {
+  unsigned* base = nullptr;
+  std::unordered_map<const void*, int> of_array;
+};
+DeviceCounters* const g_counters = new DeviceCounters[kMaxDevices];  // never destroyed: launches may come at any time
 
-void give_back_counter(void* p) {  // by the driver, when nothing that holds the recorded launch is left
-  RecordedCounter* r = static_cast<RecordedCounter*>(p);
-  {
-    std::lock_guard<std::mutex> lock(g_counter_mutex);
-    g_recorded[r->dev].free_list.push_back(r->index);
-  }
-  delete r;
-}
-
-unsigned* item_counter(cudaStream_t st) {
+unsigned* item_counter(const void* out, cudaStream_t st) {
   int dev = -1;
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  unsigned long long id = 0;
-  cudaGraph_t graph = nullptr;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices ||
-      cudaStreamGetCaptureInfo(st, &capture, &id, &graph) != cudaSuccess ||
-      (capture == cudaStreamCaptureStatusNone && cudaStreamGetId(st, &id) != cudaSuccess)) {
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
     cudaGetLastError();
     return nullptr;
   }
-  RecordedCounter* recorded = nullptr;
-  unsigned* counter = nullptr;
-  {
-    std::lock_guard<std::mutex> lock(g_counter_mutex);
-    if (g_counter_ptr[dev] == nullptr) {
-      void* p = nullptr;
-      if (capture != cudaStreamCaptureStatusNone || cudaGetSymbolAddress(&p, g_item_counters) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-      }
-      g_counter_ptr[dev] = static_cast<unsigned*>(p);
-    }
-    if (capture == cudaStreamCaptureStatusNone) {
-      auto it = g_stream_counter.find(id);
-      if (it != g_stream_counter.end()) return g_counter_ptr[dev] + it->second;
-      const int n = (int)g_stream_counter.size();
-      if (n >= kStreamCounters) return nullptr;
-      g_stream_counter.emplace(id, n);
-      return g_counter_ptr[dev] + n;
-    }
-    RecordedCounters& pool = g_recorded[dev];
-    int index = -1;
-    if (!pool.free_list.empty()) {
-      index = pool.free_list.back();
-      pool.free_list.pop_back();
-    } else if (pool.used < kRecordedCounters) {
-      index = pool.used++;
-    } else {
+  std::lock_guard<std::mutex> lock(g_counter_mutex);
+  DeviceCounters& c = g_counters[dev];
+  if (c.base == nullptr) {  // looked up once, not while a stream is being recorded
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    void* p = nullptr;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+        cudaGetSymbolAddress(&p, g_item_counters) != cudaSuccess) {
+      cudaGetLastError();
       return nullptr;
     }
-    recorded = new RecordedCounter{dev, index};
-    counter = g_counter_ptr[dev] + kStreamCounters + index;
+    c.base = static_cast<unsigned*>(p);
   }
-  // outside the lock: dropping the object calls give_back_counter
-  cudaUserObject_t obj = nullptr;
-  if (cudaUserObjectCreate(&obj, recorded, give_back_counter, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
-    cudaGetLastError();
-    give_back_counter(recorded);
-    return nullptr;
-  }
-  if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
-    cudaGetLastError();
-    cudaUserObjectRelease(obj, 1);
-    return nullptr;
-  }
-  return counter;
+  const auto it = c.of_array.find(out);
+  if (it != c.of_array.end()) return c.base + it->second;
+  const int n = (int)c.of_array.size();
+  if (n >= kCounters) return nullptr;
+  c.of_array.emplace(out, n);
+  return c.base + n;
 }
 }  // namespace
 

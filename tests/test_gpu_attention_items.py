@@ -1,5 +1,5 @@
-"""Attention forward: how its CTAs come by their work - one item each, drawn in order or as they stand, from a stream's
-counter or from a recorded launch's own, with offsets in registers, in shared memory or in global memory."""
+"""Attention forward: how its CTAs come by their work - one item each, drawn in order or as they stand, in launches and in
+recorded ones - with offsets in registers, in shared memory or in global memory."""
 import pytest
 import torch
 
@@ -51,7 +51,7 @@ def test_attention_forward_items(d, H, lengths):
     ao.fill_(7), lse.fill_(7)
     run()
     first = check()
-    run()                                         # the stream's counter is back at zero
+    run()                                         # the counter is back at zero
     assert torch.equal(check(), first)
     graphs = [torch.cuda.CUDAGraph() for _ in range(2)]
     for gr in graphs:
