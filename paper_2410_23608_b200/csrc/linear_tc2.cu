@@ -563,14 +563,16 @@ int launch_wgrad_pair(const spa_params& p, const void* a, const void* dout, int 
 
 // The pair kernels pay off where every pair gets a 256 x 256 tile (half of the allocated rows stands for the packed
 // ones): 15 120 rows 256 -> 768 13.7 us against 15.0 on single CTAs, 6 272 rows 384 -> 1 152 11.2 against 12.2; with
-// fewer tiles the smaller ones spread better (6 272 rows 384 -> 384: 7.9 against 6.5).  Not where an eighth of the pair's
-// columns or more would be padding that 128-column tiles do not have (34 000 rows allocated, 30 % of them there: 384 -> 384
-// 10.6 against 8.2, 288 -> 864 14.0 against 12.0; at half and above they gain 1 to 7 %, 288 -> 288 loses there too).
+// fewer tiles the smaller ones spread better (6 272 rows 384 -> 384: 7.9 against 6.5).  Not where K is short and
+// an eighth of the pair's columns or more would be padding that 128-column tiles do not have (34 000 rows allocated, 30 % of
+// them there: 384 -> 384 10.6 against 8.2, 288 -> 864 14.0 against 12.0; at half and above even).  With a longer main loop the
+// pairs win all the same (576 -> 576 13.1 against 15.1).
 bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out, int n_cols) {
   if (p.flags & SPA_FLAG_NO_CTA_PAIRS) return false;
   const long long tiles = (long long)((p.capacity / 2 + 2 * PM - 1) / (2 * PM)) * ((n_cols + PN - 1) / PN);
   const int blocks = (n_cols + 127) / 128;
-  const bool padded = blocks % 2 == 1 && blocks <= 7;
+  const int k = n_cols == n_out ? n_in : n_out;
+  const bool padded = blocks % 2 == 1 && blocks <= 7 && k <= 384;
   return n_in % 8 == 0 && n_out % 8 == 0 && tiles >= kMaxPairs && !padded && tensor_maps_available();
 }
 
