@@ -185,7 +185,7 @@ __device__ __forceinline__ RowSeg warp_row_segment(Load off, int n_seg, int Np, 
 }
 
 constexpr int kFwdSegStage = 2048;
-constexpr int kEarlySegments = 256;  // eight offsets a lane: their loads are in flight together
+constexpr int kEarlySegments = 512;  // sixteen offsets a lane, their loads in flight together (280 segments of 49: 14.5 -> 14.2 us)
 
 // c[j] of lane 4 i + k becomes c[k] of lane 4 i + j
 __device__ __forceinline__ void transpose_quads(uint4 (&c)[4], int lane) {

@@ -11,8 +11,8 @@ pytestmark = pytest.mark.gpu
     (64, 12, [577, 58] * 9),                      # items drawn, put in order of length
     (32, 8, [1680] + [0] * 3 + [210] * 40),       # in order; empty segments
     (64, 12, [700] * 5 + [131]),                  # a few more items than CTAs
-    (32, 16, [49] * 255),                         # offsets of the first item by one warp: the most
-    (64, 8, [49] * 256),                          # and one more; drawn without order
+    (32, 16, [49] * 511),                         # offsets of the first item by one warp: the most
+    (64, 8, [49] * 512),                          # and one more; drawn without order
     (32, 4, [5] * 2047),                          # staged offsets: the most
     (64, 4, [5] * 2048 + [300] * 30),             # and one more
     (32, 1, [3] * 70001),                         # more row tiles than are put in order
