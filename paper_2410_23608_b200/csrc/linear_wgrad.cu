@@ -39,8 +39,10 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
   const uint32_t done_bar = bar_base + 8u * 2 * kStages;
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kBars + 96);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kBars + 100);
+  constexpr int kSlot = 112;  // TMEM address, abort flag
+  static_assert(8 * (2 * kStages + 1) <= kSlot, "the barriers end in front of the words behind them");
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kBars + kSlot);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kBars + kSlot + 4);
   float* tile = reinterpret_cast<float*>(smem_al);
   float* sums = reinterpret_cast<float*>(smem_al + kBars + 128);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
