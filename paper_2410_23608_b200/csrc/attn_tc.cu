@@ -441,7 +441,8 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __rest
     auto next_q = [&](int last) {
       if (cs.n_tiles > 0 && cs.t == 0) {
         wait(bar_s, last & 1);
-        load_q(cs);
+        // after a wait that gave up the Q tile before may still be on its way
+        if (!__any_sync(0xffffffffu, ptx::lds_s32(abort_any) != 0)) load_q(cs);
       }
     };
     if (cp.n_tiles > 0) {

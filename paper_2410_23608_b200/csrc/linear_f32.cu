@@ -193,6 +193,8 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
       ok = __all_sync(0xffffffffu, ok) != 0;
       if (!ok) {
         if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
+        if (ptx::elect_one()) ptx::mma_commit(done_bar);  // the products issued so far
+        __syncwarp();
         break;
       }
       ptx::tc_fence_after_sync();
@@ -212,13 +214,13 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
       __syncwarp();
     }
   }
-  // every product has completed: the finished tile takes the stages' memory
+  // every product that was issued has completed: the finished tile takes the stages' memory
   float* tile = reinterpret_cast<float*>(smem_al);
   constexpr int kLd = kLdT<BN>;
   static_assert((BM * kLd + BM) * 4 <= kStages * kStageBytes<BN> && 32 * 128 * 4 <= kStageBytes<BN>, "fits the stages");
   float* tile_sum = tile + BM * kLd;  // column sums, one per row of the tile
   __syncwarp();
-  if (mine > 0 && !*abort_flag && !__all_sync(0xffffffffu, ptx::mbar_wait(done_bar, 0))) {
+  if (mine > 0 && !__all_sync(0xffffffffu, ptx::mbar_wait(done_bar, 0))) {
     if (lane == 0) { record_status(d_status, SPA_ERR_TIMEOUT); *abort_flag = 1; }
   }
   __syncthreads();

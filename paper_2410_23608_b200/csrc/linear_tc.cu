@@ -97,7 +97,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                const __nv_bfloat16* __restrict__ bias, OutT* __restrict__ out, long long ldo,
                long long split_stride, int M, int N, int K, const int32_t* __restrict__ cu, int n_seg, int capacity,
                int dyn_which, int k_per_split, int k_interleave, const int32_t* __restrict__ row_map,
-               RowEpilogue<kKind> epi, int32_t* d_status) {
+               RowEpilogue<kKind> epi, uint32_t wait_limit, int32_t* d_status) {
   constexpr int kStage = stage_bytes<BN>();
   pdl_launch_dependents();
 
@@ -109,8 +109,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
   auto tmem_full_bar = [&](int a) { return bar_base + 8u * (2 * kStages + a); };
   auto tmem_empty_bar = [&](int a) { return bar_base + 8u * (2 * kStages + 2 + a); };
+  const uint32_t drain_bar = bar_base + 8u * (2 * kStages + 4);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kStages * kStage + 96);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kStages * kStage + 100);
+  const uint32_t abort_s = bar_base + 100;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -121,6 +123,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       ptx::mbar_init(empty_bar(s), 1);
     }
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(tmem_full_bar(a), 1); ptx::mbar_init(tmem_empty_bar(a), 4); }
+    ptx::mbar_init(drain_bar, 1);
     *abort_flag = 0;
     ptx::fence_mbar_init();
   }
@@ -167,20 +170,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   };
 
-  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort(bar, parity, abort_s, d_status, SPA_ERR_TIMEOUT, wait_limit); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort_warp(bar, parity, abort_s, d_status, SPA_ERR_TIMEOUT, wait_limit); };
 
+  int issued = 0;       // the producer's: k-blocks whose copies have been issued
+  bool failed = false;  // a wait of this thread gave up, or it saw that another one's had
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       int it = 0;  // k-block counter over all tiles of this CTA: ring position and phase
-      for (int tile = blockIdx.x; tile < total && !*abort_flag; tile += gridDim.x) {
+      bool live = true;
+      for (int tile = blockIdx.x; tile < total && live && !*abort_flag; tile += gridDim.x) {
         const TileCoord c = coord(tile);
         int k_begin, k_end, k_step;
         k_range(c.z, k_begin, k_end, k_step);
         for (int k0 = k_begin; k0 < k_end; k0 += k_step, ++it) {
           const int s = it % kStages;
-          if (it >= kStages) wait_lane(empty_bar(s), ((it / kStages) - 1) & 1);
+          if (it >= kStages && !wait_lane(empty_bar(s), ((it / kStages) - 1) & 1)) { live = false; break; }
           const uint32_t a_dst = smem_base + s * kStage, b_dst = a_dst + kABytes;
           ptx::mbar_expect_tx(full_bar(s), kABytes + bn * BK * 2);
           if (!kAMn) {
@@ -202,26 +208,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
       }
-      if (*abort_flag) {  // let our own copies land before the CTA's shared memory goes away
-        for (int j = it > kStages ? it - kStages : 0; j < it; ++j)
-          ptx::mbar_wait(full_bar(j % kStages), (j / kStages) & 1);
-      }
+      issued = it;
+      failed = !live;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     int it = 0, tl = 0;  // k-block counter, tile counter of this CTA
+    bool live = true;    // every wait of this lane has been satisfied
     for (int tile = blockIdx.x; tile < total && !__any_sync(0xffffffffu, *abort_flag != 0); tile += gridDim.x, ++tl) {
       const TileCoord c = coord(tile);
       int k_begin, k_end, k_step;
       k_range(c.z, k_begin, k_end, k_step);
       const int acc = tl & 1;
-      if (tl >= 2) wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1);
+      if (tl >= 2) live = wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1) && live;
       ptx::tc_fence_after_sync();
       const uint32_t tmem_d = tmem_base + acc * BN;
       bool first = true;
       for (int k0 = k_begin; k0 < k_end; k0 += k_step, ++it) {
         const int s = it % kStages;
-        wait(full_bar(s), (it / kStages) & 1);
+        live = wait(full_bar(s), (it / kStages) & 1) && live;
         const uint32_t a_src = smem_base + s * kStage, b_src = a_src + kABytes;
         const int k_valid = k_end - k0;
         if ((kAMn || kBMn) && k_valid < BK) {
@@ -250,13 +255,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                         : ptx::smem_desc_sw128(b_src + k * 32, 16, 1024);
             ptx::mma_bf16(tmem_d, adesc, bdesc, idesc, (first && k == 0) ? 0u : 1u);
           }
-          ptx::mma_commit(empty_bar(s));
+          if (live) ptx::mma_commit(empty_bar(s));
         }
         first = false;
         __syncwarp();
       }
       if (!first && ptx::elect_one()) ptx::mma_commit(tmem_full_bar(acc));  // the same lane as above: it covers its products
     }
+    failed = !live;
   } else {
     // ------------------------------------------------------------------ epilogue warps
     const int q = warp & 3;          // TMEM lane quarter this warp may read
@@ -282,7 +288,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // the bias of the tile comes to L1 under the main loop: fetched where it is added, each 32 columns waited for L2
       if (bias != nullptr && lane < bn / 64 && c.n0 + lane * 64 < N) prefetch_l1(bias + c.n0 + lane * 64);
       wait(tmem_full_bar(acc), (tl >> 1) & 1);
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) { failed = true; break; }
       ptx::tc_fence_after_sync();
 #pragma unroll 1
       for (int cc = 0; cc < bn / 32; ++cc) {
@@ -339,7 +345,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   }
   ptx::tc_fence_before_sync();
-  __syncthreads();
+  if (__builtin_expect(__syncthreads_or(failed ? 1 : 0), 0)) ptx::drain_cta(issued, kStages, full_bar(0), drain_bar);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem_base, 2 * BN);
@@ -482,7 +488,7 @@ template <int BN, bool kDyn, bool kAMn, bool kBMn, typename OutT, int kKind>
 int launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, OutT* out, long long ldo,
                 long long split_stride, int M, int N, int K, const int32_t* cu, int n_seg, int capacity, int dyn_which,
                 int k_per_split, int splits, int k_interleave, const int32_t* row_map, RowEpilogue<kKind> epi,
-                int32_t* d_status, cudaStream_t st, const char* what) {
+                uint32_t wait_limit, int32_t* d_status, cudaStream_t st, const char* what) {
   auto kern = gemm_tc_kernel<BN, kDyn, kAMn, kBMn, OutT, kKind>;
   static DeviceOnce attr;  // per instantiation and device
   cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes<BN>()); });
@@ -492,7 +498,7 @@ int launch_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloa
   long long tiles = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM) * splits * (kDyn ? 2 : 1);
   const int grid = (int)(tiles < 2 * kNumSMs ? (tiles < 1 ? 1 : tiles) : 2 * kNumSMs);
   launch_pdl(kern, grid, kGemmThreads, gemm_smem_bytes<BN>(), st, tmA, tmB, bias, out, ldo, split_stride, M, N, K, cu,
-             n_seg, capacity, dyn_which, k_per_split, k_interleave, row_map, epi, d_status);
+             n_seg, capacity, dyn_which, k_per_split, k_interleave, row_map, epi, wait_limit, d_status);
   SPA_CUDA_CHECK_LAUNCH(what);
   return SPA_OK;
 }
@@ -514,7 +520,8 @@ int launch_width(TileWidth width, const CUtensorMap& tmA, const CUtensorMap& tmB
   auto run = width == kNarrow   ? launch_gemm<64, false, false, kBMn, __nv_bfloat16, kKind>
              : width == kByRows ? launch_gemm<128, true, false, kBMn, __nv_bfloat16, kKind>
                                 : launch_gemm<128, false, false, kBMn, __nv_bfloat16, kKind>;
-  return run(tmA, tmB, bias, out, n_cols, 0, p.capacity, n_cols, k, cu, p.B, p.capacity, 1, k, 1, 0, row_map, epi, d_status, st, what);
+  return run(tmA, tmB, bias, out, n_cols, 0, p.capacity, n_cols, k, cu, p.B, p.capacity, 1, k, 1, 0, row_map, epi,
+             ptx::wait_limit(p.flags), d_status, st, what);
 }
 
 }  // namespace
@@ -595,7 +602,8 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
     int rc = pair ? launch_wgrad_pair(p, a, dout, n_in, n_out, cu, part_w, db != nullptr ? part_b : nullptr, pl, d_status, st)
                   : launch_gemm<128, false, true, true, float>(tmA2, tmB2, nullptr, part_w, n_in, n_w, n_out, n_in, p.capacity,
                                                         cu, p.B, p.capacity, 2, sp.k_per_split, sp.splits, sp.splits,
-                                                        nullptr, RowEpilogue<kEpiOwn>{nullptr}, d_status, st, "gemm_tc_kernel(wgrad)");
+                                                        nullptr, RowEpilogue<kEpiOwn>{nullptr}, ptx::wait_limit(p.flags), d_status, st,
+                                                        "gemm_tc_kernel(wgrad)");
     if (rc != SPA_OK) return rc;
     const long long n_b = db != nullptr ? n_out : 0;
     int grid = (int)((n_w / 4 + 255) / 256);

@@ -16,8 +16,8 @@
 //   empty[s]       both CTAs, 1 arrival: commit of the MMAs that read stage s (multicast to the pair)
 //   tmem_full[a]   both CTAs, 1 arrival: commit after the last k-block of a tile (multicast)
 //   tmem_empty[a]  leader only, 16 arrivals: the eight epilogue warps of each CTA
-// Every wait is bounded; the two cluster-wide barriers (after set-up, before exit) are reached by every
-// thread on every path, so a CTA never leaves while its peer may still touch its shared memory.
+// Every wait is bounded; the cluster-wide barriers (after set-up, before exit, and a third where a wait has run out)
+// are reached by every thread on every path, so a CTA never leaves while its peer may still touch its shared memory.
 #include "sm100_ptx.cuh"
 #include "spa_tc.cuh"
 
@@ -44,6 +44,14 @@ __device__ __forceinline__ void cluster_sync() {
 __device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t cluster_bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_bar), "r"(bytes)
                : "memory");
+}
+__device__ __forceinline__ int ld_peer_s32(uint32_t cluster_addr) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_peer_s32(uint32_t cluster_addr, int v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
@@ -91,6 +99,45 @@ constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;  // warp 0: TMA, warp 1: M
 constexpr int kPairStage = PM * PK * 2 + (PN / 2) * PK * 2;  // 32 KB
 constexpr int kPairSmem = kPairStages * kPairStage + 1024 + 256 + kPairEpiWarps * 4096;  // ring, alignment slack, barriers, transposition
 
+// Where a wait has run out in either CTA of a pair, by all threads of both: the copies and products in flight complete
+// (each wait with a limit) before the CTAs' memory goes away.  `issued` k-blocks of a CTA have been reported to the leader's
+// full barriers, stage by stage, each phase of which takes one report of either CTA and the bytes of both.  A stage is
+// refilled only behind the products that read it, so the two counts differ by the number of stages at most: the CTA that
+// is behind reports the rest without bytes, and then the last phase of every stage completes when its copies have landed.
+//   issued_s: a word in shared memory; full0: the first full barrier; drain: a barrier of one arrival that nothing else
+//   uses; tail_bar (or 0): a barrier of this CTA with copies in flight, and the parity of its phase
+// Not inlined: inside the kernels this code cost every launch 0.1 us.
+__device__ __noinline__ void drain_pair(uint32_t rank, uint32_t issued_s, uint32_t full0, uint32_t drain,
+                                        uint32_t tail_bar, uint32_t tail_parity) {
+  if (threadIdx.x == 0) {
+    const int mine = ptx::lds_s32(issued_s), peers = ptx2::ld_peer_s32(ptx2::map_to_cta(issued_s, rank ^ 1));
+    const int all = mine > peers ? mine : peers;
+    for (int it = mine; it < all; ++it) ptx2::mbar_arrive_cluster(ptx2::map_to_cta(full0 + 8u * (it % kPairStages), 0));
+    if (tail_bar != 0) ptx::mbar_wait(tail_bar, tail_parity);
+    if (rank == 0)
+      for (int it = all > kPairStages ? all - kPairStages : 0; it < all; ++it)
+        ptx::mbar_wait(full0 + 8u * (it % kPairStages), (it / kPairStages) & 1);
+  }
+  __syncwarp();
+  if (threadIdx.x / 32 == 1) {  // the warp that issues the leader's products: they complete in both CTAs
+    if (rank == 0 && ptx::elect_one()) ptx2::mma_commit_pair(drain);
+    __syncwarp();
+    ptx::mbar_wait(drain, 0);
+  }
+  __syncthreads();
+  ptx2::cluster_sync();
+}
+
+// The end of a pair kernel: nobody leaves while the peer may still read this CTA's operands or signal its barriers; a
+// failure of one CTA (its abort flag) becomes the peer's too.
+__device__ __forceinline__ void leave_pair(uint32_t rank, uint32_t abort_s, uint32_t issued_s, uint32_t full0, uint32_t drain,
+                                           uint32_t tail_bar = 0, uint32_t tail_parity = 0) {
+  if ((threadIdx.x & 31) == 0 && ptx::lds_s32(abort_s) != 0) ptx2::st_peer_s32(ptx2::map_to_cta(abort_s, rank ^ 1), 1);
+  ptx::tc_fence_before_sync();
+  ptx2::cluster_sync();  // every thread of both CTAs
+  if (__builtin_expect(ptx::lds_s32(abort_s) != 0, 0)) drain_pair(rank, issued_s, full0, drain, tail_bar, tail_parity);
+}
+
 // kBMn: B = W is MN-major (input gradient: K = n_out rows of W, N = n_in contiguous); otherwise K-major
 // (forward: N = n_out rows of W, K = n_in contiguous).  A is always K-major, the output bf16.
 // M is the device-side packed row count.  row_map and epi as in the single-CTA kernel.
@@ -99,7 +146,7 @@ __global__ void __launch_bounds__(kPairThreads)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __nv_bfloat16* __restrict__ bias, __nv_bfloat16* __restrict__ out, long long ldo, int N, int K,
                  const int32_t* __restrict__ cu, int n_seg, int capacity, const int32_t* __restrict__ row_map,
-                 RowEpilogue<kKind> epi, int32_t* d_status) {
+                 RowEpilogue<kKind> epi, uint32_t wait_limit, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(2 * PM, PN, false, kBMn);
   pdl_launch_dependents();
 
@@ -111,8 +158,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   auto empty_bar = [&](int s) { return bar_base + 8u * (kPairStages + s); };
   auto tmem_full_bar = [&](int a) { return bar_base + 8u * (2 * kPairStages + a); };
   auto tmem_empty_bar = [&](int a) { return bar_base + 8u * (2 * kPairStages + 2 + a); };
+  const uint32_t drain_bar = bar_base + 8u * (2 * kPairStages + 4);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kPairStages * kPairStage + 192);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kPairStages * kPairStage + 196);
+  const uint32_t abort_s = bar_base + 196, issued_s = bar_base + 200;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx2::cluster_ctarank();   // 0 = leader
@@ -125,6 +174,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       ptx::mbar_init(empty_bar(s), 1);
     }
     for (int a = 0; a < 2; ++a) { ptx::mbar_init(tmem_full_bar(a), 1); ptx::mbar_init(tmem_empty_bar(a), 2 * kPairEpiWarps); }
+    ptx::mbar_init(drain_bar, 1);
     *abort_flag = 0;
     ptx::fence_mbar_init();
   }
@@ -141,19 +191,20 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int tiles_m = (M + 2 * PM - 1) / (2 * PM);
   const int total = tiles_m * tiles_n;
   const int k_blocks = (K + PK - 1) / PK;
-  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort(bar, parity, abort_s, d_status, SPA_ERR_TIMEOUT, wait_limit); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort_warp(bar, parity, abort_s, d_status, SPA_ERR_TIMEOUT, wait_limit); };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one per CTA)
     if (lane == 0) {
       int it = 0;
-      for (int tile = pair; tile < total && !*abort_flag; tile += n_pairs) {
+      bool live = true;
+      for (int tile = pair; tile < total && live && !*abort_flag; tile += n_pairs) {
         const int m0 = (tile / tiles_n) * 2 * PM + (int)rank * PM;
         const int n0 = (tile % tiles_n) * PN + (int)rank * (PN / 2);
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kPairStages;
-          if (it >= kPairStages) wait_lane(empty_bar(s), ((it / kPairStages) - 1) & 1);
+          if (it >= kPairStages && !wait_lane(empty_bar(s), ((it / kPairStages) - 1) & 1)) { live = false; break; }
           const uint32_t a_dst = smem_base + s * kPairStage, b_dst = a_dst + PM * PK * 2;
           const uint32_t lead_full = ptx2::map_to_cta(full_bar(s), 0);
           ptx2::mbar_expect_tx_cluster(lead_full, kPairStage);
@@ -168,19 +219,21 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
         }
       }
+      ptx::sts_s32(issued_s, it);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: the leader's, for the pair
     if (rank == 0) {
       int it = 0, tl = 0;
+      bool live = true;  // every wait of this lane has been satisfied
       for (int tile = pair; tile < total && !__any_sync(0xffffffffu, *abort_flag != 0); tile += n_pairs, ++tl) {
         const int acc = tl & 1;
-        if (tl >= 2) wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1);
+        if (tl >= 2) live = wait(tmem_empty_bar(acc), ((tl >> 1) - 1) & 1) && live;
         ptx::tc_fence_after_sync();
         const uint32_t tmem_d = tmem_base + acc * PN;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % kPairStages;
-          wait(full_bar(s), (it / kPairStages) & 1);
+          live = wait(full_bar(s), (it / kPairStages) & 1) && live;
           ptx::tc_fence_after_sync();
           const uint32_t a_src = smem_base + s * kPairStage, b_src = a_src + PM * PK * 2;
           if (ptx::elect_one()) {
@@ -191,7 +244,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                           : ptx::smem_desc_sw128(b_src + k * 32, 16, 1024);
               ptx2::mma_bf16_pair(tmem_d, adesc, bdesc, kIdesc, (kb == 0 && k == 0) ? 0u : 1u);
             }
-            ptx2::mma_commit_pair(empty_bar(s));
+            if (live) ptx2::mma_commit_pair(empty_bar(s));
             if (kb == k_blocks - 1) ptx2::mma_commit_pair(tmem_full_bar(acc));
           }
           __syncwarp();
@@ -264,10 +317,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (lane == 0) ptx2::mbar_arrive_cluster(lead_empty[acc]);  // this warp has drained its quarter of the accumulator
     }
   }
-  // nobody leaves while the peer may still read this CTA's operands or signal its barriers
-  ptx::tc_fence_before_sync();
-  __syncthreads();
-  ptx2::cluster_sync();
+  leave_pair(rank, abort_s, issued_s, full_bar(0), drain_bar);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx2::tmem_dealloc_pair(tmem_base, 2 * PN);
@@ -291,7 +341,7 @@ constexpr int kWgSmem = kPairSmem + 1024;  // and the 8 x 64 block of ones
 __global__ void __launch_bounds__(kPairThreads)
 wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ part,
                   float* __restrict__ part_b, int M, int N, int splits, const int32_t* __restrict__ cu, int n_seg,
-                  int capacity, int32_t* d_status) {
+                  int capacity, uint32_t wait_limit, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(2 * PM, PN, true, true);
   constexpr uint32_t kIdescOnes = ptx::idesc_bf16_f32(2 * PM, 16, true, false);
   constexpr int kBars = kPairStages * kPairStage;
@@ -304,8 +354,10 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (kPairStages + s); };
   const uint32_t tmem_full_bar = bar_base + 8u * (2 * kPairStages), tmem_empty_bar = tmem_full_bar + 8, tail_bar = tmem_full_bar + 16;
+  const uint32_t drain_bar = tmem_full_bar + 24;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kBars + 1024 + 192);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kBars + 1024 + 196);
+  const uint32_t abort_s = bar_base + 196, issued_s = bar_base + 200;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx2::cluster_ctarank();  // 0 = leader
@@ -320,6 +372,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     ptx::mbar_init(tmem_full_bar, 1);
     ptx::mbar_init(tmem_empty_bar, 2 * kPairEpiWarps);
     ptx::mbar_init(tail_bar, 1);
+    ptx::mbar_init(drain_bar, 1);
     *abort_flag = 0;
     ptx::fence_mbar_init();
   }
@@ -351,13 +404,16 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     c.n0 = c.n_t * PN;
     return c;
   };
-  auto wait_lane = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort_warp(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait_lane = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort(bar, parity, abort_s, d_status, SPA_ERR_TIMEOUT, wait_limit); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort_warp(bar, parity, abort_s, d_status, SPA_ERR_TIMEOUT, wait_limit); };
 
+  bool tail_open = false;  // copies on tail_bar that were given up on
+  uint32_t tail_parity = 0;
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one per CTA)
     int it = 0, tails = 0;
-    for (int i = pair; i < total && !__any_sync(0xffffffffu, *abort_flag != 0); i += n_pairs) {
+    bool live = true;  // lane 0: every wait has been satisfied; all lanes: so has every wait for a tail
+    for (int i = pair; i < total && !__any_sync(0xffffffffu, !live || *abort_flag != 0); i += n_pairs) {
       const Item c = item_of(i);
       const int m0 = c.m0 + (int)rank * PM, n0 = c.n0 + (int)rank * (PN / 2);
       for (int kb = c.z; kb < k_blocks; kb += n_splits, ++it) {
@@ -366,8 +422,9 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint32_t lead_full = ptx2::map_to_cta(full_bar(s), 0);
         const bool tail = k0 + PK > K;
         if (lane == 0) {
-          if (it >= kPairStages) wait_lane(empty_bar(s), ((it / kPairStages) - 1) & 1);
-          if (!tail) {
+          live = (it < kPairStages || wait_lane(empty_bar(s), ((it / kPairStages) - 1) & 1)) && live;
+          if (!live) {
+          } else if (!tail) {
             ptx2::mbar_expect_tx_cluster(lead_full, kPairStage);
 #pragma unroll
             for (int j = 0; j < 2; ++j) ptx2::tma_load_2d_pair(a_dst + j * (PK * 128), &tmA, lead_full, m0 + 64 * j, k0);
@@ -381,9 +438,10 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             for (int j = 0; j < 2; ++j) ptx::tma_load_2d(b_dst + j * (PK * 128), &tmB, tail_bar, n0 + 64 * j, k0);
           }
         }
-        __syncwarp();
+        if (!__shfl_sync(0xffffffffu, live, 0)) { live = false; break; }
         if (tail) {
-          wait(tail_bar, tails & 1);
+          live = __all_sync(0xffffffffu, wait(tail_bar, tails & 1)) != 0;
+          if (!live) { tail_open = true; break; }
           ++tails;
           const int first = K - k0;  // lines of the four boxes from here on hold no packed row
           for (int q = lane; q < 4 * (PK - first) * 8; q += 32) {
@@ -396,19 +454,22 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
       }
     }
+    if (lane == 0) ptx::sts_s32(issued_s, it);
+    tail_parity = tails & 1;
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: the leader's, for the pair
     if (rank == 0) {
       const uint64_t ones_desc = ptx::smem_desc_sw128(ones_s, 16, 1024);
       int it = 0, tl = 0;
+      bool live = true;  // every wait of this lane has been satisfied
       for (int i = pair; i < total && !__any_sync(0xffffffffu, *abort_flag != 0); i += n_pairs, ++tl) {
         const Item c = item_of(i);
-        if (tl > 0) wait(tmem_empty_bar, (tl - 1) & 1);
+        if (tl > 0) live = wait(tmem_empty_bar, (tl - 1) & 1) && live;
         ptx::tc_fence_after_sync();
         bool first = true, first_sum = true;
         for (int kb = c.z; kb < k_blocks; kb += n_splits, ++it) {
           const int s = it % kPairStages;
-          wait(full_bar(s), (it / kPairStages) & 1);
+          live = wait(full_bar(s), (it / kPairStages) & 1) && live;
           ptx::tc_fence_after_sync();
           const uint32_t a_src = smem_base + s * kPairStage, b_src = a_src + PM * PK * 2;
           const bool sum = part_b != nullptr && (kb / n_splits) % tiles_n == c.n_t;
@@ -423,7 +484,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 ptx2::mma_bf16_pair(tmem + PN, ptx::smem_desc_sw128(a_src + k * 2048, PK * 128, 1024), ones_desc, kIdescOnes,
                                     (first_sum && k == 0) ? 0u : 1u);
             }
-            ptx2::mma_commit_pair(empty_bar(s));
+            if (live) ptx2::mma_commit_pair(empty_bar(s));
             if (kb + n_splits >= k_blocks) ptx2::mma_commit_pair(tmem_full_bar);
           }
           first = false;
@@ -482,10 +543,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       if (lane == 0) ptx2::mbar_arrive_cluster(lead_empty);  // this warp has drained its quarter of the accumulator
     }
   }
-  // nobody leaves while the peer may still read this CTA's operands or signal its barriers
-  ptx::tc_fence_before_sync();
-  __syncthreads();
-  ptx2::cluster_sync();
+  leave_pair(rank, abort_s, issued_s, full_bar(0), drain_bar, tail_open ? tail_bar : 0u, tail_parity);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx2::tmem_dealloc_pair(tmem, 2 * PN);
@@ -520,14 +578,14 @@ int launch_clusters(void (*kern)(KArgs...), int pairs, int smem, cudaStream_t st
 template <bool kBMn, int kKind>
 int launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, const __nv_bfloat16* bias, __nv_bfloat16* out, long long ldo,
                 int N, int K, const int32_t* cu, int n_seg, int capacity, const int32_t* row_map, RowEpilogue<kKind> epi,
-                int32_t* d_status, cudaStream_t st, const char* what) {
+                uint32_t wait_limit, int32_t* d_status, cudaStream_t st, const char* what) {
   auto kern = gemm_pair_kernel<kBMn, kKind>;
   static DeviceOnce smem_attr;  // per instantiation and device
   cudaError_t ea = smem_attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem); });
   if (ea != cudaSuccess) { set_cuda_error(ea, what); return SPA_ERR_CUDA; }
   const long long tiles = (long long)((N + PN - 1) / PN) * ((capacity + 2 * PM - 1) / (2 * PM));
   const int pairs = (int)(tiles < kMaxPairs ? (tiles < 1 ? 1 : tiles) : kMaxPairs);
-  return launch_clusters(kern, pairs, kPairSmem, st, what, tmA, tmB, bias, out, ldo, N, K, cu, n_seg, capacity, row_map, epi, d_status);
+  return launch_clusters(kern, pairs, kPairSmem, st, what, tmA, tmB, bias, out, ldo, N, K, cu, n_seg, capacity, row_map, epi, wait_limit, d_status);
 }
 
 }  // namespace
@@ -558,7 +616,7 @@ int launch_wgrad_pair(const spa_params& p, const void* a, const void* dout, int 
   if (ea != cudaSuccess) { set_cuda_error(ea, "wgrad_pair_kernel"); return SPA_ERR_CUDA; }
   const int tiles = pl.tiles * pl.splits;
   return launch_clusters(wgrad_pair_kernel, tiles < kMaxPairs ? tiles : kMaxPairs, kWgSmem, st, "wgrad_pair_kernel", tmA, tmB, part,
-                         part_b, n_out, n_in, pl.splits, cu, p.B, p.capacity, d_status);
+                         part_b, n_out, n_in, pl.splits, cu, p.B, p.capacity, ptx::wait_limit(p.flags), d_status);
 }
 
 // The pair kernels pay off where every pair gets a 256 x 256 tile (half of the allocated rows stands for the packed
@@ -585,7 +643,7 @@ int launch_linear_fwd_pair(const spa_params& p, const void* a, const void* W, co
     return SPA_ERR_UNSUPPORTED;
   auto go = [&](auto row_epi) {
     return launch_pair<false>(tmA, tmB, (const __nv_bfloat16*)bias, (__nv_bfloat16*)out, n_out, n_out, n_in, cu, p.B, p.capacity,
-                              row_map, row_epi, d_status, st, "gemm_pair_kernel(fwd)");
+                              row_map, row_epi, ptx::wait_limit(p.flags), d_status, st, "gemm_pair_kernel(fwd)");
   };
   if (epi.h != nullptr) return go(RowEpilogue<kEpiGelu>{(__nv_bfloat16*)epi.h});
   if (epi.add != nullptr && epi.add != out) return go(RowEpilogue<kEpiAdd>{(__nv_bfloat16*)const_cast<void*>(epi.add)});
@@ -602,7 +660,7 @@ int launch_linear_dgrad_pair(const spa_params& p, const void* W, const void* dou
     return SPA_ERR_UNSUPPORTED;
   auto go = [&](auto row_epi) {
     return launch_pair<true>(tmA, tmB, nullptr, (__nv_bfloat16*)da, n_in, n_in, n_out, cu, p.B, p.capacity, row_map, row_epi,
-                             d_status, st, "gemm_pair_kernel(dgrad)");
+                             ptx::wait_limit(p.flags), d_status, st, "gemm_pair_kernel(dgrad)");
   };
   return epi.u != nullptr ? go(RowEpilogue<kEpiGeluGrad>{(__nv_bfloat16*)const_cast<void*>(epi.u)})
                           : go(RowEpilogue<kEpiOwn>{epi.add != nullptr ? (__nv_bfloat16*)da : nullptr});

@@ -28,7 +28,7 @@ template <int kStages>
 __global__ void __launch_bounds__(kThreads, kStages == 3 ? 2 : 1)
 wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ dW,
                      float* __restrict__ db, int M, int N, const int32_t* __restrict__ cu, int n_seg, int capacity,
-                     int32_t* d_status) {
+                     uint32_t wait_limit, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(kT, kT, true, true);
   constexpr uint32_t kIdescOnes = ptx::idesc_bf16_f32(kT, 16, true, false);
   extern __shared__ uint8_t smem_raw[];
@@ -38,9 +38,9 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const uint32_t bar_base = smem_base + kBars;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
-  const uint32_t done_bar = bar_base + 8u * 2 * kStages;
+  const uint32_t done_bar = bar_base + 8u * 2 * kStages, drain_bar = done_bar + 8;
   constexpr int kSlot = 112;  // TMEM address, abort flag
-  static_assert(8 * (2 * kStages + 1) <= kSlot, "the barriers end in front of the words behind them");
+  static_assert(8 * (2 * kStages + 2) <= kSlot, "the barriers end in front of the words behind them");
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_al + kBars + kSlot);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_al + kBars + kSlot + 4);
   float* tile = reinterpret_cast<float*>(smem_al);
@@ -52,6 +52,7 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     ptx::prefetch_tensormap(&tmB);
     for (int s = 0; s < kStages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
     ptx::mbar_init(done_bar, 1);
+    ptx::mbar_init(drain_bar, 1);
     *abort_flag = 0;
     ptx::fence_mbar_init();
   }
@@ -72,13 +73,15 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const int k_blocks = (K + BK - 1) / BK;
   const int mine = z < k_blocks ? (k_blocks - z + split - 1) / split : 0;  // k-blocks z, z + split, ...
   const bool with_sums = db != nullptr && blockIdx.x == 0;
-  auto wait = [&](uint32_t bar, uint32_t parity) { ptx::mbar_wait_or_abort(bar, parity, ptx::smem_u32(const_cast<int*>(abort_flag)), d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { return ptx::mbar_wait_or_abort(bar, parity, bar_base + kSlot + 4, d_status, SPA_ERR_TIMEOUT, wait_limit); };
 
+  int issued = 0;  // the producer's: k-blocks whose copies have been issued
   if (warp == 0) {
     if (lane == 0) {
-      for (int i = 0; i < mine; ++i) {
+      int i = 0;
+      for (; i < mine; ++i) {
         const int s = i % kStages, k0 = (z + i * split) * BK;
-        if (i >= kStages) wait(empty_bar(s), ((i / kStages) - 1) & 1);
+        if (i >= kStages && !wait(empty_bar(s), ((i / kStages) - 1) & 1)) break;
         const uint32_t a_dst = smem_base + s * 2 * kOp, b_dst = a_dst + kOp;
         ptx::mbar_expect_tx(full_bar(s), 2 * kOp);
 #pragma unroll
@@ -86,16 +89,16 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 #pragma unroll
         for (int j = 0; j < 2; ++j) ptx::tma_load_2d(b_dst + j * (BK * 128), &tmB, full_bar(s), n0 + 64 * j, k0);
       }
-      if (*abort_flag)  // let our own copies land before the memory takes the finished tile
-        for (int i = mine > kStages ? mine - kStages : 0; i < mine; ++i) ptx::mbar_wait(full_bar(i % kStages), (i / kStages) & 1);
+      issued = i;
     }
     __syncwarp();
   } else if (warp == 1) {
     // both 8-row groups of the ones operand are the same eight lines: a stride of zero between them
     const uint64_t ones_desc = ptx::smem_desc_sw128(smem_base + kOnes, 16, 0);
+    bool live = true;  // every wait of this lane has been satisfied
     for (int i = 0; i < mine; ++i) {
       const int s = i % kStages;
-      wait(full_bar(s), (i / kStages) & 1);
+      live = wait(full_bar(s), (i / kStages) & 1) && live;
       __syncwarp();
       const int k_valid = K - (z + i * split) * BK;
       if (k_valid < BK) {  // lines of the four boxes past the last packed row
@@ -118,7 +121,7 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
           for (int k = 0; k < BK / 16; ++k)
             ptx::mma_bf16(tmem + kT, ptx::smem_desc_sw128(a_src + k * 2048, BK * 128, 1024), ones_desc, kIdescOnes, (i > 0 || k > 0) ? 1u : 0u);
         }
-        ptx::mma_commit(empty_bar(s));
+        if (live) ptx::mma_commit(empty_bar(s));
         if (i == mine - 1) ptx::mma_commit(done_bar);
       }
       __syncwarp();
@@ -157,7 +160,8 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   }
   __syncwarp();
   if (split > 1) cluster_sync_all(); else __syncthreads();
-  if (!*abort_flag) {
+  const bool failed = *abort_flag != 0;
+  if (!failed) {
     const int rows = M - m0 < kT ? M - m0 : kT, my_rows = rows > z ? (rows - z + split - 1) / split : 0;
     for (int e = tid; e < my_rows * (kT / 4); e += kThreads) {
       const int r = z + (e / (kT / 4)) * split, c = (e % (kT / 4)) * 4;
@@ -173,6 +177,7 @@ wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       }
   }
   if (split > 1) cluster_sync_all(); else __syncthreads();  // nobody leaves while a partial tile is still being read
+  if (__builtin_expect(failed, 0)) ptx::drain_cta(issued, kStages, full_bar(0), drain_bar);
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem, 2 * kT);
@@ -208,7 +213,7 @@ int launch_stages(dim3 grid, const CUtensorMap& tmA, const CUtensorMap& tmB, flo
   }
   cfg.attrs = attr;
   cfg.numAttrs = n;
-  e = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, dW, db, n_out, n_in, cu, p.B, p.capacity, d_status);
+  e = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, dW, db, n_out, n_in, cu, p.B, p.capacity, ptx::wait_limit(p.flags), d_status);
   if (e != cudaSuccess) { set_cuda_error(e, "wgrad_cluster_kernel"); return SPA_ERR_CUDA; }
   SPA_CUDA_CHECK_LAUNCH("wgrad_cluster_kernel");
   return SPA_OK;

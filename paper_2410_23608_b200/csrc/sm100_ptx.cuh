@@ -7,10 +7,13 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "spa.h"
+
 namespace spa {
 namespace ptx {
 
 constexpr uint32_t kWaitLimit = 1u << 22;  // polls of mbarrier.try_wait before giving up (~ a second)
+inline uint32_t wait_limit(int flags) { return (flags & SPA_FLAG_SHORT_WAITS) ? 0u : kWaitLimit; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -59,28 +62,32 @@ __device__ __forceinline__ void sts_s32(uint32_t addr, int v) {
   asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// Wait inside a pipeline loop: returns once the phase has completed.  After kWaitLimit polls, or when another thread of
-// the CTA has given up, it returns all the same with the abort flag (an address in shared memory) set; the caller goes on without looking (every later
-// wait then returns at once, the loops end, and results are dropped after the CTA's next barrier), so a warp never
-// diverges here and the ready case is one instruction and a branch: with a poll of the flag and two votes around it a
-// satisfied wait took 160 clocks of a GEMM's 668 per k-block.
-__device__ __forceinline__ void mbar_wait_or_abort(uint32_t bar, uint32_t parity, uint32_t abort_flag, int32_t* d_status,
-                                                   int timeout_code) {
-  if (mbar_try_wait(bar, parity)) return;
+// Wait inside a pipeline loop: true once the phase has completed.  After `limit` polls, or when another thread of the CTA
+// has given up, it returns false with the abort flag (an address in shared memory) set.  Warps do not branch on it (every
+// later wait then returns at once, the loops end, and results are dropped after the CTA's next barrier), so the ready case
+// is one instruction and a branch: with a poll of the flag and two votes around it a satisfied wait took 160 clocks of a
+// GEMM's 668 per k-block.  But a thread that issues copies issues none from its first false on, and one that issues
+// products reports no stage as read from then on: a stage is refilled only if its last copy has landed and been read, so
+// that what is in flight at the end is known and can be waited for.
+__device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity, uint32_t abort_flag, int32_t* d_status,
+                                                   int timeout_code, uint32_t limit = kWaitLimit) {
+  if (mbar_try_wait(bar, parity)) return true;
 #pragma unroll 1
-  for (uint32_t i = 0; i < kWaitLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return;
-    if ((i & 63u) == 0u && lds_s32(abort_flag)) return;
+  for (uint32_t i = 0; i < limit; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 63u) == 0u && lds_s32(abort_flag)) return false;
   }
   if (d_status != nullptr) atomicCAS(d_status, 0, timeout_code);
   sts_s32(abort_flag, 1);
+  return false;
 }
 // The same by all lanes of a warp, which are converged again when it returns: lanes may have polled a different number of
-// times, and elect_one() in a diverged warp would elect a lane of each part.
-__device__ __forceinline__ void mbar_wait_or_abort_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag, int32_t* d_status,
-                                                        int timeout_code) {
-  mbar_wait_or_abort(bar, parity, abort_flag, d_status, timeout_code);
+// times, and elect_one() in a diverged warp would elect a lane of each part.  Each lane gets its own answer.
+__device__ __forceinline__ bool mbar_wait_or_abort_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag, int32_t* d_status,
+                                                        int timeout_code, uint32_t limit = kWaitLimit) {
+  const bool ok = mbar_wait_or_abort(bar, parity, abort_flag, d_status, timeout_code, limit);
   __syncwarp();
+  return ok;
 }
 
 // True in exactly one lane of a converged warp (all 32 lanes must execute it together).  Work that one thread has to
@@ -195,6 +202,21 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, ui
 // Arrive on `bar` once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// The end of a single-CTA pipeline in which a wait gave up, by all its threads behind a barrier: the copies of the last
+// `stages` of the `issued` k-blocks that thread 0 has issued, and the products that warp 1 has, complete (each wait with
+// a limit) before the CTA's memory goes away.  full0: the first of the stages' barriers; drain: a barrier of one arrival
+// that nothing else uses.  Not inlined: inside the kernels this code cost every launch 0.1 us.
+inline __device__ __noinline__ void drain_cta(int issued, int stages, uint32_t full0, uint32_t drain) {
+  if (threadIdx.x == 0)
+    for (int j = issued > stages ? issued - stages : 0; j < issued; ++j) mbar_wait(full0 + 8u * (j % stages), (j / stages) & 1);
+  if (threadIdx.x / 32 == 1) {
+    if (elect_one()) mma_commit(drain);
+    __syncwarp();
+    mbar_wait(drain, 0);
+  }
+  __syncwarp();
 }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp receives row (lane base + t).
