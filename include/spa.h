@@ -334,7 +334,7 @@ int spa_gelu_bwd(const spa_params* p, const void* dh, const void* u, int32_t n_c
  *   every backward field    for spa_block_fwd;
  *   labels .. train_workspace unless `trainable` is non-zero.
  * The forward pass leaves scores, mask, cu_seqlens, idx, inv, x_packed, qkv, attn_out, lse for the backward pass. */
-typedef struct spa_overlap spa_overlap;  /* a second stream and the two events that fork to it and join it */
+typedef struct spa_overlap spa_overlap;  /* two more streams and the two events that fork to them and join them */
 
 typedef struct spa_block_buffers {
   /* inputs of the forward pass */
@@ -372,7 +372,7 @@ typedef struct spa_block_buffers {
   float* db_qkv;              /* float[3C]                                                           */
   float* dW_o;                /* float[C][C]                                                         */
   float* db_o;                /* float[C]                                                            */
-  void* workspace;            /* spa_workspace_bytes()                                               */
+  void* workspace;            /* spa_workspace_bytes(); with `overlap` the second streams use it too */
   void* workspace_side;       /* a second area of that size; needed when `overlap` is given          */
   void* pack_state;           /* spa_pack_state_bytes(), zeroed once by the caller, or NULL: gate and
                                  packing then run as two kernels                                     */

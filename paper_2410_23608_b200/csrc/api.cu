@@ -436,15 +436,16 @@ int spa_gelu_bwd(const spa_params* p, const void* dh, const void* u, int32_t n_c
 
 // ---- the block as one unit: sequencing only ------------------------------------------------------------------
 struct spa_overlap {
-  cudaStream_t side;
+  cudaStream_t side, side2;
   cudaEvent_t fork, join;
 };
 
 int spa_overlap_create(spa_overlap** out) {
   if (out == nullptr) return SPA_ERR_INVALID_ARG;
-  spa_overlap* ov = new (std::nothrow) spa_overlap{nullptr, nullptr, nullptr};
+  spa_overlap* ov = new (std::nothrow) spa_overlap{nullptr, nullptr, nullptr, nullptr};
   if (ov == nullptr) return SPA_ERR_INVALID_ARG;
   cudaError_t e = cudaStreamCreateWithFlags(&ov->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ov->side2, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ov->fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ov->join, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -460,6 +461,7 @@ int spa_overlap_destroy(spa_overlap* ov) {
   if (ov == nullptr) return SPA_OK;
   if (ov->join != nullptr) cudaEventDestroy(ov->join);
   if (ov->fork != nullptr) cudaEventDestroy(ov->fork);
+  if (ov->side2 != nullptr) cudaStreamDestroy(ov->side2);
   if (ov->side != nullptr) cudaStreamDestroy(ov->side);
   delete ov;
   return SPA_OK;
@@ -484,15 +486,21 @@ int qkv_bwd_scatter(const spa_params* p, const spa_block_buffers* b, float* dW, 
   return linear_bwd_other(*p, b->x_packed, b->W_qkv, b->dqkv, p->C, 3 * p->C, b->cu_seqlens, b->dX, dW, db, b->d_status, stream,
                           b->idx, (p->flags & SPA_FLAG_RESIDUAL) != 0);
 }
-// the second stream starts after everything enqueued on the main stream so far
-inline int fork_side(const spa_overlap* ov, cudaStream_t main) {
+inline bool is_recorded(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s == cudaStreamCaptureStatusActive;
+  cudaGetLastError();
+  return false;
+}
+// `side` (a stream of ov) starts after everything enqueued on the main stream so far
+inline int fork_side(const spa_overlap* ov, cudaStream_t main, cudaStream_t side) {
   cudaError_t e = cudaEventRecord(ov->fork, main);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->side, ov->fork, 0);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ov->fork, 0);
   if (e != cudaSuccess) { set_cuda_error(e, "spa_block_bwd: fork"); return SPA_ERR_CUDA; }
   return SPA_OK;
 }
-inline int join_side(const spa_overlap* ov, cudaStream_t main) {
-  cudaError_t e = cudaEventRecord(ov->join, ov->side);
+inline int join_side(const spa_overlap* ov, cudaStream_t main, cudaStream_t side) {
+  cudaError_t e = cudaEventRecord(ov->join, side);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(main, ov->join, 0);
   if (e != cudaSuccess) { set_cuda_error(e, "spa_block_bwd: join"); return SPA_ERR_CUDA; }
   return SPA_OK;
@@ -557,13 +565,21 @@ int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream)
     SPA_STEP(spa_select_loss(p, b->scores, b->labels, b->alpha, b->ds, b->loss, b->train_workspace, stream));
   // dz = rows of dY at the selected tokens; dX = dY on the tokens that passed through
   SPA_STEP(spa_unpack_scatter_bwd(p, b->dY, b->idx, b->inv, b->cu_seqlens, b->dz, b->dX, stream));
-  bool forked = false;
+  // In a recorded step the QKV layer's weight gradient has a stream of its own, with scratch of its own: `workspace`, whose
+  // D_i the attention backward in front of it was the last to read.  Behind the projection's on one stream it would have two
+  // predecessors, and such a kernel of a graph is not launched early (programmatic launch).  One graph per step, 64 images
+  // of 196 tokens of 384 channels 127.6 -> 122.0 us, 2 of 4 200 of 256 133.0 -> 126.6, 128 of 196 of 768 245 -> 242.5.  The
+  // second fork and join cost 2 us, more than that gives on small batches (16 images of 196 tokens of 768 channels 98 ->
+  // 100, of 384 76.5 -> 75.0) and 1 to 2 us in a step that is not recorded.
+  const bool apart = ov != nullptr && b->workspace != nullptr && p->capacity >= 4096 && is_recorded(main);
+  cudaStream_t side_qkv = ov == nullptr ? nullptr : (apart ? ov->side2 : ov->side);
+  bool forked = false, forked_qkv = false;
   int rc_side = SPA_OK;
   if (ov == nullptr) {
     SPA_STEP(spa_packed_linear_bwd(p, b->attn_out, b->W_o, b->dz, C, C, b->cu_seqlens, b->d_attn_out, b->dW_o, b->db_o,
                                    b->workspace, b->d_status, stream));
   } else {
-    SPA_STEP(fork_side(ov, main));
+    SPA_STEP(fork_side(ov, main, ov->side));
     forked = true;
     rc_side = spa_packed_linear_bwd(p, b->attn_out, b->W_o, b->dz, C, C, b->cu_seqlens, nullptr, b->dW_o, b->db_o,
                                     b->workspace_side, b->d_status, side);
@@ -575,11 +591,12 @@ int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream)
                                   b->d_status, stream);
   if (rc == SPA_OK && rc_side == SPA_OK) {
     if (ov != nullptr) {
-      // the second stream's next call reads dqkv: it waits for the attention backward
-      rc_side = fork_side(ov, main);
+      // it reads dqkv: behind the attention backward
+      rc_side = fork_side(ov, main, side_qkv);
+      forked_qkv = rc_side == SPA_OK;
       if (rc_side == SPA_OK)
         rc_side = spa_packed_linear_bwd(p, b->x_packed, b->W_qkv, b->dqkv, C, 3 * C, b->cu_seqlens, nullptr, b->dW_qkv,
-                                        b->db_qkv, b->workspace_side, b->d_status, side);
+                                        b->db_qkv, apart ? b->workspace : b->workspace_side, b->d_status, (void*)side_qkv);
     }
     float* dW = ov != nullptr ? nullptr : b->dW_qkv;
     float* db = ov != nullptr ? nullptr : b->db_qkv;
@@ -602,7 +619,11 @@ int spa_block_bwd(const spa_params* p, const spa_block_buffers* b, void* stream)
   if (rc == SPA_OK && rc_side == SPA_OK && b->trainable)
     rc = spa_gate_bwd(p, b->x, b->w_g, b->scores, b->s_up, b->ds, b->dX, b->dw_g, b->db_g, b->ds_up, b->train_workspace, stream);
   if (forked) {  // joined on every path, so that a recording stream is never left forked
-    const int rj = join_side(ov, main);
+    int rj = join_side(ov, main, ov->side);
+    if (forked_qkv && side_qkv != ov->side) {
+      const int rq = join_side(ov, main, side_qkv);
+      if (rj == SPA_OK) rj = rq;
+    }
     if (rc == SPA_OK) rc = rc_side != SPA_OK ? rc_side : rj;
   }
   return rc;
@@ -710,7 +731,7 @@ int spa_layer_bwd(const spa_params* p, const spa_layer_buffers* l, void* stream)
   auto fork = [&]() -> int {
     if (ov == nullptr) return SPA_OK;
     forked = true;
-    return fork_side(ov, st);
+    return fork_side(ov, st, ov->side);
   };
   auto run = [&]() -> int {
     SPA_STEP(fork());
@@ -737,7 +758,7 @@ int spa_layer_bwd(const spa_params* p, const spa_layer_buffers* l, void* stream)
   };
   rc = run();
   if (forked) {  // joined on every path, so that a recording stream is never left forked
-    const int rj = join_side(ov, st);
+    const int rj = join_side(ov, st, ov->side);
     if (rc == SPA_OK) rc = rj;
   }
   return rc;
