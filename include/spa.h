@@ -437,7 +437,9 @@ typedef struct spa_layer_buffers {
                                  stream of blk->overlap; or NULL                                     */
 } spa_layer_buffers;
 
-/* Forward pass of the block.  blk->pack_state, order, s_up, seg_offsets and container_len are not looked at. */
+/* Forward pass of the block.  blk->pack_state, order, s_up, seg_offsets and container_len are not looked at.  `flags` must hold
+ * SPA_FLAG_RESIDUAL; SPA_FLAG_INPLACE changes nothing (under SPA_FLAG_UNFUSED, where it would reach spa_unpack_scatter, it is
+ * refused). */
 int spa_layer_fwd(const spa_params* p, const spa_layer_buffers* l, void* stream);
 
 /* Backward pass for the last spa_layer_fwd on the same buffers: dX, dW1, db1, dW2, db2, the LayerNorms' dg and dbe, and

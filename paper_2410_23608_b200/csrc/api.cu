@@ -675,7 +675,7 @@ int check_layer(const spa_params* p, const spa_layer_buffers* l) {
   SPA_PTR(l->x); SPA_PTR(l->g1); SPA_PTR(l->be1); SPA_PTR(l->g2); SPA_PTR(l->be2);
   SPA_PTR(l->z); SPA_PTR(l->y1); SPA_PTR(l->t); SPA_PTR(l->out); SPA_PTR(l->u); SPA_PTR(l->h);
   SPA_REQUIRE(l->m1 != nullptr && l->r1 != nullptr && l->m2 != nullptr && l->r2 != nullptr && l->eps > 0.f, SPA_ERR_INVALID_ARG);
-  SPA_REQUIRE((p->flags & SPA_FLAG_RESIDUAL) && !(p->flags & SPA_FLAG_INPLACE), SPA_ERR_INVALID_ARG);
+  SPA_REQUIRE((p->flags & SPA_FLAG_RESIDUAL) != 0, SPA_ERR_INVALID_ARG);
   return SPA_OK;
 }
 }  // namespace

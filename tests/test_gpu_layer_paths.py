@@ -54,3 +54,19 @@ def test_linear_tile_widths(rows, n_in, n_out, slack):
     for got, ref in ((out[:rows], a[:rows].double() @ W.double().T + b.double()), (da[:rows], dout[:rows].double() @ W.double())):
         assert float(((got.double() - ref).abs() / (1e-2 * ref.abs() + 1e-2 * ref.abs().mean())).max()) < 1
     assert bool((out[rows:] == 7).all()) and bool((da[rows:] == 7).all())
+
+
+def test_inplace_flag_changes_nothing():
+    from paper_2410_23608_b200 import binding as L
+    from paper_2410_23608_b200.layer import SpaLayer
+    cfg, inp, x, prm, _ = layer_problem(2, 1)
+    dprm = {k: (dev(v, cfg.dtype) if isinstance(v, np.ndarray) else v) for k, v in prm.items()}
+    runs = []
+    for flags in (0, L.SPA_FLAG_INPLACE):
+        lay = SpaLayer(cfg.B, cfg.N, cfg.C, cfg.H, cfg.dtype, flags=flags)
+        xd = dev(x, cfg.dtype)
+        out, dX = lay.forward(xd, dprm), lay.backward(dev(inp.dY, cfg.dtype))
+        torch.cuda.synchronize()
+        assert lay.read_status() == 0 and torch.equal(xd, dev(x, cfg.dtype))
+        runs.append((out, dX, lay.dW1, lay.blk.dW_qkv))
+    assert all(torch.equal(a, b) for a, b in zip(*runs))

@@ -100,3 +100,22 @@ def test_later_entry_points_validate_on_the_host(lib):
     assert L.spa_fused_scatter_supported(ctypes.byref(f32)) == 0          # tensor-core problems only
     assert L.spa_packed_proj_scatter(ctypes.byref(f32), None, None, None, None, None, None, None, None) in (inv, uns)
     assert L.spa_train_workspace_bytes(pp) > 0 and L.spa_train_workspace_bytes(None) == 0
+
+
+def test_transformer_block_takes_the_inplace_flag(lib):
+    """An empty batch passes every check and does no device work: SPA_FLAG_INPLACE is accepted, the residual is wanted."""
+    L = lib.lib()
+    word = 1 << 20   # any aligned address: nothing is read
+    blk = lib.SpaBlockBuffers()
+    for name, kind in lib.SpaBlockBuffers._fields_:
+        if kind is ctypes.c_void_p:
+            setattr(blk, name, word)
+    lay = lib.SpaLayerBuffers(blk=ctypes.pointer(blk), hidden=256, eps=1e-5)
+    for name, kind in lib.SpaLayerBuffers._fields_:
+        if kind is ctypes.c_void_p:
+            setattr(lay, name, word)
+    res, inp = lib.SPA_FLAG_RESIDUAL, lib.SPA_FLAG_INPLACE
+    for flags, rc in ((res, 0), (res | inp, 0), (inp, lib.SPA_ERR_INVALID_ARG), (0, lib.SPA_ERR_INVALID_ARG)):
+        none = lib.make_params(0, 16, 64, 2, "bf16", flags=flags)
+        assert L.spa_layer_fwd(ctypes.byref(none), ctypes.byref(lay), None) == rc
+        assert L.spa_layer_bwd(ctypes.byref(none), ctypes.byref(lay), None) == rc
