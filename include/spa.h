@@ -431,11 +431,14 @@ typedef struct spa_layer_buffers {
   void* dh;                   /* T[B*N][hidden]: gradient to u                                       */
   void *dt, *dy1, *dX;        /* T[B][N][C]                                                          */
   float *dW1, *db1, *dW2, *db2, *dg1, *dbe1, *dg2, *dbe2;
-  void* workspace;            /* at least spa_workspace_bytes(), spa_train_workspace_bytes() and
-                                 32 (hidden C + max(hidden, C)) floats + 1 KB                        */
-  void* workspace_side;       /* a second area of that size: the weight gradients then run on the second
+  void* workspace;            /* spa_layer_workspace_bytes(p, hidden, 0); without workspace_side or without blk->overlap
+                                 the larger of that and spa_layer_workspace_bytes(p, hidden, 1)      */
+  void* workspace_side;       /* spa_layer_workspace_bytes(p, hidden, 1): the weight gradients then run on the second
                                  stream of blk->overlap; or NULL                                     */
 } spa_layer_buffers;
+
+/* Bytes of scratch of spa_layer_bwd: side = 0 for what runs on the caller's stream, 1 for the weight gradients. */
+size_t spa_layer_workspace_bytes(const spa_params* p, int32_t hidden, int32_t side);
 
 /* Forward pass of the block.  blk->pack_state, order, s_up, seg_offsets and container_len are not looked at.  `flags` must hold
  * SPA_FLAG_RESIDUAL; SPA_FLAG_INPLACE changes nothing (under SPA_FLAG_UNFUSED, where it would reach spa_unpack_scatter, it is

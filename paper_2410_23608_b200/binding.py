@@ -33,7 +33,7 @@ EXPORTS = (
     "spa_fused_scatter_supported", "spa_gate_prefill", "spa_unpack_prefill", "spa_packed_proj_scatter", "spa_packed_linear_bwd_scatter",
     "spa_select_pack_ordered", "spa_train_workspace_bytes", "spa_score_pool", "spa_select_loss", "spa_select_pack_bwd_gated", "spa_gate_bwd",
     "spa_packed_linear", "spa_layer_norm", "spa_layer_norm_bwd", "spa_gelu", "spa_gelu_bwd",
-    "spa_overlap_create", "spa_overlap_destroy", "spa_block_fwd", "spa_block_bwd", "spa_layer_fwd", "spa_layer_bwd",
+    "spa_overlap_create", "spa_overlap_destroy", "spa_block_fwd", "spa_block_bwd", "spa_layer_fwd", "spa_layer_bwd", "spa_layer_workspace_bytes",
     "spa_probe_exp2", "spa_probe_wait_expiry", "spa_probe_mma_issue", "spa_pack_state_bytes", "spa_gate_select_pack_supported",
     "spa_gate_select_pack", "spa_container_max_segments", "spa_container_offsets",
 )
@@ -132,6 +132,8 @@ def lib() -> C.CDLL:
         L.spa_block_bwd.argtypes = [pp, C.POINTER(SpaBlockBuffers), vp]
         L.spa_layer_fwd.argtypes = [pp, C.POINTER(SpaLayerBuffers), vp]
         L.spa_layer_bwd.argtypes = [pp, C.POINTER(SpaLayerBuffers), vp]
+        L.spa_layer_workspace_bytes.restype = C.c_size_t
+        L.spa_layer_workspace_bytes.argtypes = [pp, i32, i32]
         L.spa_pack_state_bytes.restype = C.c_size_t
         L.spa_pack_state_bytes.argtypes = [pp]
         L.spa_gate_select_pack_supported.argtypes = [pp]
@@ -143,7 +145,7 @@ def lib() -> C.CDLL:
         L.spa_probe_mma_issue.argtypes = [i32, i32, vp, vp, vp]
         L.spa_read_status.argtypes = [vp, vp]
         for name in EXPORTS:
-            if name not in ("spa_workspace_bytes", "spa_train_workspace_bytes", "spa_pack_state_bytes", "spa_status_string", "spa_last_cuda_error",
+            if name not in ("spa_workspace_bytes", "spa_layer_workspace_bytes", "spa_train_workspace_bytes", "spa_pack_state_bytes", "spa_status_string", "spa_last_cuda_error",
                             "spa_launch_count"):
                 getattr(L, name).restype = C.c_int
         L.spa_status_string.restype = C.c_char_p
@@ -188,6 +190,10 @@ def _check(rc: int, where: str):
 
 def spa_workspace_bytes(p: SpaParams) -> int:
     return int(lib().spa_workspace_bytes(C.byref(p)))
+
+
+def spa_layer_workspace_bytes(p: SpaParams, hidden: int, side: bool) -> int:
+    return int(lib().spa_layer_workspace_bytes(C.byref(p), int(hidden), int(side)))
 
 
 def spa_gate(p, x, w_g, b_g, s_up, scores, mask, stream=None):

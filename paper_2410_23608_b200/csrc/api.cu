@@ -680,6 +680,20 @@ int check_layer(const spa_params* p, const spa_layer_buffers* l) {
 }
 }  // namespace
 
+size_t spa_layer_workspace_bytes(const spa_params* p, int32_t hidden, int32_t side) {
+  if (check_params(p) != SPA_OK || hidden <= 0) return 0;
+  size_t most = 0;
+  auto at_least = [&](size_t bytes) { most = bytes > most ? bytes : most; };
+  if (side != 0) {  // the weight gradients
+    const int layers[4][2] = {{hidden, p->C}, {p->C, hidden}, {p->C, p->C}, {p->C, 3 * p->C}};
+    for (const auto& l : layers) at_least(tc_weight_grad_workspace_bytes(*p, l[0], l[1]));
+  } else {  // D_i of the attention backward, the per-CTA sums of the LayerNorm backward
+    at_least(tc_attention_workspace_bytes(*p));
+    at_least(layer_norm_workspace_bytes(*p));
+  }
+  return (most + 255) & ~(size_t)255;
+}
+
 // Eight kernels instead of the twelve that the calls one by one take (a kernel boundary costs 2.6 us, more than the work of
 // most of them on a small batch): LN1 also writes the gate's scores and the residual stream, the first feed-forward product
 // writes its activation too, the second adds the residual from where it lies.  8 x 196 tokens of 384 channels: 78 -> 67 us.

@@ -530,6 +530,10 @@ bool tc_linear_supported(int n_in, int n_out) {
   return n_in % 8 == 0 && n_out % 8 == 0 && n_in >= 64 && n_out >= 64 && encode_fn() != nullptr;
 }
 
+size_t tc_weight_grad_workspace_bytes(const spa_params& p, int n_in, int n_out) {
+  return p.dtype == SPA_BF16 && tc_linear_supported(n_in, n_out) ? wgrad_workspace_bytes(p.capacity, n_in, n_out) : 0;
+}
+
 size_t tc_linear_workspace_bytes(const spa_params& p) {
   if (p.dtype != SPA_BF16 || !tc_linear_supported(p.C, 3 * p.C)) return 0;
   const size_t a = wgrad_workspace_bytes(p.capacity, p.C, 3 * p.C);

@@ -50,6 +50,7 @@ template <int kKind> struct RowEpilogue {
 };
 
 size_t tc_linear_workspace_bytes(const spa_params& p);
+size_t tc_weight_grad_workspace_bytes(const spa_params& p, int n_in, int n_out);
 size_t tc_attention_workspace_bytes(const spa_params& p);
 
 bool tc_linear_supported(int n_in, int n_out);

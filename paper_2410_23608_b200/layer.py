@@ -35,10 +35,9 @@ class SpaLayer:
         f = lambda *s: torch.empty(*s, dtype=torch.float32, device=dev)
         self.dW1, self.db1, self.dW2, self.db2 = f(self.hidden, C), f(self.hidden), f(C, self.hidden), f(C)
         self.dg1, self.dbe1, self.dg2, self.dbe2 = f(C), f(C), f(C), f(C)
-        # split-K partials of the widest weight gradient (at most 32 splits) and the per-CTA sums of the LayerNorm backward
-        ws = max(L.spa_workspace_bytes(self.p), 32 * self.hidden * C * 4 + 32 * max(self.hidden, C) * 4 + 1024,
-                 L.spa_train_workspace_bytes(self.p))
-        self.workspace, self.workspace_side = (torch.empty(ws, dtype=torch.uint8, device=dev) for _ in range(2))
+        # one area for the caller's stream, one for the weight gradients on the library's second stream
+        need = (max(L.spa_layer_workspace_bytes(self.p, self.hidden, side), 256) for side in (False, True))
+        self.workspace, self.workspace_side = (torch.empty(n, dtype=torch.uint8, device=dev) for n in need)
         self.blk._bufs.overlap = self.blk._overlap  # the weight gradients on the library's second stream
         self._lib = L.lib()
         own = ("cu_all", "z", "y1", "t", "out", "u", "h", "m1", "r1", "m2", "r2", "dh", "dt", "dy1", "dX", "dW1", "db1", "dW2", "db2",
