@@ -1892,7 +1892,7 @@ int bwd_launch(const spa_params& p, const void* qkv, const void* ao, const float
 }
 
 // The counter that a launch which writes `out` draws its items from, or nullptr (then a static stride assigns them).
-unsigned* item_counter(const void* out, cudaStream_t st);
+unsigned* item_counter(const void* out);
 
 template <int D>
 int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao, float* lse,
@@ -1910,7 +1910,7 @@ int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_s
   // 400 rows (and cost 1 us in front of short items), and 8 to 12 % from 576 rows on.
   const bool even_items = (long long)p.capacity <= 512ll * (n_seg > 0 ? n_seg : 1);
   launch_pdl(kern, grid, kFwdThreads, FwdSmem<D>::kBytes, st, tm, seg, n_seg, p.capacity, p.C, p.H,
-             softmax_scale_of(p) * 1.4426950408889634f, (__nv_bfloat16*)ao, lse, items > grid ? item_counter(ao, st) : nullptr, even_items, d_status);
+             softmax_scale_of(p) * 1.4426950408889634f, (__nv_bfloat16*)ao, lse, items > grid ? item_counter(ao) : nullptr, even_items, d_status);
   SPA_CUDA_CHECK_LAUNCH("attn_fwd_tc_kernel");
   return SPA_OK;
 }
@@ -1975,7 +1975,18 @@ struct DeviceCounters {
 };
 DeviceCounters* const g_counters = new DeviceCounters[kMaxDevices];  // never destroyed: launches may come at any time
 
-unsigned* item_counter(const void* out, cudaStream_t st) {
+// Device address of a variable of this library.  Also while the calling thread records a stream: loading what holds the
+// variable is then not part of the recording.
+template <typename T> cudaError_t symbol_address(void** p, const T& symbol) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  e = cudaGetSymbolAddress(p, symbol);
+  const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+  return e != cudaSuccess ? e : back;
+}
+
+unsigned* item_counter(const void* out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
     cudaGetLastError();
@@ -1983,11 +1994,9 @@ unsigned* item_counter(const void* out, cudaStream_t st) {
   }
   std::lock_guard<std::mutex> lock(g_counter_mutex);
   DeviceCounters& c = g_counters[dev];
-  if (c.base == nullptr) {  // looked up once, not while a stream is being recorded
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (c.base == nullptr) {
     void* p = nullptr;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
-        cudaGetSymbolAddress(&p, g_item_counters) != cudaSuccess) {
+    if (symbol_address(&p, g_item_counters) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
@@ -2011,7 +2020,7 @@ int static_attention_scratch(void** out) {
   std::lock_guard<std::mutex> lock(g_scratch_mutex);
   if (g_scratch_ptr[dev] == nullptr) {
     void* ptr = nullptr;
-    e = cudaGetSymbolAddress(&ptr, g_static_scratch);
+    e = symbol_address(&ptr, g_static_scratch);
     if (e != cudaSuccess || ptr == nullptr) {
       set_cuda_error(e, "spa_packed_attention_bwd_static: cudaGetSymbolAddress");
       return SPA_ERR_CUDA;
