@@ -4,7 +4,8 @@
 // An fp32 value is the exact sum of three bf16 values (8 + 8 + 8 bits of its 24): x = x0 + x1 + x2.  Of the nine
 // products of two such sums the six largest are formed - x0 y0; x0 y1, x1 y0, x0 y2, x1 y1, x2 y0 - and what is left
 // out lies below 2^-26 of |x||y|, under the rounding of an fp32 product.  x0 y0 has an accumulator of its own: the
-// small terms then add no rounding steps at the magnitude of the result; the two are added at the end.
+// small terms then add no rounding steps at the magnitude of the result; the two are added at the end.  (The method:
+// Henry, Tang, Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype For Higher-Precision Computations", 2019.)
 //   forward  A = a (K contiguous),     B = W (K contiguous),   M = packed rows (device)
 //   dgrad    A = dout (K contiguous),  B = W (N contiguous),   M = packed rows (device)
 //   wgrad    A = dout (M contiguous),  B = a (N contiguous),   K = packed rows (device)
@@ -13,9 +14,14 @@
 // operands follow from it.  A ninth warp issues the products.  The finished tile goes through shared memory, where a
 // cluster that splits K adds its partial tiles in a fixed order over distributed shared memory: no scratch in global
 // memory, bitwise reproducible.
+// Infinities: an infinite part times a zero part is NaN where the product of the values is not, and a finite value next to
+// fp32's largest rounds to an infinite first part.  Either leaves an infinity or NaN in the result, so results that are not
+// finite are formed again as a chain of fp32 FMAs over K (fma_chain), which is what they are by definition.
 // Bound: 24 products per 64-k block and tile (1 650 clocks at BN = 128) against about 800 issue clocks of splitting.
 // 1 568 x 1 152 x 384: forward 18, dgrad 23, wgrad 23 us, where fp32 FMAs on 64 x 64 tiles took 73, 99 and 141; error
 // against fp64 1e-7 to 5e-7 relative, that of the FMA kernels 2e-7 to 1e-6.
+#include <math_constants.h>
+
 #include "simt_stage.cuh"
 #include "sm100_ptx.cuh"
 #include "spa_common.cuh"
@@ -41,7 +47,7 @@ __device__ __forceinline__ float4 ld_values(const float* p) {
 
 struct Tile8 { float4 a, b; };  // eight consecutive values of a line
 
-// Two values into their three bf16 parts, packed pairwise.  A value beyond bf16's range keeps its infinite first part.
+// Two values into their three bf16 parts, packed pairwise.  An infinite first part has no rest.
 __device__ __forceinline__ void split2(float x, float y, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
   auto pack = [](float u, float v) { __nv_bfloat162 h = __floats2bfloat162_rn(u, v); return *reinterpret_cast<uint32_t*>(&h); };
   auto rest = [](float v, uint32_t part) { return (part & 0x7f800000u) != 0x7f800000u ? v - __uint_as_float(part) : 0.f; };
@@ -98,6 +104,25 @@ template <int R, bool kMn> struct Operand {
 
 __device__ __forceinline__ uint64_t operand_desc(uint32_t addr, int k, bool mn) {
   return mn ? ptx::smem_desc_sw128(addr + k * 2048, BK * 128, 1024) : ptx::smem_desc_sw128(addr + k * 32, 16, 1024);
+}
+
+// Results m, n .. n + 3 as chains of FMAs over K, for those that the three parts leave infinite or NaN: rare, so not inlined.
+// Chains that are all NaN stay NaN.
+template <bool kAMn, bool kBMn>
+__device__ __noinline__ float4 fma_chain(const float* A, long long lda, const float* B, long long ldb, int m, int n, int K) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k = 0; k < K; ++k) {
+    const float a = A[kAMn ? (long long)k * lda + m : (long long)m * lda + k];
+    float b[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = B[kBMn ? (long long)k * ldb + n + j : (long long)(n + j) * ldb + k];
+    v.x = fmaf(a, b[0], v.x);
+    v.y = fmaf(a, b[1], v.y);
+    v.z = fmaf(a, b[2], v.z);
+    v.w = fmaf(a, b[3], v.w);
+    if (v.x != v.x && v.y != v.y && v.z != v.z && v.w != v.w) break;
+  }
+  return v;
 }
 
 // dyn_which: 1 = M is the device-side packed row count, 2 = K is.
@@ -272,6 +297,7 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
       if (n0 + c >= N) continue;
       const float* src = tile + r * kLd + c;
       float4 v = split > 1 ? sum_dsmem4(src, split) : *reinterpret_cast<const float4*>(src);
+      if (!(fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(v.w) < CUDART_INF_F)) v = fma_chain<kAMn, kBMn>(A, lda, Bm, ldb, m0 + r, n0 + c, K);
       if (bias != nullptr) {
         const float4 w = __ldg(reinterpret_cast<const float4*>(bias + n0 + c));
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
