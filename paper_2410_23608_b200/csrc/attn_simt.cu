@@ -88,6 +88,22 @@ __device__ __forceinline__ void weighted(float (*o)[D / kTX], const float* p, co
   }
 }
 
+// A zero weight times an infinity or NaN of another segment in the same tile is NaN.  Sums that are not finite, where the
+// CTA's rows are of several segments, are therefore formed again from their own segment's rows alone: rare, one value after
+// the other from global memory.  (Tiles looked at as they come in, or a second pass over the tiles: 3 us of 69 each.)
+template <int W> __device__ __forceinline__ bool finite_sums(const float* o) {
+  float s = 0.f;
+#pragma unroll
+  for (int d = 0; d < W; ++d) s += fabsf(o[d]);
+  return s < CUDART_INF_F;
+}
+template <typename T, int D> __device__ __forceinline__ float row_dot(const T* a, const T* b) {
+  float s = 0.f;
+#pragma unroll 1
+  for (int e = 0; e < D; ++e) s = fmaf(to_f32<T>(a[e]), to_f32<T>(b[e]), s);
+  return s;
+}
+
 // W consecutive values of one row
 template <typename T, int W> __device__ __forceinline__ void store_row(T* dst, const float* v) {
 #pragma unroll
@@ -150,6 +166,7 @@ attn_fwd_simt_kernel(const T* __restrict__ qkv, const int32_t* __restrict__ seg,
     cp_async_commit();
   };
   const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
+  const bool several = seg_s[0].hi < all.hi;  // segments that the CTA's rows are of
   stage(0);
 
   float o[4][W] = {}, m[4], l[4] = {};
@@ -196,6 +213,17 @@ attn_fwd_simt_kernel(const T* __restrict__ qkv, const int32_t* __restrict__ seg,
   for (int i = 0; i < 4; ++i) {
     const int row = i0 + ty + kTY * i;
     if (row >= Np) continue;
+    if (several && !finite_sums<W>(o[i])) {
+#pragma unroll
+      for (int d = 0; d < W; ++d) o[i][d] = 0.f;
+#pragma unroll 1
+      for (int k = mine[i].lo; k < mine[i].hi; ++k) {
+        const T* key = qkv + k * ld + C + h * D;
+        const float p = expf(row_dot<T, D>(qkv + row * ld + h * D, key) * scale - m[i]);
+#pragma unroll
+        for (int d = 0; d < W; ++d) o[i][d] = fmaf(p, to_f32<T>(key[C + tx * W + d]), o[i][d]);
+      }
+    }
     const float inv_l = 1.f / l[i];
 #pragma unroll
     for (int d = 0; d < W; ++d) o[i][d] *= inv_l;
@@ -267,6 +295,7 @@ attn_bwd_simt_kernel(const T* __restrict__ qkv, const T* __restrict__ ao, const 
     }
   };
   const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
+  const bool several = seg_s[0].hi < all.hi;  // segments that the CTA's rows are of
   stage(0);
 
   RowSeg mine[4];
@@ -314,6 +343,22 @@ attn_bwd_simt_kernel(const T* __restrict__ qkv, const T* __restrict__ ao, const 
   for (int i = 0; i < 4; ++i) {
     const int row = i0 + ty + kTY * i;
     if (row >= Np) continue;
+    if (several && !(finite_sums<W>(acc1[i]) && finite_sums<W>(acc2[i]))) {
+#pragma unroll
+      for (int d = 0; d < W; ++d) acc1[i][d] = acc2[i][d] = 0.f;
+#pragma unroll 1
+      for (int k = mine[i].lo; k < mine[i].hi; ++k) {
+        const int q = dq ? row : k, j = dq ? k : row;  // query and key of the pair
+        const T *Q = qkv + q * ld + h * D, *K = qkv + j * ld + C + h * D, *dO = dao + (long long)q * C + h * D;
+        const float p = expf(row_dot<T, D>(Q, K) * scale - lse[(long long)h * capacity + q]);
+        const float ds = p * (row_dot<T, D>(dO, K + C) - row_dot<T, D>(dO, ao + (long long)q * C + h * D));
+#pragma unroll
+        for (int d = 0; d < W; ++d) {
+          acc1[i][d] = fmaf(ds, to_f32<T>((dq ? K : Q)[tx * W + d]), acc1[i][d]);
+          if (!dq) acc2[i][d] = fmaf(p, to_f32<T>(dO[tx * W + d]), acc2[i][d]);
+        }
+      }
+    }
     T* dst = dqkv + (long long)row * ld + h * D + tx * W;
 #pragma unroll
     for (int d = 0; d < W; ++d) acc1[i][d] *= scale;
