@@ -27,7 +27,7 @@ template <int D> constexpr int kLd = D + 4;  // rows 4 banks apart
 
 // Rows [row0, row0 + kRows) of one head's slice (column col0 of a [*, ld] matrix); rows from row_end on become zero.
 template <typename T, int D, int kRows>
-__device__ __forceinline__ void stage_rows(float* dst, const T* __restrict__ src, long long ld, int col0, int row0, int row_end,
+__device__ __forceinline__ void stage_rows(float* dst, const T* src, long long ld, int col0, int row0, int row_end,
                                            int tid) {
   constexpr int E = Vec16<T>::kElems, kPer = D / E;
 #pragma unroll
@@ -128,7 +128,7 @@ __device__ __forceinline__ float sum16(float v) {
 }
 
 // Segments of the CTA's 32 rows in seg_s[32] (threads 0-31 search one each); returns the range they span together.
-__device__ __forceinline__ RowSeg tile_segments(RowSeg* seg_s, const int32_t* __restrict__ seg, int n_seg, int Np, int i0,
+__device__ __forceinline__ RowSeg tile_segments(RowSeg* seg_s, const int32_t* seg, int n_seg, int Np, int i0,
                                                 int tid) {
   if (tid < kR) seg_s[tid] = row_segment(seg, n_seg, Np, i0 + tid);
   __syncthreads();
@@ -141,7 +141,7 @@ template <int D> constexpr int kFwdFloats = (kR + 4 * kT) * kLd<D> + kR * kLdP; 
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads)
-attn_fwd_simt_kernel(const T* __restrict__ qkv, const int32_t* __restrict__ seg, int n_seg, int capacity, int C,
+attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ ao, float* __restrict__ lse) {
   pdl_entry();
   constexpr int W = D / kTX;
@@ -241,8 +241,8 @@ template <int D> constexpr int kBwdFloats = (2 * kR + 4 * kT) * kLd<D> + 2 * kR 
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads)
-attn_bwd_simt_kernel(const T* __restrict__ qkv, const T* __restrict__ ao, const float* __restrict__ lse,
-                     const T* __restrict__ dao, const int32_t* __restrict__ seg, int n_seg, int capacity, int C,
+attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
+                     const T* dao, const int32_t* seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ dqkv) {
   pdl_entry();
   constexpr int W = D / kTX, E = Vec16<T>::kElems;

@@ -225,7 +225,7 @@ template <int D> struct FwdSmem {
 // 128 segments of 98 to 196 rows, 12 heads of 64: 54 -> 51; one segment of 98 rows: 6.0 us, as before.
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 2)
-attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* __restrict__ seg, int n_seg, int capacity,
+attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* seg, int n_seg, int capacity,
                    int C, int H, float scale_log2e, __nv_bfloat16* __restrict__ ao, float* __restrict__ lse,
                    unsigned* counter, bool even_items, int32_t* d_status) {
   using HT = HeadTile<D>;
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2)
 attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_constant__ CUtensorMap tm_do,
                    const __grid_constant__ CUtensorMap tm_qkv_y, const __grid_constant__ CUtensorMap tm_do_y,
                    const __grid_constant__ CUtensorMap tm_o,
-                   const float* __restrict__ lse, float* __restrict__ delta, const int32_t* __restrict__ seg, int n_seg,
+                   const float* lse, float* delta, const int32_t* seg, int n_seg,
                    int capacity, int C, int H, float scale, __nv_bfloat16* __restrict__ dqkv, int skip_short, int32_t* d_status) {
   using HT = HeadTile<D>;
   constexpr int kTile = HT::kTileBytes;             // own tiles: 128 rows
@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2)
 attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_constant__ CUtensorMap tm_do,
                    const __grid_constant__ CUtensorMap tm_qkv_y, const __grid_constant__ CUtensorMap tm_do_y,
                    const __grid_constant__ CUtensorMap tm_o,
-                   const float* __restrict__ lse, float* __restrict__ delta, const int32_t* __restrict__ seg, int n_seg,
+                   const float* lse, float* delta, const int32_t* seg, int n_seg,
                    int capacity, int C, int H, float scale, __nv_bfloat16* __restrict__ dqkv, int skip_short, int32_t* d_status) {
   using HT = HeadTile<D>;
   constexpr int kTile = HT::kTileBytes;             // own tiles: 128 rows
@@ -1619,8 +1619,8 @@ template <int D> __host__ __device__ constexpr int short_smem_bytes() {
 template <int D>
 __global__ void __launch_bounds__(kShortThreads, 2)
 attn_bwd_short_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_constant__ CUtensorMap tm_do,
-                      const __grid_constant__ CUtensorMap tm_o, const float* __restrict__ lse,
-                      const int32_t* __restrict__ seg, int n_seg, int capacity, int C, float scale,
+                      const __grid_constant__ CUtensorMap tm_o, const float* lse,
+                      const int32_t* seg, int n_seg, int capacity, int C, float scale,
                       __nv_bfloat16* __restrict__ dqkv, int32_t* d_status) {
   using HT = HeadTile<D>;
   constexpr int kTile = HT::kTileBytes;

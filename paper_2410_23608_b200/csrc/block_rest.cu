@@ -16,9 +16,9 @@ constexpr int kLnChunks = 4;  // 16-byte chunks of a row per lane: C <= 128 chun
 // adds to): one pass over x instead of three kernels that read x or its normalisation again.
 template <typename T, bool kGate>
 __global__ void __launch_bounds__(kRestThreads)
-layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, const T* __restrict__ beta, float eps,
+layer_norm_kernel(const uint4* x16, const T* gamma, const T* beta, float eps,
                   int rows, int C, uint4* __restrict__ y16, float* __restrict__ mean, float* __restrict__ rstd,
-                  const T* __restrict__ w_g, float b_g, float tau, float* __restrict__ scores, uint8_t* __restrict__ mask,
+                  const T* w_g, float b_g, float tau, float* __restrict__ scores, uint8_t* __restrict__ mask,
                   uint4* __restrict__ copy16) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
@@ -34,7 +34,7 @@ layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, co
     for (int k = 0; k < kLnChunks; ++k) {
       const int q = lane + 32 * k;
       if (q < Q) {
-        const uint4 raw = ld_nc16(x16 + (long long)t * Q + q);
+        const uint4 raw = ld_stream16(x16 + (long long)t * Q + q);
         if (kGate) copy16[(long long)t * Q + q] = raw;
         Vec16<T>::to_float(raw, v[k]);
 #pragma unroll
@@ -57,15 +57,15 @@ layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, co
       const int q = lane + 32 * k;
       if (q < Q) {
         float o[E], g[E], b[E];
-        Vec16<T>::to_float(__ldg(g16 + q), g);
-        Vec16<T>::to_float(__ldg(b16 + q), b);
+        Vec16<T>::to_float(g16[q], g);
+        Vec16<T>::to_float(b16[q], b);
 #pragma unroll
         for (int e = 0; e < E; ++e) o[e] = (v[k][e] - mu) * rs * g[e] + b[e];
         const uint4 out = Vec16<T>::from_float(o);
         y16[(long long)t * Q + q] = out;
         if (kGate) {
           Vec16<T>::to_float(out, o);
-          Vec16<T>::to_float(__ldg(w16 + q), g);
+          Vec16<T>::to_float(w16[q], g);
 #pragma unroll
           for (int e = 0; e < E; ++e) dot = fmaf(o[e], g[e], dot);
         }
@@ -90,10 +90,10 @@ layer_norm_kernel(const uint4* __restrict__ x16, const T* __restrict__ gamma, co
 // CTA's sums met bank conflicts of eight, the reduction read a sector for every value).
 template <typename T, int kCh>
 __global__ void __launch_bounds__(kRestThreads, kCh <= 3 ? 2 : 1)
-layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ x16, const T* __restrict__ gamma,
-                      const float* __restrict__ mean, const float* __restrict__ rstd, const uint4* add16, int rows,
-                      int C, uint4* dx16, float* __restrict__ part, const int32_t* __restrict__ dy_row,
-                      const int32_t* __restrict__ dz_row, uint4* __restrict__ dz16) {
+layer_norm_bwd_kernel(const uint4* dy16, const uint4* x16, const T* gamma,
+                      const float* mean, const float* rstd, const uint4* add16, int rows,
+                      int C, uint4* dx16, float* __restrict__ part, const int32_t* dy_row,
+                      const int32_t* dz_row, uint4* __restrict__ dz16) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
   extern __shared__ __align__(16) float acc_s[];  // [8 warps][2C]
@@ -112,14 +112,14 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
 #pragma unroll
     for (int k = 0; k < kCh; ++k) {
       const int q = lane + 32 * k;
-      xr[k] = q < Q ? ld_nc16(x16 + (long long)t * Q + q) : zero;
+      xr[k] = q < Q ? ld_stream16(x16 + (long long)t * Q + q) : zero;
       ar[k] = q < Q && add16 != nullptr ? add16[(long long)t * Q + q] : zero;
     }
     const float mu = mean[t], rs = rstd[t];
 #pragma unroll
     for (int k = 0; k < kCh; ++k) {
       const int q = lane + 32 * k;
-      dr[k] = q < Q && src >= 0 ? ld_nc16(dy16 + (long long)src * Q + q) : zero;
+      dr[k] = q < Q && src >= 0 ? ld_stream16(dy16 + (long long)src * Q + q) : zero;
     }
     if (src < 0) {  // no gradient into this row: what the residual branch brings, or nothing
 #pragma unroll
@@ -140,7 +140,7 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
         float dy[E], xv[E], gm[E];
         Vec16<T>::to_float(dr[k], dy);
         Vec16<T>::to_float(xr[k], xv);
-        Vec16<T>::to_float(__ldg(reinterpret_cast<const uint4*>(gamma) + q), gm);
+        Vec16<T>::to_float(reinterpret_cast<const uint4*>(gamma)[q], gm);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const float xh = (xv[e] - mu) * rs, g = dy[e] * gm[e];
@@ -160,7 +160,7 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
         Vec16<T>::to_float(dr[k], dy);
         Vec16<T>::to_float(xr[k], xv);
         Vec16<T>::to_float(ar[k], a);
-        Vec16<T>::to_float(__ldg(reinterpret_cast<const uint4*>(gamma) + q), gm);
+        Vec16<T>::to_float(reinterpret_cast<const uint4*>(gamma)[q], gm);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const float xh = (xv[e] - mu) * rs, g = dy[e] * gm[e];
@@ -196,12 +196,12 @@ layer_norm_bwd_kernel(const uint4* __restrict__ dy16, const uint4* __restrict__ 
 // out = gelu(u) (kBwd = false) or out = dh * gelu'(u) (kBwd = true), over `total` 16-byte chunks
 template <typename T, bool kBwd>
 __global__ void __launch_bounds__(kRestThreads)
-gelu_kernel(const uint4* __restrict__ u16, const uint4* dh16, long long total, uint4* out16) {
+gelu_kernel(const uint4* u16, const uint4* dh16, long long total, uint4* out16) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
   for (long long k = (long long)blockIdx.x * kRestThreads + threadIdx.x; k < total; k += (long long)gridDim.x * kRestThreads) {
     float u[E], o[E];
-    Vec16<T>::to_float(ld_nc16(u16 + k), u);
+    Vec16<T>::to_float(ld_stream16(u16 + k), u);
     if (kBwd) {
       float d[E];
       Vec16<T>::to_float(dh16[k], d);

@@ -14,7 +14,7 @@ constexpr int kGateRows = 2;  // rows per warp per iteration
 
 template <typename T>
 __global__ void __launch_bounds__(kGateThreads)
-gate_kernel(const T* __restrict__ x, const T* __restrict__ w_g, float b_g, const float* __restrict__ s_up,
+gate_kernel(const T* x, const T* w_g, float b_g, const float* s_up,
             float tau, int rows, int C, float* __restrict__ scores, uint8_t* __restrict__ mask, uint4* __restrict__ y16) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
@@ -37,7 +37,7 @@ gate_kernel(const T* __restrict__ x, const T* __restrict__ w_g, float b_g, const
       uint4 v[kGateRows];
 #pragma unroll
       for (int k = 0; k < kGateRows; ++k)
-        if (r0 + k < rows) v[k] = ld_nc16(x16 + (size_t)(r0 + k) * Q + q);
+        if (r0 + k < rows) v[k] = ld_stream16(x16 + (size_t)(r0 + k) * Q + q);
       if (y16 != nullptr) {  // pass-through copy y = x rides on the one read of x
 #pragma unroll
         for (int k = 0; k < kGateRows; ++k)

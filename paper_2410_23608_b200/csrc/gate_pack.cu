@@ -46,7 +46,7 @@ __device__ __forceinline__ uint4 scaled16(uint4 v, float s) {
 // kChunks: 16-byte chunks of a row held by one lane (row = up to 32 * kChunks chunks); kRows: rows per warp.
 template <typename T, int kChunks, int kRows, bool kGateScale>
 __global__ void __launch_bounds__(kGpThreads)
-gate_pack_kernel(const uint4* __restrict__ x16, const T* __restrict__ w_g, float b_g, const float* __restrict__ s_up,
+gate_pack_kernel(const uint4* x16, const T* w_g, float b_g, const float* s_up,
                  float tau, int rows, int N, int B, int Q, int capacity, float* __restrict__ scores,
                  uint8_t* __restrict__ mask, uint4* __restrict__ y16, uint4* __restrict__ xp16,
                  int32_t* __restrict__ idx, int32_t* __restrict__ inv, int32_t* __restrict__ cu, uint32_t* state,
@@ -69,7 +69,7 @@ gate_pack_kernel(const uint4* __restrict__ x16, const T* __restrict__ w_g, float
     for (int c = 0; c < kChunks; ++c) {
       const int q = lane + 32 * c;
       v[k][c] = make_uint4(0u, 0u, 0u, 0u);
-      if (row0 + k < rows && q < Q) v[k][c] = ld_nc16(x16 + (size_t)(row0 + k) * Q + q);
+      if (row0 + k < rows && q < Q) v[k][c] = ld_stream16(x16 + (size_t)(row0 + k) * Q + q);
     }
   }
   if (y16 != nullptr) {
@@ -112,7 +112,7 @@ gate_pack_kernel(const uint4* __restrict__ x16, const T* __restrict__ w_g, float
     float s = warp_sum(acc[k]) + b_g;
     const int r = row0 + k;
     if (r < rows) {
-      if (s_up != nullptr) s = fmaxf(s, __ldg(s_up + r));
+      if (s_up != nullptr) s = fmaxf(s, s_up[r]);
       if (s > tau) sel_bits |= 1u << k;
       if (lane == 0) {
         scores[r] = s;

@@ -69,7 +69,7 @@ template <int R, bool kMn> struct Operand {
     if (!kMn) { row = line; k = chunk * 8; off = line * 128 + ((chunk ^ (line & 7)) << 4); }
     else { const int kl = line & 63, box = line >> 6; row = box * 64 + chunk * 8; k = kl; off = box * 8192 + kl * 128 + ((chunk ^ (kl & 7)) << 4); }
   }
-  __device__ static __forceinline__ void load(Tile8* t, const float* __restrict__ src, long long ld, int r0, int rows, int k0,
+  __device__ static __forceinline__ void load(Tile8* t, const float* src, long long ld, int r0, int rows, int k0,
                                               int k_end, int tid) {
 #pragma unroll
     for (int i = 0; i < kUnits; ++i) {
@@ -130,10 +130,10 @@ __device__ __noinline__ float4 fma_chain(const float* A, long long lda, const fl
 // colsum (optional, wgrad): colsum[m] = sum_k A(m,k), by the CTAs of the first column of tiles from the lines they load.
 template <int BN, bool kAMn, bool kBMn>
 __global__ void __launch_bounds__(kThreads, 1)
-gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restrict__ Bm, long long ldb,
-                const float* __restrict__ bias, float* out, long long ldo, int M, int N, int K,
-                const int32_t* __restrict__ cu, int n_seg, int capacity, int dyn_which, const float* add, const float* u, float* h,
-                const int32_t* __restrict__ row_map, float* __restrict__ colsum, int32_t* d_status) {
+gemm_f32_kernel(const float* A, long long lda, const float* Bm, long long ldb,
+                const float* bias, float* out, long long ldo, int M, int N, int K,
+                const int32_t* cu, int n_seg, int capacity, int dyn_which, const float* add, const float* u, float* h,
+                const int32_t* row_map, float* __restrict__ colsum, int32_t* d_status) {
   using OpA = Operand<BM, kAMn>;
   using OpB = Operand<BN, kBMn>;
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(BM, BN, kAMn, kBMn);
@@ -299,7 +299,7 @@ gemm_f32_kernel(const float* __restrict__ A, long long lda, const float* __restr
       float4 v = split > 1 ? sum_dsmem4(src, split) : *reinterpret_cast<const float4*>(src);
       if (!(fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(v.w) < CUDART_INF_F)) v = fma_chain<kAMn, kBMn>(A, lda, Bm, ldb, m0 + r, n0 + c, K);
       if (bias != nullptr) {
-        const float4 w = __ldg(reinterpret_cast<const float4*>(bias + n0 + c));
+        const float4 w = ld_values(bias + n0 + c);
         v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
       }
       const int m = m0 + r;

@@ -14,10 +14,10 @@ constexpr int kThreads = 256;
 // dyn_which: 0 = sizes as given, 1 = M is the device-side packed row count, 2 = K is.
 template <typename T, typename TO>
 __global__ void __launch_bounds__(kThreads)
-gemm_simt_kernel(const T* __restrict__ A, long long sAm, long long sAk, const T* __restrict__ Bm, long long sBn,
-                 long long sBk, const T* __restrict__ bias, TO* __restrict__ out, long long ldo, int M, int N, int K,
-                 const int32_t* __restrict__ cu, int n_seg, int capacity, int dyn_which, int accumulate,
-                 const int32_t* __restrict__ row_map) {
+gemm_simt_kernel(const T* A, long long sAm, long long sAk, const T* Bm, long long sBn,
+                 long long sBk, const T* bias, TO* out, long long ldo, int M, int N, int K,
+                 const int32_t* cu, int n_seg, int capacity, int dyn_which, int accumulate,
+                 const int32_t* row_map) {
   pdl_entry();
   if (dyn_which != 0) {
     const int rows = packed_rows(cu, n_seg, capacity);
@@ -81,7 +81,7 @@ gemm_simt_kernel(const T* __restrict__ A, long long sAm, long long sAk, const T*
 // db[j] = sum over packed rows of dout[i][j], rows added in a fixed order.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-colsum_kernel(const T* __restrict__ dout, int n_out, const int32_t* __restrict__ cu, int n_seg, int capacity,
+colsum_kernel(const T* dout, int n_out, const int32_t* cu, int n_seg, int capacity,
               float* __restrict__ db) {
   pdl_entry();
   const int rows = packed_rows(cu, n_seg, capacity);

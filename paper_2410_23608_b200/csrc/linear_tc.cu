@@ -94,9 +94,9 @@ struct TileCoord { int m0, n0, z, n_t; };
 template <int BN, bool kDyn, bool kAMn, bool kBMn, typename OutT, int kKind>
 __global__ void __launch_bounds__(kGemmThreads)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __nv_bfloat16* __restrict__ bias, OutT* __restrict__ out, long long ldo,
-               long long split_stride, int M, int N, int K, const int32_t* __restrict__ cu, int n_seg, int capacity,
-               int dyn_which, int k_per_split, int k_interleave, const int32_t* __restrict__ row_map,
+               const __nv_bfloat16* bias, OutT* __restrict__ out, long long ldo,
+               long long split_stride, int M, int N, int K, const int32_t* cu, int n_seg, int capacity,
+               int dyn_which, int k_per_split, int k_interleave, const int32_t* row_map,
                RowEpilogue<kKind> epi, uint32_t wait_limit, int32_t* d_status) {
   constexpr int kStage = stage_bytes<BN>();
   pdl_launch_dependents();
@@ -360,7 +360,7 @@ constexpr int kColsumChunks = 64;  // row chunks over the allocated rows (rows p
 inline int colsum_rows_per_chunk(int capacity) { return (((capacity + kColsumChunks - 1) / kColsumChunks) + 7) & ~7; }
 
 __global__ void __launch_bounds__(256)
-colsum_partial_kernel(const __nv_bfloat16* __restrict__ dout, int n_out, const int32_t* __restrict__ cu, int n_seg,
+colsum_partial_kernel(const __nv_bfloat16* dout, int n_out, const int32_t* cu, int n_seg,
                       int capacity, int rows_per_chunk, float* __restrict__ part) {
   pdl_entry();
   const int rows = packed_rows(cu, n_seg, capacity);
@@ -377,7 +377,7 @@ colsum_partial_kernel(const __nv_bfloat16* __restrict__ dout, int n_out, const i
       uint4 v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (i0 + 32 * u < r_end) v[u] = ld_nc16(dout + (long long)(i0 + 32 * u) * n_out + col);
+        if (i0 + 32 * u < r_end) v[u] = ld_stream16(dout + (long long)(i0 + 32 * u) * n_out + col);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (i0 + 32 * u < r_end) {
@@ -408,9 +408,14 @@ colsum_partial_kernel(const __nv_bfloat16* __restrict__ dout, int n_out, const i
 // optionally, the bias-gradient partials, one per row chunk or (rows_per_chunk2 = 0) tiles_n2 per split - up to hundreds
 // of them for a few thousand outputs, so there a warp owns four outputs: lane l adds chunks l, l + 32, ... in order and a fixed shuffle
 // tree adds the lanes.  The first ceil(n2 / 32) blocks take the second array.
+__device__ __forceinline__ float4 ld_part(const float* part, long long j) {
+  const uint4 v = ld_stream16(reinterpret_cast<const float4*>(part) + j);
+  return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+
 __global__ void __launch_bounds__(256)
-split_reduce_kernel(const float* __restrict__ part, long long n, const float* __restrict__ part2, long long n2,
-                    int splits, int rows_per_chunk2, int tiles_n2, const int32_t* __restrict__ cu, int n_seg, int capacity,
+split_reduce_kernel(const float* part, long long n, const float* part2, long long n2,
+                    int splits, int rows_per_chunk2, int tiles_n2, const int32_t* cu, int n_seg, int capacity,
                     float* __restrict__ out, float* __restrict__ out2) {
   pdl_entry();
   const int rows = packed_rows(cu, n_seg, capacity);
@@ -425,7 +430,7 @@ split_reduce_kernel(const float* __restrict__ part, long long n, const float* __
     const int lane = threadIdx.x & 31;
     float4 s4 = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int z = lane; z < valid2; z += 32) {
-      const float4 v = __ldcs(reinterpret_cast<const float4*>(part2 + (long long)z * n2) + j);
+      const float4 v = ld_part(part2 + (long long)z * n2, j);
       s4.x += v.x; s4.y += v.y; s4.z += v.z; s4.w += v.w;
     }
 #pragma unroll
@@ -443,7 +448,7 @@ split_reduce_kernel(const float* __restrict__ part, long long n, const float* __
     float4 s4 = make_float4(0.f, 0.f, 0.f, 0.f);
     // four splits' loads in flight at a time; the additions stay in split order
     auto add = [&](const float4& v) { s4.x += v.x; s4.y += v.y; s4.z += v.z; s4.w += v.w; };
-    auto at = [&](int z) { return __ldcs(reinterpret_cast<const float4*>(part + (long long)z * n) + j); };
+    auto at = [&](int z) { return ld_part(part + (long long)z * n, j); };
     int z = 0;
     for (; z + 4 <= valid1; z += 4) {
       const float4 v0 = at(z), v1 = at(z + 1), v2 = at(z + 2), v3 = at(z + 3);

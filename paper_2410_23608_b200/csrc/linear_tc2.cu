@@ -144,8 +144,8 @@ __device__ __forceinline__ void leave_pair(uint32_t rank, uint32_t abort_s, uint
 template <bool kBMn, int kKind>
 __global__ void __launch_bounds__(kPairThreads)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const __nv_bfloat16* __restrict__ bias, __nv_bfloat16* __restrict__ out, long long ldo, int N, int K,
-                 const int32_t* __restrict__ cu, int n_seg, int capacity, const int32_t* __restrict__ row_map,
+                 const __nv_bfloat16* bias, __nv_bfloat16* __restrict__ out, long long ldo, int N, int K,
+                 const int32_t* cu, int n_seg, int capacity, const int32_t* row_map,
                  RowEpilogue<kKind> epi, uint32_t wait_limit, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(2 * PM, PN, false, kBMn);
   pdl_launch_dependents();
@@ -340,7 +340,7 @@ constexpr int kWgSmem = kPairSmem + 1024;  // and the 8 x 64 block of ones
 
 __global__ void __launch_bounds__(kPairThreads)
 wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ part,
-                  float* __restrict__ part_b, int M, int N, int splits, const int32_t* __restrict__ cu, int n_seg,
+                  float* __restrict__ part_b, int M, int N, int splits, const int32_t* cu, int n_seg,
                   int capacity, uint32_t wait_limit, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(2 * PM, PN, true, true);
   constexpr uint32_t kIdescOnes = ptx::idesc_bf16_f32(2 * PM, 16, true, false);

@@ -27,7 +27,7 @@ static_assert(kT * kLd * 4 <= 3 * 2 * kOp, "the finished tile takes the stages' 
 template <int kStages>
 __global__ void __launch_bounds__(kThreads, kStages == 3 ? 2 : 1)
 wgrad_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ dW,
-                     float* __restrict__ db, int M, int N, const int32_t* __restrict__ cu, int n_seg, int capacity,
+                     float* __restrict__ db, int M, int N, const int32_t* cu, int n_seg, int capacity,
                      uint32_t wait_limit, int32_t* d_status) {
   constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(kT, kT, true, true);
   constexpr uint32_t kIdescOnes = ptx::idesc_bf16_f32(kT, 16, true, false);

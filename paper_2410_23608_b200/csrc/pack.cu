@@ -45,8 +45,8 @@ __device__ __forceinline__ uint4 add16(uint4 a, uint4 b) {
 // token b*N + order[j]; mask, scores, idx and inv stay indexed by the original token.
 template <typename T, bool kGateScale, bool kOrdered>
 __global__ void __launch_bounds__(kPackThreads)
-select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ mask, const float* __restrict__ scores,
-                   const int32_t* __restrict__ order, int rows, int N, int B, int Q, int tile, int capacity,
+select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
+                   const int32_t* order, int rows, int N, int B, int Q, int tile, int capacity,
                    uint4* __restrict__ xp16,
                    int32_t* __restrict__ idx, int32_t* __restrict__ inv, int32_t* __restrict__ cu,
                    int32_t* d_status) {
@@ -69,7 +69,7 @@ select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ ma
     const int img0 = (tile_start / N) * N;
     for (int k = tid; k < (img0 >> 4); k += kPackThreads) cnt += count_nonzero_bytes(ld_dep16(mask16 + k));
     for (int k = (img0 & ~15) + tid; k < img0; k += kPackThreads) cnt += ld_dep(mask + k) != 0;
-    for (int j = tid; j < tile_start - img0; j += kPackThreads) cnt += ld_dep(mask + img0 + __ldg(order + j)) != 0;
+    for (int j = tid; j < tile_start - img0; j += kPackThreads) cnt += ld_dep(mask + img0 + ld_dep(order + j)) != 0;
   }
   cnt = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
   if (lane == 0) warp_cnt[wid] = cnt;
@@ -78,7 +78,7 @@ select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ ma
   const int t = tile_start + tid;
   const bool in_tile = tid < tile && t < rows;
   int tok = t;  // the token that position t of the visiting order stands for
-  if (kOrdered && in_tile) tok = (t / N) * N + __ldg(order + t % N);
+  if (kOrdered && in_tile) tok = (t / N) * N + ld_dep(order + t % N);
   const bool sel = in_tile && ld_dep(mask + tok) != 0;
   const unsigned ballot = __ballot_sync(0xffffffffu, sel);
   if (lane == 0) warp_sel[wid] = __popc(ballot);
@@ -121,7 +121,7 @@ select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ ma
       if (k < total) {
         r[u] = k / Q;
         q[u] = k - r[u] * Q;
-        v[u] = ld_nc16(x16 + (size_t)sel_tok[r[u]] * Q + q[u]);
+        v[u] = ld_stream16(x16 + (size_t)sel_tok[r[u]] * Q + q[u]);
       }
     }
 #pragma unroll
@@ -139,8 +139,8 @@ select_pack_kernel(const uint4* __restrict__ x16, const uint8_t* __restrict__ ma
 // Out of place: every row of y is written, from z (selected) or x (pass-through).
 template <typename T, bool kResidual>
 __global__ void __launch_bounds__(kPackThreads)
-unpack_scatter_kernel(const uint4* __restrict__ z16, const uint4* __restrict__ x16, const int32_t* __restrict__ inv,
-                      const int32_t* __restrict__ cu, int B, int capacity, long long total, int Q,
+unpack_scatter_kernel(const uint4* z16, const uint4* x16, const int32_t* inv,
+                      const int32_t* cu, int B, int capacity, long long total, int Q,
                       uint4* __restrict__ y16) {
   pdl_entry();
   const int Np = packed_rows(cu, B, capacity);
@@ -155,10 +155,10 @@ unpack_scatter_kernel(const uint4* __restrict__ z16, const uint4* __restrict__ x
         const int q = (int)(k - t * Q);
         const int i = ld_dep(inv + t);
         if (i >= 0 && i < Np) {
-          v[u] = ld_nc16(z16 + (size_t)i * Q + q);
-          if (kResidual) v[u] = add16<T>(v[u], ld_nc16(x16 + k));
+          v[u] = ld_stream16(z16 + (size_t)i * Q + q);
+          if (kResidual) v[u] = add16<T>(v[u], ld_stream16(x16 + k));
         } else {
-          v[u] = ld_nc16(x16 + k);
+          v[u] = ld_stream16(x16 + k);
         }
       }
     }
@@ -175,8 +175,8 @@ unpack_scatter_kernel(const uint4* __restrict__ z16, const uint4* __restrict__ x
 // (dst = dX, add = dY under the residual flag).  `add` may alias `dst`.
 template <typename T, bool kAdd>
 __global__ void __launch_bounds__(kPackThreads)
-row_scatter_kernel(const uint4* __restrict__ src16, const uint4* addp, const int32_t* __restrict__ idx,
-                   const int32_t* __restrict__ cu, int B, int capacity, int Q, uint4* dst16) {
+row_scatter_kernel(const uint4* src16, const uint4* addp, const int32_t* idx,
+                   const int32_t* cu, int B, int capacity, int Q, uint4* dst16) {
   pdl_entry();
   const long long total = (long long)packed_rows(cu, B, capacity) * Q;
   const long long stride = (long long)gridDim.x * kPackThreads;
@@ -190,7 +190,7 @@ row_scatter_kernel(const uint4* __restrict__ src16, const uint4* addp, const int
         const long long i = k / Q;
         const int q = (int)(k - i * Q);
         o[u] = (size_t)ld_dep(idx + i) * Q + q;
-        v[u] = ld_nc16(src16 + k);
+        v[u] = ld_stream16(src16 + k);
         if (kAdd) v[u] = add16<T>(v[u], addp[o[u]]);
       }
     }
@@ -204,8 +204,8 @@ row_scatter_kernel(const uint4* __restrict__ src16, const uint4* addp, const int
 
 // Transpose of the unpack: one pass over dY; selected rows go to dz, the others to dX.
 __global__ void __launch_bounds__(kPackThreads)
-unpack_scatter_bwd_kernel(const uint4* __restrict__ dY16, const int32_t* __restrict__ inv,
-                          const int32_t* __restrict__ cu, int B, int capacity, long long total, int Q,
+unpack_scatter_bwd_kernel(const uint4* dY16, const int32_t* inv,
+                          const int32_t* cu, int B, int capacity, long long total, int Q,
                           uint4* __restrict__ dz16, uint4* dX16, bool copy_pass_through, bool copy_selected) {
   pdl_entry();
   const int Np = packed_rows(cu, B, capacity);
@@ -223,7 +223,7 @@ unpack_scatter_bwd_kernel(const uint4* __restrict__ dY16, const int32_t* __restr
         const int i = ld_dep(inv + t);
         if (i >= 0 && i < Np) o[u] = (long long)i * Q + q;
         else if (copy_pass_through) o[u] = -1;
-        if (o[u] != -2) v[u] = ld_nc16(dY16 + k);
+        if (o[u] != -2) v[u] = ld_stream16(dY16 + k);
       }
     }
 #pragma unroll
@@ -249,14 +249,14 @@ int stream_grid(long long total_chunks) {
 // dst = src over `total` 16-byte chunks: the pass-through rows of the unpack step written ahead of
 // time, so that the projection (or the input-gradient product) only has to scatter the selected rows.
 __global__ void __launch_bounds__(kPackThreads)
-copy_chunks_kernel(const uint4* __restrict__ src16, uint4* __restrict__ dst16, long long total) {
+copy_chunks_kernel(const uint4* src16, uint4* __restrict__ dst16, long long total) {
   pdl_entry();
   const long long stride = (long long)gridDim.x * kPackThreads;
   for (long long k0 = (long long)blockIdx.x * kPackThreads + threadIdx.x; k0 < total; k0 += stride * kBatch) {
     uint4 v[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
-      if (k0 + u * stride < total) v[u] = ld_nc16(src16 + k0 + u * stride);
+      if (k0 + u * stride < total) v[u] = ld_stream16(src16 + k0 + u * stride);
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
       if (k0 + u * stride < total) dst16[k0 + u * stride] = v[u];
@@ -278,7 +278,7 @@ constexpr int kCutThreads = 1024;
 constexpr int kCutMaxOffsets = 4096;  // B + 1 offsets and their prefix counts are held in shared memory
 
 __global__ void __launch_bounds__(kCutThreads)
-container_offsets_kernel(const int32_t* __restrict__ cu, int B, int L, int n_max, int32_t* __restrict__ out) {
+container_offsets_kernel(const int32_t* cu, int B, int L, int n_max, int32_t* __restrict__ out) {
   pdl_entry();
   __shared__ int32_t cu_s[kCutMaxOffsets];
   __shared__ int32_t pre_s[kCutMaxOffsets + 1];  // pre_s[b] = distinct non-multiple offsets among cu[0..b)

@@ -17,7 +17,7 @@ __device__ __forceinline__ float sigmoid_f(float s) { return 1.f / (1.f + __expf
 __device__ __forceinline__ float softplus_f(float s) { return fmaxf(s, 0.f) + log1pf(__expf(-fabsf(s))); }
 
 __global__ void __launch_bounds__(kTrainThreads)
-score_pool_kernel(const float* __restrict__ prev, int B, int rows, int cols, float* __restrict__ s_up) {
+score_pool_kernel(const float* prev, int B, int rows, int cols, float* __restrict__ s_up) {
   pdl_entry();
   const long long total = (long long)B * rows * cols;
   for (long long t = (long long)blockIdx.x * kTrainThreads + threadIdx.x; t < total;
@@ -34,7 +34,7 @@ score_pool_kernel(const float* __restrict__ prev, int B, int rows, int cols, flo
 // ds[t] = alpha (Sigmoid(s_t) - y_t); part[blockIdx] = this CTA's share of the loss (tokens in a fixed
 // grid-stride order, tree reduction of fixed shape).  labels == nullptr: ds = 0, loss = 0.
 __global__ void __launch_bounds__(kTrainThreads)
-select_loss_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ labels, float alpha, long long total,
+select_loss_kernel(const float* scores, const uint8_t* labels, float alpha, long long total,
                    float* __restrict__ ds, float* __restrict__ part) {
   pdl_entry();
   float acc = 0.f;
@@ -67,7 +67,7 @@ select_loss_kernel(const float* __restrict__ scores, const uint8_t* __restrict__
 constexpr int kSumThreads = 1024;
 template <bool kWide>
 __global__ void __launch_bounds__(kWide ? kSumThreads : kTrainThreads)
-partial_sum_kernel(const float* __restrict__ part, int n_blocks, int stride, int n_out, float* __restrict__ out, int n_out2,
+partial_sum_kernel(const float* part, int n_blocks, int stride, int n_out, float* __restrict__ out, int n_out2,
                    float* __restrict__ out2) {
   pdl_entry();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -99,9 +99,9 @@ partial_sum_kernel(const float* __restrict__ part, int n_blocks, int stride, int
 // ds_t += Sigmoid'(s_t) (dxp_i . x_t).
 template <typename T, bool kResidual>
 __global__ void __launch_bounds__(kTrainThreads)
-pack_bwd_gated_kernel(const uint4* __restrict__ dxp16, const uint4* __restrict__ x16, const float* __restrict__ scores,
-                      const uint4* dY16, const int32_t* __restrict__ idx, const int32_t* __restrict__ cu, int B,
-                      int capacity, int Q, uint4* dX16, float* __restrict__ ds) {
+pack_bwd_gated_kernel(const uint4* dxp16, const uint4* x16, const float* scores,
+                      const uint4* dY16, const int32_t* idx, const int32_t* cu, int B,
+                      int capacity, int Q, uint4* dX16, float* ds) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
   const int Np = packed_rows(cu, B, capacity);
@@ -112,8 +112,8 @@ pack_bwd_gated_kernel(const uint4* __restrict__ dxp16, const uint4* __restrict__
     const float p = sigmoid_f(scores[t]);
     float dot = 0.f;
     for (int q = lane; q < Q; q += 32) {
-      const uint4 g = ld_nc16(dxp16 + (long long)i * Q + q);
-      const uint4 xv = ld_nc16(x16 + t * Q + q);
+      const uint4 g = ld_stream16(dxp16 + (long long)i * Q + q);
+      const uint4 xv = ld_stream16(x16 + t * Q + q);
       float fg[E], fx[E];
       Vec16<T>::to_float(g, fg);
       Vec16<T>::to_float(xv, fx);
@@ -144,8 +144,8 @@ constexpr int kGbChunks = 4;   // 16-byte chunks of a row per lane: C <= 128 chu
 
 template <typename T>
 __global__ void __launch_bounds__(kTrainThreads)
-gate_bwd_kernel(const uint4* __restrict__ x16, const T* __restrict__ w_g, const float* __restrict__ scores,
-                const float* __restrict__ s_up, const float* __restrict__ ds, int rows, int C, uint4* dX16,
+gate_bwd_kernel(const uint4* x16, const T* w_g, const float* scores,
+                const float* s_up, const float* ds, int rows, int C, uint4* dX16,
                 float* __restrict__ ds_up, float* __restrict__ part) {
   pdl_entry();
   constexpr int E = Vec16<T>::kElems;
@@ -185,7 +185,7 @@ gate_bwd_kernel(const uint4* __restrict__ x16, const T* __restrict__ w_g, const 
 #pragma unroll
       for (int r = 0; r < kGbRows; ++r)
         if (d[r] != 0.f) {  // warp-uniform
-          xv[r] = ld_nc16(x16 + (long long)(t0 + r) * Q + q);
+          xv[r] = ld_stream16(x16 + (long long)(t0 + r) * Q + q);
           gv[r] = dX16[(long long)(t0 + r) * Q + q];
         }
 #pragma unroll
