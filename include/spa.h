@@ -297,7 +297,9 @@ int spa_gate_bwd(const spa_params* p, const void* x, const void* w_g, const floa
 
 /* ---- The rest of the pre-norm transformer block around SPA (Sec. 3.2: selected tokens go through attention,
  * the others straight to the feed-forward network).  The paper prints no formula for these standard parts;
- * they are: LayerNorm over the channels, linear layers over all tokens, the exact (erf) GELU. --------------- */
+ * they are: LayerNorm over the channels, linear layers over all tokens, the GELU by the normal distribution function
+ * (not its tanh form).  spa_gelu and spa_gelu_bwd take erff; the bf16 products of the transformer block, which apply it on
+ * their way out, a formula with an error of 3e-7 (the results of both are within a bf16 rounding, less in the far tail). */
 
 /* out[i][:] = b + W a[i][:] for the rows that cu_seqlens[B] counts (W: T[n_out][n_in], b: T[n_out] or NULL,
  * a: T[capacity][n_in], out: T[capacity][n_out]).  accumulate != 0 adds the result to what out holds (a residual

@@ -1,5 +1,5 @@
 // The rest of the pre-norm transformer block around SPA (Sec. 3.2: selected tokens go through attention, the
-// others straight to the feed-forward network): LayerNorm over the channels and the exact GELU, forward and
+// others straight to the feed-forward network): LayerNorm over the channels and the GELU (by erff), forward and
 // backward.  The two feed-forward products are the library's linear layers run over all B*N tokens.
 // Row-wise streaming kernels: one warp per token row, 16-byte accesses, fp32 arithmetic; the per-channel sums
 // of the LayerNorm backward are taken per CTA in a fixed order and combined by the shared reduction kernel.

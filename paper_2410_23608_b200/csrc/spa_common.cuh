@@ -120,8 +120,11 @@ __device__ __forceinline__ float gelu_grad_f(float u) {
 }
 
 // Standard normal distribution function and density, Phi(u) and phi(u), from Abramowitz and Stegun 7.1.26: erfc(x) =
-// t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) e^(-x^2), t = 1 / (1 + 0.3275911 x), |error| <= 1.5e-7, x >= 0 (the tail is
-// the product itself, so it keeps its relative accuracy).  About half of erff's instructions.
+// t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) e^(-x^2), t = 1 / (1 + 0.3275911 x), x >= 0, |error| <= 1.5e-7 (Phi: 7e-8, in fp32
+// 3e-7; by erff 6e-8).  For results stored as bf16, whose rounding is 2e-3 of them: gelu and gelu' come out the same but for 2
+// and 0 of the 3 064 bf16 values of 0.001 < |u| < 4, with the same error; below, the tail's relative error grows (5e-5 at u =
+// -3, 5e-4 at -4, 4e-3 at -6, 1e-2 at -8), less than that of 1 + erff, which has no digits left there.  About half of erff's
+// instructions: 8 192 x 3 072 forward and backward in a layer's training, 509 -> 518 us by erff.
 __device__ __forceinline__ void normal_cdf_pdf(float u, float& cdf, float& pdf) {
   const float x = fabsf(u) * 0.70710678118654752f;
   const float e = __expf(-x * x);

@@ -8,8 +8,8 @@ namespace spa {
 // The same on the device, for eight bf16 values of a row at element offset `at` of the result: `fetch` ahead of time what the
 // result is combined with, `finish` behind the product.  One kind per kernel: a second set of fetched values spills, and a
 // result that is not known to be apart from what it is combined with costs the plain products 1 us.  kEpiOwn: the result as
-// it is, or joined to what `out` holds (other = out).  gelu reads the rounded result, so a layer and its activation in one
-// kernel equal the two calls.
+// it is, or joined to what `out` holds (other = out).  gelu reads the rounded result, as spa_gelu would; that call takes erff,
+// this one normal_cdf_pdf, so the two may differ by a rounding.
 enum EpiKind { kEpiOwn, kEpiAdd, kEpiGeluGrad, kEpiGelu };
 template <int kKind> struct RowEpilogue {
   __nv_bfloat16* other;  // out or null; add; u; h

@@ -70,3 +70,19 @@ def test_inplace_flag_changes_nothing():
         assert lay.read_status() == 0 and torch.equal(xd, dev(x, cfg.dtype))
         runs.append((out, dX, lay.dW1, lay.blk.dW_qkv))
     assert all(torch.equal(a, b) for a, b in zip(*runs))
+
+
+def test_activation_of_the_product_is_that_of_the_call_within_a_rounding():
+    from paper_2410_23608_b200 import binding as L
+    from paper_2410_23608_b200.layer import SpaLayer
+    cfg, inp, x, prm, _ = layer_problem(2, 2)
+    dprm = {k: (dev(v, cfg.dtype) if isinstance(v, np.ndarray) else v) for k, v in prm.items()}
+    lay = SpaLayer(cfg.B, cfg.N, cfg.C, cfg.H, cfg.dtype)
+    lay.forward(dev(x, cfg.dtype), dprm)
+    by_call = torch.empty_like(lay.h)
+    L.spa_gelu(lay.p, lay.u, lay.hidden, by_call)
+    exact = torch.nn.functional.gelu(lay.u.double())
+    for h in (lay.h.double(), by_call.double()):
+        # the rounding to eight bits (at most 2^-8 of the value), and the error of the distribution function times |u|
+        assert bool(((h - exact).abs() <= 2.0 ** -8 * exact.abs() + 6e-7 * lay.u.double().abs() + 1e-30).all())
+    assert float((lay.h != by_call).double().mean()) < 2e-3
