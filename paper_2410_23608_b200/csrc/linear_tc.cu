@@ -591,7 +591,9 @@ int launch_linear_bwd_tc(const spa_params& p, const void* a, const void* W, cons
   if (dW == nullptr && db == nullptr) return SPA_OK;
   const PairWgradPlan pl = pair_wgrad_plan(p.capacity, n_in, n_out);
   // CTA pairs where there are enough of their 256 x 256 tiles and enough rows to split between them (768 x 768 over 9 216
-  // rows: 18 us on pairs, 30 on clusters; 1 536 x 512 over 3 402: 17 either way; 1 536 x 384 over 1 568: 14 and 12)
+  // rows: 18 us on pairs, 30 on clusters; 1 536 x 512 over 3 402: 17 either way; 1 536 x 384 over 1 568: 14 and 12).  The line
+  // runs through 768 x 768 and 8 192 allocated rows and is on the safe side: at 6 144, all or half of them there, pairs are
+  // ahead too (768 x 768 14.1 against 21.1 and 11.7 against 14.2, 576 x 576 13.7 against 15.3 and 11.4 against 11.7).
   if (dW != nullptr && wgrad_on_pairs(p) && (pl.tiles < 9 || p.capacity < 128 * BK))
     return launch_wgrad_cluster(p, a, dout, n_in, n_out, cu, dW, db, d_status, st);
   const SplitPlan sp = plan_splits(p.capacity, n_in, n_out);

@@ -624,7 +624,8 @@ int launch_wgrad_pair(const spa_params& p, const void* a, const void* dout, int 
 // fewer tiles the smaller ones spread better (6 272 rows 384 -> 384: 7.9 against 6.5).  Not where K is short and
 // an eighth of the pair's columns or more would be padding that 128-column tiles do not have (34 000 rows allocated, 30 % of
 // them there: 384 -> 384 10.6 against 8.2, 288 -> 864 14.0 against 12.0; at half and above even).  With a longer main loop the
-// pairs win all the same (576 -> 576 13.1 against 15.1).
+// pairs win all the same (576 -> 576 13.1 against 15.1, 512 -> 640 10.7 against 12.3; no padded width lies between 384 and 512
+// in what was measured).
 bool tc_pair_linear_supported(const spa_params& p, int n_in, int n_out, int n_cols) {
   if (p.flags & SPA_FLAG_NO_CTA_PAIRS) return false;
   const long long tiles = (long long)((p.capacity / 2 + 2 * PM - 1) / (2 * PM)) * ((n_cols + PN - 1) / PN);
