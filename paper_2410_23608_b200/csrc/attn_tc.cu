@@ -749,8 +749,9 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   auto stage_of = [&](int t_) { return (t_ + kShift) % kStages; };
   auto use_of = [&](int t_) { return (uint32_t)(((t_ + kShift) / kStages) & 1); };  // parity of that stage's barrier
   constexpr int kStatBase = kYBase + kStages * 2 * kYTile;
-  float* stat_lse = reinterpret_cast<float*>(smem_al + kStatBase);  // [3][64] lse_i * log2e of the staged query tile
-  float* stat_D = stat_lse + 3 * kBwdY;                              // [3][64] D_i
+  float* stat_lse = reinterpret_cast<float*>(smem_al + kStatBase);  // [3][64] -lse_i * log2e of the staged query tile
+  float* stat_D = stat_lse + 3 * kBwdY;                              // [3][64] -D_i
+  const uint32_t stat_s = smem_base + kStatBase;
   constexpr int kBarBase = kStatBase + kBwdStatBytes;
   const uint32_t bar_base = smem_base + kBarBase;
   const uint32_t bar_x = bar_base, bar_s = bar_base + 56, bar_acc = bar_base + 64;
@@ -882,7 +883,7 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
       if (mine.hi > mine.lo) my_lse = lse[(long long)h * capacity + row] * kLog2e;
     } else if (half == 0 && rl < kBwdY) {
       const int i = o_lo + rl;
-      if (i < o_hi) { nxt_lse = lse[(long long)h * capacity + i] * kLog2e; nxt_D = delta[(long long)h * capacity + i]; }
+      if (i < o_hi) { nxt_lse = -lse[(long long)h * capacity + i] * kLog2e; nxt_D = -delta[(long long)h * capacity + i]; }
     }
   }
 
@@ -920,7 +921,7 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
       stat_D[(t_ % 3) * kBwdY + rl] = nxt_D;
       const int i = y0 + kBwdY + rl;
       nxt_lse = 0.f; nxt_D = 0.f;
-      if (i < o_hi) { nxt_lse = lse[(long long)h * capacity + i] * kLog2e; nxt_D = delta[(long long)h * capacity + i]; }
+      if (i < o_hi) { nxt_lse = -lse[(long long)h * capacity + i] * kLog2e; nxt_D = -delta[(long long)h * capacity + i]; }
     }
     return ok;
   };
@@ -1070,22 +1071,39 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
           for (int j = 0; j < kPc; ++j)
             if ((unsigned)(yc0 + j - mine.lo) >= span) { rs[j] = 0xff800000u; rp[j] = 0u; }  // p = 2^-inf = 0, dP = 0
         }
-        const float* sl = stat_lse + (t % 3) * kBwdY + col0;
-        const float* sd = stat_D + (t % 3) * kBwdY + col0;
+        if constexpr (kDQ) {
+          // All exponents, then all exponentials, then what uses them.  Value by value, in the order of the formula, a warp
+          // waits out the exponential unit's latency with every pair: dQ pass of 16 segments of 210 to 1 680 rows, 8 heads of
+          // 32: 89.2 -> 84.9 us, of 32 of 58 to 518, 12 heads of 64: 44.3 -> 42.8.  (The other pass at d = 32 has no registers
+          // left for it: 132 -> 135.)
+          const uint64_t scale2 = ptx::pair(scale_log2e, scale_log2e), lse2 = ptx::pair(-my_lse, -my_lse), D2 = ptx::pair(-my_D, -my_D);
 #pragma unroll
-        for (int j = 0; j < kPc; j += 2) {
-          float pv[2], dsv[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const float l2 = kDQ ? my_lse : sl[j + u];
-            const float Dv = kDQ ? my_D : sd[j + u];
-            pv[u] = ptx::ex2_approx(fmaf(__uint_as_float(rs[j + u]), scale_log2e, -l2));
-            dsv[u] = pv[u] * (__uint_as_float(rp[j + u]) - Dv);
+          for (int j = 0; j < kPc; j += 2) {
+            ptx::unpair(ptx::fma2(ptx::pair(rs[j], rs[j + 1]), scale2, lse2), rs[j], rs[j + 1]);
+            ptx::unpair(ptx::add2(ptx::pair(rp[j], rp[j + 1]), D2), rp[j], rp[j + 1]);
           }
-          __nv_bfloat162 bds = __floats2bfloat162_rn(dsv[0], dsv[1]);
-          pk_ds[j >> 1] = *reinterpret_cast<uint32_t*>(&bds);
-          __nv_bfloat162 bp = __floats2bfloat162_rn(pv[0], pv[1]);
-          pk_p[j >> 1] = *reinterpret_cast<uint32_t*>(&bp);
+#pragma unroll
+          for (int j = 0; j < kPc; ++j) rs[j] = __float_as_uint(ptx::ex2_approx(__uint_as_float(rs[j])));
+#pragma unroll
+          for (int j = 0; j < kPc; j += 2) {
+            float d0, d1;
+            ptx::unpair(ptx::mul2(ptx::pair(rs[j], rs[j + 1]), ptx::pair(rp[j], rp[j + 1])), d0, d1);
+            pk_ds[j >> 1] = ptx::bf16_pair(d0, d1);
+          }
+        } else {
+          const float* sl = stat_lse + (t % 3) * kBwdY + col0;
+          const float* sd = stat_D + (t % 3) * kBwdY + col0;
+#pragma unroll
+          for (int j = 0; j < kPc; j += 2) {
+            float pv[2], dsv[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              pv[u] = ptx::ex2_approx(fmaf(__uint_as_float(rs[j + u]), scale_log2e, sl[j + u]));
+              dsv[u] = pv[u] * (__uint_as_float(rp[j + u]) + sd[j + u]);
+            }
+            pk_ds[j >> 1] = ptx::bf16_pair(dsv[0], dsv[1]);
+            pk_p[j >> 1] = ptx::bf16_pair(pv[0], pv[1]);
+          }
         }
       } else {
 #pragma unroll
@@ -1211,8 +1229,9 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
   constexpr int kPBase = kYBase + kStages * 2 * kYTile;   // P^T of the current tile: [128 keys][64 queries] bf16, K-major
   const uint32_t p_s = smem_base + kPBase;
   constexpr int kStatBase = kPBase + kTile;
-  float* stat_lse = reinterpret_cast<float*>(smem_al + kStatBase);  // [3][64] lse_i * log2e of the staged query tile
-  float* stat_D = stat_lse + 3 * kBwdY;                              // [3][64] D_i
+  float* stat_lse = reinterpret_cast<float*>(smem_al + kStatBase);  // [3][64] -lse_i * log2e of the staged query tile
+  float* stat_D = stat_lse + 3 * kBwdY;                              // [3][64] -D_i
+  const uint32_t stat_s = smem_base + kStatBase;
   constexpr int kBarBase = kStatBase + kBwdStatBytes;
   const uint32_t bar_base = smem_base + kBarBase;
   const uint32_t bar_x = bar_base, bar_s = bar_base + 32, bar_dp = bar_base + 40, bar_acc = bar_base + 48;
@@ -1337,7 +1356,7 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
   float nxt_lse = 0.f, nxt_D = 0.f;  // prefetched values of the next streamed query tile, row rl < 64
   if (is_math && half == 0 && rl < kBwdY) {
     const int i = o_lo + rl;
-    if (i < o_hi) { nxt_lse = lse[(long long)h * capacity + i] * kLog2e; nxt_D = delta[(long long)h * capacity + i]; }
+    if (i < o_hi) { nxt_lse = -lse[(long long)h * capacity + i] * kLog2e; nxt_D = -delta[(long long)h * capacity + i]; }
   }
 
   constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(128, kBwdY, false, false);
@@ -1372,7 +1391,7 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
       stat_D[(t_ % 3) * kBwdY + rl] = nxt_D;
       const int i = y0 + kBwdY + rl;
       nxt_lse = 0.f; nxt_D = 0.f;
-      if (i < o_hi) { nxt_lse = lse[(long long)h * capacity + i] * kLog2e; nxt_D = delta[(long long)h * capacity + i]; }
+      if (i < o_hi) { nxt_lse = -lse[(long long)h * capacity + i] * kLog2e; nxt_D = -delta[(long long)h * capacity + i]; }
     }
     return ok;
   };
@@ -1458,6 +1477,7 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
     // ---------------------------------------------------------------- arithmetic: two threads per key row
     constexpr int kPc = kBwdY / 2;  // fp32 columns of each tile owned by this thread
     const int col0 = half * kPc;
+    const uint64_t scale2 = ptx::pair(scale_log2e, scale_log2e);
     // no barrier joins the arithmetic warps inside the loop, so a warp whose wait gave up may leave it alone: the
     // others see the flag in their own waits
     auto fail = [&]() {
@@ -1497,16 +1517,20 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
           for (int j = 0; j < kPc; ++j)
             if ((unsigned)(yc0 + j - mine.lo) >= span) rs[j] = 0xff800000u;  // p = 2^-inf = 0
         }
-        const float* sl = stat_lse + (t % 3) * kBwdY + col0;
+        // all exponents, all exponentials, then what uses them: see the dQ pass (32 segments of 58 to 518 rows, 12 heads: 66.1 ->
+        // 61.1 us, 64 of 39 to 157, 6 heads: 16.4 -> 15.6)
+        const uint32_t sl = stat_s + ((t % 3) * kBwdY + col0) * 4;
 #pragma unroll
-        for (int j = 0; j < kPc; j += 2) {
-          const float p0 = ptx::ex2_approx(fmaf(__uint_as_float(rs[j]), scale_log2e, -sl[j]));
-          const float p1 = ptx::ex2_approx(fmaf(__uint_as_float(rs[j + 1]), scale_log2e, -sl[j + 1]));
-          rs[j] = __float_as_uint(p0);
-          rs[j + 1] = __float_as_uint(p1);
-          __nv_bfloat162 bp = __floats2bfloat162_rn(p0, p1);
-          pk[j >> 1] = *reinterpret_cast<uint32_t*>(&bp);
+        for (int j = 0; j < kPc; j += 4) {
+          uint64_t l2[2];
+          ptx::lds_pairs(sl + j * 4, l2[0], l2[1]);
+          ptx::unpair(ptx::fma2(ptx::pair(rs[j], rs[j + 1]), scale2, l2[0]), rs[j], rs[j + 1]);
+          ptx::unpair(ptx::fma2(ptx::pair(rs[j + 2], rs[j + 3]), scale2, l2[1]), rs[j + 2], rs[j + 3]);
         }
+#pragma unroll
+        for (int j = 0; j < kPc; ++j) rs[j] = __float_as_uint(ptx::ex2_approx(__uint_as_float(rs[j])));
+#pragma unroll
+        for (int j = 0; j < kPc; j += 2) pk[j >> 1] = ptx::bf16_pair(__uint_as_float(rs[j]), __uint_as_float(rs[j + 1]));
       } else {
 #pragma unroll
         for (int j = 0; j < kPc / 2; ++j) pk[j] = 0u;
@@ -1529,14 +1553,19 @@ attn_bwd_kv_split_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __gri
       ptx::tmem_ld_32x32(tmem + lane_base + kColS2 + col0, rp);  // by the whole warp: the load is a collective
       ptx::tmem_ld_wait();
       if (some) {
-        const float* sd = stat_D + (t % 3) * kBwdY + col0;
+        // a masked column has p = 0 exactly and a finite dP^T (rows past the last valid one are zeroed): dS^T = 0
+        const uint32_t sd = stat_s + ((t % 3 + 3) * kBwdY + col0) * 4;
 #pragma unroll
-        for (int j = 0; j < kPc; j += 2) {
-          // a masked column has p = 0 exactly and a finite dP^T (rows past the last valid one are zeroed): dS^T = 0
-          const float d0 = __uint_as_float(rs[j]) * (__uint_as_float(rp[j]) - sd[j]);
-          const float d1 = __uint_as_float(rs[j + 1]) * (__uint_as_float(rp[j + 1]) - sd[j + 1]);
-          __nv_bfloat162 bds = __floats2bfloat162_rn(d0, d1);
-          pk[j >> 1] = *reinterpret_cast<uint32_t*>(&bds);
+        for (int j = 0; j < kPc; j += 4) {
+          uint64_t d2[2];
+          ptx::lds_pairs(sd + j * 4, d2[0], d2[1]);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int i = j + 2 * u;
+            float d0, d1;
+            ptx::unpair(ptx::mul2(ptx::pair(rs[i], rs[i + 1]), ptx::add2(ptx::pair(rp[i], rp[i + 1]), d2[u])), d0, d1);
+            pk[i >> 1] = ptx::bf16_pair(d0, d1);
+          }
         }
       }
       ptx::tmem_st_32x16(tmem + lane_base + kColS2 + col0, pk);
