@@ -3,13 +3,16 @@
 // workload and the bring-up reference of the tensor-core kernels.
 //
 // Work split: a CTA owns 32 consecutive packed rows and one head, wherever segment boundaries fall, and walks the
-// rows of the other side that the segments of its rows span, in tiles of 64 staged in shared memory as fp32, two
-// tiles in flight.  128 threads form a grid of 8 x 16: a product tile of 32 x 64 is 4 x 4 values per thread (8
+// rows of the other side that the segments of its rows span, in tiles of 64 staged in shared memory as fp32.  Two groups of
+// 128 threads take them in turn, each with a stage of its own, and the first joins the two results at the end: one group's copies
+// and softmax run under the other's products, and a CTA's chain, which bounds all but the largest problems, is half as long.
+// A group is a grid of 8 x 16 threads: a product tile of 32 x 64 is 4 x 4 values per thread (8
 // vector reads of shared memory per 64 multiply-adds), its softmax statistics are shuffles among 16 lanes, and the
-// second product gives a thread 4 rows x D / 16 head dimensions.  Small problems are bound by the length of one CTA's
-// chain: 32-row tiles halve it and double the CTAs.  (235 rows of 3 heads: 7 us forward, 15 us backward,
-// where one thread per row, one key after the other, took 32 and 90; 1 568 rows of 6 heads: 22 us forward, before 75.)  No padding token is ever
-// computed, nothing is atomically accumulated, and every sum runs in a fixed order.
+// second product gives a thread 4 rows x D / 16 head dimensions.  No padding token is ever computed, nothing is atomically
+// accumulated, and every sum runs in a fixed order.  With one group, and two tiles in flight, against two, us: one image of
+// 4 200 tokens, 8 heads of 32, forward 81.5 -> 46.1, backward 200.5 -> 151.8; 4 of 196 tokens, 3 heads of 32, 7.4 -> 7.2 and
+// 15.8 -> 14.4; 16 of 196, 6 heads of 64, 22.6 -> 21.7 and 76.2 -> 73.0; 64 of them 71.2 -> 68.8 and 256 -> 246.  What bounds it
+// then is shared memory: a vector read of 16 bytes per eight multiply-adds, 30 of the 75 TFLOP/s of the multiply-adds.
 #include <math_constants.h>
 
 #include "simt_stage.cuh"
@@ -20,18 +23,19 @@ namespace {
 
 constexpr int kR = 32;          // packed rows per CTA
 constexpr int kT = 64;          // rows of a streamed tile
-constexpr int kThreads = 128;
-constexpr int kTX = 16, kTY = 8;  // thread (ty, tx): rows ty + 8 i (i < 4), streamed rows tx + 16 j (j < 4)
+constexpr int kGroups = 2;      // of threads: group q takes the streamed tiles q, q + 2, ..
+constexpr int kGroup = 128, kThreads = kGroups * kGroup;
+constexpr int kTX = 16, kTY = 8;  // thread (ty, tx) of a group: rows ty + 8 i (i < 4), streamed rows tx + 16 j (j < 4)
 constexpr int kLdP = kT + 4;    // leading dimension of the probability tiles
 template <int D> constexpr int kLd = D + 4;  // rows 4 banks apart
 
 // Rows [row0, row0 + kRows) of one head's slice (column col0 of a [*, ld] matrix); rows from row_end on become zero.
-template <typename T, int D, int kRows>
+template <typename T, int D, int kRows, int kBy>
 __device__ __forceinline__ void stage_rows(float* dst, const T* src, long long ld, int col0, int row0, int row_end,
                                            int tid) {
   constexpr int E = Vec16<T>::kElems, kPer = D / E;
 #pragma unroll
-  for (int c = tid; c < kRows * kPer; c += kThreads) {
+  for (int c = tid; c < kRows * kPer; c += kBy) {
     const int r = c / kPer, cc = (c % kPer) * E;
     stage16<T>(dst + r * kLd<D> + cc, src + (long long)(row0 + r) * ld + col0 + cc, row0 + r < row_end, src);
   }
@@ -116,6 +120,8 @@ template <> __device__ __forceinline__ void store_row<float, 2>(float* dst, cons
   *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
 }
 
+__device__ __forceinline__ void group_sync(int q) { asm volatile("bar.sync %0, %1;" ::"r"(q + 1), "n"(kGroup) : "memory"); }
+
 __device__ __forceinline__ float max16(float v) {
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -137,47 +143,49 @@ __device__ __forceinline__ RowSeg tile_segments(RowSeg* seg_s, const int32_t* se
 }
 
 // ------------------------------------------------------------------------------------ forward
-template <int D> constexpr int kFwdFloats = (kR + 4 * kT) * kLd<D> + kR * kLdP;  // Q, two stages of K and V, P
+template <int D> constexpr int kFwdFloats = (kR + kGroups * 2 * kT) * kLd<D> + kGroups * kR * kLdP;  // Q; per group K and V, P
 
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ ao, float* __restrict__ lse) {
   pdl_entry();
   constexpr int W = D / kTX;
   extern __shared__ __align__(16) float sm[];
   __shared__ RowSeg seg_s[kR];
-  float* Qs = sm;
-  float* KV = sm + kR * kLd<D>;              // stage s: K at s * 2 tiles, V behind it
-  float* Ps = KV + 4 * kT * kLd<D>;
   constexpr int kTile = kT * kLd<D>;
   const int Np = packed_rows(seg, n_seg, capacity);
   const int i0 = blockIdx.x * kR;
   if (i0 >= Np) return;
-  const int tid = threadIdx.x, tx = tid % kTX, ty = tid / kTX, h = blockIdx.y;
+  const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup, tx = tid % kTX, ty = tid / kTX, h = blockIdx.y;
+  float* Qs = sm;
+  float* Ks = sm + kR * kLd<D> + grp * 2 * kTile;  // this group's K, V behind it
+  float* Ps = sm + kR * kLd<D> + kGroups * 2 * kTile + grp * kR * kLdP;
   const long long ld = 3LL * C;
-  stage_rows<T, D, kR>(Qs, qkv, ld, h * D, i0, Np, tid);
-  const RowSeg all = tile_segments(seg_s, seg, n_seg, Np, i0, tid);
-  auto stage = [&](int t) {
-    const int kv0 = all.lo + t * kT;
-    float* dst = KV + (t & 1) * 2 * kTile;
-    stage_rows<T, D, kT>(dst, qkv, ld, C + h * D, kv0, all.hi, tid);
-    stage_rows<T, D, kT>(dst + kTile, qkv, ld, 2 * C + h * D, kv0, all.hi, tid);
-    cp_async_commit();
-  };
+  stage_rows<T, D, kR, kThreads>(Qs, qkv, ld, h * D, i0, Np, threadIdx.x);
+  cp_async_commit();
+  const RowSeg all = tile_segments(seg_s, seg, n_seg, Np, i0, threadIdx.x);
   const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
   const bool several = seg_s[0].hi < all.hi;  // segments that the CTA's rows are of
-  stage(0);
+  auto stage = [&](int t) {
+    const int kv0 = all.lo + t * kT;
+    stage_rows<T, D, kT, kGroup>(Ks, qkv, ld, C + h * D, kv0, all.hi, tid);
+    cp_async_commit();
+    stage_rows<T, D, kT, kGroup>(Ks + kTile, qkv, ld, 2 * C + h * D, kv0, all.hi, tid);
+    cp_async_commit();
+  };
+  if (grp < n_tiles) stage(grp);
 
   float o[4][W] = {}, m[4], l[4] = {};
   RowSeg mine[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) { m[i] = -CUDART_INF_F; mine[i] = seg_s[ty + kTY * i]; }
-  for (int t = 0; t < n_tiles; ++t) {
-    if (t + 1 < n_tiles) { stage(t + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
-    __syncthreads();
+  cp_async_wait<2>();
+  __syncthreads();  // Q, of which every thread has copied a part
+  for (int t = grp; t < n_tiles; t += kGroups) {
+    cp_async_wait<1>();
+    group_sync(grp);  // K; V is waited for behind the first product
     const int kv0 = all.lo + t * kT;
-    const float* Ks = KV + (t & 1) * 2 * kTile;
     float s[4][4] = {};
     dots<D>(s, Qs, Ks, ty, tx);
 #pragma unroll
@@ -204,10 +212,35 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
       for (int d = 0; d < W; ++d) o[i][d] *= alpha;
       m[i] = m_new;
     }
-    __syncwarp();  // the rows of P that this warp reads are the ones its own lanes wrote
+    cp_async_wait<0>();
+    group_sync(grp);  // V, and the rows of P
     const int n = all.hi - kv0 < kT ? all.hi - kv0 : kT;
     weighted<D>(o, Ps, Ks + kTile, n, ty, tx);
-    __syncthreads();  // the stage is free for the tile after next
+    group_sync(grp);  // the stage is free
+    if (t + kGroups < n_tiles) stage(t + kGroups);
+  }
+  // the second group's share of every row, in the memory of its stage
+  float* part = sm + kR * kLd<D> + 2 * kTile + tid;  // [4 (W + 2)][kGroup]
+  if (grp == 1) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      part[(i * (W + 2)) * kGroup] = m[i];
+      part[(i * (W + 2) + 1) * kGroup] = l[i];
+#pragma unroll
+      for (int d = 0; d < W; ++d) part[(i * (W + 2) + 2 + d) * kGroup] = o[i][d];
+    }
+  }
+  __syncthreads();
+  if (grp == 1) return;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float m1 = part[(i * (W + 2)) * kGroup], l1 = part[(i * (W + 2) + 1) * kGroup];
+    const float m_new = fmaxf(m[i], m1), m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
+    const float a0 = expf(m[i] - m_use), a1 = expf(m1 - m_use);
+    l[i] = l[i] * a0 + l1 * a1;
+#pragma unroll
+    for (int d = 0; d < W; ++d) o[i][d] = o[i][d] * a0 + part[(i * (W + 2) + 2 + d) * kGroup] * a1;
+    m[i] = m_new;
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -237,10 +270,10 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
 // holds), so that they share the GPU: blockIdx.z = 0: own rows are queries, streamed rows keys,
 //   S = Q K^T, dP = dO V^T, dS = P (dP - D), dQ += dS K;
 // blockIdx.z = 1: own rows are keys, streamed rows queries, everything transposed: dV += P^T dO, dK += dS^T Q.
-template <int D> constexpr int kBwdFloats = (2 * kR + 4 * kT) * kLd<D> + 2 * kR * kLdP + 4 * kT;
+template <int D> constexpr int kBwdFloats = (2 * kR + kGroups * 2 * kT) * kLd<D> + kGroups * (kR * kLdP + 2 * kT);
 
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
                      const T* dao, const int32_t* seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ dqkv) {
@@ -249,17 +282,17 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
   constexpr int kTile = kT * kLd<D>;
   extern __shared__ __align__(16) float sm[];
   __shared__ RowSeg seg_s[kR];
+  const int grp = threadIdx.x / kGroup, tid = threadIdx.x % kGroup, tx = tid % kTX, ty = tid / kTX, h = blockIdx.y;
   float* A1 = sm;                       // Q | K of the own rows
   float* A2 = A1 + kR * kLd<D>;         // dO | V
-  float* Y = A2 + kR * kLd<D>;          // stage s: K | Q at s * 2 tiles, V | dO behind it
-  float* Ps = Y + 4 * kTile;            // P^T (second pass)
-  float* Ds = Ps + kR * kLdP;           // dS | dS^T
-  float* st = Ds + kR * kLdP;           // second pass, stage s: lse_i at s * 2 * kT, D_i behind it
+  float* Y1 = A2 + kR * kLd<D> + grp * 2 * kTile;  // this group's K | Q
+  float* Y2 = Y1 + kTile;                          // V | dO
+  float* Ps = A2 + kR * kLd<D> + kGroups * 2 * kTile + grp * (kR * kLdP + 2 * kT);  // P^T, then dS | dS^T
+  float* s2 = Ps + kR * kLdP;           // second pass: lse_i of the streamed rows, D_i behind it
   const bool dq = blockIdx.z == 0;
   const int Np = packed_rows(seg, n_seg, capacity);
   const int i0 = blockIdx.x * kR;
   if (i0 >= Np) return;
-  const int tid = threadIdx.x, tx = tid % kTX, ty = tid / kTX, h = blockIdx.y;
   const long long ld = 3LL * C;
   // D of packed row i: eight or sixteen 16-byte loads, all in flight together
   auto row_D = [&](int i) {
@@ -276,27 +309,26 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
     }
     return s;
   };
-  stage_rows<T, D, kR>(A1, qkv, ld, (dq ? 0 : C) + h * D, i0, Np, tid);
-  if (dq) stage_rows<T, D, kR>(A2, dao, (long long)C, h * D, i0, Np, tid);
-  else stage_rows<T, D, kR>(A2, qkv, ld, 2 * C + h * D, i0, Np, tid);
-  const RowSeg all = tile_segments(seg_s, seg, n_seg, Np, i0, tid);
+  stage_rows<T, D, kR, kThreads>(A1, qkv, ld, (dq ? 0 : C) + h * D, i0, Np, threadIdx.x);
+  if (dq) stage_rows<T, D, kR, kThreads>(A2, dao, (long long)C, h * D, i0, Np, threadIdx.x);
+  else stage_rows<T, D, kR, kThreads>(A2, qkv, ld, 2 * C + h * D, i0, Np, threadIdx.x);
+  cp_async_commit();
+  const RowSeg all = tile_segments(seg_s, seg, n_seg, Np, i0, threadIdx.x);
+  const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
+  const bool several = seg_s[0].hi < all.hi;  // segments that the CTA's rows are of
   auto stage = [&](int t) {
     const int y0 = all.lo + t * kT;
-    float* dst = Y + (t & 1) * 2 * kTile;
-    stage_rows<T, D, kT>(dst, qkv, ld, (dq ? C : 0) + h * D, y0, all.hi, tid);
-    if (dq) stage_rows<T, D, kT>(dst + kTile, qkv, ld, 2 * C + h * D, y0, all.hi, tid);
-    else stage_rows<T, D, kT>(dst + kTile, dao, (long long)C, h * D, y0, all.hi, tid);
+    stage_rows<T, D, kT, kGroup>(Y1, qkv, ld, (dq ? C : 0) + h * D, y0, all.hi, tid);
+    if (dq) stage_rows<T, D, kT, kGroup>(Y2, qkv, ld, 2 * C + h * D, y0, all.hi, tid);
+    else stage_rows<T, D, kT, kGroup>(Y2, dao, (long long)C, h * D, y0, all.hi, tid);
     cp_async_commit();
     if (!dq && tid < kT) {
-      float* s2 = st + (t & 1) * 2 * kT;
       const bool in = y0 + tid < all.hi;
       s2[tid] = in ? lse[(long long)h * capacity + y0 + tid] : 0.f;
       s2[kT + tid] = in ? row_D(y0 + tid) : 0.f;
     }
   };
-  const int n_tiles = (all.hi - all.lo + kT - 1) / kT;
-  const bool several = seg_s[0].hi < all.hi;  // segments that the CTA's rows are of
-  stage(0);
+  if (grp < n_tiles) stage(grp);
 
   RowSeg mine[4];
   float my_lse[4] = {}, my_D[4] = {};
@@ -313,13 +345,12 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
     }
   }
   float acc1[4][W] = {}, acc2[4][W] = {};  // dQ | dK and dV
-  for (int t = 0; t < n_tiles; ++t) {
-    if (t + 1 < n_tiles) { stage(t + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
-    __syncthreads();
+  cp_async_wait<1>();
+  __syncthreads();  // the own rows, of which every thread has copied a part
+  for (int t = grp; t < n_tiles; t += kGroups) {
+    cp_async_wait<0>();
+    group_sync(grp);
     const int y0 = all.lo + t * kT;
-    const float* Y1 = Y + (t & 1) * 2 * kTile;
-    const float* Y2 = Y1 + kTile;
-    const float* s2 = st + (t & 1) * 2 * kT;
     float s[4][4] = {}, dp[4][4] = {};
     dots<D>(s, A1, Y1, ty, tx);
     dots<D>(dp, A2, Y2, ty, tx);
@@ -331,14 +362,43 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
         const float l = dq ? my_lse[i] : s2[c], Dv = dq ? my_D[i] : s2[kT + c];
         const float p = (ya >= mine[i].lo && ya < mine[i].hi) ? expf(s[i][j] * scale - l) : 0.f;
         if (!dq) Ps[(ty + kTY * i) * kLdP + c] = p;
-        Ds[(ty + kTY * i) * kLdP + c] = p * (dp[i][j] - Dv);
+        dp[i][j] = p * (dp[i][j] - Dv);
       }
-    __syncwarp();  // the rows of P and dS that this warp reads are the ones its own lanes wrote
     const int n = all.hi - y0 < kT ? all.hi - y0 : kT;
-    weighted<D>(acc1, Ds, Y1, n, ty, tx);
-    if (!dq) weighted<D>(acc2, Ps, Y2, n, ty, tx);
-    __syncthreads();  // the stage is free for the tile after next
+    if (!dq) {
+      __syncwarp();  // the rows of P and dS that this warp reads are the ones its own lanes wrote
+      weighted<D>(acc2, Ps, Y2, n, ty, tx);
+      __syncwarp();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) Ps[(ty + kTY * i) * kLdP + tx + kTX * j] = dp[i][j];
+    __syncwarp();
+    weighted<D>(acc1, Ps, Y1, n, ty, tx);
+    group_sync(grp);  // the stage is free
+    if (t + kGroups < n_tiles) stage(t + kGroups);
   }
+  // the second group's share of every sum, in the memory of its stage
+  float* part = A2 + kR * kLd<D> + 2 * kTile + tid;  // [8 W][kGroup]
+  if (grp == 1) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int d = 0; d < W; ++d) {
+        part[(i * W + d) * kGroup] = acc1[i][d];
+        part[((4 + i) * W + d) * kGroup] = acc2[i][d];
+      }
+  }
+  __syncthreads();
+  if (grp == 1) return;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int d = 0; d < W; ++d) {
+      acc1[i][d] += part[(i * W + d) * kGroup];
+      acc2[i][d] += part[((4 + i) * W + d) * kGroup];
+    }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int row = i0 + ty + kTY * i;
