@@ -1,0 +1,49 @@
+"""Packing and the transpose of the unpacking at the edges of their batches: rows of 4 to 128 chunks, masks of one load per
+thread and of many, tiles of few and of many selected rows."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,N,C,dtype,keep,flag", [
+    (1, 1, 32, "bf16", 1.0, 0),             # one row of four chunks
+    (1, 16 * 256, 32, "bf16", 0.5, 0),      # as many mask chunks as threads
+    (1, 16 * 256 + 33, 96, "f32", 1.0, 0),  # and more; everything selected
+    (3, 1357, 384, "bf16", 0.3, "RESIDUAL"),
+    (16, 4200, 64, "bf16", 0.9, 0),         # more than one batch of mask loads
+    (5, 301, 1024, "bf16", 0.0, 0),         # nothing selected
+    (2, 500, 512, "f32", 0.7, "RESIDUAL"),  # 128 chunks a row
+    (7, 77, 768, "bf16", 0.6, 0),
+])
+def test_pack_and_its_transposes_move_rows(B, N, C, dtype, keep, flag):
+    from paper_2410_23608_b200 import binding as L
+    T = torch.float32 if dtype == "f32" else torch.bfloat16
+    flags = getattr(L, "SPA_FLAG_" + flag) if flag else 0
+    p = L.make_params(B, N, C, max(C // 32, 1), dtype, B * N, flags)
+    g = torch.Generator(device="cuda").manual_seed(B * N + C)
+    x, dY = (torch.randn(B * N, C, generator=g, device="cuda").to(T) for _ in range(2))
+    mask = (torch.rand(B * N, generator=g, device="cuda") < keep).to(torch.uint8)
+    sel = mask.nonzero()[:, 0].int()
+    Np = sel.numel()
+    e = lambda *s, dt=torch.int32: torch.full(s, 7, device="cuda", dtype=dt)
+    xp, idx, inv, cu, status = e(B * N, C, dt=T), e(B * N), e(B * N), e(B + 1), torch.zeros(4, dtype=torch.int32, device="cuda")
+    L.spa_select_pack(p, x, mask, None, xp, idx, inv, cu, status)
+    assert L.spa_read_status(status) == 0
+    assert torch.equal(xp[:Np], x[sel.long()]) and bool((xp[Np:] == 7).all())
+    assert torch.equal(idx[:Np], sel) and bool((idx[Np:] == 7).all())
+    want = torch.full_like(inv, -1)
+    want[sel.long()] = torch.arange(Np, device="cuda", dtype=torch.int32)
+    assert torch.equal(inv, want)
+    assert cu.tolist() == [0] + mask.view(B, N).sum(1).cumsum(0).tolist()
+    for in_place in (False, True):
+        d = dY.clone()
+        dz, dX = e(B * N, C, dt=T), d if in_place else e(B * N, C, dt=T)
+        L.spa_unpack_scatter_bwd(p, d, idx, inv, cu, dz, dX)
+        torch.cuda.synchronize()
+        assert torch.equal(dz[:Np], dY[sel.long()]) and bool((dz[Np:] == 7).all())
+        if in_place:
+            assert torch.equal(dX, dY)
+        else:
+            assert torch.equal(dX[mask == 0], dY[mask == 0])
+            assert torch.equal(dX[mask == 1], dY[mask == 1]) if flag else bool((dX[mask == 1] == 7).all())
