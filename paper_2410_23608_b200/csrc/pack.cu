@@ -20,6 +20,26 @@ __device__ __forceinline__ int count_nonzero_bytes(uint4 m) {
          __popc(__vcmpne4(m.z, 0u) & 0x01010101u) + __popc(__vcmpne4(m.w, 0u) & 0x01010101u);
 }
 
+// Selected tokens among the first `n` chunks of 16 mask bytes, this thread's share: kCount loads in flight together.  One after
+// the other they were 10 000 of the clocks of a CTA behind 60 000 tokens.
+constexpr int kCount = 8;
+__device__ __forceinline__ int count_mask(const uint4* mask16, int n, int tid) {
+  int cnt = 0;
+  if (n <= kPackThreads) return tid < n ? count_nonzero_bytes(ld_dep16(mask16 + tid)) : 0;
+  for (int k0 = tid; k0 < n; k0 += kPackThreads * kCount) {
+    uint4 m[kCount];
+#pragma unroll
+    for (int u = 0; u < kCount; ++u) {
+      const int k = k0 + u * kPackThreads;
+      m[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (k < n) m[u] = ld_dep16(mask16 + k);
+    }
+#pragma unroll
+    for (int u = 0; u < kCount; ++u) cnt += count_nonzero_bytes(m[u]);
+  }
+  return cnt;
+}
+
 template <typename T>
 __device__ __forceinline__ uint4 scale16(uint4 v, float s) {
   float f[Vec16<T>::kElems];
@@ -37,6 +57,32 @@ __device__ __forceinline__ uint4 add16(uint4 a, uint4 b) {
 #pragma unroll
   for (int e = 0; e < Vec16<T>::kElems; ++e) fa[e] += fb[e];
   return Vec16<T>::from_float(fa);
+}
+
+// Chunk k of a tile's selected rows is (row k / Q, 16-byte column k % Q): kLoads of them in flight per thread.
+template <typename T, bool kGateScale, int kLoads>
+__device__ __forceinline__ void gather_rows(const uint4* x16, uint4* xp16, const int* sel_tok, const float* sel_scale, int total,
+                                            int Q, int tid) {
+  for (int k0 = tid; k0 < total; k0 += kPackThreads * kLoads) {
+    uint4 v[kLoads];
+    int r[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int k = k0 + u * kPackThreads;
+      if (k < total) {
+        r[u] = k / Q;
+        v[u] = ld_stream16(x16 + (size_t)sel_tok[r[u]] * Q + (k - r[u] * Q));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int k = k0 + u * kPackThreads;
+      if (k < total) {
+        if (kGateScale) v[u] = scale16<T>(v[u], sel_scale[r[u]]);
+        xp16[k] = v[u];
+      }
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------ select + pack
@@ -58,28 +104,32 @@ select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int tile_start = blockIdx.x * tile;  // multiple of 16
 
-  // 1. number of selected tokens before this tile
+  // 1. whether this thread's token is selected, on its way while the others are counted
+  const int t = tile_start + tid;
+  const bool in_tile = tid < tile && t < rows;
+  int tok = t;  // the token that position t of the visiting order stands for
+  if (kOrdered && in_tile) tok = (t / N) * N + ld_dep(order + t % N);
+  uint32_t own = 0;
+  if (in_tile) own = ld_dep(mask + tok);
+
+  // 2. number of selected tokens before this tile
   int cnt = 0;
   const uint4* mask16 = reinterpret_cast<const uint4*>(mask);
   if (!kOrdered) {
-    for (int k = tid; k < (tile_start >> 4); k += kPackThreads) cnt += count_nonzero_bytes(ld_dep16(mask16 + k));
+    cnt = count_mask(mask16, tile_start >> 4, tid);
   } else {
     // whole images before the tile's first image: any order visits the same bytes; then the positions of
     // that image which the given order visits before the tile
     const int img0 = (tile_start / N) * N;
-    for (int k = tid; k < (img0 >> 4); k += kPackThreads) cnt += count_nonzero_bytes(ld_dep16(mask16 + k));
+    cnt = count_mask(mask16, img0 >> 4, tid);
     for (int k = (img0 & ~15) + tid; k < img0; k += kPackThreads) cnt += ld_dep(mask + k) != 0;
     for (int j = tid; j < tile_start - img0; j += kPackThreads) cnt += ld_dep(mask + img0 + ld_dep(order + j)) != 0;
   }
   cnt = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
   if (lane == 0) warp_cnt[wid] = cnt;
 
-  // 2. ranks inside the tile
-  const int t = tile_start + tid;
-  const bool in_tile = tid < tile && t < rows;
-  int tok = t;  // the token that position t of the visiting order stands for
-  if (kOrdered && in_tile) tok = (t / N) * N + ld_dep(order + t % N);
-  const bool sel = in_tile && ld_dep(mask + tok) != 0;
+  // 3. ranks inside the tile
+  const bool sel = own != 0;
   const unsigned ballot = __ballot_sync(0xffffffffu, sel);
   if (lane == 0) warp_sel[wid] = __popc(ballot);
   __syncthreads();
@@ -108,31 +158,14 @@ select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
   if (tid == 0 && tile_start + tile >= rows) cu[B] = base + tile_total;
   __syncthreads();
 
-  // 3. gather the selected rows: chunk k of the tile is (row k / Q, 16-byte column k % Q)
+  // 4. gather the selected rows
   int n_ok = capacity - base;
   n_ok = n_ok < 0 ? 0 : (n_ok < tile_total ? n_ok : tile_total);
   const int total = n_ok * Q;
-  for (int k0 = tid; k0 < total; k0 += kPackThreads * kBatch) {
-    uint4 v[kBatch];
-    int r[kBatch], q[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int k = k0 + u * kPackThreads;
-      if (k < total) {
-        r[u] = k / Q;
-        q[u] = k - r[u] * Q;
-        v[u] = ld_stream16(x16 + (size_t)sel_tok[r[u]] * Q + q[u]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int k = k0 + u * kPackThreads;
-      if (k < total) {
-        if (kGateScale) v[u] = scale16<T>(v[u], sel_scale[r[u]]);
-        xp16[(size_t)(base + r[u]) * Q + q[u]] = v[u];
-      }
-    }
-  }
+  uint4* dst16 = xp16 + (size_t)base * Q;
+  // eight in flight where they fill more than one batch: the longer code costs a CTA of one or two batches of four 0.5 us
+  if (total <= 2 * kPackThreads * kBatch) gather_rows<T, kGateScale, kBatch>(x16, dst16, sel_tok, sel_scale, total, Q, tid);
+  else gather_rows<T, kGateScale, 2 * kBatch>(x16, dst16, sel_tok, sel_scale, total, Q, tid);
 }
 
 // ------------------------------------------------------------------------------ unpack
@@ -205,7 +238,7 @@ row_scatter_kernel(const uint4* src16, const uint4* addp, const int32_t* idx,
 // Transpose of the unpack: one pass over dY; selected rows go to dz, the others to dX.  A warp has kBwdRows rows, as in the
 // gate kernel: their chunks are read before it is known where they go, so the look-up of the rows' places runs beside them instead of in
 // front of each.  Alone, us: 16 x 4 200 rows of 256 channels 14.5 -> 12.9, 32 x 576 of 768 12.8 -> 11.4, 128 x 196 of 768 16.4 -> 15.5,
-// 64 x 196 of 384 4.9 -> 4.6, 1 x 3 901 of 256 3.1 -> 2.3 (the first three at 0.8 of the copy bandwidth, launch apart).
+// 64 x 196 of 384 4.9 -> 4.6, 1 x 3 901 of 256 3.1 -> 2.3; 96 x 4 200 of 64 23.8 -> 18.6 (the first three at 0.8 of the copy bandwidth, launch apart).
 constexpr int kBwdRows = 4;
 __global__ void __launch_bounds__(kPackThreads)
 unpack_scatter_bwd_kernel(const uint4* dY16, const int32_t* inv,
@@ -215,6 +248,30 @@ unpack_scatter_bwd_kernel(const uint4* dY16, const int32_t* inv,
   const int lane = threadIdx.x & 31, warp = blockIdx.x * (kPackThreads / 32) + (threadIdx.x >> 5);
   const int n_warps = gridDim.x * (kPackThreads / 32);
   const int Np = packed_rows(cu, B, capacity);
+  if (Q < 32) {  // rows shorter than a warp: 32 of them, chunk k of the 32 Q being (row k / Q, column k % Q)
+    for (int r0 = warp * 32; r0 < rows; r0 += n_warps * 32) {
+      int at = r0 + lane < rows ? ld_dep(inv + r0 + lane) : -1;
+      if (at >= Np) at = -1;
+      for (int k0 = lane; k0 < 32 * Q; k0 += 32 * kBwdRows) {
+        uint4 v[kBwdRows];
+        int r[kBwdRows];
+#pragma unroll
+        for (int u = 0; u < kBwdRows; ++u) {
+          const int k = k0 + 32 * u;
+          r[u] = k / Q;
+          if (k < 32 * Q && r0 + r[u] < rows) v[u] = ld_stream16(dY16 + (size_t)r0 * Q + k);
+        }
+#pragma unroll
+        for (int u = 0; u < kBwdRows; ++u) {
+          const int k = k0 + 32 * u, place = __shfl_sync(0xffffffffu, at, r[u] & 31);
+          if (k >= 32 * Q || r0 + r[u] >= rows) continue;
+          if (place >= 0) dz16[(size_t)place * Q + (k - r[u] * Q)] = v[u];
+          if (place >= 0 ? copy_selected : copy_pass_through) dX16[(size_t)r0 * Q + k] = v[u];
+        }
+      }
+    }
+    return;
+  }
   for (int r0 = warp * kBwdRows; r0 < rows; r0 += n_warps * kBwdRows) {
     int at = -1;  // lane u < kBwdRows: the packed place of row r0 + u
     if (lane < kBwdRows && r0 + lane < rows) at = ld_dep(inv + r0 + lane);
@@ -350,9 +407,14 @@ int launch_select_pack(const spa_params& p, const void* x, const uint8_t* mask, 
                        const int32_t* order, void* xp, int32_t* idx, int32_t* inv, int32_t* cu, int32_t* d_status,
                        cudaStream_t st) {
   const int rows = p.B * p.N;
-  int tile = 256;
-  while (tile > 32 && (rows + tile - 1) / tile < 2 * kNumSMs) tile >>= 1;
-  const int grid = (rows + tile - 1) / tile;
+  // Selected tokens come in regions, and a CTA in one copies nearly all of its tile: six CTAs per SM even that out (128 x 196
+  // rows of 768 channels 11.1 -> 9.3 us, in a forward pass 88.5 -> 85.2; with two per SM 11.3 and 86.9), while what they
+  // read of the mask in front of their tiles, half of it each, stays within what the L2 delivers in 4 us.
+  int tile = 256, grid = (rows + tile - 1) / tile;
+  while (tile > 32 && (grid < 2 * kNumSMs || (grid < 6 * kNumSMs && (long long)grid * rows <= 40000000ll))) {
+    tile >>= 1;
+    grid = (rows + tile - 1) / tile;
+  }
   const bool gs = (p.flags & SPA_FLAG_GATE_SCALE) != 0;
 #define SPA_PACK_LAUNCH(T, GS, ORD)                                                                              \
   launch_pdl(select_pack_kernel<T, GS, ORD>, grid, kPackThreads, 0, st, (const uint4*)x, mask, scores, order, rows, p.N, \
@@ -396,7 +458,7 @@ int launch_unpack_scatter_bwd(const spa_params& p, const void* dY, const int32_t
                               const int32_t* cu, void* dz, void* dX, cudaStream_t st) {
   (void)idx;
   const int Q = p.dtype == SPA_F32 ? chunks_per_row<float>(p.C) : chunks_per_row<__nv_bfloat16>(p.C);
-  const int rows = p.B * p.N, per_cta = kPackThreads / 32 * kBwdRows;
+  const int rows = p.B * p.N, per_cta = kPackThreads / 32 * (Q < 32 ? 32 : kBwdRows);
   int grid = (rows + per_cta - 1) / per_cta;
   if (grid > kNumSMs * 8) grid = kNumSMs * 8;
   const bool copy = dX != nullptr && dX != dY;
