@@ -586,14 +586,14 @@ int kv_launch(const spa_params& p, const void* qkv, const float* lse, const floa
 // is.  dQ and dK / dV together, us, the other kernels -> this one, at tiles per SM of
 //   5: 32 images of 196 tokens, 6 heads of 64, 20.2 -> 20.8;  10: 64 of them 24.5 -> 27.8, 4 x 4 200 tokens in containers of 49,
 //   8 heads of 32, 19.8 -> 21.2;  11: 24 x 315 tokens, 8 heads of 64, 27.3 -> 29.2;  15.6: 32 x 256, 12 heads of 64, 39.0 -> 37.0,
-//   but in a transformer block's step, whose weight gradients then have to wait for whole SMs, 503 -> 506 (the line lies above it);
-//   16: 8 x 576 35.7 -> 36.1;  20: 128 x 196, 6 heads of 64, 45.6 -> 44.6, of 32 38.5 -> 38.9, 8 x 4 200 in containers 33.9 -> 33.3;
-//   32: 16 x 576 58.3 -> 53.1;  40: 128 x 196, 12 heads, 55.5 -> 52.0;  60: 1 x 4 200, 8 heads of 32, 34.2 -> 29.4;
+//   but in a transformer block's step, whose weight gradients then wait for whole SMs, 503 -> 506;  16: 8 x 576 35.7 -> 36.1;
+//   20: 128 x 196, 6 heads of 64, 45.6 -> 44.6 (a transformer block's step 538 -> 544), of 32 38.5 -> 38.9, 8 x 4 200 in
+//   containers 33.9 -> 33.3;  the line;  32: 16 x 576 58.3 -> 53.1;  40: 128 x 196, 12 heads, 55.5 -> 52.0;  60: 1 x 4 200, 8 heads of 32, 34.2 -> 29.4;
 //   900: 16 x 4 200 210.6 -> 175.7.
 bool attention_bwd_kv_applies(const spa_params& p, int n_seg) {
   const long long items = (long long)p.H * ((p.capacity + 127) / 128);
   const long long segment = p.capacity / (n_seg > 0 ? n_seg : 1);
-  return items * (128 + segment) >= 17ll * 128 * kNumSMs;
+  return items * (128 + segment) >= 24ll * 128 * kNumSMs;
 }
 
 int launch_attention_bwd_kv(const spa_params& p, const void* qkv, const float* lse, const float* delta, const void* dao,
