@@ -552,7 +552,8 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm, const int32_t* seg, i
 // fp32 values in registers and when its bf16 operands are in TMEM.
 // The bf16 operands have TMEM columns of their own, so the next tile's fp32 products are issued as soon as
 // the current ones are in registers and run under the arithmetic.  That needs room in TMEM: this kernel serves
-// the dQ pass and the dK/dV pass at d = 32; the dK/dV pass at d = 64 is attn_bwd_kv_split_kernel below.
+// the dQ pass and the dK/dV pass at d = 32; the dK/dV pass at d = 64 is attn_bwd_kv_split_kernel below.  Large problems run
+// the dK/dV pass in attn_bwd_kv.cu.
 constexpr int kBwdMath = 256;      // arithmetic threads: two per TMEM lane (row)
 constexpr int kBwdThreads = kBwdMath + 32;
 constexpr int kBwdY = 64;          // rows of a streamed tile
