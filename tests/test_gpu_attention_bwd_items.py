@@ -15,10 +15,10 @@ pytestmark = pytest.mark.gpu
     (32, 8, 67200, [1680] + [0] * 3 + [210] * 40),          # empty segments
     (64, 12, 34000, [128] * 40 + [1] * 128 + [256, 384]),   # boundaries on the tiles; items of one tile
     (32, 16, 34000, [49] * 511),                            # the first item by one warp: the most segments
-    (64, 8, 34000, [49] * 512),                             # and one more
-    (32, 8, 34000, [5] * 2047),                             # staged offsets: the most
-    (64, 4, 80000, [5] * 2048 + [300] * 30),                # and one more
-    (32, 1, 140000, [3] * 40001),                           # more row tiles than are put in order
+    (64, 12, 34000, [49] * 512),                             # and one more
+    (32, 16, 34000, [5] * 2047),                             # staged offsets: the most
+    (64, 8, 80000, [5] * 2048 + [300] * 30),                # and one more
+    (32, 4, 140000, [3] * 40001),                           # more row tiles than are put in order
     (64, 2, 300, [100, 77, 123]),                           # too small: the other kernels
 ])
 def test_attention_backward_items(d, H, cap, lengths):
