@@ -13,6 +13,8 @@
 // 4 200 tokens, 8 heads of 32, forward 81.5 -> 46.1, backward 200.5 -> 151.8; 4 of 196 tokens, 3 heads of 32, 7.4 -> 7.2 and
 // 15.8 -> 14.4; 16 of 196, 6 heads of 64, 22.6 -> 21.7 and 76.2 -> 73.0; 64 of them 71.2 -> 68.8 and 256 -> 246.  What bounds it
 // then is shared memory: a vector read of 16 bytes per eight multiply-adds, 30 of the 75 TFLOP/s of the multiply-adds.
+// Errors against fp64 are smaller, the sums being two (4 000 rows of one segment, 2 heads of 64: outputs 1.18e-6 -> 8.6e-7,
+// gradients 1.25e-6 -> 9.6e-7; short segments 0.95 of before).
 #include <math_constants.h>
 
 #include "simt_stage.cuh"
