@@ -124,6 +124,15 @@ template <> __device__ __forceinline__ void store_row<float, 2>(float* dst, cons
 
 __device__ __forceinline__ void group_sync(int q) { asm volatile("bar.sync %0, %1;" ::"r"(q + 1), "n"(kGroup) : "memory"); }
 
+// The CTA's own rows are there, of which every thread has copied a part: kBehind is the number of copy groups that a thread
+// with a streamed tile has committed behind its part.  One without a tile has none behind it and waits for all it has:
+// counted like the others, its part could still be on its way behind the barrier.
+template <int kBehind> __device__ __forceinline__ void own_rows_landed(bool has_tile) {
+  if (has_tile) cp_async_wait<kBehind>();
+  else cp_async_wait<0>();
+  __syncthreads();
+}
+
 __device__ __forceinline__ float max16(float v) {
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -182,8 +191,7 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
   RowSeg mine[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) { m[i] = -CUDART_INF_F; mine[i] = seg_s[ty + kTY * i]; }
-  cp_async_wait<2>();
-  __syncthreads();  // Q, of which every thread has copied a part
+  own_rows_landed<2>(grp < n_tiles);  // Q; K and V of the first tile may be on their way
   for (int t = grp; t < n_tiles; t += kGroups) {
     cp_async_wait<1>();
     group_sync(grp);  // K; V is waited for behind the first product
@@ -347,8 +355,7 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
     }
   }
   float acc1[4][W] = {}, acc2[4][W] = {};  // dQ | dK and dV
-  cp_async_wait<1>();
-  __syncthreads();  // the own rows, of which every thread has copied a part
+  own_rows_landed<1>(grp < n_tiles);
   for (int t = grp; t < n_tiles; t += kGroups) {
     cp_async_wait<0>();
     group_sync(grp);

@@ -25,3 +25,26 @@ def test_no_load_can_move_above_the_wait_for_the_kernel_before(name):
         assert load == "volatile"
     # an array that one pass of a kernel writes and another only reads
     assert not re.search(r"__restrict__\s+delta\b", text)
+
+
+@pytest.mark.parametrize("kernel", ["attn_fwd_simt_kernel", "attn_bwd_simt_kernel"])
+@pytest.mark.parametrize("has_tile", [True, False])
+def test_own_rows_have_landed_before_the_barrier_that_publishes_them(kernel, has_tile):
+    """fp32 attention: a thread's own rows are its oldest group of asynchronous copies.  The wait in front of the barrier leaves
+    the newest n groups in flight, which must not be all that a thread without a streamed tile (segments of one) has."""
+    text = code("attn_simt.cu")
+    body = text[text.index(kernel + "("):]
+    body = body[:body.index("for (int t = grp; t < n_tiles")]
+    staging = re.search(r"auto stage = \[&\]\(int t\) \{(.*?)\n  \};", body, re.S)
+    assert body[:staging.start()].count("cp_async_commit();") == 1
+    rest = body[staging.end():]
+    assert len(re.findall(r"if \(grp < n_tiles\) stage\(grp\);", rest)) == 1 and "cp_async_commit" not in rest
+    committed = 1 + (staging.group(1).count("cp_async_commit();") if has_tile else 0)
+    helper = re.search(r"void own_rows_landed\(bool has_tile\) \{(.*?)\n\}", text, re.S)
+    if helper:
+        branch = re.sub(r"\s+", " ", helper.group(1)).strip()
+        assert branch == "if (has_tile) cp_async_wait<kBehind>(); else cp_async_wait<0>(); __syncthreads();"
+    left = None
+    for wait in re.finditer(r"cp_async_wait<(\d)>\(\);|own_rows_landed<(\d)>\(grp < n_tiles\);", rest):
+        left = int(wait.group(1)) if wait.group(1) else int(wait.group(2)) if has_tile else 0
+    assert left is not None and left < committed
