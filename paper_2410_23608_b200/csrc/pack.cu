@@ -235,71 +235,73 @@ row_scatter_kernel(const uint4* src16, const uint4* addp, const int32_t* idx,
   }
 }
 
-// Transpose of the unpack: one pass over dY; selected rows go to dz, the others to dX.  A warp has kBwdRows rows, as in the
-// gate kernel: their chunks are read before it is known where they go, so the look-up of the rows' places runs beside them instead of in
-// front of each.  Alone, us: 16 x 4 200 rows of 256 channels 14.5 -> 12.9, 32 x 576 of 768 12.8 -> 11.4, 128 x 196 of 768 16.4 -> 15.5,
-// 64 x 196 of 384 4.9 -> 4.6, 1 x 3 901 of 256 3.1 -> 2.3; 96 x 4 200 of 64 23.8 -> 18.6 (the first three at 0.8 of the copy bandwidth, launch apart).
-constexpr int kBwdRows = 4;
+// Transpose of the unpack: one pass over dY; selected rows go to dz, the others to dX (unless that is dY or there is none).
+// Chunk k is (row k / Q, column k % Q), kLoads of them to a thread: the row's place and the chunk are read side by side, so
+// one round trip to memory is all that a small call takes, and what bounds a large one is memory.  us, with whole rows to a warp
+// (32 narrow ones or four wide ones) -> this: 784 rows of 96 fp32 channels 4.8 -> 1.6, 6 272 of 192 bf16 4.9 -> 2.1, 196 of 768 2.9 ->
+// 1.6, 12 544 of 384 4.4 -> 3.4, 8 192 of 768 5.9 -> 4.1, 18 432 of 768 7.6 -> 7.0, 25 088 of 768 11.0 -> 9.4, 67 200 of 256 8.7 ->
+// 8.6, 403 200 of 64 13.8 -> 12.9.
+template <int kLoads>
 __global__ void __launch_bounds__(kPackThreads)
-unpack_scatter_bwd_kernel(const uint4* dY16, const int32_t* inv,
-                          const int32_t* cu, int B, int capacity, int rows, int Q,
+unpack_scatter_bwd_kernel(const uint4* dY16, const int32_t* inv, const int32_t* cu, int B, int capacity, long long total, int Q,
                           uint4* __restrict__ dz16, uint4* dX16, bool copy_pass_through, bool copy_selected) {
   pdl_entry();
-  const int lane = threadIdx.x & 31, warp = blockIdx.x * (kPackThreads / 32) + (threadIdx.x >> 5);
-  const int n_warps = gridDim.x * (kPackThreads / 32);
-  const int Np = packed_rows(cu, B, capacity);
-  if (Q < 32) {  // rows shorter than a warp: 32 of them, chunk k of the 32 Q being (row k / Q, column k % Q)
-    for (int r0 = warp * 32; r0 < rows; r0 += n_warps * 32) {
-      int at = r0 + lane < rows ? ld_dep(inv + r0 + lane) : -1;
-      if (at >= Np) at = -1;
-      for (int k0 = lane; k0 < 32 * Q; k0 += 32 * kBwdRows) {
-        uint4 v[kBwdRows];
-        int r[kBwdRows];
+  constexpr int kStep = kPackThreads * kLoads;
+  const int Np = packed_rows(cu, B, capacity), tid = threadIdx.x;
+  for (long long first = (long long)blockIdx.x * kStep; first < total; first += (long long)gridDim.x * kStep) {
+    const long long row = first / Q;
+    const int col = (int)(first - row * Q) + tid;
+    const int n = total - first < kStep ? (int)(total - first) : kStep;
+    int at[kLoads], q[kLoads];
+    uint4 v[kLoads];
 #pragma unroll
-        for (int u = 0; u < kBwdRows; ++u) {
-          const int k = k0 + 32 * u;
-          r[u] = k / Q;
-          if (k < 32 * Q && r0 + r[u] < rows) v[u] = ld_stream16(dY16 + (size_t)r0 * Q + k);
-        }
-#pragma unroll
-        for (int u = 0; u < kBwdRows; ++u) {
-          const int k = k0 + 32 * u, place = __shfl_sync(0xffffffffu, at, r[u] & 31);
-          if (k >= 32 * Q || r0 + r[u] >= rows) continue;
-          if (place >= 0) dz16[(size_t)place * Q + (k - r[u] * Q)] = v[u];
-          if (place >= 0 ? copy_selected : copy_pass_through) dX16[(size_t)r0 * Q + k] = v[u];
-        }
+    for (int u = 0; u < kLoads; ++u) {
+      const int k = tid + u * kPackThreads, r = (col + u * kPackThreads) / Q;
+      q[u] = col + u * kPackThreads - r * Q;
+      at[u] = -1;
+      if (k < n) {
+        at[u] = ld_dep(inv + row + r);
+        if (copy_pass_through) v[u] = ld_stream16(dY16 + first + k);
       }
     }
-    return;
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      if (at[u] >= Np) at[u] = -1;
+      if (!copy_pass_through && at[u] >= 0) v[u] = ld_stream16(dY16 + first + tid + u * kPackThreads);
+    }
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int k = tid + u * kPackThreads;
+      if (at[u] >= 0) dz16[(size_t)at[u] * Q + q[u]] = v[u];
+      if (k < n && (at[u] >= 0 ? copy_selected : copy_pass_through)) dX16[first + k] = v[u];
+    }
   }
-  for (int r0 = warp * kBwdRows; r0 < rows; r0 += n_warps * kBwdRows) {
-    int at = -1;  // lane u < kBwdRows: the packed place of row r0 + u
-    if (lane < kBwdRows && r0 + lane < rows) at = ld_dep(inv + r0 + lane);
+}
+
+// The same where nothing goes to dX, for many rows of 32 chunks and more: kRows rows to a warp, which passes over those that
+// were not selected without a look at each of their chunks.
+constexpr int kRows = 2;
+__global__ void __launch_bounds__(kPackThreads)
+unpack_gather_kernel(const uint4* dY16, const int32_t* inv, const int32_t* cu, int B, int capacity, int rows, int Q,
+                     uint4* __restrict__ dz16) {
+  pdl_entry();
+  const int lane = threadIdx.x & 31, n_warps = gridDim.x * (kPackThreads / 32);
+  const int Np = packed_rows(cu, B, capacity);
+  for (long long r0 = (long long)(blockIdx.x * (kPackThreads / 32) + (threadIdx.x >> 5)) * kRows; r0 < rows; r0 += (long long)n_warps * kRows) {
+    int at = -1;  // lane u < kRows: the packed place of row r0 + u
+    if (lane < kRows && r0 + lane < rows) at = ld_dep(inv + r0 + lane);
     if (at >= Np) at = -1;
-    int place[kBwdRows];
-    bool read[kBwdRows];
+    int place[kRows];
 #pragma unroll
-    for (int u = 0; u < kBwdRows; ++u) read[u] = r0 + u < rows;
-    if (!copy_pass_through) {
+    for (int u = 0; u < kRows; ++u) place[u] = __shfl_sync(0xffffffffu, at, u);
+    for (int q = lane; q < Q; q += 32) {
+      uint4 v[kRows];
 #pragma unroll
-      for (int u = 0; u < kBwdRows; ++u) read[u] = __shfl_sync(0xffffffffu, at, u) >= 0;
-    }
-    for (int q0 = 0; q0 < Q; q0 += 32) {
-      const int q = q0 + lane;
-      uint4 v[kBwdRows];
+      for (int u = 0; u < kRows; ++u)
+        if (place[u] >= 0) v[u] = ld_stream16(dY16 + (size_t)(r0 + u) * Q + q);
 #pragma unroll
-      for (int u = 0; u < kBwdRows; ++u)
-        if (read[u] && q < Q) v[u] = ld_stream16(dY16 + (size_t)(r0 + u) * Q + q);
-      if (q0 == 0) {
-#pragma unroll
-        for (int u = 0; u < kBwdRows; ++u) place[u] = __shfl_sync(0xffffffffu, at, u);
-      }
-#pragma unroll
-      for (int u = 0; u < kBwdRows; ++u) {
-        if (!read[u] || q >= Q) continue;
+      for (int u = 0; u < kRows; ++u)
         if (place[u] >= 0) dz16[(size_t)place[u] * Q + q] = v[u];
-        if (place[u] >= 0 ? copy_selected : copy_pass_through) dX16[(size_t)(r0 + u) * Q + q] = v[u];
-      }
     }
   }
 }
@@ -329,7 +331,6 @@ copy_chunks_kernel(const uint4* src16, uint4* __restrict__ dst16, long long tota
 }
 
 template <typename T> int chunks_per_row(int C) { return C / Vec16<T>::kElems; }
-
 
 // ------------------------------------------------------------------------------ container cuts
 // Attention segments of the paper's fixed-length containers (Sec. 3.2 "Token Packing": the packed tokens fill
@@ -458,12 +459,27 @@ int launch_unpack_scatter_bwd(const spa_params& p, const void* dY, const int32_t
                               const int32_t* cu, void* dz, void* dX, cudaStream_t st) {
   (void)idx;
   const int Q = p.dtype == SPA_F32 ? chunks_per_row<float>(p.C) : chunks_per_row<__nv_bfloat16>(p.C);
-  const int rows = p.B * p.N, per_cta = kPackThreads / 32 * (Q < 32 ? 32 : kBwdRows);
-  int grid = (rows + per_cta - 1) / per_cta;
-  if (grid > kNumSMs * 8) grid = kNumSMs * 8;
-  const bool copy = dX != nullptr && dX != dY;
-  launch_pdl(unpack_scatter_bwd_kernel, grid < 1 ? 1 : grid, kPackThreads, 0, st, (const uint4*)dY, inv, cu, p.B, p.capacity,
-             rows, Q, (uint4*)dz, (uint4*)dX, copy, copy && (p.flags & SPA_FLAG_RESIDUAL) != 0);
+  const int rows = p.B * p.N;
+  const long long total = (long long)rows * Q;
+  const bool copy = dX != nullptr && dX != dY, copy_selected = copy && (p.flags & SPA_FLAG_RESIDUAL) != 0;
+  // Two chunks to a thread as long as all CTAs (eight per SM) are resident together, up to 12 544 rows of 384 bf16 channels: 3.3
+  // us, with four 3.8.  Beyond, four: 8 192 rows of 768 4.0 us, with two 4.3; 25 088 rows 9.2 and 10.1.  Where only selected rows are
+  // read, the kernel with whole rows takes over there: 67 200 rows of 256 channels 5.9 -> 5.1 us, 25 088 of 768 6.6 -> 5.2, but
+  // 8 192 of 768 3.8 -> 4.4.  (Four of those to a warp: 4.9, 6.0 and 5.1.)
+  const bool wide = !copy && Q >= 32;
+  auto grid = [&](long long n, int per_cta, int per_sm) {
+    const long long g = (n + per_cta - 1) / per_cta;
+    return (int)(g < 1 ? 1 : (g > per_sm * kNumSMs ? per_sm * kNumSMs : g));
+  };
+  if (total <= 8ll * kNumSMs * 2 * kPackThreads)
+    launch_pdl(unpack_scatter_bwd_kernel<2>, grid(total, 2 * kPackThreads, 8), kPackThreads, 0, st, (const uint4*)dY, inv, cu, p.B,
+               p.capacity, total, Q, (uint4*)dz, (uint4*)dX, copy, copy_selected);
+  else if (!wide)
+    launch_pdl(unpack_scatter_bwd_kernel<4>, grid(total, 4 * kPackThreads, 16), kPackThreads, 0, st, (const uint4*)dY, inv, cu, p.B,
+               p.capacity, total, Q, (uint4*)dz, (uint4*)dX, copy, copy_selected);
+  else
+    launch_pdl(unpack_gather_kernel, grid(rows, kPackThreads / 32 * kRows, 16), kPackThreads, 0, st, (const uint4*)dY, inv, cu, p.B,
+               p.capacity, rows, Q, (uint4*)dz);
   SPA_CUDA_CHECK_LAUNCH("unpack_scatter_bwd_kernel");
   return SPA_OK;
 }

@@ -47,3 +47,37 @@ def test_pack_and_its_transposes_move_rows(B, N, C, dtype, keep, flag):
         else:
             assert torch.equal(dX[mask == 0], dY[mask == 0])
             assert torch.equal(dX[mask == 1], dY[mask == 1]) if flag else bool((dX[mask == 1] == 7).all())
+
+
+@pytest.mark.parametrize("rows,C,dtype,keep,flag", [
+    (7, 8, "bf16", 0.5, 0),                  # one chunk a row: every chunk of a thread in another row
+    (784, 96, "f32", 0.3, 0),                # 24 chunks a row: rows across warps and CTAs
+    (301, 8192, "f32", 0.4, "RESIDUAL"),     # 2 048 chunks a row: longer than a CTA's step
+    (18944, 256, "bf16", 0.3, 0),            # two chunks a thread: the most
+    (18945, 256, "bf16", 0.3, "RESIDUAL"),   # four, and whole rows to a warp where nothing is copied
+    (15001, 328, "bf16", 0.6, 0),            # 41 chunks a row: a warp's second pass is partly empty
+    (86017, 56, "bf16", 0.2, 0),             # 7 chunks a row
+    (42000, 1024, "bf16", 0.1, 0),           # more than one step for a CTA
+])
+def test_transpose_of_the_unpacking(rows, C, dtype, keep, flag):
+    from paper_2410_23608_b200 import binding as L
+    T = torch.float32 if dtype == "f32" else torch.bfloat16
+    p = L.make_params(1, rows, C, 1, dtype, rows, getattr(L, "SPA_FLAG_" + flag) if flag else 0)
+    g = torch.Generator(device="cuda").manual_seed(rows + C)
+    dY = torch.randn(rows, C, generator=g, device="cuda").to(T)
+    sel = torch.rand(rows, generator=g, device="cuda") < keep
+    Np = int(sel.sum())
+    for n_valid in (Np, Np - Np // 3):                      # all packed rows, and fewer than the places say
+        inv = torch.where(sel, sel.cumsum(0) - 1, -1).int()
+        cu = torch.tensor([0, n_valid], dtype=torch.int32, device="cuda")
+        taken = sel & (inv < n_valid)
+        for target in ("dX", "dY", None):
+            d, dz = dY.clone(), torch.full((rows, C), 7, device="cuda", dtype=T)
+            dX = torch.full((rows, C), 7, device="cuda", dtype=T) if target == "dX" else d if target else None
+            L.spa_unpack_scatter_bwd(p, d, None, inv, cu, dz, dX)
+            torch.cuda.synchronize()
+            assert torch.equal(dz[:n_valid], dY[taken]) and bool((dz[n_valid:] == 7).all())
+            assert torch.equal(d, dY)
+            if target == "dX":
+                assert torch.equal(dX[~taken], dY[~taken])
+                assert torch.equal(dX[taken], dY[taken]) if flag else bool((dX[taken] == 7).all())
