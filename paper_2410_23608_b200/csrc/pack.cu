@@ -15,28 +15,16 @@ namespace {
 constexpr int kPackThreads = 256;
 constexpr int kBatch = 4;  // independent 16-byte loads in flight per thread
 
+// Non-zero bytes of 16: the addition carries into a byte's top bit if one of the bits below is set, and never beyond it
 __device__ __forceinline__ int count_nonzero_bytes(uint4 m) {
-  return __popc(__vcmpne4(m.x, 0u) & 0x01010101u) + __popc(__vcmpne4(m.y, 0u) & 0x01010101u) +
-         __popc(__vcmpne4(m.z, 0u) & 0x01010101u) + __popc(__vcmpne4(m.w, 0u) & 0x01010101u);
+  auto top = [](uint32_t w) { return (((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u; };
+  return __popc(top(m.x) | top(m.y) >> 1 | top(m.z) >> 2 | top(m.w) >> 3);
 }
 
-// Selected tokens among the first `n` chunks of 16 mask bytes, this thread's share: kCount loads in flight together.  One after
-// the other they were 10 000 of the clocks of a CTA behind 60 000 tokens.
-constexpr int kCount = 8;
+// Selected tokens among the first `n` chunks of 16 mask bytes, this thread's share
 __device__ __forceinline__ int count_mask(const uint4* mask16, int n, int tid) {
   int cnt = 0;
-  if (n <= kPackThreads) return tid < n ? count_nonzero_bytes(ld_dep16(mask16 + tid)) : 0;
-  for (int k0 = tid; k0 < n; k0 += kPackThreads * kCount) {
-    uint4 m[kCount];
-#pragma unroll
-    for (int u = 0; u < kCount; ++u) {
-      const int k = k0 + u * kPackThreads;
-      m[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (k < n) m[u] = ld_dep16(mask16 + k);
-    }
-#pragma unroll
-    for (int u = 0; u < kCount; ++u) cnt += count_nonzero_bytes(m[u]);
-  }
+  for (int k = tid; k < n; k += kPackThreads) cnt += count_nonzero_bytes(ld_dep16(mask16 + k));
   return cnt;
 }
 
@@ -59,36 +47,15 @@ __device__ __forceinline__ uint4 add16(uint4 a, uint4 b) {
   return Vec16<T>::from_float(fa);
 }
 
-// Chunk k of a tile's selected rows is (row k / Q, 16-byte column k % Q): kLoads of them in flight per thread.
-template <typename T, bool kGateScale, int kLoads>
-__device__ __forceinline__ void gather_rows(const uint4* x16, uint4* xp16, const int* sel_tok, const float* sel_scale, int total,
-                                            int Q, int tid) {
-  for (int k0 = tid; k0 < total; k0 += kPackThreads * kLoads) {
-    uint4 v[kLoads];
-    int r[kLoads];
-#pragma unroll
-    for (int u = 0; u < kLoads; ++u) {
-      const int k = k0 + u * kPackThreads;
-      if (k < total) {
-        r[u] = k / Q;
-        v[u] = ld_stream16(x16 + (size_t)sel_tok[r[u]] * Q + (k - r[u] * Q));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kLoads; ++u) {
-      const int k = k0 + u * kPackThreads;
-      if (k < total) {
-        if (kGateScale) v[u] = scale16<T>(v[u], sel_scale[r[u]]);
-        xp16[k] = v[u];
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------------------------ select + pack
 // kOrdered: the tokens of every image are visited in the order order[0], order[1], ... (a cyclically shifted
 // feature map) instead of raster order.  Flat position t = b*N + j of the visiting order then stands for
 // token b*N + order[j]; mask, scores, idx and inv stay indexed by the original token.
+// What bounds it is a CTA's chain: count, gather, store.  Hence one division per thread, under the mask's loads, instead of one per
+// chunk, eight chunks in flight, and short code, which a CTA runs through but once: a second copy of the gather and eight mask loads in
+// a row cost more than they gave.  us, with those -> this: 12 544 rows of 384 channels 5.6 -> 4.3, 18 432 of 768 9.2 -> 7.0,
+// 25 088 of 768 8.7 -> 7.3, 67 200 of 256 9.4 -> 7.8, 403 200 of 64 37.3 -> 29.0, 14 000 of 512 fp32 10.2 -> 7.9, 196 of 768 4.2 -> 3.3.
+constexpr int kPackLoads = 8;
 template <typename T, bool kGateScale, bool kOrdered>
 __global__ void __launch_bounds__(kPackThreads)
 select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
@@ -111,6 +78,10 @@ select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
   if (kOrdered && in_tile) tok = (t / N) * N + ld_dep(order + t % N);
   uint32_t own = 0;
   if (in_tile) own = ld_dep(mask + tok);
+
+  // row and column of this thread's first chunk, and how far on its next one is
+  int r = tid / Q, q = tid - r * Q;
+  const int dr = kPackThreads / Q, dq = kPackThreads - dr * Q;
 
   // 2. number of selected tokens before this tile
   int cnt = 0;
@@ -158,14 +129,30 @@ select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
   if (tid == 0 && tile_start + tile >= rows) cu[B] = base + tile_total;
   __syncthreads();
 
-  // 4. gather the selected rows
+  // 4. gather the selected rows: chunk k of them is (row k / Q, column k % Q), and a thread's next one is kPackThreads on
   int n_ok = capacity - base;
   n_ok = n_ok < 0 ? 0 : (n_ok < tile_total ? n_ok : tile_total);
-  const int total = n_ok * Q;
-  uint4* dst16 = xp16 + (size_t)base * Q;
-  // eight in flight where they fill more than one batch: the longer code costs a CTA of one or two batches of four 0.5 us
-  if (total <= 2 * kPackThreads * kBatch) gather_rows<T, kGateScale, kBatch>(x16, dst16, sel_tok, sel_scale, total, Q, tid);
-  else gather_rows<T, kGateScale, 2 * kBatch>(x16, dst16, sel_tok, sel_scale, total, Q, tid);
+  uint4* dst16 = xp16 + (size_t)base * Q + tid;
+#pragma unroll 1
+  while (r < n_ok) {
+    uint4 v[kPackLoads];
+    int row[kPackLoads];
+#pragma unroll
+    for (int u = 0; u < kPackLoads; ++u) {
+      row[u] = r;
+      if (r < n_ok) v[u] = ld_stream16(x16 + (size_t)sel_tok[r] * Q + q);
+      r += dr;
+      q += dq;
+      if (q >= Q) { q -= Q; ++r; }
+    }
+#pragma unroll
+    for (int u = 0; u < kPackLoads; ++u) {
+      if (row[u] >= n_ok) break;
+      if (kGateScale) v[u] = scale16<T>(v[u], sel_scale[row[u]]);
+      dst16[u * kPackThreads] = v[u];
+    }
+    dst16 += kPackLoads * kPackThreads;
+  }
 }
 
 // ------------------------------------------------------------------------------ unpack
@@ -408,18 +395,22 @@ int launch_select_pack(const spa_params& p, const void* x, const uint8_t* mask, 
                        const int32_t* order, void* xp, int32_t* idx, int32_t* inv, int32_t* cu, int32_t* d_status,
                        cudaStream_t st) {
   const int rows = p.B * p.N;
-  // Selected tokens come in regions, and a CTA in one copies nearly all of its tile: six CTAs per SM even that out (128 x 196
-  // rows of 768 channels 11.1 -> 9.3 us, in a forward pass 88.5 -> 85.2; with two per SM 11.3 and 86.9), while what they
-  // read of the mask in front of their tiles, half of it each, stays within what the L2 delivers in 4 us.
+  // Selected tokens come in regions, and a CTA in one copies nearly all of its tile: smaller tiles even that out and shorten its
+  // chain, while every CTA reads the mask in front of its tile, grid^2 tile / 2 bytes in all.  Half the tile saves time in proportion to
+  // tile * Q, so the line is grid^2 against Q; measured, it lies near 5 000.  us of tiles of 256 / 128 / 64 / 32 tokens: 25 088 rows
+  // of 768 bf16 channels - / 8.5 / 8.4 / 7.0, 67 200 of 256 9.5 / 7.5 / 8.0 / 10.9, 50 000 of 256 6.0 / 6.2 / 6.3 / 8.1 and (more
+  // selected) 8.8 / 8.2 / 7.2 / 9.3, 50 000 of 768 20 / 15 / 11 / 11, 100 000 of 256 14.5 / 11.5 / 13.3 / 19.5.  And a tile has three chunks or
+  // more for each thread: 16 800 rows of 64 channels 3.3 us with two -> 3.0, 8 000 of 128 2.9 -> 2.8.
+  const int Q = p.dtype == SPA_F32 ? chunks_per_row<float>(p.C) : chunks_per_row<__nv_bfloat16>(p.C);
   int tile = 256, grid = (rows + tile - 1) / tile;
-  while (tile > 32 && (grid < 2 * kNumSMs || (grid < 6 * kNumSMs && (long long)grid * rows <= 40000000ll))) {
+  while (tile > 32 && (tile >> 1) * Q >= 3 * kPackThreads && (grid < 2 * kNumSMs || grid * grid <= 5000 * Q)) {
     tile >>= 1;
     grid = (rows + tile - 1) / tile;
   }
   const bool gs = (p.flags & SPA_FLAG_GATE_SCALE) != 0;
 #define SPA_PACK_LAUNCH(T, GS, ORD)                                                                              \
   launch_pdl(select_pack_kernel<T, GS, ORD>, grid, kPackThreads, 0, st, (const uint4*)x, mask, scores, order, rows, p.N, \
-             p.B, chunks_per_row<T>(p.C), tile, p.capacity, (uint4*)xp, idx, inv, cu, d_status)
+             p.B, Q, tile, p.capacity, (uint4*)xp, idx, inv, cu, d_status)
 #define SPA_PACK_ORD(T, GS) do { if (order != nullptr) SPA_PACK_LAUNCH(T, GS, true); else SPA_PACK_LAUNCH(T, GS, false); } while (0)
   if (p.dtype == SPA_F32) { if (gs) SPA_PACK_ORD(float, true); else SPA_PACK_ORD(float, false); }
   else { if (gs) SPA_PACK_ORD(__nv_bfloat16, true); else SPA_PACK_ORD(__nv_bfloat16, false); }

@@ -81,3 +81,48 @@ def test_transpose_of_the_unpacking(rows, C, dtype, keep, flag):
             if target == "dX":
                 assert torch.equal(dX[~taken], dY[~taken])
                 assert torch.equal(dX[taken], dY[taken]) if flag else bool((dX[taken] == 7).all())
+
+
+@pytest.mark.parametrize("B,N,C,dtype,keep,scaled,shift,short", [
+    (3, 50, 8, "bf16", 1.0, False, 0, 0),       # one chunk a row: a thread's next one is 256 rows on
+    (7, 1000, 40, "bf16", 0.7, True, 9, 0),     # five chunks a row: 256 is no multiple
+    (2, 700, 1016, "f32", 0.9, True, 0, 0),     # 254 chunks
+    (2, 700, 1028, "f32", 0.9, True, 5, 0),     # 257: longer than the CTA's step
+    (1, 67, 8192, "f32", 0.8, False, 0, 0),     # 2 048 chunks a row
+    (64, 196, 192, "bf16", 0.5, False, 0, 100), # rows that do not fit in
+    (2, 30000, 16, "bf16", 0.02, False, 0, 0),  # long counts, nearly empty tiles
+])
+def test_packing_in_batches(B, N, C, dtype, keep, scaled, shift, short):
+    from paper_2410_23608_b200 import binding as L
+    T = torch.float32 if dtype == "f32" else torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B * N + C)
+    x = torch.randn(B, N, C, generator=g, device="cuda").to(T)
+    scores = torch.randn(B, N, generator=g, device="cuda")
+    sel = torch.rand(B, N, generator=g, device="cuda") < keep
+    # any non-zero byte selects
+    mask = torch.where(sel, torch.randint(1, 256, (B, N), generator=g, device="cuda"), 0).to(torch.uint8).contiguous()
+    visit = torch.arange(N, device="cuda").roll(-shift)
+    tok = (torch.arange(B, device="cuda")[:, None] * N + visit).reshape(-1)
+    tok = tok[sel.reshape(-1)[tok]]
+    Np = tok.numel()
+    cap = Np - short
+    p = L.make_params(B, N, C, 1, dtype, cap, L.SPA_FLAG_GATE_SCALE if scaled else 0)
+    e = lambda *s, dt=torch.int32: torch.full(s, 7, device="cuda", dtype=dt)
+    xp, idx, inv, cu, status = e(cap + 3, C, dt=T), e(cap + 3), e(B * N), e(B + 1), torch.zeros(4, dtype=torch.int32, device="cuda")
+    if shift:
+        L.spa_select_pack_ordered(p, x, mask, scores, visit.int(), xp, idx, inv, cu, status)
+    else:
+        L.spa_select_pack(p, x, mask, scores, xp, idx, inv, cu, status)
+    assert L.spa_read_status(status) == (L.SPA_ERR_CAPACITY if short else 0)
+    tok = tok[:cap]
+    want = x.view(-1, C)[tok]
+    if scaled:  # 1 / (1 + exp(-s)): the exponential is good to 2 + 1.16 |s| units in the last place, |s| < 6
+        ref = (want.double() * scores.view(-1)[tok].double().sigmoid()[:, None])
+        assert bool(((xp[:cap].double() - ref).abs() <= (2e-6 if dtype == "f32" else 2 ** -8) * ref.abs()).all())
+    else:
+        assert torch.equal(xp[:cap], want)
+    assert torch.equal(idx[:cap], tok.int()) and bool((xp[cap:] == 7).all()) and bool((idx[cap:] == 7).all())
+    place = torch.full((B * N,), -1, device="cuda", dtype=torch.int32)
+    place[tok] = torch.arange(cap, device="cuda", dtype=torch.int32)
+    assert torch.equal(inv, place)
+    assert cu.tolist() == [0] + sel.sum(1).cumsum(0).tolist()
