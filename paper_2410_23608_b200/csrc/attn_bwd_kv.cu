@@ -518,6 +518,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
         ptx::tmem_ld_32x32(lane_base + kColDP + col0, rp);  // by the whole warp: the load is a collective
         ptx::tmem_ld_wait();
         ptx::tc_fence_before_sync();
+        __syncwarp();
         if (lane == 0) ptx::mbar_arrive(bar_dpfree);
         if (some) {
           if (partial) {

@@ -48,3 +48,11 @@ def test_own_rows_have_landed_before_the_barrier_that_publishes_them(kernel, has
     for wait in re.finditer(r"cp_async_wait<(\d)>\(\);|own_rows_landed<(\d)>\(grp < n_tiles\);", rest):
         left = int(wait.group(1)) if wait.group(1) else int(wait.group(2)) if has_tile else 0
     assert left is not None and left < committed
+
+
+@pytest.mark.parametrize("name", FILES)
+def test_a_warp_comes_together_before_one_lane_arrives_for_it(name):
+    """An arrival orders what its own thread did.  What the other lanes did (loads of TMEM that the next product overwrites, stores
+    that it reads) is ordered by the barrier among them in front of it."""
+    for before in re.findall(r"([^;{}]*[;{}])\s*if \(lane == 0\) \{?\s*ptx::mbar_arrive\(", code(name)):
+        assert re.fullmatch(r"\s*(__syncwarp\(\)|ptx::named_barrier\([^;]*\));", before), before
