@@ -69,3 +69,37 @@ def test_attention_backward_items(d, H, cap, lengths):
     for _ in range(20):
         gr.replay()
     assert torch.equal(check(), first)
+
+
+@pytest.mark.parametrize("d,H", [(64, 12), (32, 16)])
+@pytest.mark.parametrize("rows", [129, 300, 320, 384])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_what_is_not_finite_stays_with_the_tiles_of_its_image(d, H, rows, bad):
+    """dK and dV of 128 packed rows read the images that have rows among them, and no row behind those images."""
+    from paper_2410_23608_b200 import binding as L
+    C, cap, lengths = H * d, 34000, [rows, 500, 128 * 4 - (rows + 500) % 128, 777]
+    Np = sum(lengths)
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    qkv = torch.randn(cap, 3 * C, generator=g, device="cuda").to(torch.bfloat16)
+    dao = torch.randn(cap, C, generator=g, device="cuda").to(torch.bfloat16)
+    ao, lse = torch.empty(cap, C, device="cuda", dtype=torch.bfloat16), torch.empty(H, cap, device="cuda")
+    cu = torch.tensor([0] + lengths, device="cuda").cumsum(0).int()
+    p = L.make_params(1, cap, C, H, "bf16", cap)
+    ws = torch.empty(max(L.spa_workspace_bytes(p), 256), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    L.spa_packed_attention_fwd(p, qkv, cu, 4, ao, lse, status)
+
+    def backward():
+        out = torch.empty(cap, 3 * C, device="cuda", dtype=torch.bfloat16)
+        L.spa_packed_attention_bwd(p, qkv, ao, lse, dao, cu, 4, out, ws, status)
+        assert L.spa_read_status(status) == 0
+        return out[:Np, C:]
+
+    want = backward()
+    bad_rows = slice(rows, rows + 500)                      # the second image
+    dao[bad_rows] = bad
+    got = backward()
+    alone = torch.ones(Np, dtype=torch.bool, device="cuda")
+    alone[rows // 128 * 128:(rows + 500 + 127) // 128 * 128] = False
+    assert torch.equal(got[alone], want[alone])
+    assert not bool(torch.isfinite(got[bad_rows]).any())
