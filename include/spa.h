@@ -57,8 +57,9 @@ enum {
   SPA_FLAG_NO_CTA_PAIRS = 16,/* wide linear layers: keep the one-CTA tensor-core kernels (no CTA pairs) */
   SPA_FLAG_UNFUSED = 32,  /* spa_block_fwd / spa_block_bwd: separate projection, scatter and gather kernels even
                              where the fused calls apply                                                      */
-  SPA_FLAG_SHORT_WAITS = 128, /* diagnostics: the device-side waits of the linear layers' tensor-core kernels give up at the
-                             first poll that fails, so that a test sees what a wait that ran out leaves behind        */
+  SPA_FLAG_SHORT_WAITS = 128, /* diagnostics: the device-side waits of the linear layers' tensor-core kernels and of the
+                             attention backward's dK/dV pipeline (large problems) give up at the first poll that fails,
+                             so that a test sees what a wait that ran out leaves behind                               */
   SPA_FLAG_ONE_PASS_BWD = 64 /* attention backward (tensor-core problems): segments of at most 128 rows are handled by
                              a kernel that owns a whole segment and evaluates S, P, dP, dS once; the two-pass kernels
                              take the longer segments only.  Same results within the stated tolerances               */

@@ -50,7 +50,8 @@ template <int D>
 __global__ void __launch_bounds__(kKvThreads, 1)
 attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_constant__ CUtensorMap tm_do, const float* lse,
                    const float* delta, const int32_t* seg, int n_seg, int capacity, int C, int H, float scale,
-                   __nv_bfloat16* __restrict__ dqkv, bool skip_short, unsigned* counter, bool even_items, int32_t* d_status) {
+                   __nv_bfloat16* __restrict__ dqkv, bool skip_short, unsigned* counter, bool even_items, uint32_t wait_limit,
+                   int32_t* d_status) {
   using HT = HeadTile<D>;
   using SM = KvSmem<D>;
   constexpr int kTile = SM::kTile, kStages = SM::kStages;
@@ -75,7 +76,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   // phase of one barrier completing under a wait for the first would look like neither
   auto bar_ds = [&](int g, int grp) { return bar + 128 + 16 * (g & 1) + 8 * grp; };
   const uint32_t bar_order = bar + 176;   // 16: the order of the items is there
-  const uint32_t bar_drain = bar + 184;   // only behind a wait that gave up
+  const uint32_t bar_drain = bar + 184;   // 3: the products of an issuing warp have completed, all of them
   auto bar_y = [&](int st) { return bar + 192 + 8 * st; };   // 2: copies of a stage have landed, its statistics are there
   auto bar_free = [&](int st) { return bar + 240 + 8 * st; };  // the products that read a stage have completed
   const uint32_t tmem_slot = bar + 288, abort_any = bar + 292;
@@ -160,17 +161,18 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   ptx::tc_fence_after_sync();
   const uint32_t tmem = (uint32_t)ptx::lds_s32(tmem_slot);
   // Bounded; nobody branches on a wait that gave up inside an item (see mbar_wait_or_abort)
-  auto wait = [&](uint32_t b, uint32_t parity) { return ptx::mbar_wait_or_abort_warp(b, parity, abort_any, d_status, SPA_ERR_TIMEOUT); };
+  auto wait = [&](uint32_t b, uint32_t parity) { return ptx::mbar_wait_or_abort_warp(b, parity, abort_any, d_status, SPA_ERR_TIMEOUT, wait_limit); };
   const bool is_math = warp < kMathWarps;
   auto aborted = [&]() { return __any_sync(0xffffffffu, ptx::lds_s32(abort_any) != 0) != 0; };
+
+  int n = 0, filled = 0;  // items whose copies have been issued or looked at, tiles whose copies have been
 
   if (warp == kWarpLoad) {
     // ---------------------------------------------------------------- items, copies and statistics: one warp
     int own = blockIdx.x, drawn = blockIdx.x;
     if (draws && (int)blockIdx.x >= given && lane == 0) drawn = draw_item(counter, given, n_items, own);
     bool order_ready = false, ok = true;
-    int n = 0, st = 0, use = 0;  // items announced; stage of the next tile and how often it has been filled
-    int filled = 0;              // tiles whose copies have been issued
+    int st = 0, use = 0;  // stage of the next tile and how often it has been filled
     int v;
     auto wait_all = [&](uint32_t b, uint32_t parity) { ok = __all_sync(0xffffffffu, wait(b, parity)) != 0 && ok; };
     for (;;) {
@@ -284,14 +286,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
         ptx::mbar_arrive(bar_item(n));
       }
     }
-    if (aborted()) {
-      // copies in flight land before shared memory is released; the numbers drawn have to add up all the same
-      if (lane == 0) {
-        for (int i = filled > kStages ? filled - kStages : 0; i < filled; ++i) ptx::mbar_wait(bar_y(i % kStages), (i / kStages) & 1);
-        for (int i = n > 2 ? n - 2 : 0; i <= n; ++i) ptx::mbar_wait(bar_x(i), (i >> 1) & 1, 1u << 14);
-        while (draws && drawn < n_items) drawn = draw_item(counter, given, n_items, own);
-      }
-    }
+    while (draws && lane == 0 && drawn < n_items) drawn = draw_item(counter, given, n_items, own);  // after a wait that gave up: the numbers have to add up
     __syncwarp();
   } else if (!is_math) {
     // ---------------------------------------------------------------- products: three warps, whose lanes all follow the tiles
@@ -410,11 +405,8 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
         c = advance(c, c_first);
       }
     }
-    if (aborted()) {  // products in flight complete before their memory goes away
-      if (ptx::elect_one()) ptx::mma_commit(bar_drain);
-      __syncwarp();
-      ptx::mbar_wait(bar_drain, 0);
-    }
+    __syncwarp();
+    if (ptx::elect_one()) ptx::mma_commit(bar_drain);
     __syncwarp();
   } else {
     // ---------------------------------------------------------------- arithmetic: four threads per key row, two of each group.
@@ -460,7 +452,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(bar_drained(item));
     };
-    int g = 0, st = 0, n = 0;
+    int g = 0, st = 0;
     uint32_t use = 0;
     for (;; ++n) {
       wait(bar_item(n), (n >> 1) & 1);
@@ -570,7 +562,14 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
+  // Products complete before the CTA's memory goes, and so do copies, which have been waited for unless a wait gave up.  Here, because
+  // that may have been in a warp whose partners had left their loops in good order.
+  if (warp == kWarpLoad && aborted() && lane == 0) {
+    for (int i = filled > kStages ? filled - kStages : 0; i < filled; ++i) ptx::mbar_wait(bar_y(i % kStages), (i / kStages) & 1);
+    for (int i = n > 2 ? n - 2 : 0; i <= n; ++i) ptx::mbar_wait(bar_x(i), (i >> 1) & 1, 1u << 14);
+  }
   if (warp == kWarpS) {
+    ptx::mbar_wait(bar_drain, 0);
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem, 512);
   }
@@ -591,7 +590,8 @@ int kv_launch(const spa_params& p, const void* qkv, const float* lse, const floa
   const int grid = (int)(items < kNumSMs ? items : kNumSMs);
   const bool even_items = (long long)p.capacity <= 512ll * (n_seg > 0 ? n_seg : 1);  // as in the forward
   launch_pdl(kern, grid, kKvThreads, KvSmem<D>::kBytes, st, tm_qkv, tm_do, lse, delta, seg, n_seg, p.capacity, p.C, p.H,
-             softmax_scale_of(p), (__nv_bfloat16*)dqkv, skip_short, items > grid ? item_counter(dqkv) : nullptr, even_items, d_status);
+             softmax_scale_of(p), (__nv_bfloat16*)dqkv, skip_short, items > grid ? item_counter(dqkv) : nullptr, even_items,
+             ptx::wait_limit(p.flags), d_status);
   SPA_CUDA_CHECK_LAUNCH("attn_bwd_kv_kernel");
   return SPA_OK;
 }

@@ -35,3 +35,31 @@ def test_short_waits_leave_nothing_in_flight(rows, n_in, n_out, pairs):
         assert all(torch.equal(x, y) for x, y in zip(got, want))
     assert [L.spa_read_status(s) for s in clean] == [0, 0, 0]
     assert [L.spa_read_status(s) for s in expired] == [L.SPA_ERR_TIMEOUT] * 3
+
+
+# items drawn in order of length; given and drawn, one or two tiles each; one per CTA; two CTAs
+@pytest.mark.parametrize("d,H,cap,lengths", [(64, 12, 18432, [577, 58] * 9), (32, 16, 34000, [49] * 511), (64, 12, 34000, [700]),
+                                             (32, 2, 1 << 18, [100])])
+def test_short_waits_in_the_attention_backward(d, H, cap, lengths):
+    from paper_2410_23608_b200 import binding as L
+    C, Np, n_seg = H * d, sum(lengths), len(lengths)
+    g = torch.Generator(device="cuda").manual_seed(Np)
+    qkv = torch.randn(cap, 3 * C, generator=g, device="cuda").to(torch.bfloat16)
+    dao = torch.randn(cap, C, generator=g, device="cuda").to(torch.bfloat16)
+    ao, lse = torch.empty(cap, C, device="cuda", dtype=torch.bfloat16), torch.empty(H, cap, device="cuda")
+    cu = torch.tensor([0] + lengths, device="cuda").cumsum(0).int()
+    p, short = (L.make_params(1, cap, C, H, "bf16", cap, flags=f) for f in (0, L.SPA_FLAG_SHORT_WAITS))
+    ws = torch.empty(max(L.spa_workspace_bytes(p), 256), dtype=torch.uint8, device="cuda")
+    clean, expired = torch.zeros(4, dtype=torch.int32, device="cuda"), torch.zeros(4, dtype=torch.int32, device="cuda")
+    L.spa_packed_attention_fwd(p, qkv, cu, n_seg, ao, lse, clean)
+    out = torch.full((cap, 3 * C), 7.0, device="cuda", dtype=torch.bfloat16)
+    run = lambda p, status: L.spa_packed_attention_bwd(p, qkv, ao, lse, dao, cu, n_seg, out, ws, status)
+    run(p, clean)
+    want = out.clone()
+    for _ in range(10):
+        run(short, expired)
+        assert bool((out[Np:] == 7).all())
+        run(p, clean)                         # the same array: its items are counted from zero again
+        assert torch.equal(out, want)
+    assert L.spa_read_status(clean) == 0
+    assert L.spa_read_status(expired) == L.SPA_ERR_TIMEOUT
