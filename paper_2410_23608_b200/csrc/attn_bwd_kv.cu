@@ -19,7 +19,7 @@ namespace {
 //         over its own columns of S^T of tile g;
 //   dP^T  one buffer: issued as soon as the warps hold that of tile g in registers, under the exponentials of tile g + 1.
 // Sixteen arithmetic warps: four threads per key row, 32 of the 128 queries each, in two groups of eight that need not be in
-// step.  Three warps issue the products (S^T and dP^T | dV | dK): one for all of them was what the tiles waited for, 20 to 28
+// step.  Three warps issue the products (S^T and dP^T | dV | dK): one for all of them was what the tiles waited for, 20 or 24
 // products and seven waits in 2 800 clocks a tile.  The last warp draws the items, looks up their rows' segments, issues every
 // copy and stages the queries' statistics, up to kStages tiles and an item ahead.  A finished item's accumulators are
 // drained behind the exponentials of the next item's first tile, when the wait for its last products is over.

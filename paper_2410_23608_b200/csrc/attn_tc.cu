@@ -613,7 +613,6 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   constexpr int kStatBase = kYBase + kStages * 2 * kYTile;
   float* stat_lse = reinterpret_cast<float*>(smem_al + kStatBase);  // [3][64] -lse_i * log2e of the staged query tile
   float* stat_D = stat_lse + 3 * kBwdY;                              // [3][64] -D_i
-  const uint32_t stat_s = smem_base + kStatBase;
   constexpr int kBarBase = kStatBase + kBwdStatBytes;
   const uint32_t bar_base = smem_base + kBarBase;
   const uint32_t bar_x = bar_base, bar_s = bar_base + 56, bar_acc = bar_base + 64;
@@ -1842,8 +1841,8 @@ int launch_attention_fwd_tc(const spa_params& p, const void* qkv, const int32_t*
 // device, with that device current, and cached.
 static __device__ __align__(256) unsigned char g_static_scratch[SPA_STATIC_SCRATCH_BYTES];
 
-// Item counters of the attention forward kernel: zero when the library is loaded and after every launch.  A launch uses the
-// one that belongs to its output array: two launches that write the same array cannot run side by side, on whatever
+// Item counters of the attention forward kernel and of the backward's dK/dV pipeline, so up to two per block that is trained: zero
+// when the library is loaded and after every launch.  A launch uses the one that belongs to its output array: two launches that write the same array cannot run side by side, on whatever
 // streams or in whatever graphs they are.  (One per recorded launch, given back by a user object of its graph, made every
 // replay of the graph 40 to 100 us slower.)  An array keeps its counter while the library is loaded; the arrays past the
 // first 16 384 get none, and their launches stride over the items.

@@ -1,4 +1,4 @@
-"""Attention backward in one pipeline per CTA over all its items (attn_bwd_kv.cu, large problems): items given, strided, drawn
+"""Attention backward in one pipeline per CTA over all its items (attn_bwd_kv.cu, large problems): items given, drawn
 and put in order, one tile and many, offsets in shared memory and in global memory, and what the other kernels take."""
 import pytest
 import torch
@@ -18,7 +18,9 @@ pytestmark = pytest.mark.gpu
     (64, 12, 34000, [49] * 512),                             # and one more
     (32, 16, 34000, [5] * 2047),                             # staged offsets: the most
     (64, 8, 80000, [5] * 2048 + [300] * 30),                # and one more
-    (32, 4, 140000, [3] * 40001),                           # more row tiles than are put in order
+    (32, 4, 140000, [3] * 40001),                           # offsets in global memory, many row tiles
+    (64, 2, 80000, [300, 700] * 75 + [8]),                  # 512 drawn row tiles: the most that are put in order
+    (64, 2, 80000, [300, 700] * 75 + [9]),                  # and one more
     (64, 2, 300, [100, 77, 123]),                           # too small: the other kernels
 ])
 def test_attention_backward_items(d, H, cap, lengths):
