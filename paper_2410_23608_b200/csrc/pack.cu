@@ -55,8 +55,7 @@ __device__ __forceinline__ uint4 add16(uint4 a, uint4 b) {
 // chunk, eight chunks in flight, and short code, which a CTA runs through but once: a second copy of the gather and eight mask loads in
 // a row cost more than they gave.  us, with those -> this: 12 544 rows of 384 channels 5.6 -> 4.3, 18 432 of 768 9.2 -> 7.0,
 // 25 088 of 768 8.7 -> 7.3, 67 200 of 256 9.4 -> 7.8, 403 200 of 64 37.3 -> 29.0, 14 000 of 512 fp32 10.2 -> 7.9, 196 of 768 4.2 -> 3.3.
-constexpr int kPackLoads = 8;
-template <typename T, bool kGateScale, bool kOrdered>
+template <typename T, bool kGateScale, bool kOrdered, int kPackLoads>
 __global__ void __launch_bounds__(kPackThreads)
 select_pack_kernel(const uint4* x16, const uint8_t* mask, const float* scores,
                    const int32_t* order, int rows, int N, int B, int Q, int tile, int capacity,
@@ -397,25 +396,30 @@ int launch_select_pack(const spa_params& p, const void* x, const uint8_t* mask, 
   const int rows = p.B * p.N;
   // Selected tokens come in regions, and a CTA in one copies nearly all of its tile: smaller tiles even that out and shorten its
   // chain, while every CTA reads the mask in front of its tile, grid^2 tile / 2 bytes in all.  Half the tile saves time in proportion to
-  // tile * Q, so the line is grid^2 against Q; measured, it lies near 5 000.  us of tiles of 256 / 128 / 64 / 32 tokens: 25 088 rows
-  // of 768 bf16 channels - / 8.5 / 8.4 / 7.0, 67 200 of 256 9.5 / 7.5 / 8.0 / 10.9, 50 000 of 256 6.0 / 6.2 / 6.3 / 8.1 and (more
-  // selected) 8.8 / 8.2 / 7.2 / 9.3, 50 000 of 768 20 / 15 / 11 / 11, 100 000 of 256 14.5 / 11.5 / 13.3 / 19.5.  And a tile has three chunks or
-  // more for each thread: 16 800 rows of 64 channels 3.3 us with two -> 3.0, 8 000 of 128 2.9 -> 2.8.
+  // tile * Q, so from a CTA per SM on the line is grid^2 against Q; measured, it lies near 5 000.  us of tiles of 256 / 128 / 64 / 32
+  // tokens: 25 088 rows of 768 bf16 channels - / 8.5 / 8.4 / 7.0, 67 200 of 256 9.5 / 7.5 / 8.0 / 10.9, 50 000 of 256 6.0 / 6.2 / 6.3 /
+  // 8.1 and (more selected) 8.8 / 8.2 / 7.2 / 9.3, 50 000 of 768 20 / 15 / 11 / 11, 100 000 of 256 14.5 / 11.5 / 13.3 / 19.5, 16 800
+  // of 64 3.4 / 2.8 / 3.0 / 3.6.
   const int Q = p.dtype == SPA_F32 ? chunks_per_row<float>(p.C) : chunks_per_row<__nv_bfloat16>(p.C);
   int tile = 256, grid = (rows + tile - 1) / tile;
-  while (tile > 32 && (tile >> 1) * Q >= 3 * kPackThreads && (grid < 2 * kNumSMs || grid * grid <= 5000 * Q)) {
+  while (tile > 32 && (grid < kNumSMs || grid * grid <= 5000 * Q)) {
     tile >>= 1;
     grid = (rows + tile - 1) / tile;
   }
   const bool gs = (p.flags & SPA_FLAG_GATE_SCALE) != 0;
-#define SPA_PACK_LAUNCH(T, GS, ORD)                                                                              \
-  launch_pdl(select_pack_kernel<T, GS, ORD>, grid, kPackThreads, 0, st, (const uint4*)x, mask, scores, order, rows, p.N, \
+  // Eight chunks in flight where a full tile has six or more per thread and the SMs have two CTAs each to keep memory busy: 18 432 rows of 768
+  // channels 7.8 -> 6.9 us, 67 200 of 256 8.3 -> 7.5; below, the longer code only costs: 8 000 of 128 2.6 -> 2.9, 7 560 of 512 4.1 -> 4.3.
+  const bool deep = tile * Q >= 6 * kPackThreads && grid >= 2 * kNumSMs;
+#define SPA_PACK_LOADS(T, GS, ORD, LOADS)                                                                                 \
+  launch_pdl(select_pack_kernel<T, GS, ORD, LOADS>, grid, kPackThreads, 0, st, (const uint4*)x, mask, scores, order, rows, p.N, \
              p.B, Q, tile, p.capacity, (uint4*)xp, idx, inv, cu, d_status)
+#define SPA_PACK_LAUNCH(T, GS, ORD) do { if (deep) SPA_PACK_LOADS(T, GS, ORD, 8); else SPA_PACK_LOADS(T, GS, ORD, 4); } while (0)
 #define SPA_PACK_ORD(T, GS) do { if (order != nullptr) SPA_PACK_LAUNCH(T, GS, true); else SPA_PACK_LAUNCH(T, GS, false); } while (0)
   if (p.dtype == SPA_F32) { if (gs) SPA_PACK_ORD(float, true); else SPA_PACK_ORD(float, false); }
   else { if (gs) SPA_PACK_ORD(__nv_bfloat16, true); else SPA_PACK_ORD(__nv_bfloat16, false); }
 #undef SPA_PACK_ORD
 #undef SPA_PACK_LAUNCH
+#undef SPA_PACK_LOADS
   SPA_CUDA_CHECK_LAUNCH("select_pack_kernel");
   return SPA_OK;
 }
