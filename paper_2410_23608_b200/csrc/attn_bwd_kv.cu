@@ -80,7 +80,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   auto bar_y = [&](int st) { return bar + 192 + 8 * st; };   // 2: copies of a stage have landed, its statistics are there
   auto bar_free = [&](int st) { return bar + 240 + 8 * st; };  // the products that read a stage have completed
   const uint32_t tmem_slot = bar + 288, abort_any = bar + 292;
-  auto item_slot = [&](int item) { return bar + 304 + 16 * (item & 3); };   // {r0, h, first streamed row, tiles * 128 + back}
+  auto item_slot = [&](int item) { return bar + 304 + 16 * (item & 3); };   // {r0, h, first streamed row, tiles * 128 + over}
   auto row_s = [&](int item) { return smem_base + SM::kRows + (item & 3) * 1024; };
   int32_t* seg_s = reinterpret_cast<int32_t*>(smem_al + SM::kSeg);
   ItemOrder* order = reinterpret_cast<ItemOrder*>(smem_al + SM::kOrder);
@@ -228,12 +228,12 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
         hi = __reduce_max_sync(0xffffffffu, hi_rows);
       }
       const int n_tiles = hi > lo ? (hi - lo + 127) / 128 : 0;  // none: every row belongs to the one-pass kernel
-      // The last tile of several ends with the item's rows: `back` rows ahead of its turn, which its threads take for masked.  Rows
-      // behind it are another image's, and an infinity or NaN there times the zeros of P^T and dS^T would be NaN in this one's sums.
-      // (One tile alone has 128 rows of the item's own segments, or ends with the last valid row.)  Whole backward: containers of 49 rows, in
-      // which more threads then have a part of the last tile, 54.3 -> 55.2 us; one image of 4 200 rows, whose last tile needed its lines
-      // behind the last valid row cleared, 149.1 -> 143.7.
-      const int back = n_tiles > 1 ? lo + n_tiles * 128 - hi : 0;
+      // The last tile's `over` queries behind the item's segments are another image's, or no one's, and an infinity or NaN there times the
+      // zeros of P^T and dS^T would be NaN in this image's sums.  So the products that sum over queries leave out the groups of
+      // 16 that have none of the item's, and the rest of the group that has both is cleared in shared memory.
+      // (Whole backward: 16 segments of 210 to 1 680 rows, 8 heads of 32, 174.7 -> 168.6 us, one of 4 200 rows 148.8 -> 135.6, in
+      // containers of 49 54.2 -> 53.2: before, only lines behind the last valid row were cleared, all of them.)
+      const int over = n_tiles * 128 - (hi - lo);
       if (n_tiles > 0) {
         if (skip_short) load_own(n, r0, h);
         float sl[4], sd[4];  // statistics of the next tile's queries, on their way
@@ -250,23 +250,22 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
           ptx::sts_s32(item_slot(n), r0);
           ptx::sts_s32(item_slot(n) + 4, h);
           ptx::sts_s32(item_slot(n) + 8, lo);
-          ptx::sts_s32(item_slot(n) + 12, n_tiles * 128 + back);
+          ptx::sts_s32(item_slot(n) + 12, n_tiles * 128 + over);
         }
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(bar_item(n));
-        auto first_row = [&](int t) { return lo + t * 128 - (t == n_tiles - 1 ? back : 0); };
         for (int t = 0; t < n_tiles; ++t) {
           if (t == n_tiles - 1 && lane == 0) drawn = draw_item(counter, given, n_items, own);  // the next item
           if (use > 0) wait_all(bar_free(st), (use - 1) & 1);
           if (!ok) break;
-          if (!(started && t == 0)) load_tile(st, first_row(t), h);
+          if (!(started && t == 0)) load_tile(st, lo + t * 128, h);
           const uint32_t stat = smem_base + SM::kStat + st * 1024 + lane * 4;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             ptx::sts_s32(stat + 128 * i, __float_as_int(-sl[i] * kLog2e));
             ptx::sts_s32(stat + 512 + 128 * i, __float_as_int(-sd[i]));
           }
-          if (t + 1 < n_tiles) fetch_stats(first_row(t + 1));
+          if (t + 1 < n_tiles) fetch_stats(lo + (t + 1) * 128);
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(bar_y(st));
           ++filled;
@@ -293,44 +292,37 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
     // and take every wait together; one elected lane issues (see ptx::elect_one)
     constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(128, 128, false, false);
     constexpr uint32_t kIdescAcc = ptx::idesc_bf16_f32(128, D, false, true);
-    struct Tile { int item, left, y0, back, st; uint32_t use; };  // left: tiles of the item from this one on; 0: past the end
+    struct Tile { int item, left, over, st; uint32_t use; };  // left: tiles of the item from this one on; 0: past the end
     auto open = [&](Tile& t) {  // the item's slot
       wait(bar_item(t.item), (t.item >> 1) & 1);
       const bool gone = aborted();
-      t.y0 = __shfl_sync(0xffffffffu, ptx::lds_s32(item_slot(t.item) + 8), 0);
       const int tiles = __shfl_sync(0xffffffffu, ptx::lds_s32(item_slot(t.item) + 12), 0);
       t.left = gone ? 0 : tiles >> 7;
-      t.back = tiles & 127;
+      t.over = tiles & 127;
     };
     auto advance = [&](Tile t, bool& first) {
-      t.y0 += 128;
       if (++t.st == kStages) { t.st = 0; t.use ^= 1u; }
       first = --t.left == 0;
       if (first) {
         ++t.item;
         open(t);
-      } else if (t.left == 1) {
-        t.y0 -= t.back;
       }
       return t;
     };
     const uint32_t y_lo = HT::desc_lo(y_s(0, 0)), x_lo = HT::desc_lo(smem_base);
     constexpr uint32_t kTileLo = kTile / 16;
-    Tile c{0, 0, 0, 0, 0, 0};
+    Tile c{0, 0, 0, 0, 0};
     bool c_first = true;  // the tile opens an item
     open(c);
     if (warp == kWarpS) {
       auto issue_s = [&](const Tile& t, int g, bool first) {
         if (first) wait(bar_x(t.item), (t.item >> 1) & 1);
         wait(bar_y(t.st), t.use);
-        if (t.y0 + 128 > Np) {
-          // lines past the last valid packed row are unspecified memory, and would be summed over
-          const int line0 = Np - t.y0;
+        if (t.left == 1 && (t.over & 15) != 0) {
           constexpr int kChunks = HT::kRowBytes / 16;
-          for (int i = lane; i < (128 - line0) * kChunks * 2; i += 32) {
-            const int w = i / ((128 - line0) * kChunks), j = i - w * (128 - line0) * kChunks;
-            *reinterpret_cast<uint4*>(smem_al + SM::kY + kTile * (2 * t.st + w) + line0 * HT::kRowBytes + j * 16) = make_uint4(0, 0, 0, 0);
-          }
+          const int n_chunks = (t.over & 15) * kChunks, at = SM::kY + 2 * kTile * t.st + (128 - t.over) * HT::kRowBytes;
+          for (int i = lane; i < 2 * n_chunks; i += 32)
+            *reinterpret_cast<uint4*>(smem_al + at + (i < n_chunks ? i : kTile / 16 + i - n_chunks) * 16) = make_uint4(0, 0, 0, 0);
           ptx::fence_proxy_async_smem();
           __syncwarp();
         }
@@ -383,6 +375,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
         // k-step k (16 queries): columns that the threads of column group k / 2 have written over their S
         const uint32_t a = tmem + 128 * (g & 1) + (is_v ? 0 : 16), b = b_lo + 2 * kTileLo * c.st;
         const uint32_t acc = c_first ? 0u : 1u;
+        const int steps = c.left == 1 ? 8 - (c.over >> 4) : 8;
         bool gone = false;
 #pragma unroll
         for (int grp = 0; grp < 2; ++grp) {  // dV += P^T dO | dK += dS^T Q: queries 64 grp ..
@@ -393,7 +386,8 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
           if (!gone && ptx::elect_one()) {
 #pragma unroll
             for (int k = 4 * grp; k < 4 * grp + 4; ++k)
-              ptx::mma_bf16_ts(out, a + (k >> 1) * 32 + (k & 1) * 8, HT::desc(b + k * HT::kStepMN), kIdescAcc, k == 0 ? acc : 1u);
+              if (k < steps)
+                ptx::mma_bf16_ts(out, a + (k >> 1) * 32 + (k & 1) * 8, HT::desc(b + k * HT::kStepMN), kIdescAcc, k == 0 ? acc : 1u);
             if (grp == 1) {
               ptx::mma_commit(bar_free(c.st));
               if (c.left == 1) ptx::mma_commit(bar_acc(c.item));
@@ -457,8 +451,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
     for (;; ++n) {
       wait(bar_item(n), (n >> 1) & 1);
       const bool gone = aborted();
-      const int tiles = ptx::lds_s32(item_slot(n) + 12), back = tiles & 127;
-      int left = tiles >> 7;
+      int left = ptx::lds_s32(item_slot(n) + 12) >> 7;
       if (gone || left == 0) break;
       // the row's segment relative to this thread's first column of the tile; it moves down tile by tile
       int lo = ptx::lds_s32(row_s(n) + rl * 4), hi = ptx::lds_s32(row_s(n) + 512 + rl * 4);
@@ -469,10 +462,6 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
         hi -= y0;
       }
       for (bool first = true; left > 0; --left, ++g, lo -= 128, hi -= 128, first = false) {
-        if (left == 1 && back > 0) {  // the last tile: not the rows that the one before it had
-          lo = (lo > -col0 ? lo : -col0) + back;
-          hi += back;
-        }
         const uint32_t s_col = lane_base + 128 * (g & 1) + col0;
         const uint32_t stat = smem_base + SM::kStat + st * 1024 + col0 * 4;
         // ---- P^T = 2^(S^T - lse).  A thread whose 32 queries lie wholly outside its row's segment writes zeros without the
