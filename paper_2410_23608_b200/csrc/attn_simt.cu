@@ -3,18 +3,20 @@
 // workload and the bring-up reference of the tensor-core kernels.
 //
 // Work split: a CTA owns 32 consecutive packed rows and one head, wherever segment boundaries fall, and walks the
-// rows of the other side that the segments of its rows span, in tiles of 64 staged in shared memory as fp32.  Two groups of
-// 128 threads take them in turn, each with a stage of its own, and the first joins the two results at the end: one group's copies
-// and softmax run under the other's products, and a CTA's chain, which bounds all but the largest problems, is half as long.
+// rows of the other side that the segments of its rows span, in tiles of 64 staged in shared memory as fp32.  Where there are few CTAs, two
+// groups of 128 threads take them in turn, each with a stage of its own, and the first joins the two results at the end: one group's copies
+// and softmax run under the other's products, and a CTA's chain, which bounds such problems, is half as long.  Else one group takes
+// them all, and other CTAs run under its copies (see one_group).
 // A group is a grid of 8 x 16 threads: a product tile of 32 x 64 is 4 x 4 values per thread (8
 // vector reads of shared memory per 64 multiply-adds), its softmax statistics are shuffles among 16 lanes, and the
 // second product gives a thread 4 rows x D / 16 head dimensions.  No padding token is ever computed, nothing is atomically
-// accumulated, and every sum runs in a fixed order.  With one group, and two tiles in flight, against two, us: one image of
+// accumulated, and every sum runs in a fixed order.  Against one group with two tiles in flight for all, us: one image of
 // 4 200 tokens, 8 heads of 32, forward 81.5 -> 46.1, backward 200.5 -> 151.8; 4 of 196 tokens, 3 heads of 32, 7.4 -> 7.2 and
-// 15.8 -> 14.4; 16 of 196, 6 heads of 64, 22.6 -> 21.7 and 76.2 -> 73.0; 64 of them 71.2 -> 68.8 and 256 -> 246.  What bounds it
+// 15.8 -> 14.4; 16 of 196, 6 heads of 64, 22.6 -> 21.7 and 76.2 -> 73.0; 64 of them 70.4 -> 62.6 and 254 -> 229.  What bounds it
 // then is shared memory: a vector read of 16 bytes per eight multiply-adds, 30 of the 75 TFLOP/s of the multiply-adds.
-// Errors against fp64 are smaller, the sums being two (4 000 rows of one segment, 2 heads of 64: outputs 1.18e-6 -> 8.6e-7,
-// gradients 1.25e-6 -> 9.6e-7; short segments 0.95 of before).
+// Errors against fp64: a tile's terms are summed by themselves and then added, so that no chain is longer than 64 terms and the
+// number of tiles (4 000 rows of one segment, 2 heads of 64: outputs 1.16e-6 with one chain, 8.5e-7 with one per group, 3.5e-7 now,
+// gradients 1.24e-6, 9.4e-7 and 5.2e-7; 64 images of 186 rows, 8 heads of 32: 3.2e-7, 2.8e-7, 2.6e-7).
 #include <math_constants.h>
 
 #include "simt_stage.cuh"
@@ -25,8 +27,7 @@ namespace {
 
 constexpr int kR = 32;          // packed rows per CTA
 constexpr int kT = 64;          // rows of a streamed tile
-constexpr int kGroups = 2;      // of threads: group q takes the streamed tiles q, q + 2, ..
-constexpr int kGroup = 128, kThreads = kGroups * kGroup;
+constexpr int kGroup = 128;     // threads; of kGroups groups, one or two, group q takes the streamed tiles q, q + kGroups, ..
 constexpr int kTX = 16, kTY = 8;  // thread (ty, tx) of a group: rows ty + 8 i (i < 4), streamed rows tx + 16 j (j < 4)
 constexpr int kLdP = kT + 4;    // leading dimension of the probability tiles
 template <int D> constexpr int kLd = D + 4;  // rows 4 banks apart
@@ -65,6 +66,12 @@ __device__ __forceinline__ void dots(float (*s)[4], const float* a, const float*
   }
 }
 
+template <int W> __device__ __forceinline__ void add_to(float (*sum)[W], const float (*v)[W]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int d = 0; d < W; ++d) sum[i][d] += v[i][d];
+}
 // o[i][d] += sum over the tile's rows k < n of p[ty + 8 i][k] * v[k][tx * (D / 16) + d]
 template <int D>
 __device__ __forceinline__ void weighted(float (*o)[D / kTX], const float* p, const float* v, int n, int ty, int tx) {
@@ -154,14 +161,14 @@ __device__ __forceinline__ RowSeg tile_segments(RowSeg* seg_s, const int32_t* se
 }
 
 // ------------------------------------------------------------------------------------ forward
-template <int D> constexpr int kFwdFloats = (kR + kGroups * 2 * kT) * kLd<D> + kGroups * kR * kLdP;  // Q; per group K and V, P
+template <int D, int kGroups> constexpr int kFwdFloats = (kR + kGroups * 2 * kT) * kLd<D> + kGroups * kR * kLdP;  // Q; per group K and V, P
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads, 2)
+template <typename T, int D, int kGroups>
+__global__ void __launch_bounds__(kGroups * kGroup, 4 / kGroups)
 attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ ao, float* __restrict__ lse) {
   pdl_entry();
-  constexpr int W = D / kTX;
+  constexpr int W = D / kTX, kThreads = kGroups * kGroup;
   extern __shared__ __align__(16) float sm[];
   __shared__ RowSeg seg_s[kR];
   constexpr int kTile = kT * kLd<D>;
@@ -196,7 +203,7 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
     cp_async_wait<1>();
     group_sync(grp);  // K; V is waited for behind the first product
     const int kv0 = all.lo + t * kT;
-    float s[4][4] = {};
+    float s[4][4] = {}, alpha[4];
     dots<D>(s, Qs, Ks, ty, tx);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -209,7 +216,7 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
       }
       const float m_new = fmaxf(m[i], max16(cm));
       const float m_use = m_new == -CUDART_INF_F ? 0.f : m_new;  // no key of this row so far
-      const float alpha = expf(m[i] - m_use);
+      alpha[i] = expf(m[i] - m_use);
       float rs = 0.f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -217,40 +224,45 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
         rs += p;
         Ps[(ty + kTY * i) * kLdP + tx + kTX * j] = p;
       }
-      l[i] = l[i] * alpha + sum16(rs);
-#pragma unroll
-      for (int d = 0; d < W; ++d) o[i][d] *= alpha;
+      l[i] = l[i] * alpha[i] + sum16(rs);
       m[i] = m_new;
     }
     cp_async_wait<0>();
     group_sync(grp);  // V, and the rows of P
     const int n = all.hi - kv0 < kT ? all.hi - kv0 : kT;
-    weighted<D>(o, Ps, Ks + kTile, n, ty, tx);
+    float tile[4][W] = {};  // a sum of its own: the chain is a tile long and then a term per tile
+    weighted<D>(tile, Ps, Ks + kTile, n, ty, tx);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int d = 0; d < W; ++d) o[i][d] = fmaf(o[i][d], alpha[i], tile[i][d]);
     group_sync(grp);  // the stage is free
     if (t + kGroups < n_tiles) stage(t + kGroups);
   }
-  // the second group's share of every row, in the memory of its stage
-  float* part = sm + kR * kLd<D> + 2 * kTile + tid;  // [4 (W + 2)][kGroup]
-  if (grp == 1) {
+  if (kGroups > 1 && n_tiles == 1 && grp == 1) return;
+  if (kGroups > 1 && n_tiles > 1) {  // the second group's share of every row, in the memory of its stage
+    float* part = sm + kR * kLd<D> + 2 * kTile + tid;  // [4 (W + 2)][kGroup]
+    if (grp == 1) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        part[(i * (W + 2)) * kGroup] = m[i];
+        part[(i * (W + 2) + 1) * kGroup] = l[i];
+#pragma unroll
+        for (int d = 0; d < W; ++d) part[(i * (W + 2) + 2 + d) * kGroup] = o[i][d];
+      }
+    }
+    __syncthreads();
+    if (grp == 1) return;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      part[(i * (W + 2)) * kGroup] = m[i];
-      part[(i * (W + 2) + 1) * kGroup] = l[i];
+      const float m1 = part[(i * (W + 2)) * kGroup], l1 = part[(i * (W + 2) + 1) * kGroup];
+      const float m_new = fmaxf(m[i], m1), m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
+      const float a0 = expf(m[i] - m_use), a1 = expf(m1 - m_use);
+      l[i] = l[i] * a0 + l1 * a1;
 #pragma unroll
-      for (int d = 0; d < W; ++d) part[(i * (W + 2) + 2 + d) * kGroup] = o[i][d];
+      for (int d = 0; d < W; ++d) o[i][d] = o[i][d] * a0 + part[(i * (W + 2) + 2 + d) * kGroup] * a1;
+      m[i] = m_new;
     }
-  }
-  __syncthreads();
-  if (grp == 1) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float m1 = part[(i * (W + 2)) * kGroup], l1 = part[(i * (W + 2) + 1) * kGroup];
-    const float m_new = fmaxf(m[i], m1), m_use = m_new == -CUDART_INF_F ? 0.f : m_new;
-    const float a0 = expf(m[i] - m_use), a1 = expf(m1 - m_use);
-    l[i] = l[i] * a0 + l1 * a1;
-#pragma unroll
-    for (int d = 0; d < W; ++d) o[i][d] = o[i][d] * a0 + part[(i * (W + 2) + 2 + d) * kGroup] * a1;
-    m[i] = m_new;
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -280,13 +292,14 @@ attn_fwd_simt_kernel(const T* qkv, const int32_t* seg, int n_seg, int capacity, 
 // holds), so that they share the GPU: blockIdx.z = 0: own rows are queries, streamed rows keys,
 //   S = Q K^T, dP = dO V^T, dS = P (dP - D), dQ += dS K;
 // blockIdx.z = 1: own rows are keys, streamed rows queries, everything transposed: dV += P^T dO, dK += dS^T Q.
-template <int D> constexpr int kBwdFloats = (2 * kR + kGroups * 2 * kT) * kLd<D> + kGroups * (kR * kLdP + 2 * kT);
+template <int D, int kGroups> constexpr int kBwdFloats = (2 * kR + kGroups * 2 * kT) * kLd<D> + kGroups * (kR * kLdP + 2 * kT);
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads, 2)
+template <typename T, int D, int kGroups>
+__global__ void __launch_bounds__(kGroups * kGroup, 4 / kGroups)
 attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
                      const T* dao, const int32_t* seg, int n_seg, int capacity, int C,
                      float scale, T* __restrict__ dqkv) {
+  constexpr int kThreads = kGroups * kGroup;
   pdl_entry();
   constexpr int W = D / kTX, E = Vec16<T>::kElems;
   constexpr int kTile = kT * kLd<D>;
@@ -376,7 +389,9 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
     const int n = all.hi - y0 < kT ? all.hi - y0 : kT;
     if (!dq) {
       __syncwarp();  // the rows of P and dS that this warp reads are the ones its own lanes wrote
-      weighted<D>(acc2, Ps, Y2, n, ty, tx);
+      float tile[4][W] = {};
+      weighted<D>(tile, Ps, Y2, n, ty, tx);
+      add_to<W>(acc2, tile);
       __syncwarp();
     }
 #pragma unroll
@@ -384,30 +399,34 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
 #pragma unroll
       for (int j = 0; j < 4; ++j) Ps[(ty + kTY * i) * kLdP + tx + kTX * j] = dp[i][j];
     __syncwarp();
-    weighted<D>(acc1, Ps, Y1, n, ty, tx);
+    float tile[4][W] = {};
+    weighted<D>(tile, Ps, Y1, n, ty, tx);
+    add_to<W>(acc1, tile);
     group_sync(grp);  // the stage is free
     if (t + kGroups < n_tiles) stage(t + kGroups);
   }
-  // the second group's share of every sum, in the memory of its stage
-  float* part = A2 + kR * kLd<D> + 2 * kTile + tid;  // [8 W][kGroup]
-  if (grp == 1) {
+  if (kGroups > 1 && n_tiles == 1 && grp == 1) return;
+  if (kGroups > 1 && n_tiles > 1) {  // the second group's share of every sum, in the memory of its stage
+    float* part = A2 + kR * kLd<D> + 2 * kTile + tid;  // [8 W][kGroup]
+    if (grp == 1) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int d = 0; d < W; ++d) {
+          part[(i * W + d) * kGroup] = acc1[i][d];
+          part[((4 + i) * W + d) * kGroup] = acc2[i][d];
+        }
+    }
+    __syncthreads();
+    if (grp == 1) return;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int d = 0; d < W; ++d) {
-        part[(i * W + d) * kGroup] = acc1[i][d];
-        part[((4 + i) * W + d) * kGroup] = acc2[i][d];
+        acc1[i][d] += part[(i * W + d) * kGroup];
+        acc2[i][d] += part[((4 + i) * W + d) * kGroup];
       }
   }
-  __syncthreads();
-  if (grp == 1) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int d = 0; d < W; ++d) {
-      acc1[i][d] += part[(i * W + d) * kGroup];
-      acc2[i][d] += part[((4 + i) * W + d) * kGroup];
-    }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int row = i0 + ty + kTY * i;
@@ -436,54 +455,68 @@ attn_bwd_simt_kernel(const T* qkv, const T* ao, const float* lse,
   }
 }
 
-template <typename T, int D>
+template <typename T, int D, int kGroups>
 int fwd_launch(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao, float* lse,
                cudaStream_t st) {
-  auto kern = attn_fwd_simt_kernel<T, D>;
-  constexpr int kSmem = kFwdFloats<D> * (int)sizeof(float);
+  auto kern = attn_fwd_simt_kernel<T, D, kGroups>;
+  constexpr int kSmem = kFwdFloats<D, kGroups> * (int)sizeof(float);
   static DeviceOnce attr;
   cudaError_t e = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem); });
   if (e != cudaSuccess) { set_cuda_error(e, "attn_fwd_simt_kernel"); return SPA_ERR_CUDA; }
-  launch_pdl(kern, dim3((p.capacity + kR - 1) / kR, p.H), kThreads, kSmem, st, (const T*)qkv, seg, n_seg, p.capacity, p.C,
+  launch_pdl(kern, dim3((p.capacity + kR - 1) / kR, p.H), kGroups * kGroup, kSmem, st, (const T*)qkv, seg, n_seg, p.capacity, p.C,
              softmax_scale_of(p), (T*)ao, lse);
   SPA_CUDA_CHECK_LAUNCH("attn_fwd_simt_kernel");
   return SPA_OK;
 }
 
-template <typename T, int D>
+template <typename T, int D, int kGroups>
 int bwd_launch(const spa_params& p, const void* qkv, const void* ao, const float* lse, const void* dao,
                const int32_t* seg, int n_seg, void* dqkv, cudaStream_t st) {
-  auto kern = attn_bwd_simt_kernel<T, D>;
-  constexpr int kSmem = kBwdFloats<D> * (int)sizeof(float);
+  auto kern = attn_bwd_simt_kernel<T, D, kGroups>;
+  constexpr int kSmem = kBwdFloats<D, kGroups> * (int)sizeof(float);
   static DeviceOnce attr;
   cudaError_t e = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem); });
   if (e != cudaSuccess) { set_cuda_error(e, "attn_bwd_simt_kernel"); return SPA_ERR_CUDA; }
-  launch_pdl(kern, dim3((p.capacity + kR - 1) / kR, p.H, 2), kThreads, kSmem, st, (const T*)qkv, (const T*)ao, lse,
+  launch_pdl(kern, dim3((p.capacity + kR - 1) / kR, p.H, 2), kGroups * kGroup, kSmem, st, (const T*)qkv, (const T*)ao, lse,
              (const T*)dao, seg, n_seg, p.capacity, p.C, softmax_scale_of(p), (T*)dqkv);
   SPA_CUDA_CHECK_LAUNCH("attn_bwd_simt_kernel");
   return SPA_OK;
 }
 
+// One group where the CTAs that the capacity may fill are many per SM: four of them run on an SM (three in the backward at
+// d = 64) instead of two, and none has a second group that idles over an odd tile.  By the capacity, of which a part is rows: 12
+// per SM, 6 where segments have 64 rows or fewer and most CTAs one tile (10 in the forward at d = 64, where few CTAs land unevenly).
+// us, two groups -> one, forward and backward: 8 heads of 32, 64 images of 196 tokens, half selected, 55.7 -> 47.9 and 170 -> 151, a
+// fifth 19.6 -> 16.2 and 51 -> 42; 4 x 4 200 tokens in containers of 49, two thirds selected, 64 -> 49 and 202 -> 158; 6 heads of 64, 64
+// images 68 -> 63 and 245 -> 229.  Below the line: 3 heads of 32, 16 images 13.7 -> 14.9 and 26.9 -> 35.2, 6 of 64 23.3 -> 31.8 and
+// 76.5 -> 80.4.  Not with more than 8 tiles, which two groups share evenly: 2 heads of 64, 4 images of 4 039 tokens 129 -> 132 and
+// 360 -> 400.
+bool one_group(const spa_params& p, int n_seg, bool forward) {
+  const long long ctas = (long long)((p.capacity + kR - 1) / kR) * p.H * (forward ? 1 : 2), tile = (long long)kT * n_seg;
+  const int per_sm = p.capacity > tile ? 12 : forward && p.C / p.H == 64 ? 10 : 6;
+  return p.capacity <= 8 * tile && ctas >= per_sm * kNumSMs;
+}
+
 }  // namespace
+
+#define SPA_SIMT_LAUNCH(WHICH, FORWARD, ...)                                                                               \
+  const int d = p.C / p.H;                                                                                               \
+  if (one_group(p, n_seg, FORWARD)) {                                                                                             \
+    if (p.dtype == SPA_F32) return d == 32 ? WHICH<float, 32, 1>(__VA_ARGS__) : WHICH<float, 64, 1>(__VA_ARGS__);        \
+    return d == 32 ? WHICH<__nv_bfloat16, 32, 1>(__VA_ARGS__) : WHICH<__nv_bfloat16, 64, 1>(__VA_ARGS__);                \
+  }                                                                                                                      \
+  if (p.dtype == SPA_F32) return d == 32 ? WHICH<float, 32, 2>(__VA_ARGS__) : WHICH<float, 64, 2>(__VA_ARGS__);          \
+  return d == 32 ? WHICH<__nv_bfloat16, 32, 2>(__VA_ARGS__) : WHICH<__nv_bfloat16, 64, 2>(__VA_ARGS__)
 
 int launch_attention_fwd_simt(const spa_params& p, const void* qkv, const int32_t* seg, int n_seg, void* ao,
                               float* lse, cudaStream_t st) {
-  const int d = p.C / p.H;
-  if (p.dtype == SPA_F32)
-    return d == 32 ? fwd_launch<float, 32>(p, qkv, seg, n_seg, ao, lse, st)
-                   : fwd_launch<float, 64>(p, qkv, seg, n_seg, ao, lse, st);
-  return d == 32 ? fwd_launch<__nv_bfloat16, 32>(p, qkv, seg, n_seg, ao, lse, st)
-                 : fwd_launch<__nv_bfloat16, 64>(p, qkv, seg, n_seg, ao, lse, st);
+  SPA_SIMT_LAUNCH(fwd_launch, true, p, qkv, seg, n_seg, ao, lse, st);
 }
 
 int launch_attention_bwd_simt(const spa_params& p, const void* qkv, const void* ao, const float* lse,
                               const void* dao, const int32_t* seg, int n_seg, void* dqkv, cudaStream_t st) {
-  const int d = p.C / p.H;
-  if (p.dtype == SPA_F32)
-    return d == 32 ? bwd_launch<float, 32>(p, qkv, ao, lse, dao, seg, n_seg, dqkv, st)
-                   : bwd_launch<float, 64>(p, qkv, ao, lse, dao, seg, n_seg, dqkv, st);
-  return d == 32 ? bwd_launch<__nv_bfloat16, 32>(p, qkv, ao, lse, dao, seg, n_seg, dqkv, st)
-                 : bwd_launch<__nv_bfloat16, 64>(p, qkv, ao, lse, dao, seg, n_seg, dqkv, st);
+  SPA_SIMT_LAUNCH(bwd_launch, false, p, qkv, ao, lse, dao, seg, n_seg, dqkv, st);
 }
+#undef SPA_SIMT_LAUNCH
 
 }  // namespace spa
