@@ -24,9 +24,10 @@ namespace {
 // copy and stages the queries' statistics, up to kStages tiles and an item ahead.  A finished item's accumulators are
 // drained behind the exponentials of the next item's first tile, when the wait for its last products is over.
 // What bounds it: the exponentials are 1 024 clocks of a tile's 2 500 (16 segments of 210 to 1 680 rows, 8 heads of 32), the
-// rest is the chain wait - load - arithmetic - store - announcement of a warp, four of which share a scheduler.  That
-// workload: 132.7 -> 99.1 us against two CTAs per SM on 64-query tiles with a prologue per item; cut into containers of 49
-// rows 43.3 -> 35.4; 32 segments of 58 to 518 rows, 12 heads of 64: 60.4 -> 51.7.
+// rest is the chain wait - load - arithmetic - store - announcement of a warp, four of which share a scheduler (96 registers, of
+// which 16 to 28 bytes are spilled).  The whole backward with it, against two CTAs per SM on 64-query tiles with a prologue per
+// item: that workload 211.5 -> 169.5 us, cut into containers of 49 rows 61.5 -> 54.0; 32 segments of 58 to 518 rows, 12 heads of 64,
+// 96.9 -> 84.5.
 constexpr int kMathWarps = 16, kMathThreads = 32 * kMathWarps;
 // warps behind the arithmetic ones: products S^T and dP^T | dV | dK; items and copies
 constexpr int kWarpS = kMathWarps, kWarpV = kMathWarps + 1, kWarpK = kMathWarps + 2, kWarpLoad = kMathWarps + 3;
@@ -590,12 +591,13 @@ int kv_launch(const spa_params& p, const void* qkv, const float* lse, const floa
 // By the 128 x 128 tiles that the capacity may hold, items times the tiles that one spans (its own 128 rows and what a segment
 // adds), per SM: with few of them the start of the pipeline, a copy, a look-up and a cold instruction cache long, is all there
 // is.  dQ and dK / dV together, us, the other kernels -> this one, at tiles per SM of
-//   5: 32 images of 196 tokens, 6 heads of 64, 20.2 -> 20.8;  10: 64 of them 24.5 -> 27.8, 4 x 4 200 tokens in containers of 49,
-//   8 heads of 32, 19.8 -> 21.2;  11: 24 x 315 tokens, 8 heads of 64, 27.3 -> 29.2;  15.6: 32 x 256, 12 heads of 64, 39.0 -> 37.0,
-//   but in a transformer block's step, whose weight gradients then wait for whole SMs, 503 -> 506;  16: 8 x 576 35.7 -> 36.1;
-//   20: 128 x 196, 6 heads of 64, 45.6 -> 44.6 (a transformer block's step 538 -> 544), of 32 38.5 -> 38.9, 8 x 4 200 in
-//   containers 33.9 -> 33.3;  the line;  32: 16 x 576 58.3 -> 53.1;  40: 128 x 196, 12 heads, 55.5 -> 52.0;  60: 1 x 4 200, 8 heads of 32, 34.2 -> 29.4;
-//   900: 16 x 4 200 210.6 -> 175.7.
+//   5: 32 images of 196 tokens, 6 heads of 64, 20.1 -> 18.9;  10: 64 of them 24.6 -> 26.2, 4 x 4 200 tokens in containers of 49,
+//   8 heads of 32, 19.5 -> 20.4;  11: 24 x 315 tokens, 8 heads of 64, 27.8 -> 27.0;  15.6: 32 x 256, 12 heads of 64, 40.0 -> 37.5,
+//   but in a transformer block's step, whose weight gradients then wait for whole SMs, 503 -> 506 when the kernel was new;  16: 8 x 576
+//   43.0 -> 38.1;  20: 128 x 196, 6 heads of 64, 45.5 -> 43.3 (a transformer block's step then 538 -> 544), of 32 38.9 -> 37.6, 8 x
+//   4 200 in containers 35.3 -> 32.4;  the line;  32: 16 x 576 59.4 -> 51.8;  40: 128 x 196, 12 heads, 56.5 -> 51.5;  60: 1 x 4 200,
+//   8 heads of 32, 33.9 -> 27.8;  960: 16 x 4 200 211.5 -> 169.5.  Rows are a part of the capacity; with 1 to 3 % of 16 x 4 200 tokens
+//   selected 52 -> 34, of 32 x 576 23.4 -> 19.5.
 bool attention_bwd_kv_applies(const spa_params& p, int n_seg) {
   const long long items = (long long)p.H * ((p.capacity + 127) / 128);
   const long long segment = p.capacity / (n_seg > 0 ? n_seg : 1);
