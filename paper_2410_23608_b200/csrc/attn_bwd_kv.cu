@@ -32,7 +32,8 @@ constexpr int kMathWarps = 16, kMathThreads = 32 * kMathWarps;
 // warps behind the arithmetic ones: products S^T and dP^T | dV | dK; items and copies
 constexpr int kWarpS = kMathWarps, kWarpV = kMathWarps + 1, kWarpK = kMathWarps + 2, kWarpLoad = kMathWarps + 3;
 constexpr int kKvThreads = kMathThreads + 128;
-constexpr int kKvSegStage = 2048;
+// Up to so many segments, whose offsets are searched in shared memory; its size goes by them.
+constexpr int kKvSegStage = 12288;
 constexpr uint32_t kColDP = 256, kColDV = 384, kColDK = 448;  // S^T: columns 0 and 128
 
 template <int D> struct KvSmem {
@@ -42,9 +43,11 @@ template <int D> struct KvSmem {
   static constexpr int kStat = kY + kStages * 2 * kTile;      // [kStages][2][128]: -lse_i log2e, -D_i of the queries
   static constexpr int kRows = kStat + kStages * 2 * 128 * 4;
   static constexpr int kBar = kRows + 4 * 2 * 128 * 4;        // rows' segments of four items: [lo][hi]
-  static constexpr int kSeg = kBar + 512;                     // barriers, item slots
-  static constexpr int kOrder = kSeg + (kKvSegStage + 4) * 4;
-  static constexpr int kBytes = kOrder + (int)sizeof(ItemOrder) + 1024;  // and the alignment of the base
+  static constexpr int kOrder = kBar + 512;                   // barriers, item slots
+  static constexpr int kSeg = kOrder + (int)sizeof(ItemOrder);
+  static constexpr int bytes(int offsets) { return kSeg + offsets * 4 + 1024; }  // and the alignment of the base
+  static constexpr int kMaxBytes = bytes(kKvSegStage);
+  static_assert(kMaxBytes <= 227 * 1024, "shared memory of a CTA");
 };
 
 template <int D>
@@ -113,9 +116,8 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
     ptx::fence_mbar_init();
   }
   pdl_entry();
-  const bool staged = n_seg < kKvSegStage;
-  if (staged)
-    for (int i = tid; i <= n_seg; i += kKvThreads) seg_s[i] = ld_dep(seg + i);
+#pragma unroll 4
+  for (int i = tid; i <= n_seg; i += kKvThreads) seg_s[i] = ld_dep(seg + i);
   const int Np = packed_rows(seg, n_seg, capacity);
   const int row_tiles = (Np + 127) / 128, n_items = row_tiles * H;
   if ((int)blockIdx.x >= n_items) return;
@@ -123,7 +125,7 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
   // see the forward kernel
   const bool draws = counter != nullptr && n_items > (int)gridDim.x;
   const int given = draws ? (int)gridDim.x / H * H : n_items;
-  const bool ordered = !even_items && draws && staged && 2 * n_items >= 3 * (int)gridDim.x && row_tiles - given / H <= kMaxOrder;
+  const bool ordered = !even_items && draws && 2 * n_items >= 3 * (int)gridDim.x && row_tiles - given / H <= kMaxOrder;
   // The loading warp gets the streamed rows of the CTA's first item straight from the offsets, of which a lane takes a few, and
   // starts its copies before the CTA comes together.
   const bool early = warp == kWarpLoad && n_seg < kEarlySegments && !skip_short && !(draws && (int)blockIdx.x >= given);
@@ -192,25 +194,20 @@ attn_bwd_kv_kernel(const __grid_constant__ CUtensorMap tm_qkv, const __grid_cons
       if (!skip_short && !started) load_own(n, r0, h);
       // the segments of its rows, four to a lane, in step
       RowSeg s[4];
-      if (staged) {
-        int a[4] = {}, b[4];  // seg_s[a] <= row < seg_s[b]
+      int a[4] = {}, b[4];  // seg_s[a] <= row < seg_s[b]
 #pragma unroll
-        for (int i = 0; i < 4; ++i) b[i] = n_seg;
-        for (int step = 32 - __clz(n_seg - 1 > 0 ? n_seg - 1 : 0); step > 0; --step) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int mid = (a[i] + b[i]) >> 1;  // = a once b = a + 1: no change then
-            if (seg_s[mid] <= r0 + 32 * i + lane) a[i] = mid; else b[i] = mid;
-          }
-        }
+      for (int i = 0; i < 4; ++i) b[i] = n_seg;
+      for (int step = 32 - __clz(n_seg - 1 > 0 ? n_seg - 1 : 0); step > 0; --step) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int end = seg_s[a[i] + 1];
-          s[i] = r0 + 32 * i + lane < Np ? RowSeg{seg_s[a[i]], end < Np ? end : Np} : RowSeg{0, 0};
+          const int mid = (a[i] + b[i]) >> 1;  // = a once b = a + 1: no change then
+          if (seg_s[mid] <= r0 + 32 * i + lane) a[i] = mid; else b[i] = mid;
         }
-      } else {
+      }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) s[i] = warp_row_segment([&](int j) { return ld_dep(seg + j); }, n_seg, Np, r0 + 32 * i);
+      for (int i = 0; i < 4; ++i) {
+        const int end = seg_s[a[i] + 1];
+        s[i] = r0 + 32 * i + lane < Np ? RowSeg{seg_s[a[i]], end < Np ? end : Np} : RowSeg{0, 0};
       }
       const uint32_t rs = row_s(n) + lane * 4;
       int lo_rows = 0x7fffffff, hi_rows = 0;
@@ -574,12 +571,13 @@ int kv_launch(const spa_params& p, const void* qkv, const float* lse, const floa
     return SPA_ERR_UNSUPPORTED;
   auto kern = attn_bwd_kv_kernel<D>;
   static DeviceOnce attr;
-  cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, KvSmem<D>::kBytes); });
+  cudaError_t ea = attr.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, KvSmem<D>::kMaxBytes); });
   if (ea != cudaSuccess) { set_cuda_error(ea, "attn_bwd_kv_kernel"); return SPA_ERR_CUDA; }
   const long long items = (long long)p.H * ((p.capacity + 127) / 128);
   const int grid = (int)(items < kNumSMs ? items : kNumSMs);
   const bool even_items = (long long)p.capacity <= 512ll * (n_seg > 0 ? n_seg : 1);  // as in the forward
-  launch_pdl(kern, grid, kKvThreads, KvSmem<D>::kBytes, st, tm_qkv, tm_do, lse, delta, seg, n_seg, p.capacity, p.C, p.H,
+  const int offsets = n_seg < 2048 ? 2048 : n_seg + 1;
+  launch_pdl(kern, grid, kKvThreads, KvSmem<D>::bytes(offsets), st, tm_qkv, tm_do, lse, delta, seg, n_seg, p.capacity, p.C, p.H,
              softmax_scale_of(p), (__nv_bfloat16*)dqkv, skip_short, items > grid ? item_counter(dqkv) : nullptr, even_items,
              ptx::wait_limit(p.flags), d_status);
   SPA_CUDA_CHECK_LAUNCH("attn_bwd_kv_kernel");
@@ -598,10 +596,13 @@ int kv_launch(const spa_params& p, const void* qkv, const float* lse, const floa
 //   4 200 in containers 35.3 -> 32.4;  the line;  32: 16 x 576 59.4 -> 51.8;  40: 128 x 196, 12 heads, 56.5 -> 51.5;  60: 1 x 4 200,
 //   8 heads of 32, 33.9 -> 27.8;  960: 16 x 4 200 211.5 -> 169.5.  Rows are a part of the capacity; with 1 to 3 % of 16 x 4 200 tokens
 //   selected 52 -> 34, of 32 x 576 23.4 -> 19.5.
+// And by the segments: searched in global memory, their offsets are what the tiles of short segments wait for.  42 images of 2 782 tokens in
+// containers of 49 rows (2 394 segments), 8 heads of 32: the other kernels 230, so 257.7, from shared memory 204.3;  14 000 images
+// of 49 tokens, whose offsets do not fit there, 691 -> 746.
 bool attention_bwd_kv_applies(const spa_params& p, int n_seg) {
   const long long items = (long long)p.H * ((p.capacity + 127) / 128);
   const long long segment = p.capacity / (n_seg > 0 ? n_seg : 1);
-  return items * (128 + segment) >= 24ll * 128 * kNumSMs;
+  return n_seg < kKvSegStage && items * (128 + segment) >= 24ll * 128 * kNumSMs;
 }
 
 int launch_attention_bwd_kv(const spa_params& p, const void* qkv, const float* lse, const float* delta, const void* dao,

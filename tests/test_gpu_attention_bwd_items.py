@@ -1,5 +1,5 @@
 """Attention backward in one pipeline per CTA over all its items (attn_bwd_kv.cu, large problems): items given, drawn
-and put in order, one tile and many, offsets in shared memory and in global memory, and what the other kernels take."""
+and put in order, one tile and many, few offsets and many, and what the other kernels take."""
 import pytest
 import torch
 
@@ -16,9 +16,11 @@ pytestmark = pytest.mark.gpu
     (64, 12, 34000, [128] * 40 + [1] * 128 + [256, 384]),   # boundaries on the tiles; items of one tile
     (32, 16, 34000, [49] * 511),                            # the first item by one warp: the most segments
     (64, 12, 34000, [49] * 512),                             # and one more
-    (32, 16, 34000, [5] * 2047),                             # staged offsets: the most
-    (64, 8, 80000, [5] * 2048 + [300] * 30),                # and one more
-    (32, 4, 140000, [3] * 40001),                           # offsets in global memory, many row tiles
+    (32, 16, 34000, [5] * 2047),                             # offsets in the least shared memory that is asked for
+    (64, 8, 80000, [5] * 2048 + [300] * 30),                # and more
+    (64, 4, 100000, [8] * 12287),                            # staged offsets: the most
+    (32, 4, 100000, [8] * 12288),                            # and one more: the other kernels
+    (32, 4, 140000, [3] * 40001),                           # offsets in global memory: the other kernels, many row tiles
     (64, 2, 80000, [300, 700] * 75 + [8]),                  # 512 drawn row tiles: the most that are put in order
     (64, 2, 80000, [300, 700] * 75 + [9]),                  # and one more
     (64, 2, 300, [100, 77, 123]),                           # too small: the other kernels
